@@ -334,7 +334,11 @@ bm_status upload_tables(PlanDev& P) {
   if (P.dtab[di]) { cudaFree(P.dtab[di]); P.dtab[di] = nullptr; }
   if (!img.empty()) {
     BM_CUDA(cudaMalloc(&P.dtab[di], img.size()));
+    // a copy from pageable memory may return before it has landed, and the
+    // first kernels that read the tables run on streams that do not wait for
+    // the default stream
     BM_CUDA(cudaMemcpy(P.dtab[di], img.data(), img.size(), cudaMemcpyHostToDevice));
+    BM_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
   }
   P.dev[di] = dev;
   auto& G = glevels<T>(P);
