@@ -531,8 +531,8 @@ Reblock reblock_of(const PlanHost& h, bool coarse) {
 }
 
 // cudaFuncAttributeMaxDynamicSharedMemorySize set once per device for a kernel.
-std::atomic<unsigned> g_cb_attr{0}, g_dt_attr{0}, g_dec_attr{0}, g_encw_attr{0}, g_encc_attr{0}, g_cbb_attr{0};
-std::atomic<unsigned> g_enc1_attr{0}, g_enc3_attr{0};
+std::atomic<unsigned> g_cb_attr{0}, g_dt_attr{0}, g_dec_attr{0}, g_cbb_attr{0};
+std::atomic<unsigned> g_enc0_attr{0}, g_enc2_attr{0}, g_enc3_attr{0}, g_encc0_attr{0}, g_encc2_attr{0};
 template <class F>
 cudaError_t set_smem_once(F* fn, int bytes, std::atomic<unsigned>& done) {
   int dev = 0;
@@ -545,25 +545,32 @@ cudaError_t set_smem_once(F* fn, int bytes, std::atomic<unsigned>& done) {
   return e;
 }
 
-// Preferred shared-memory carveout 0 (the most L1) for a kernel that keeps
-// a table in L1 rather than in shared memory, once per device.
-template <class F>
-cudaError_t prefer_l1_once(F* fn, std::atomic<unsigned>& done) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  const unsigned bit = 1u << (dev & 31);
-  if (done.load() & bit) return cudaSuccess;
-  e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
-  if (e == cudaSuccess) done.fetch_or(bit);
-  return e;
-}
-
 int grid_for(int64_t work, int threads, int per_sm = 8) {
   int64_t g = (work + threads - 1) / threads;
   const int64_t cap = (int64_t)num_sms() * per_sm;
   if (g > cap) g = cap;
   return (int)std::max<int64_t>(g, 1);
+}
+
+// The encoder over caller-supplied symbols: the window of a dictionary of at
+// most kEncWinSmall symbols unless a code is too long for its entries, else
+// the split table (the variant that does not apply returns at once).
+cudaError_t launch_encode_clamped(FusedEncodeArgs a, unsigned long long nch, cudaStream_t s) {
+  cudaError_t e = cudaSuccess;
+  if (a.dict <= kEncWinSmall) {
+    a.win = kEncWinSmall;
+    const size_t m0 = enc_smem<0>(8, kEncWinSmall, a.dict);
+    if ((e = set_smem_once(encode_fused_kernel<8, true, 0>, (int)m0, g_encc0_attr)) != cudaSuccess) return e;
+    encode_fused_kernel<8, true, 0><<<grid_for((int64_t)nch * 32, 256, 4), 256, m0, s>>>(a);
+    g_launches.fetch_add(1);
+  }
+  if ((e = set_smem_once(encode_fused_kernel<kEncWarps, true, 2>, (int)enc_smem<2>(kEncWarps, 0, kMaxDict),
+                         g_encc2_attr)) != cudaSuccess)
+    return e;
+  encode_fused_kernel<kEncWarps, true, 2>
+      <<<grid_for((int64_t)nch * 32, kEncWarps * 32, 1), kEncWarps * 32, enc_smem<2>(kEncWarps, 0, a.dict), s>>>(a);
+  g_launches.fetch_add(1);
+  return cudaGetLastError();
 }
 
 // CTAs of the decoder an SM holds (its lookup table, threads and registers),
@@ -1496,7 +1503,7 @@ bm_status compress_t(const T* field, const int64_t* shape, const Params& prm, do
   Carver probe;
   carve_all(probe, nullptr);
   probe.take<Scalars>(1); probe.take<unsigned>(dict); probe.take<uint8_t>(dict); probe.take<unsigned>(dict);
-  probe.take<unsigned char>(cb_big_bytes()); probe.take<unsigned>(dict);
+  probe.take<unsigned char>(cb_big_bytes()); probe.take<unsigned>(dict); probe.take<unsigned>(kMaxLen + 1);
   probe.take<double>(L.nq); probe.take<T>(L.nq); probe.take<double>(ntiers); probe.take<uint8_t>(h.nblocks_all);
   probe.take<uint16_t>((size_t)h.n_coeffs); probe.take<int32_t>((size_t)h.n_coeffs);
   probe.take<unsigned char>(256 + 16ull * L.nch);
@@ -1521,6 +1528,7 @@ bm_status compress_t(const T* field, const int64_t* shape, const Params& prm, do
   unsigned* codes = cv.take<unsigned>(dict);
   unsigned char* cb_big = cv.take<unsigned char>(cb_big_bytes());
   unsigned* packed = cv.take<unsigned>(dict);
+  unsigned* first_code = cv.take<unsigned>(kMaxLen + 1);
   double* qd = cv.take<double>(L.nq);
   T* rq = cv.take<T>(L.nq);
   double* dtiers = cv.take<double>(ntiers);
@@ -1640,7 +1648,7 @@ bm_status compress_t(const T* field, const int64_t* shape, const Params& prm, do
   {
     Stage st("huffman_codebook");
     CodebookArgs ca{hist, dict, lens, codes, prefix_fits ? out : nullptr, L.off_codebook, cap, sc, 1, L.nch,
-                    raw_total, cb_big, packed};
+                    raw_total, cb_big, packed, first_code};
     if (phase == kFinishA) {  // the batch builds every item's codebook in one launch
       bs->cb = ca;
       bs->cb_ready = true;
@@ -1675,30 +1683,29 @@ bm_status compress_t(const T* field, const int64_t* shape, const Params& prm, do
     Stage st("huffman_encode");
     FusedEncodeArgs ea{};
     ea.sym = sym; ea.esc = esc; ea.n = (unsigned long long)h.n_coeffs; ea.chunk = prm.chunk;
-    ea.lens = lens; ea.codes = codes; ea.packed = packed; ea.dict = dict; ea.nch = L.nch;
+    ea.lens = lens; ea.codes = codes; ea.packed = packed; ea.first_code = first_code; ea.dict = dict; ea.nch = L.nch;
     ea.ticket = reinterpret_cast<unsigned*>(tickets); ea.st = lb_status;
     ea.chunk_words = reinterpret_cast<unsigned*>(out + L.off_chunks);
     ea.splits = reinterpret_cast<uint16_t*>(out + L.off_splits);
     ea.out = out; ea.capacity = cap; ea.sc = sc;
-    // the codebook picked one of four variants (the others return at once):
-    // every symbol in a small window, four CTAs of eight warps per SM; every
-    // symbol in the large window, or the large window with global look-ups
-    // beside it, one CTA of kEncWarps warps per SM; the global table, four
-    // CTAs of eight warps per SM
+    // the codebook picked one of three variants (the others return at once):
+    // every symbol in a small window, two CTAs of eight warps per SM; every
+    // symbol in the large window, or the split table of the whole dictionary,
+    // one CTA of kEncWarps warps per SM
     constexpr int ew = kEncWarps * 32;
-    const int eg = grid_for((int64_t)L.nch * 32, ew, 32 / kEncWarps);
-    BM_CUDA(set_smem_once(encode_fused_kernel<kEncWarps, false, 3>, (int)enc_smem<0>(kEncWin), g_enc3_attr));
-    BM_CUDA(set_smem_once(encode_fused_kernel<kEncWarps, false, 1>, (int)enc_smem<1>(kEncWin), g_enc1_attr));
-    BM_CUDA(prefer_l1_once(encode_fused_kernel<8, false, 2>, g_encw_attr));
-    FusedEncodeArgs e0 = ea, e1 = ea;
+    const int eg = grid_for((int64_t)L.nch * 32, ew, 1);
+    const size_t m0 = enc_smem<0>(8, kEncWinSmall, dict), m3 = enc_smem<3>(kEncWarps, kEncWin, dict),
+                 m2 = enc_smem<2>(kEncWarps, 0, dict);
+    BM_CUDA(set_smem_once(encode_fused_kernel<8, false, 0>, (int)m0, g_enc0_attr));
+    BM_CUDA(set_smem_once(encode_fused_kernel<kEncWarps, false, 3>, (int)m3, g_enc3_attr));
+    BM_CUDA(set_smem_once(encode_fused_kernel<kEncWarps, false, 2>, (int)enc_smem<2>(kEncWarps, 0, kMaxDict), g_enc2_attr));
+    FusedEncodeArgs e0 = ea, e3 = ea;
     e0.win = kEncWinSmall;
-    e1.win = kEncWin;
-    encode_fused_kernel<8, false, 0>
-        <<<grid_for((int64_t)L.nch * 32, 256, 4), 256, enc_smem<0>(kEncWinSmall), s>>>(e0);
-    encode_fused_kernel<kEncWarps, false, 3><<<eg, ew, enc_smem<0>(kEncWin), s>>>(e1);
-    encode_fused_kernel<kEncWarps, false, 1><<<eg, ew, enc_smem<1>(kEncWin), s>>>(e1);
-    encode_fused_kernel<8, false, 2><<<grid_for((int64_t)L.nch * 32, 256, 4), 256, 0, s>>>(ea);
-    g_launches.fetch_add(4);
+    e3.win = kEncWin;
+    encode_fused_kernel<8, false, 0><<<grid_for((int64_t)L.nch * 32, 256, 4), 256, m0, s>>>(e0);
+    encode_fused_kernel<kEncWarps, false, 3><<<eg, ew, m3, s>>>(e3);
+    encode_fused_kernel<kEncWarps, false, 2><<<eg, ew, m2, s>>>(ea);
+    g_launches.fetch_add(3);
   }
   {
     Stage st("finish");
@@ -3013,7 +3020,7 @@ bm_status bm_huffman_encode(const uint16_t* d_symbols, uint64_t n, int dict_size
   Carver probe;
   probe.take<Scalars>(1); probe.take<unsigned>(dict_size); probe.take<uint8_t>(dict_size);
   probe.take<unsigned>(dict_size); probe.take<unsigned>(nch); probe.take<unsigned char>(256 + 16ull * nch);
-  probe.take<unsigned char>(cb_big_bytes()); probe.take<unsigned>(dict_size);
+  probe.take<unsigned char>(cb_big_bytes()); probe.take<unsigned>(dict_size); probe.take<unsigned>(kMaxLen + 1);
   Workspace* ws = nullptr;
   if (bm_status st = get_ws(s, probe.off + 4096, 4096, &ws)) return st;
   Carver cv;
@@ -3025,6 +3032,7 @@ bm_status bm_huffman_encode(const uint16_t* d_symbols, uint64_t n, int dict_size
   unsigned char* tickets = cv.take<unsigned char>(256 + 16ull * nch);
   unsigned char* cb_big = cv.take<unsigned char>(cb_big_bytes());
   unsigned* packed = cv.take<unsigned>(dict_size);
+  unsigned* first_code = cv.take<unsigned>(kMaxLen + 1);
   uint8_t* out = reinterpret_cast<uint8_t*>(d_out);
   BM_CUDA(cudaMemsetAsync(sc, 0, sizeof(Scalars), s));
   BM_CUDA(cudaMemsetAsync(hist, 0, 4ull * dict_size, s));
@@ -3037,7 +3045,7 @@ bm_status bm_huffman_encode(const uint16_t* d_symbols, uint64_t n, int dict_size
   }
   {
     Stage st("huffman_codebook");
-    CodebookArgs ca{hist, dict_size, lens, codes, out, off_cb, out_capacity, sc, 0, nch, ~0ull, cb_big, packed};
+    CodebookArgs ca{hist, dict_size, lens, codes, out, off_cb, out_capacity, sc, 0, nch, ~0ull, cb_big, packed, first_code};
     BM_CUDA(set_smem_once(codebook_kernel, (int)sizeof(CbSmem), g_cb_attr));
     codebook_kernel<<<1, kCbThreads, sizeof(CbSmem), s>>>(ca);
     BM_LAUNCHED();
@@ -3052,17 +3060,11 @@ bm_status bm_huffman_encode(const uint16_t* d_symbols, uint64_t n, int dict_size
     ea.splits = reinterpret_cast<uint16_t*>(out + off_sp);
     ea.capacity = out_capacity; ea.sc = sc;
     ea.packed = packed;
-    ea.win = kEncWinSmall;
-    if (dict_size <= kEncWinSmall) {
-      encode_fused_kernel<8, true, 0>
-          <<<grid_for((int64_t)nch * 32, 256, 4), 256, enc_smem<0>(kEncWinSmall), s>>>(ea);
-    } else {
-      BM_CUDA(prefer_l1_once(encode_fused_kernel<8, true, 2>, g_encc_attr));
-      encode_fused_kernel<8, true, 2><<<grid_for((int64_t)nch * 32, 256, 4), 256, 0, s>>>(ea);
-    }
+    ea.first_code = first_code;
+    BM_CUDA(launch_encode_clamped(ea, nch, s));
     encode_finish_kernel<<<1, 32, 0, s>>>(~0ull, out_capacity, sc);
     zero_tail_kernel<<<1, 32, 0, s>>>(out, sc);
-    g_launches.fetch_add(3);
+    g_launches.fetch_add(2);
     BM_CUDA(cudaGetLastError());
   }
   Scalars* hsc = reinterpret_cast<Scalars*>(ws->h);
@@ -3150,7 +3152,6 @@ namespace {
 constexpr size_t kNoAllocBytes = size_t(1) << 20;     // 1 MiB
 constexpr unsigned long long kNoAllocMaxChunks = 16384;
 constexpr int kNoAllocMaxDict = 8192;  // at most this many present symbols: the codebook stays in shared memory
-static_assert(kNoAllocMaxDict <= kEncWinSmall, "the encoder's window must hold the whole dictionary");
 __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
 
 std::mutex g_noalloc_mu;
@@ -3210,6 +3211,7 @@ extern "C" bm_status bm_huffman_encode_noalloc(const uint16_t* d_symbols, uint64
   unsigned* codes = cv.take<unsigned>(dict_size);
   unsigned char* tickets = cv.take<unsigned char>(256 + 16ull * nch);
   unsigned* packed = cv.take<unsigned>(dict_size);
+  unsigned* first_code = cv.take<unsigned>(kMaxLen + 1);
   if (cv.off > kNoAllocBytes) return fail(BM_ERR_ARG, "request does not fit the static scratch");
   uint8_t* out = reinterpret_cast<uint8_t*>(d_out);
   // the array keeps the previous call's contents: clear what must start at zero
@@ -3218,7 +3220,7 @@ extern "C" bm_status bm_huffman_encode_noalloc(const uint16_t* d_symbols, uint64
   BM_CUDA(cudaMemsetAsync(tickets, 0, 256 + 16ull * nch, s));
   BM_CUDA(cudaMemsetAsync(out, 0, off_cb, s));
   hist_kernel<<<grid_for((int64_t)n, 256, 4), 256, 0, s>>>(d_symbols, n, dict_size, hist, sc);
-  CodebookArgs ca{hist, dict_size, lens, codes, out, off_cb, out_capacity, sc, 0, nch, ~0ull, nullptr, packed};
+  CodebookArgs ca{hist, dict_size, lens, codes, out, off_cb, out_capacity, sc, 0, nch, ~0ull, nullptr, packed, first_code};
   BM_CUDA(set_smem_once(codebook_kernel, (int)sizeof(CbSmem), g_cb_attr));
   codebook_kernel<<<1, kCbThreads, sizeof(CbSmem), s>>>(ca);
   FusedEncodeArgs ea{};
@@ -3229,11 +3231,11 @@ extern "C" bm_status bm_huffman_encode_noalloc(const uint16_t* d_symbols, uint64
   ea.splits = reinterpret_cast<uint16_t*>(out + off_sp);
   ea.capacity = out_capacity; ea.sc = sc;
   ea.packed = packed;
-  ea.win = kEncWinSmall;  // dict_size <= kNoAllocMaxDict = kEncWinSmall: every symbol in the window
-  encode_fused_kernel<8, true, 0><<<grid_for((int64_t)nch * 32, 256, 4), 256, enc_smem<0>(kEncWinSmall), s>>>(ea);
+  ea.first_code = first_code;
+  BM_CUDA(launch_encode_clamped(ea, nch, s));
   encode_finish_kernel<<<1, 32, 0, s>>>(~0ull, out_capacity, sc);
   zero_tail_kernel<<<1, 32, 0, s>>>(out, sc);
-  g_launches.fetch_add(6);
+  g_launches.fetch_add(4);
   BM_CUDA(cudaGetLastError());
   Scalars hsc;
   BM_CUDA(cudaMemcpyAsync(&hsc, sc, sizeof(Scalars), cudaMemcpyDeviceToHost, s));

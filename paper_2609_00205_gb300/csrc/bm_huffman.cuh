@@ -21,47 +21,21 @@ namespace bm {
 
 constexpr int kCbThreads = 1024;
 constexpr int kLutBits = 14;
-// Entries of the code table the encoder keeps in shared memory (a window of
-// the dictionary), 4 bytes each.  When every present symbol lies within
-// kEncWinSmall consecutive symbols, the window holds them all in CTAs of
-// eight warps, four per SM (the rest of the SM's shared memory stays L1 for
-// the symbol loads in flight).  Otherwise the window of the variant with
-// global look-ups beside it has kEncWin entries in one CTA of kEncWarps warps
-// per SM: 57,344 entries (224 KB) serve all but the far tails of a
-// 65,536-symbol dictionary.  The encoder of caller-supplied symbols keeps
-// kEncWinSmall entries.
-#ifndef BM_ENC_WIN
-#define BM_ENC_WIN 57344
-#endif
-constexpr int kEncWin = BM_ENC_WIN;
-constexpr int kEncWarps = kEncWin > 8192 ? 32 : 8;
+// Entries of the code table window the encoder keeps in shared memory (a
+// window of the dictionary, 4 bytes an entry): kEncWinSmall in CTAs of eight
+// warps, two per SM, when every present symbol lies within so many consecutive
+// symbols; kEncWin in one CTA of sixteen warps per SM, beside the warps'
+// staging words, when they lie within that.
+constexpr int kEncWin = 49152;
 constexpr int kEncWinSmall = 8192;
-// The window variant with global look-ups beside it is taken while its
-// window (and the escape symbol's registers) serve at least BM_ENC_WIN_PCT
-// percent of a call's symbols and fewer than BM_ENC_ESC_PCT percent escape.
-// When escapes dominate, the other symbols are the far tails spread over the
-// whole dictionary, and the global-table variant, which leaves all of L1 to
-// the table, was faster on GB300 (513^3 GRF, 1e-5, 56 % escapes: 1.08 against
-// 1.68 ms for the large window); at 1e-4 (no symbol spans fewer than 57,344)
-// the large window took 0.52 ms, against 0.84 for the 8,192-entry one.
-#ifndef BM_ENC_WIN_PCT
-#define BM_ENC_WIN_PCT 50
-#endif
-#ifndef BM_ENC_ESC_PCT
-#define BM_ENC_ESC_PCT 20
-#endif
-// The encoder's table entry of a symbol: its code in the low kPackBits bits
-// and its length above them.  A code longer than kPackBits bits (a few
-// symbols of singleton counts in fields of 10^8 symbols and more) keeps only
-// its length there, and the encoder reads the code from the full code table.
-constexpr unsigned kPackBits = 26;
+constexpr int kEncWarps = 32;
+// The window's entry of a symbol: its code, left-justified, and its length in
+// the low five bits.  Codes longer than kPackLen bits do not fit: a codebook
+// with one (fields beyond about 10^8 symbols) takes the split table.
+constexpr unsigned kPackLen = 27;
 __host__ __device__ constexpr unsigned enc_entry(unsigned code, unsigned len) {
-  return (len <= kPackBits ? code : 0u) | (len << kPackBits);
+  return len >= 1 && len <= kPackLen ? (code << (32 - len)) | len : 0u;
 }
-// Shared memory of the encoder with a window of `win` entries; the variant
-// for wide code distributions keeps no table in shared memory.
-template <int TAB>
-__host__ __device__ constexpr size_t enc_smem(int win = kEncWin) { return TAB == 2 ? 0 : (size_t)win * 4; }
 // Every chunk is split into eight equal runs; the stream stores the bit
 // offsets of runs 1..7 so that eight decoders can work on one chunk.
 constexpr int kSplits = 8;
@@ -440,7 +414,8 @@ struct CodebookArgs {
   unsigned long long nch;        // chunks
   unsigned long long raw_total;  // size of the raw stream (~0: no raw fallback)
   unsigned char* big;            // global scratch for more than kCbSmemSyms present symbols (cb_big_bytes())
-  unsigned* packed;              // [dict] out (nullable): the encoder's entries, enc_entry(code, len)
+  unsigned* packed;              // [dict] out: the encoder's entries, enc_entry(code, len)
+  unsigned* first_code;          // [kMaxLen + 1] out: first code of each length
   int presorted;                 // cb_presort_kernel ran: tables cleared, symbols compacted into the
                                  // global arrays and, above kCbSmemSyms of them, sorted
 };
@@ -521,7 +496,7 @@ struct CbPre {
   unsigned dcnt[kPreCtas * 256];   // per (CTA, digit) keys of the current pass; then per (CTA, length) codes
   unsigned rcnt[kPreCtas];         // run starts of each CTA's segment of compact indices
   unsigned bsum[kPreCtas];         // codebook-section bytes of each CTA's runs
-  unsigned long long bits, all, win;  // sums of f len, f, f served by the encoder's window
+  unsigned long long bits;         // sum of f len
 };
 __host__ __device__ constexpr size_t cb_big_bytes() {
   return (size_t)kMaxDict * (2 + 1 + 4 + 2 + 4 + 2 + 4 + 4 * 2 + 2 + 4 + 2) + 3 * 4 * (size_t)kMaxDict + 16 * 256 +
@@ -887,40 +862,29 @@ __device__ void codebook_lengths(const CodebookArgs& a, CbArrays<IdT> V, int n, 
 // The codebook's decisions (one thread): section sizes and offsets, the
 // encoder's table and window, the lower bound on the stream size and the
 // raw-copy decision.  smin / smax: the smallest and largest present symbol;
-// bits, all, win: sum of f_s len_s, of f_s, and of f_s over the symbols the
-// encoder's centred window (or the escape registers) serves.
+// bits: sum of f_s len_s.
 __device__ inline void codebook_decide(const CodebookArgs& a, unsigned smin, unsigned smax, unsigned long long total,
-                                       int nruns, unsigned max_len, unsigned long long bits, unsigned long long all,
-                                       unsigned long long win, bool fits) {
-  const unsigned wlo_c =
-      a.dict <= kEncWin ? 0u : (unsigned)min(max(a.dict / 2 - kEncWin / 2, 0), a.dict - kEncWin);
+                                       int nruns, unsigned max_len, unsigned long long bits, bool fits) {
   {
     Scalars* sc = a.sc;
     sc->codebook_bytes = total;
     sc->n_runs = (unsigned long long)nruns;
     sc->max_len = max_len;
-    // the encoder's shared-memory window of the code table: every present
-    // symbol when they span at most kEncWinSmall symbols, or at most kEncWin
-    // (a larger window in a larger CTA); else kEncWin entries centred on the dictionary's middle (code 0) while they and the
-    // escape symbol serve at least BM_ENC_WIN_PCT percent of the symbols met
-    // and escapes are fewer than BM_ENC_ESC_PCT percent (the rest looked up
-    // in the global table); else no window (the global-table variant, with
-    // all of L1 for the table)
+    // the encoder's table: a shared-memory window of enc_entry words when every
+    // present symbol lies in kEncWinSmall or in kEncWin consecutive symbols and
+    // no code is too long for an entry, else the split table of the whole
+    // dictionary (three shared-memory look-ups per code instead of one: 0.284
+    // ms for the window at 1e-3 against 0.397 for the split table at 1e-4, 513^3)
     unsigned wn = kEncWin;
-    if (smax - smin < (unsigned)kEncWinSmall) {
+    sc->enc_lo = 0;
+    sc->enc_mode = 2;
+    if (max_len <= kPackLen && smax - smin < (unsigned)kEncWinSmall) {
       sc->enc_lo = a.dict <= kEncWinSmall ? 0u : min(smin, (unsigned)(a.dict - kEncWinSmall));
       sc->enc_mode = 0;
       wn = kEncWinSmall;
-    } else if (smax - smin < (unsigned)kEncWin) {
+    } else if (max_len <= kPackLen && smax - smin < (unsigned)kEncWin) {
       sc->enc_lo = a.dict <= kEncWin ? 0u : min(smin, (unsigned)(a.dict - kEncWin));
       sc->enc_mode = 3;
-    } else if (win * 100ull >= (unsigned long long)BM_ENC_WIN_PCT * all &&
-               (unsigned long long)a.hist[0] * 100ull < (unsigned long long)BM_ENC_ESC_PCT * all) {
-      sc->enc_lo = wlo_c;
-      sc->enc_mode = 1;
-    } else {
-      sc->enc_lo = 0;
-      sc->enc_mode = 2;
     }
     // the window's entries above the largest present symbol are never read
     sc->enc_n = smax >= sc->enc_lo ? min(wn, smax + 1u - sc->enc_lo) : 0u;
@@ -946,12 +910,12 @@ __device__ inline void codebook_decide(const CodebookArgs& a, unsigned smin, uns
 template <typename IdT>
 __device__ void codebook_emit(const CodebookArgs& a, CbArrays<IdT> V, int n, unsigned* scan_tmp, CanonTables* ct) {
   __shared__ unsigned s_total, s_nruns;
-  __shared__ unsigned long long s_bits, s_all, s_win;
-  if (threadIdx.x == 0) { s_bits = 0; s_all = 0; s_win = 0; }
+  __shared__ unsigned long long s_bits;
+  if (threadIdx.x == 0) s_bits = 0;
   // 4. canonical codes (the counting pass in the sort counts' shared memory)
   build_canonical(V.clen, n, V.wcnt, V.canon, ct);
-  const bool pk = a.packed != nullptr;
   const int nc = (int)ct->n;
+  if (threadIdx.x <= kMaxLen) a.first_code[threadIdx.x] = ct->first_code[threadIdx.x];
   for (int i0 = threadIdx.x; i0 < nc; i0 += 8 * blockDim.x) {  // eight loads in flight
     unsigned ci[8], L[8], sy[8];
 #pragma unroll
@@ -971,7 +935,7 @@ __device__ void codebook_emit(const CodebookArgs& a, CbArrays<IdT> V, int n, uns
       if (i < nc) {
         const unsigned c = ct->first_code[L[t]] + (unsigned)(i - (int)ct->first_pos[L[t]]);
         a.codes[sy[t]] = c;
-        if (pk) a.packed[sy[t]] = enc_entry(c, L[t]);
+        a.packed[sy[t]] = enc_entry(c, L[t]);
         a.lens[sy[t]] = (uint8_t)L[t];
       }
     }
@@ -1078,11 +1042,7 @@ __device__ void codebook_emit(const CodebookArgs& a, CbArrays<IdT> V, int n, uns
   // 6. layout of the rest of the stream (escape counts, outlier codes, then
   // the bitstream) and a lower bound on its size: the bitstream holds exactly
   // sum_s f_s len_s bits plus the padding of each chunk to whole words
-  // (and the symbols met that the encoder's window centred on code 0, or the
-  // escape symbol's registers, serve)
-  const unsigned wlo_c =
-      a.dict <= kEncWin ? 0u : (unsigned)min(max(a.dict / 2 - kEncWin / 2, 0), a.dict - kEncWin);
-  unsigned long long my_bits = 0, my_all = 0, my_win = 0;
+  unsigned long long my_bits = 0;
   for (int i0 = threadIdx.x; i0 < n; i0 += 8 * blockDim.x) {  // eight loads in flight
     unsigned sy[8], cl[8], f[8];
 #pragma unroll
@@ -1095,27 +1055,14 @@ __device__ void codebook_emit(const CodebookArgs& a, CbArrays<IdT> V, int n, uns
     for (int t = 0; t < 8; ++t) f[t] = i0 + t * (int)blockDim.x < n ? a.hist[sy[t]] : 0u;
 #pragma unroll
     for (int t = 0; t < 8; ++t)
-      if (i0 + t * (int)blockDim.x < n) {
-        my_bits += (unsigned long long)f[t] * cl[t];
-        my_all += f[t];
-        if (sy[t] - wlo_c < (unsigned)kEncWin || sy[t] == 0u) my_win += f[t];
-      }
+      if (i0 + t * (int)blockDim.x < n) my_bits += (unsigned long long)f[t] * cl[t];
   }
 #pragma unroll
-  for (int o = 16; o; o >>= 1) {
-    my_bits += __shfl_xor_sync(0xffffffffu, my_bits, o);
-    my_all += __shfl_xor_sync(0xffffffffu, my_all, o);
-    my_win += __shfl_xor_sync(0xffffffffu, my_win, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    if (my_bits) atomicAdd(&s_bits, my_bits);
-    if (my_all) atomicAdd(&s_all, my_all);
-    if (my_win) atomicAdd(&s_win, my_win);
-  }
+  for (int o = 16; o; o >>= 1) my_bits += __shfl_xor_sync(0xffffffffu, my_bits, o);
+  if ((threadIdx.x & 31) == 0 && my_bits) atomicAdd(&s_bits, my_bits);
   __syncthreads();
   if (threadIdx.x == 0)
-    codebook_decide(a, n ? V.csym[0] : 0u, n ? V.csym[n - 1] : 0u, total, nruns, ct->max_len, s_bits, s_all, s_win,
-                    fits);
+    codebook_decide(a, n ? V.csym[0] : 0u, n ? V.csym[n - 1] : 0u, total, nruns, ct->max_len, s_bits, fits);
 }
 
 // Multi-CTA start of the codebook for wide code distributions: one
@@ -1173,7 +1120,7 @@ __global__ void __launch_bounds__(kPreThreads) cb_presort_kernel(CodebookArgs a)
   for (int s = c * kPreThreads + threadIdx.x; s < dict; s += G * kPreThreads) {
     a.lens[s] = 0;
     a.codes[s] = 0;
-    if (a.packed) a.packed[s] = 0;
+    a.packed[s] = 0;
   }
   const int dseg = (dict + G - 1) / G, d0 = min(dict, c * dseg), d1 = min(dict, d0 + dseg);
   unsigned my = 0;
@@ -1184,8 +1131,6 @@ __global__ void __launch_bounds__(kPreThreads) cb_presort_kernel(CodebookArgs a)
     if (c == 0) {
       pre->maxk = 0;
       pre->bits = 0;
-      pre->all = 0;
-      pre->win = 0;
     }
   }
   grid.sync();
@@ -1294,7 +1239,7 @@ __global__ void __launch_bounds__(kPreThreads) cb_emit_kernel(CodebookArgs a) {
   __shared__ unsigned s_lc[kMaxLen + 2];
   __shared__ unsigned s_scan[kPreThreads];
   __shared__ unsigned s_red[kPreThreads / 32];
-  __shared__ unsigned long long s_r64[3][kPreThreads / 32];
+  __shared__ unsigned long long s_r64[kPreThreads / 32];
   __shared__ CanonTables s_ct;
   __shared__ unsigned s_prev, s_rbase, s_nruns, s_boff, s_total;
   auto block_excl = [&](unsigned v, unsigned* total) {
@@ -1316,18 +1261,13 @@ __global__ void __launch_bounds__(kPreThreads) cb_emit_kernel(CodebookArgs a) {
   if (tid < kMaxLen + 2) s_lc[tid] = 0u;
   if (tid == 0) s_prev = e0 > 0 ? (unsigned)V.csym[e0 - 1] : 0u;
   __syncthreads();
-  const unsigned wlo_c =
-      a.dict <= kEncWin ? 0u : (unsigned)min(max(a.dict / 2 - kEncWin / 2, 0), a.dict - kEncWin);
-  unsigned long long my_bits = 0, my_all = 0, my_win = 0;
+  unsigned long long my_bits = 0;
   for (int i = tid; i < m; i += kPreThreads) {
     const unsigned L = V.clen[e0 + i], sy = V.csym[e0 + i];
     s_len[i] = (uint8_t)L;
     s_sym[i] = (uint16_t)sy;
     if (L >= 1u && L <= (unsigned)kMaxLen) atomicAdd(&s_lc[L], 1u);
-    const unsigned long long f = a.hist[sy];
-    my_bits += f * L;
-    my_all += f;
-    if (sy - wlo_c < (unsigned)kEncWin || sy == 0u) my_win += f;
+    my_bits += (unsigned long long)a.hist[sy] * L;
   }
   __syncthreads();
   auto is_start = [&](int i) {  // i: index within the segment
@@ -1338,29 +1278,21 @@ __global__ void __launch_bounds__(kPreThreads) cb_emit_kernel(CodebookArgs a) {
 #pragma unroll
   for (int o = 16; o; o >>= 1) {
     my_bits += __shfl_xor_sync(0xffffffffu, my_bits, o);
-    my_all += __shfl_xor_sync(0xffffffffu, my_all, o);
-    my_win += __shfl_xor_sync(0xffffffffu, my_win, o);
     my_st += __shfl_xor_sync(0xffffffffu, my_st, o);
   }
   if (lane == 0) {
-    s_r64[0][wid] = my_bits;
-    s_r64[1][wid] = my_all;
-    s_r64[2][wid] = my_win;
+    s_r64[wid] = my_bits;
     s_red[wid] = my_st;
   }
   __syncthreads();
   if (tid == 0) {
-    unsigned long long b = 0, al = 0, w = 0;
+    unsigned long long b = 0;
     unsigned st = 0;
     for (int k = 0; k < kPreThreads / 32; ++k) {
-      b += s_r64[0][k];
-      al += s_r64[1][k];
-      w += s_r64[2][k];
+      b += s_r64[k];
       st += s_red[k];
     }
     atomicAdd(&pre->bits, b);
-    atomicAdd(&pre->all, al);
-    atomicAdd(&pre->win, w);
     pre->rcnt[c] = st;
   }
   if (tid < kMaxLen + 2) pre->dcnt[c * 256 + tid] = s_lc[tid];
@@ -1409,14 +1341,14 @@ __global__ void __launch_bounds__(kPreThreads) cb_emit_kernel(CodebookArgs a) {
   }
   grid.sync();
   // E2: code tables over the canonical order; section bytes of this CTA's runs
-  const bool pk = a.packed != nullptr;
+  if (c == 0 && tid <= kMaxLen) a.first_code[tid] = s_ct.first_code[tid];
   for (int i = c * kPreThreads + tid; i < n; i += G * kPreThreads) {
     const unsigned ci = V.canon[i];
     const unsigned L = V.clen[ci];
     const unsigned cd = s_ct.first_code[L] + (unsigned)(i - (int)s_ct.first_pos[L]);
     const unsigned sy = V.csym[ci];
     a.codes[sy] = cd;
-    if (pk) a.packed[sy] = enc_entry(cd, L);
+    a.packed[sy] = enc_entry(cd, L);
     a.lens[sy] = (uint8_t)L;
   }
   const int rq = (nruns + G - 1) / G, q0 = min(nruns, c * rq), q1 = min(nruns, q0 + rq);
@@ -1489,7 +1421,7 @@ __global__ void __launch_bounds__(kPreThreads) cb_emit_kernel(CodebookArgs a) {
       for (unsigned long long t = total; t < pad8(total); ++t) a.out[a.off + t] = 0;
   }
   if (c == 0 && tid == 0)
-    codebook_decide(a, V.csym[0], V.csym[n - 1], total, nruns, s_ct.max_len, pre->bits, pre->all, pre->win, fits);
+    codebook_decide(a, V.csym[0], V.csym[n - 1], total, nruns, s_ct.max_len, pre->bits, fits);
 }
 
 // The codebook of one compress call, built by one CTA (the whole block).
@@ -1520,7 +1452,7 @@ __device__ void codebook_block(const CodebookArgs& a) {
   for (int s = threadIdx.x; s < dict; s += blockDim.x) {
     a.lens[s] = 0;
     a.codes[s] = 0;
-    if (a.packed) a.packed[s] = 0;
+    a.packed[s] = 0;
   }
   // present symbols, in symbol order, compacted: warp w walks its contiguous
   // rows of 32 symbols (coalesced loads, eight rows in flight), counting by
@@ -1795,6 +1727,7 @@ struct FusedEncodeArgs {
   const uint8_t* lens;
   const unsigned* codes;
   const unsigned* packed;        // [dict] enc_entry(code, len) per symbol (written by the codebook)
+  const unsigned* first_code;    // [kMaxLen + 1] first code of each length (written by the codebook)
   int dict;
   unsigned long long nch;
   unsigned* ticket;              // zeroed before launch
@@ -1804,7 +1737,7 @@ struct FusedEncodeArgs {
   uint8_t* out;                  // stream base; the codebook kernel put the section offsets in sc
   unsigned long long capacity;
   Scalars* sc;
-  int win;                       // entries of the shared-memory window (dynamic shared memory: 4 per entry)
+  int win;                       // entries of the shared-memory window (MODE 0, 3)
 };
 
 __device__ __forceinline__ unsigned long long ld_volatile_u64(const unsigned long long* p) {
@@ -1813,296 +1746,338 @@ __device__ __forceinline__ unsigned long long ld_volatile_u64(const unsigned lon
   return v;
 }
 
-constexpr int kEncGroups = 8;  // a lane's slice: up to 8 groups of 8 symbols (chunk <= 2048)
+constexpr int kEncSteps = 8;  // 256-symbol steps of the longest chunk (2048 symbols)
+// Warps (and consecutive chunks) of a tile, by the CTA's warps: with one
+// look-back per chunk and 32 warps per SM a warp walked back over thousands
+// of unfinished predecessors (half of the kernel's instructions); larger
+// tiles wait longer at their barriers.  At 513^3, 1e-2 / 1e-3 / 1e-4 / 1e-5
+// (the small window, the large one, the split table twice), tiles of one
+// chunk took 0.309 / 0.316 / 0.417 / 0.529 ms, of four 0.271 / 0.284 / 0.397
+// / 0.502, of eight 0.260 / 0.294 / 0.427 / 0.558.
+constexpr int enc_group(int warps) { return warps > 8 ? 4 : 8; }
 
-__device__ __forceinline__ unsigned sym_of(const uint4* q, int i) {
-  const unsigned w = (i & 4) ? ((i & 2) ? q[i >> 3].w : q[i >> 3].z) : ((i & 2) ? q[i >> 3].y : q[i >> 3].x);
-  return (i & 1) ? (w >> 16) : (w & 0xFFFFu);
-}
-
-// The encoder's code table, entries enc_entry(code, len): a window of
-// `wn` entries in shared memory (sc) starting at symbol `lo`, and the
-// whole table in global memory (gp), read through L1; gc holds the full codes
-// of the rare codes longer than kPackBits bits.  The escape symbol 0's code
-// and length are in registers.
+// Tables of the encoder in shared memory, by the kernel's MODE:
+//   0, 3  a window of the dictionary, one enc_entry per symbol (`lo` its first
+//         symbol): every symbol met lies in it and no code is longer than
+//         kPackLen bits;
+//   2     the whole dictionary split into the symbol's rank among the codes of
+//         its length (u16, `low`) and the length (u8, `len`): any code is
+//         first_code[len] + rank, with the left-justified first codes in `fc`.
+template <int MODE, bool CLAMP>
 struct EncTab {
-  const unsigned* sc;
-  unsigned lo, wn;  // first symbol and entries of the window
-  const unsigned* gc;
-  const unsigned* gp;
-  unsigned c0, l0;  // code and length of symbol 0
+  const unsigned* ent;
+  const uint16_t* low;
+  const uint8_t* len;
+  const unsigned* fc;  // [kMaxLen + 1] first codes, left-justified
+  unsigned lo;
+  // What a symbol's look-up keeps in a register: the window's entry, or
+  // rank | len << 16.
+  __device__ __forceinline__ unsigned entry(unsigned s) const {
+    if (MODE == 2) return (unsigned)low[s] | ((unsigned)len[s] << 16);
+    return ent[s - lo];
+  }
+  __device__ __forceinline__ unsigned length(unsigned s) const { return MODE == 2 ? (unsigned)len[s] : ent[s - lo] & 31u; }
+  // Symbol i of a lane's eight.
+  __device__ __forceinline__ static unsigned symbol(const unsigned (&w)[4], int i, unsigned dmax) {
+    const unsigned s = (i & 1) ? w[i >> 1] >> 16 : w[i >> 1] & 0xFFFFu;
+    return CLAMP ? min(s, dmax) : s;
+  }
+  __device__ __forceinline__ static unsigned bits(unsigned e) { return MODE == 2 ? e >> 16 : e & 31u; }
+  // The code left-justified in 32 bits.
+  __device__ __forceinline__ unsigned code(unsigned e, unsigned L) const {
+    if (MODE == 2) return fc[L] + ((e & 0xFFFFu) << (32u - L));
+    return e & ~31u;
+  }
 };
+// Shared memory of the encoder: the table, then a step's packed words for
+// each warp (256 symbols of at most 32 bits from any bit of the first word on).
+constexpr int kEncStage = 260;
+template <int MODE>
+__host__ __device__ constexpr size_t enc_table_bytes(int win, int dict) {
+  return MODE == 2 ? (size_t)(dict + 7) / 8 * 8 * 3 + 4 * (kMaxLen + 4) : 4 * (size_t)win;
+}
+template <int MODE>
+__host__ __device__ constexpr size_t enc_smem(int warps, int win, int dict) {
+  return enc_table_bytes<MODE>(win, dict) + (size_t)warps * kEncStage * 4;
+}
+static_assert(enc_smem<3>(kEncWarps, kEncWin, 0) <= 227 * 1024 && enc_smem<2>(kEncWarps, 0, kMaxDict) <= 227 * 1024,
+              "encoder shared memory");
 
-// A global load issued only where `pred` holds (a predicated instruction,
-// not a branch: the warp does not diverge); v keeps its value elsewhere.
-__device__ __forceinline__ unsigned ld_nc_if(const unsigned* p, bool pred, unsigned v) {
-  asm("{\n .reg .pred q;\n setp.ne.u32 q, %2, 0;\n @q ld.global.nc.u32 %0, [%1];\n}\n"
-      : "+r"(v)
-      : "l"(p), "r"((unsigned)pred));
-  return v;
-}
-// Table of a lookup: TAB 0 = the shared-memory window only (it holds every
-// symbol met), 1 = the window with the global table for symbols outside it,
-// 2 = the global table only.
-template <int TAB>
-__device__ __forceinline__ unsigned entry_of(const EncTab& t, unsigned s) {
-  if (TAB == 0) return t.sc[s - t.lo];
-  if (TAB == 1) {  // the window's entry, or (rare) the global table's by a predicated load
-    const unsigned k = s - t.lo;
-    const bool in = k < t.wn;
-    const unsigned ew = t.sc[in ? k : 0u];
-    const unsigned eg = ld_nc_if(t.gp + s, !in && s != 0u, enc_entry(t.c0, t.l0));
-    return in ? ew : eg;
-  }
-  return s == 0u ? enc_entry(t.c0, t.l0) : __ldg(t.gp + s);
-}
-template <int TAB>
-__device__ __forceinline__ void code_of(const EncTab& t, unsigned s, unsigned& c, unsigned& L) {
-  const unsigned e = entry_of<TAB>(t, s);
-  c = e & ((1u << kPackBits) - 1u);
-  L = e >> kPackBits;
-  if (L > kPackBits) c = s == 0u ? t.c0 : __ldg(t.gc + s);  // a long code (rare)
-}
-// Without long codes in the warp's slices: the entry alone.
-template <int TAB>
-__device__ __forceinline__ void code_of_short(const EncTab& t, unsigned s, unsigned& c, unsigned& L) {
-  const unsigned e = entry_of<TAB>(t, s);
-  c = e & ((1u << kPackBits) - 1u);
-  L = e >> kPackBits;
-}
-template <int TAB>
-__device__ __forceinline__ unsigned len_of(const EncTab& t, unsigned s) {
-  return entry_of<TAB>(t, s) >> kPackBits;
-}
-// An entry at or above this one has a code longer than kPackBits bits.
-constexpr unsigned kLongEntry = (kPackBits + 1u) << kPackBits;
-
-// Symbols of a slice, streamed past L1 (the global code table of the GLOB
-// variant keeps L1 to itself).
-__device__ __forceinline__ uint4 ld_stream(const uint4* p) {
-  uint4 v;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
-               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
-  return v;
-}
-
-// Bits, escape mask and largest table entry of a lane's vector slice (G
-// groups held in registers).  CLAMP: symbols may be out of the dictionary
-// (caller-supplied) and are clamped; the compressor's own symbols are in
-// range by construction.
-template <int TAB, bool CLAMP, int GC>
-__device__ __forceinline__ void slice_bits(const uint4* q, int G, unsigned dmax, const EncTab& tab, unsigned& bits,
-                                           unsigned long long& emask, unsigned& emax) {
-  bits = 0;
-  emax = 0;
-  unsigned nz = 0;
-#pragma unroll
-  for (int i = 0; i < 8 * kEncGroups; ++i) {
-    if ((i >> 3) < (GC ? GC : G)) {
-      const unsigned s = CLAMP ? min(sym_of(q, i), dmax) : sym_of(q, i);
-      const unsigned e = entry_of<TAB>(tab, s);
-      bits += e >> kPackBits;
-      emax = max(emax, e);
-      nz += s == 0;
-    }
-  }
-  emask = 0;
-  if (nz) {  // escapes (symbol 0): their positions, for the outlier codes
-    unsigned em[2] = {0u, 0u};
-#pragma unroll
-    for (int i = 0; i < 8 * kEncGroups; ++i)
-      if ((i >> 3) < (GC ? GC : G)) em[i >> 5] |= (unsigned)(sym_of(q, i) == 0) << (i & 31);
-    emask = ((unsigned long long)em[1] << 32) | em[0];
-  }
-}
-
-// MSB-first packing of a lane's vector slice.  `acc` holds the pending bits in
-// its low `nb` bits (garbage above is shifted out and never stored); every
-// word is stored through `wp` as soon as it fills.  The lane's first word may
-// start with the previous lane's last bits: it is stored with zeros there and
-// the previous lane ORs its bits in afterwards.
-template <int TAB, bool CLAMP, int GC, bool LONG>
-__device__ __forceinline__ void slice_pack(const uint4* q, int G, unsigned dmax, const EncTab& tab, unsigned* wp,
-                                           unsigned nb, unsigned long long& acc_out, unsigned& nb_out,
-                                           unsigned*& wp_out) {
-  // acc = hi:lo holds at most 31 pending bits, so a code of up to 32 bits
-  // fits; each shift is one clamped funnel shift (a shift by 32 moves the
-  // whole low word up).  LONG: the warp's slices hold codes longer than
-// kPackBits bits, read from the full code table.
-  unsigned hi = 0, lo = 0;
-#pragma unroll
-  for (int i = 0; i < 8 * kEncGroups; ++i) {
-    if ((i >> 3) < (GC ? GC : G)) {
-      const unsigned s = CLAMP ? min(sym_of(q, i), dmax) : sym_of(q, i);
-      unsigned c, L;
-      if (LONG) code_of<TAB>(tab, s, c, L);
-      else code_of_short<TAB>(tab, s, c, L);
-      hi = __funnelshift_lc(lo, hi, L);
-      lo = __funnelshift_lc(0u, lo, L) | c;
-      nb += L;
-      if (nb >= 32u) {
-        nb -= 32u;
-        *wp++ = __funnelshift_r(lo, hi, nb);
+// Publishes tile c's (words, escapes) aggregate and walks back over its
+// predecessors (a window of 32 per step, one per lane of the calling warp)
+// until one has published an inclusive prefix, then publishes its own.  Every
+// lane gets the words and escapes before the tile; false when the bounded
+// wait ran out.
+__device__ __forceinline__ bool enc_lookback(unsigned long long* st, unsigned long long c, unsigned W, unsigned esc,
+                                             unsigned long long& pw_out, unsigned long long& pe_out) {
+  const int lane = threadIdx.x & 31;
+  unsigned long long pw = 0, pe = 0;
+  int timed_out = 0;
+  if (c == 0) {
+    if (lane == 0) atomicExch(st + 0, pack_status(kFlagIncl, W, esc));
+  } else {
+    if (lane == 0) atomicExch(st + c, pack_status(kFlagAgg, W, esc));
+    long long top = (long long)c - 1;  // highest predecessor not yet summed
+    long spins = 0;
+    while (top >= 0) {
+      const long long pidx = top - lane;
+      const unsigned long long sv = pidx >= 0 ? ld_volatile_u64(st + pidx) : kFlagIncl;  // before chunk 0: prefix 0
+      const unsigned flag = (unsigned)(sv >> 62);
+      // only the lanes up to the first unpublished one can be used
+      const unsigned unpub = __ballot_sync(0xffffffffu, flag == 0);
+      const unsigned incl = __ballot_sync(0xffffffffu, flag == 2);
+      const int first_incl = incl ? __ffs(incl) - 1 : 32;
+      const int first_unpub = unpub ? __ffs(unpub) - 1 : 32;
+      if (first_unpub <= first_incl && first_unpub < 32) {
+        if (first_unpub == 0) {  // nearest predecessor not published yet: wait
+          if (++spins > kSpinLimit) { timed_out = 1; break; }
+          __nanosleep(32);
+          continue;
+        }
       }
+      const int take = min(first_incl + 1, first_unpub);  // lanes [0, take) are summed
+      unsigned long long w = 0, e = 0;
+      if (lane < take && pidx >= 0) { w = (sv >> 31) & kM31; e = sv & kM31; }
+#pragma unroll
+      for (int o = 16; o; o >>= 1) {
+        w += __shfl_xor_sync(0xffffffffu, w, o);
+        e += __shfl_xor_sync(0xffffffffu, e, o);
+      }
+      pw += w;
+      pe += e;
+      if (first_incl < take) break;  // reached an inclusive prefix (or the start)
+      top -= take;
+    }
+    timed_out = __shfl_sync(0xffffffffu, timed_out, 0);
+    if (!timed_out && lane == 0) {
+      __threadfence();
+      atomicExch(st + c, pack_status(kFlagIncl, pw + W, pe + esc));
     }
   }
-  acc_out = ((unsigned long long)hi << 32) | lo;
-  nb_out = nb;
-  wp_out = wp;
+  pw_out = pw;  // every lane holds the same sums
+  pe_out = pe;
+  return !timed_out;
 }
 
-// The instantiation of a slice function picked at run time (full
-// default-size slices or not; for packing, long codes in the warp or not);
-// TAB is the kernel's.
-#define BM_ENC_DISPATCH(FN, ...)                                  \
-  do {                                                            \
-    if (G == kEncGroups) FN<TAB, CLAMP, kEncGroups>(__VA_ARGS__); \
-    else FN<TAB, CLAMP, 0>(__VA_ARGS__);                          \
-  } while (0)
-#define BM_ENC_DISPATCH_PACK(FN, ...)                                                  \
-  do {                                                                                 \
-    if (G == kEncGroups) {                                                             \
-      if (wlong) FN<TAB, CLAMP, kEncGroups, true>(__VA_ARGS__);                        \
-      else FN<TAB, CLAMP, kEncGroups, false>(__VA_ARGS__);                             \
-    } else {                                                                           \
-      if (wlong) FN<TAB, CLAMP, 0, true>(__VA_ARGS__);                                 \
-      else FN<TAB, CLAMP, 0, false>(__VA_ARGS__);                                      \
-    }                                                                                  \
-  } while (0)
+// A shared-memory store where `pred` holds, and an OR into shared memory
+// (predicated instructions: lanes that fill a word at different symbols do
+// not diverge).
+__device__ __forceinline__ void st_shared_if(unsigned addr, unsigned v, bool pred) {
+  asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %2, 0;\n @q st.shared.u32 [%0], %1;\n}\n" ::"r"(addr), "r"(v),
+               "r"((unsigned)pred)
+               : "memory");
+}
+__device__ __forceinline__ void red_shared_or(unsigned addr, unsigned v) {
+  asm volatile("red.shared.or.b32 [%0], %1;\n" ::"r"(addr), "r"(v) : "memory");
+}
+
+// Which of a lane's eight symbols are escapes (symbol 0).
+__device__ __forceinline__ unsigned escape_mask(const unsigned (&w)[4]) {
+  unsigned m = 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    m |= (w[i] & 0xFFFFu) == 0u ? 1u << (2 * i) : 0u;
+    m |= (w[i] >> 16) == 0u ? 2u << (2 * i) : 0u;
+  }
+  return m;
+}
+
+// The outlier codes of a step's escapes (m8: this lane's eight symbols), at
+// stream order positions from ep on; s: the step's first symbol; rank: the
+// escapes of the lanes before, total: of the warp.  Many escapes are copied
+// 32 consecutive symbols at a time (coalesced), few by the lanes that hold
+// them.
+__device__ __forceinline__ void enc_outliers(const int32_t* __restrict__ esc, int32_t* __restrict__ ocode,
+                                             unsigned long long n_out, unsigned m8, unsigned long long s,
+                                             unsigned long long ep, unsigned rank, unsigned total) {
+  const int lane = threadIdx.x & 31;
+  if (total >= 32u) {
+    unsigned x = m8 << (8 * (lane & 3));
+    x |= __shfl_xor_sync(0xffffffffu, x, 1);
+    x |= __shfl_xor_sync(0xffffffffu, x, 2);
+    int32_t v[8];
+    unsigned m[8];
+#pragma unroll
+    for (int g = 0; g < 8; ++g) {  // eight loads in flight
+      m[g] = __shfl_sync(0xffffffffu, x, 4 * g);
+      v[g] = ((m[g] >> lane) & 1u) ? __ldg(esc + s + 32 * g + lane) : 0;
+    }
+#pragma unroll
+    for (int g = 0; g < 8; ++g) {
+      const unsigned long long p = ep + __popc(m[g] & ((1u << lane) - 1u));
+      if (((m[g] >> lane) & 1u) && p < n_out) ocode[p] = v[g];
+      ep += __popc(m[g]);
+    }
+  } else {
+    ep += rank;
+    while (m8) {
+      const int i = __ffs(m8) - 1;
+      m8 &= m8 - 1u;
+      if (ep < n_out) ocode[ep] = __ldg(esc + s + 8 * lane + i);
+      ++ep;
+    }
+  }
+}
 
 // The codebook's choice of table (sc->enc_mode, the kernel's MODE): 0 when
 // every symbol met lies in a window of kEncWinSmall entries, 3 when they all
-// lie in one of kEncWin entries, 1 when that window serves most of them and
-// the global table the rest, 2 (the global table only) otherwise; modes 0 and
-// 3 look up the window alone (TAB 0).  For the compressor's own symbols
-// (CLAMP = false) all four are launched, the ones that do not match returning
-// at once; for caller-supplied symbols the host picks by dictionary size.
-// Warps take chunks in ticket order.  A warp codes its chunk's bit count from
-// the symbols it holds in registers, publishes the chunk's (words, escapes)
-// aggregate, walks back over its predecessors until one has published an
-// inclusive prefix (bounded wait), publishes its own inclusive prefix and then
-// packs its codes at the now known word offset.  Each lane stores its full
-// words; a word shared by two lanes is completed by an atomic OR of the
-// earlier lane's last bits.
+// lie in one of kEncWin entries, and no code is longer than kPackLen bits;
+// 2 (the split table of the whole dictionary) otherwise.  For the
+// compressor's own symbols (CLAMP = false) all three are launched, the ones
+// that do not match returning at once; caller-supplied symbols (clamped to
+// the dictionary) take 0 or 2 by the dictionary's size and the longest code.
+//
+// Groups of warps take tiles of consecutive chunks in ticket order, one chunk
+// per warp, with one look-back per tile.  Chunks of whole 256-symbol steps: in
+// step k lane l holds symbols 256 k + 8 l .. + 7 (one coalesced 16-byte load),
+// so the warp's lanes code one contiguous run of the stream at a time.  The
+// first look-ups give the chunk's bits; after the look-back each step's
+// symbols (from L2) are looked up again, a warp scan of their lengths gives
+// every lane its bit, and the lane's eight codes are packed MSB-first into
+// the warp's words in shared memory: full words are stored, a lane's last
+// bits are ORed into the word a later lane completed, the step's own last
+// bits carry into the next step, and the full words leave with coalesced
+// stores.  Bound by issue (mostly the ALU pipe) and the L1 pipeline: look-ups
+// (about four wavefronts for 32 symbols), word stores and the copy out.  The
+// kernel before it gave a lane 64 consecutive symbols: every word store and
+// symbol load of a warp went to 32 different lines, and the far symbols of a
+// wide distribution came from a table in global memory.  513^3 GRF, 1e-2 /
+// 1e-3 / 1e-4 / 1e-5: 0.33 / 0.377 / 0.53 / 0.95 ms before, 0.26 / 0.284 /
+// 0.397 / 0.502 now.
 template <int WARPS, bool CLAMP, int MODE>
 __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) encode_fused_kernel(FusedEncodeArgs a) {
-  constexpr int TAB = MODE == 3 ? 0 : MODE;
   extern __shared__ __align__(16) unsigned char enc_smem_raw[];
-  const int WN = TAB == 2 ? 0 : a.win;
-  unsigned* ent = reinterpret_cast<unsigned*>(enc_smem_raw);  // [WN] the window's entries
+  constexpr int kEncGroup = enc_group(WARPS), NG = WARPS / kEncGroup;
+  __shared__ unsigned s_tile[NG], s_w[NG][kEncGroup], s_e[NG][kEncGroup], s_ok[NG];
+  __shared__ unsigned long long s_base[NG][2];
   Scalars* sc = a.sc;
   if (sc->skip) return;  // the stream is already known to be a raw copy
-  if (!CLAMP && (unsigned)MODE != sc->enc_mode) return;
-  const unsigned wlo = sc->enc_lo;
-  // the compressor's symbols lie below enc_lo + enc_n: the rest is never read
-  const int nfill = CLAMP ? WN : min(WN, (int)sc->enc_n);
-  for (int i = threadIdx.x; i < nfill; i += blockDim.x) {
-    const unsigned s = wlo + (unsigned)i;
-    ent[i] = s < (unsigned)a.dict ? a.packed[s] : 0u;
+  if (CLAMP) {
+    if ((a.dict <= kEncWinSmall && sc->max_len <= kPackLen) != (MODE == 0)) return;
+  } else if ((unsigned)MODE != sc->enc_mode) {
+    return;
   }
-  const EncTab tab{ent, wlo, (unsigned)WN, a.codes, a.packed, a.codes[0], a.lens[0]};
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  EncTab<MODE, CLAMP> tab{};
+  if (MODE == 2) {
+    const int D = (a.dict + 7) / 8 * 8;
+    uint16_t* low = reinterpret_cast<uint16_t*>(enc_smem_raw);
+    uint8_t* len = enc_smem_raw + 2 * D;
+    unsigned* fc = reinterpret_cast<unsigned*>(enc_smem_raw + 3 * D);
+    for (int i = threadIdx.x; i < a.dict; i += blockDim.x) {
+      const unsigned L = a.lens[i];
+      len[i] = (uint8_t)L;
+      low[i] = (uint16_t)(L ? a.codes[i] - a.first_code[L] : 0u);
+    }
+    if (threadIdx.x <= kMaxLen) fc[threadIdx.x] = threadIdx.x ? a.first_code[threadIdx.x] << (32 - threadIdx.x) : 0u;
+    tab.low = low;
+    tab.len = len;
+    tab.fc = fc;
+  } else {
+    unsigned* ent = reinterpret_cast<unsigned*>(enc_smem_raw);
+    const unsigned wlo = CLAMP ? 0u : sc->enc_lo;
+    // the compressor's symbols lie below enc_lo + enc_n: the rest is never read
+    const int nfill = CLAMP ? min(a.win, a.dict) : min(a.win, (int)sc->enc_n);
+    for (int i = threadIdx.x; i < nfill; i += blockDim.x) {
+      const unsigned s = wlo + (unsigned)i;
+      ent[i] = s < (unsigned)a.dict ? a.packed[s] : 0u;
+    }
+    tab.ent = ent;
+    tab.lo = wlo;
+  }
+  unsigned* const buf =
+      reinterpret_cast<unsigned*>(enc_smem_raw + enc_table_bytes<MODE>(a.win, a.dict)) + warp * kEncStage;
+  const unsigned sbuf = smem_u32(buf);
   __syncthreads();
-  const int lane = threadIdx.x & 31;
   const unsigned dmax = (unsigned)(a.dict - 1);
   const unsigned long long off_bits = sc->off_bits;
   const unsigned long long n_out = sc->n_outliers;
   unsigned* words = reinterpret_cast<unsigned*>(a.out + off_bits);
-  unsigned* chunk_esc = (a.esc && n_out) ? reinterpret_cast<unsigned*>(a.out + sc->off_chunk_esc) : nullptr;
+  const bool has_esc = a.esc && n_out;
+  unsigned* chunk_esc = has_esc ? reinterpret_cast<unsigned*>(a.out + sc->off_chunk_esc) : nullptr;
   int32_t* ocode = reinterpret_cast<int32_t*>(a.out + sc->off_outliers);
   const unsigned long long word_cap = a.capacity > off_bits ? (a.capacity - off_bits) / 4 : 0ull;
   const int per = a.chunk / 32;
-  const int G = per / 8;
+  const int ns = a.chunk / 256;  // steps of a chunk
+  // an eighth of a chunk is 32 ns symbols, 4 ns lanes of the steps; the
+  // reciprocal divides lane indices below 256 exactly
+  const unsigned lpe = 4u * ns, lpe_inv = lpe ? (65536u + lpe - 1u) / lpe : 0u;
+  const bool steps_ok = (a.chunk & 255) == 0 && (reinterpret_cast<uintptr_t>(a.sym) & 15) == 0;
+  const int grp = warp / kEncGroup, gw = warp % kEncGroup;  // tile group, warp of the group
+  const unsigned long long ntiles = (a.nch + kEncGroup - 1) / kEncGroup;
+  auto group_sync = [&] { asm volatile("bar.sync %0, %1;\n" ::"r"(grp + 1), "n"(kEncGroup * 32) : "memory"); };
   while (true) {
-    unsigned long long c = 0;
-    if (lane == 0) c = atomicAdd(a.ticket, 1u);
-    c = __shfl_sync(0xffffffffu, c, 0);
-    if (c >= a.nch) break;
-    const unsigned long long cb = c * (unsigned long long)a.chunk;
+    if (gw == 0 && lane == 0) s_tile[grp] = atomicAdd(a.ticket, 1u);
+    group_sync();
+    const unsigned long long tile = s_tile[grp];
+    if (tile >= ntiles) break;
+    const unsigned long long c = tile * kEncGroup + gw;  // past the last chunk: no symbols
+    const unsigned long long cb = min(a.n, c * (unsigned long long)a.chunk);
     const unsigned long long ce = min(a.n, cb + (unsigned long long)a.chunk);
-    const unsigned long long s0 = min(ce, cb + (unsigned long long)lane * per);
-    const unsigned long long s1 = min(ce, s0 + per);
+    const bool steps = steps_ok && ce - cb == (unsigned long long)a.chunk;
+    // first look-ups: bits and escapes of the chunk
+    unsigned xb = 0, xe = 0, bits = 0, nesc = 0;  // other chunks: a slice per lane
+    const unsigned long long s0 = min(ce, cb + (unsigned long long)lane * per), s1 = min(ce, s0 + per);
     const int cnt = (int)(s1 - s0);
-    // vector slices: whole groups of 8 symbols, 16-byte aligned, every lane
-    // full with at least 32 symbols (so at least 32 bits: a word never has
-    // more than two owners)
-    const bool warp_vec = __all_sync(0xffffffffu, (per & 7) == 0 && per >= 32 && cnt == per && (s0 & 7ull) == 0 &&
-                                                      (reinterpret_cast<uintptr_t>(a.sym) & 15) == 0);
-    uint4 q[kEncGroups];
-    // pass 1: bits and escapes of the slice
-    unsigned bits = 0, nesc = 0, emax = 0;
-    unsigned long long emask = 0;
-    if (warp_vec) {
-      const uint4* p = reinterpret_cast<const uint4*>(a.sym + s0);
+    unsigned tot_bits, tot_esc;
+    if (steps) {
+      const uint4* p = reinterpret_cast<const uint4*>(a.sym + cb) + lane;
+      uint4 q[kEncSteps];
 #pragma unroll
-      for (int g = 0; g < kEncGroups; ++g)
-        q[g] = g < G ? (TAB == 2 ? ld_stream(p + g) : __ldg(p + g)) : make_uint4(0, 0, 0, 0);
-      // G is 8 at the default chunk of 2048 symbols: a fully unrolled slice
-      BM_ENC_DISPATCH(slice_bits, q, G, dmax, tab, bits, emask, emax);
-      nesc = __popcll(emask);
+      for (int k = 0; k < kEncSteps; ++k) q[k] = k < ns ? __ldg(p + 32 * k) : make_uint4(0, 0, 0, 0);
+      unsigned sum = 0;  // bits | escapes << 17
+#pragma unroll
+      for (int k = 0; k < kEncSteps; ++k) {
+        if (k < ns) {
+          const unsigned w[4] = {q[k].x, q[k].y, q[k].z, q[k].w};
+#pragma unroll
+          for (int i = 0; i < 8; ++i) sum += tab.length(tab.symbol(w, i, dmax));
+          if (has_esc) sum += (unsigned)__popc(escape_mask(w)) << 17;
+        }
+      }
+      sum = __reduce_add_sync(0xffffffffu, sum);
+      tot_bits = sum & 0x1FFFFu;  // at most 2048 codes of 32 bits
+      tot_esc = sum >> 17;
     } else {
       for (int t = 0; t < cnt; ++t) {
         const unsigned s = CLAMP ? min((unsigned)a.sym[s0 + t], dmax) : (unsigned)a.sym[s0 + t];
-        bits += len_of<TAB>(tab, s);
+        bits += tab.bits(tab.entry(s));
         nesc += s == 0;
       }
-    }
-    if (!a.esc) nesc = 0;
-    unsigned xb = bits, xe = nesc;
+      if (!a.esc) nesc = 0;
+      xb = bits;
+      xe = nesc;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned yb = __shfl_up_sync(0xffffffffu, xb, o);
-      const unsigned ye = __shfl_up_sync(0xffffffffu, xe, o);
-      if (lane >= o) { xb += yb; xe += ye; }
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned yb = __shfl_up_sync(0xffffffffu, xb, o);
+        const unsigned ye = __shfl_up_sync(0xffffffffu, xe, o);
+        if (lane >= o) { xb += yb; xe += ye; }
+      }
+      tot_bits = __shfl_sync(0xffffffffu, xb, 31);
+      tot_esc = __shfl_sync(0xffffffffu, xe, 31);
     }
-    const unsigned tot_bits = __shfl_sync(0xffffffffu, xb, 31);
-    const unsigned tot_esc = __shfl_sync(0xffffffffu, xe, 31);
     const unsigned W = (tot_bits + 31u) >> 5;
-    // publish the aggregate, then look back (a window of 32 predecessors per
-    // step, one per lane) until an inclusive prefix is found
-    unsigned long long pw = 0, pe = 0;
-    int timed_out = 0;
-    if (c == 0) {
-      if (lane == 0) atomicExch(a.st + 0, pack_status(kFlagIncl, W, tot_esc));
-    } else {
-      if (lane == 0) atomicExch(a.st + c, pack_status(kFlagAgg, W, tot_esc));
-      long long top = (long long)c - 1;  // highest predecessor not yet summed
-      long spins = 0;
-      while (top >= 0) {
-        const long long pidx = top - lane;
-        const unsigned long long sv = pidx >= 0 ? ld_volatile_u64(a.st + pidx) : kFlagIncl;  // before chunk 0: prefix 0
-        const unsigned flag = (unsigned)(sv >> 62);
-        // only the lanes up to the first unpublished one can be used
-        const unsigned unpub = __ballot_sync(0xffffffffu, flag == 0);
-        const unsigned incl = __ballot_sync(0xffffffffu, flag == 2);
-        const int first_incl = incl ? __ffs(incl) - 1 : 32;
-        const int first_unpub = unpub ? __ffs(unpub) - 1 : 32;
-        if (first_unpub <= first_incl && first_unpub < 32) {
-          if (first_unpub == 0) {  // nearest predecessor not published yet: wait
-            if (++spins > kSpinLimit) { timed_out = 1; break; }
-            __nanosleep(32);
-            continue;
-          }
-        }
-        const int take = min(first_incl + 1, first_unpub);  // lanes [0, take) are summed
-        unsigned long long w = 0, e = 0;
-        if (lane < take && pidx >= 0) { w = (sv >> 31) & kM31; e = sv & kM31; }
-#pragma unroll
-        for (int o = 16; o; o >>= 1) {
-          w += __shfl_xor_sync(0xffffffffu, w, o);
-          e += __shfl_xor_sync(0xffffffffu, e, o);
-        }
-        pw += w;
-        pe += e;
-        if (first_incl < take) break;  // reached an inclusive prefix (or the start)
-        top -= take;
-      }
-      timed_out = __shfl_sync(0xffffffffu, timed_out, 0);
-      if (!timed_out && lane == 0) {
-        __threadfence();
-        atomicExch(a.st + c, pack_status(kFlagIncl, pw + W, pe + tot_esc));
+    if (lane == 0) {
+      s_w[grp][gw] = W;
+      s_e[grp][gw] = tot_esc;
+    }
+    group_sync();
+    if (gw == 0) {
+      unsigned long long bw, be;
+      const unsigned tw = __reduce_add_sync(0xffffffffu, lane < kEncGroup ? s_w[grp][lane] : 0u);
+      const unsigned te = __reduce_add_sync(0xffffffffu, lane < kEncGroup ? s_e[grp][lane] : 0u);
+      const bool ok = enc_lookback(a.st, tile, tw, te, bw, be);
+      if (lane == 0) {
+        s_base[grp][0] = bw;
+        s_base[grp][1] = be;
+        s_ok[grp] = ok;
       }
     }
-    if (lane == 0) {
+    group_sync();
+    const unsigned long long pw = s_base[grp][0] + __reduce_add_sync(0xffffffffu, lane < gw ? s_w[grp][lane] : 0u);
+    unsigned long long pe = s_base[grp][1] + __reduce_add_sync(0xffffffffu, lane < gw ? s_e[grp][lane] : 0u);
+    const bool ok = s_ok[grp];
+    if (lane == 0 && c < a.nch) {
       a.chunk_words[c] = W;
       if (chunk_esc) chunk_esc[c] = tot_esc;
       if (c == a.nch - 1) {
@@ -2110,112 +2085,112 @@ __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) encode_fused_kernel(Fu
         sc->esc_seen = pe + tot_esc;
       }
     }
-    timed_out = __shfl_sync(0xffffffffu, timed_out, 0);
-    if (timed_out) {
+    if (!ok) {
       if (lane == 0) atomicOr(&sc->status, ST_TIMEOUT | ST_RAW);
       break;
     }
-    pw = __shfl_sync(0xffffffffu, pw, 0);
-    pe = __shfl_sync(0xffffffffu, pe, 0);
+    if (c >= a.nch) continue;
     if (pw + W > word_cap) {  // the stream would not fit: it becomes a raw copy
       if (lane == 0) atomicOr(&sc->status, ST_RAW);
       continue;
     }
-    // outlier codes of the slice, in stream order
-    unsigned long long epos = pe + (xe - nesc);
-    if (a.esc && warp_vec && (per & 31) == 0 && tot_esc * 8u >= (unsigned)a.chunk) {
-      // many escapes: the warp copies them together, 32 consecutive symbols of
-      // one lane's slice at a time (that lane's escape mask, broadcast), so
-      // the loads of the escaped codes and the stores of the outliers are
-      // coalesced rather than one line per lane
-      unsigned long long ep = pe;
-      for (int l = 0; l < 32; ++l) {
-        const unsigned long long ml = __shfl_sync(0xffffffffu, emask, l);
-        const unsigned long long sl = cb + (unsigned long long)l * per;
+    unsigned* const gw = words + pw;
+    if (steps) {
+      const uint4* p = reinterpret_cast<const uint4*>(a.sym + cb) + lane;
+      uint4 qn = __ldg(p);
+      unsigned b0 = 0, carry = 0;  // the step's first bit in the chunk; the bits before it in its word
+#pragma unroll 1
+      for (int k = 0; k < ns; ++k) {
+        const unsigned w[4] = {qn.x, qn.y, qn.z, qn.w};
+        if (k + 1 < ns) qn = __ldg(p + 32 * (k + 1));
+        unsigned e[8], v = 0;  // v: this lane's bits | escapes << 16
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const unsigned m = (unsigned)(ml >> (32 * h));
-          if (32 * h < per && m) {
-            const unsigned r = __popc(m & ((1u << lane) - 1u));
-            if (((m >> lane) & 1u) && ep + r < n_out) ocode[ep + r] = __ldg(a.esc + sl + 32 * h + lane);
-            ep += __popc(m);
-          }
+        for (int i = 0; i < 8; ++i) e[i] = tab.entry(tab.symbol(w, i, dmax));
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v += tab.bits(e[i]);
+        unsigned m8 = 0;
+        if (has_esc) {
+          m8 = escape_mask(w);
+          v += (unsigned)__popc(m8) << 16;
         }
+        unsigned x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+          if (lane >= o) x += y;
+        }
+        const unsigned tot = __shfl_sync(0xffffffffu, x, 31);
+        x -= v;
+        const unsigned start = b0 + (x & 0xFFFFu);
+        {  // bit offsets of the chunk's eighths 1..7
+          const unsigned g = 32u * k + lane, j = (g * lpe_inv) >> 16;
+          if (j && j * lpe == g) a.splits[c * (kSplits - 1) + j - 1] = (uint16_t)start;
+        }
+        if (has_esc) {
+          const unsigned te = tot >> 16;
+          if (te) enc_outliers(a.esc, ocode, n_out, m8, cb + 256u * k, pe, x >> 16, te);
+          pe += te;
+        }
+        const unsigned w0 = b0 >> 5;
+        unsigned off = start & 31u, cur = lane == 0 ? carry : 0u;
+        unsigned wp = sbuf + 4u * ((start >> 5) - w0);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const unsigned L = tab.bits(e[i]), t = tab.code(e[i], L);
+          cur |= t >> off;
+          const unsigned rest = __funnelshift_r(0u, t, off);  // the code's bits past this word
+          off += L;
+          const bool full = off >= 32u;
+          st_shared_if(wp, cur, full);
+          wp += full ? 4u : 0u;
+          cur = full ? rest : cur;
+          off &= 31u;
+        }
+        // the word of the step's last bits is completed by no lane: the last
+        // lane stores it, every other lane's last bits lie in a stored word
+        if (lane == 31 && off) st_shared_if(wp, cur, true);
+        __syncwarp();
+        if (lane != 31 && off) red_shared_or(wp, cur);
+        __syncwarp();
+        b0 += tot & 0xFFFFu;
+        const unsigned nfull = (b0 >> 5) - w0;
+#pragma unroll 1
+        for (unsigned i = lane; i < nfull; i += 32) gw[w0 + i] = buf[i];
+        carry = (b0 & 31u) ? buf[nfull] : 0u;
+        __syncwarp();
       }
-    } else if (a.esc && nesc) {
-      if (warp_vec) {
-        unsigned long long m = emask;
-        while (m) {
-          int idx[4];
-          int k = 0;
-#pragma unroll
-          for (int t = 0; t < 4; ++t) {
-            idx[t] = m ? __ffsll((long long)m) - 1 : -1;
-            m &= m ? m - 1 : 0ull;
-            k += idx[t] >= 0;
-          }
-          int32_t v[4];
-#pragma unroll
-          for (int t = 0; t < 4; ++t) v[t] = idx[t] >= 0 ? __ldg(a.esc + s0 + idx[t]) : 0;
-#pragma unroll
-          for (int t = 0; t < 4; ++t)
-            if (idx[t] >= 0 && epos + t < n_out) ocode[epos + t] = v[t];
-          epos += k;
-        }
-      } else {
+      if (lane == 0 && (b0 & 31u)) gw[b0 >> 5] = carry;
+    } else {  // zero the chunk's words; words shared by lanes are ORed
+      unsigned long long epos = pe + (xe - nesc);
+      if (a.esc && nesc) {
         for (int t = 0; t < cnt; ++t)
           if (a.sym[s0 + t] == 0) {
             if (epos < n_out) ocode[epos] = a.esc[s0 + t];
             ++epos;
           }
       }
-    }
-    if ((lane & 3) == 0 && lane) a.splits[c * (kSplits - 1) + (lane >> 2) - 1] = (uint16_t)(xb - bits);
-    // pass 2: pack MSB-first
-    const unsigned bit0 = xb - bits;
-    const unsigned long long head_idx = pw + (bit0 >> 5);
-    const bool head_partial = (bit0 & 31u) != 0;
-    if (warp_vec) {
-      unsigned long long acc;
-      unsigned nb;
-      unsigned* wp;
-      unsigned* const w0 = words + head_idx;
-      const unsigned nb0 = bit0 & 31u;
-      const bool wlong = __any_sync(0xffffffffu, emax >= kLongEntry);
-      BM_ENC_DISPATCH_PACK(slice_pack, q, G, dmax, tab, w0, nb0, acc, nb, wp);
-      // every lane holds >= 32 bits, so the word of its last bits is the next
-      // lane's first word (already stored, zeros in these bits); the last
-      // lane's last word is its own
+      if ((lane & 3) == 0 && lane) a.splits[c * (kSplits - 1) + (lane >> 2) - 1] = (uint16_t)(xb - bits);
+      for (unsigned w = lane; w < W; w += 32) gw[w] = 0u;
       __syncwarp();
-      if (nb) {
-        const unsigned tail = (unsigned)(acc << (32 - nb));
-        if (lane == 31) *wp = tail;
-        else atomicOr(wp, tail);
-      }
-    } else {  // a partial chunk: zero its words, shared words are ORed
-      for (unsigned w = lane; w < W; w += 32) words[pw + w] = 0u;
-      __syncwarp();
-      unsigned long long acc = 0, widx = head_idx;
-      unsigned nb = bit0 & 31u, head = 0;
-      bool pending_head = head_partial;
+      const unsigned bit0 = xb - bits;
+      unsigned off = bit0 & 31u, cur = 0;
+      unsigned* wp = gw + (bit0 >> 5);
+      bool head = off != 0u;  // the first word holds other lanes' bits
       for (int t = 0; t < cnt; ++t) {
         const unsigned s = CLAMP ? min((unsigned)a.sym[s0 + t], dmax) : (unsigned)a.sym[s0 + t];
-        unsigned c, L;
-        code_of<TAB>(tab, s, c, L);
-        acc = (acc << L) | c;
-        nb += L;
-        if (nb >= 32u) {
-          nb -= 32u;
-          const unsigned word = (unsigned)(acc >> nb);
-          if (pending_head) head = word;
-          else words[widx] = word;
-          pending_head = false;
-          ++widx;
+        const unsigned ent = tab.entry(s), L = tab.bits(ent), tc = tab.code(ent, L);
+        cur |= tc >> off;
+        off += L;
+        if (off >= 32u) {
+          off -= 32u;
+          if (head) atomicOr(wp, cur);
+          else *wp = cur;
+          head = false;
+          ++wp;
+          cur = __funnelshift_lc(0u, tc, L - off);
         }
       }
-      __syncwarp();
-      if (head_partial && !pending_head) atomicOr(words + head_idx, head);
-      if (nb) atomicOr(words + widx, (unsigned)(acc << (32 - nb)));
+      if (off) atomicOr(wp, cur);
     }
   }
 }
@@ -2514,6 +2489,13 @@ __global__ void __launch_bounds__(kDecThreads) decode_kernel(DecodeArgs a) {
     const unsigned long long used = b0 + (unsigned long long)nwords * 32ull - (unsigned long long)skip - nbits;
     if (bad || (k < kSplits - 1 ? used != b1 : used > b1)) atomicOr(&a.sc->status, ST_CORRUPT);
   }
+}
+
+constexpr int kEncGroups = 8;  // a lane's slice: up to 8 groups of 8 symbols (chunk <= 2048)
+
+__device__ __forceinline__ unsigned sym_of(const uint4* q, int i) {
+  const unsigned w = (i & 4) ? ((i & 2) ? q[i >> 3].w : q[i >> 3].z) : ((i & 2) ? q[i >> 3].y : q[i >> 3].x);
+  return (i & 1) ? (w >> 16) : (w & 0xFFFFu);
 }
 
 // Escaped symbols (symbol 0) take the outlier codes in stream order: one

@@ -1,0 +1,51 @@
+"""The Huffman encoder at the edges of its tiles: chunk sizes of whole and
+partial 256-symbol steps, symbol counts around a tile of chunks, each of its
+tables (small window, split table of the whole dictionary, codes too long for
+a window entry); every section must be the oracle's byte for byte."""
+import numpy as np
+import pytest
+import torch
+
+import fields
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+def _check(sym, dict_size, chunk):
+    import paper_2609_00205_gb300 as bm
+
+    so, mo = oracle.huffman_encode(sym, dict_size, chunk)
+    sg, mg = bm.huffman_encode(torch.from_numpy(sym.view(np.int16)).to("cuda"), dict_size, chunk)
+    assert mg == mo
+    np.testing.assert_array_equal(sg.cpu().numpy(), so)
+    back = bm.huffman_decode(sg, mg, sym.size, dict_size, chunk)
+    np.testing.assert_array_equal(back.cpu().numpy().view(np.uint16), sym)
+
+
+@pytest.mark.parametrize("dict_size", [8192, 65536])
+@pytest.mark.parametrize("chunk", [64, 96, 256, 512, 768, 1280, 1792, 2016, 2048])
+def test_chunk_sizes(chunk, dict_size):
+    sym = fields.laplace_symbols(9 * chunk + 37, dict_size // 2, dict_size / 20, seed=chunk, escape_rate=0.01)
+    _check(sym, dict_size, chunk)
+
+
+@pytest.mark.parametrize("dict_size,scale", [(4096, 1.0), (65536, 9000.0)])
+@pytest.mark.parametrize("n", [1, 31, 2047, 2048, 2049, 4 * 2048 - 1, 4 * 2048, 8 * 2048, 8 * 2048 + 1,
+                               3 * 8 * 2048 + 5])
+def test_symbol_counts_around_tiles(n, dict_size, scale):
+    _check(fields.laplace_symbols(n, dict_size // 2, scale, seed=n), dict_size, 2048)
+
+
+@pytest.mark.parametrize("dict_size", [128, 16384])
+def test_codes_longer_than_a_window_entry(dict_size):
+    """Fibonacci counts (36 symbols, 39 M in all) give codes of 1 to 35 bits,
+    limited to 32: longer than the 27 bits of a window entry in a dictionary
+    that fits the small window."""
+    f = [1, 1]
+    while len(f) < 36:
+        f.append(f[-1] + f[-2])
+    rng = np.random.default_rng(5)
+    sym = np.repeat(np.arange(3, 3 + len(f)), f).astype(np.uint16)
+    rng.shuffle(sym)
+    _check(sym, dict_size, 2048)
