@@ -531,7 +531,7 @@ Reblock reblock_of(const PlanHost& h, bool coarse) {
 }
 
 // cudaFuncAttributeMaxDynamicSharedMemorySize set once per device for a kernel.
-std::atomic<unsigned> g_cb_attr{0}, g_dt_attr{0}, g_dec_attr{0}, g_cbb_attr{0};
+std::atomic<unsigned> g_cb_attr{0}, g_dt_attr{0}, g_cbb_attr{0};
 std::atomic<unsigned> g_enc0_attr{0}, g_enc2_attr{0}, g_enc3_attr{0}, g_encc0_attr{0}, g_encc2_attr{0};
 template <class F>
 cudaError_t set_smem_once(F* fn, int bytes, std::atomic<unsigned>& done) {
@@ -573,21 +573,23 @@ cudaError_t launch_encode_clamped(FusedEncodeArgs a, unsigned long long nch, cud
   return cudaGetLastError();
 }
 
-// CTAs of the decoder an SM holds (its lookup table, threads and registers),
-// once per device.
-int dec_per_sm() {
-  static std::atomic<int> cached[64];
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev >= 64) return 1;
-  int v = cached[dev].load();
-  if (v <= 0) {
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, decode_kernel, kDecThreads, kDecSmem) != cudaSuccess || v < 1) {
-      cudaGetLastError();
-      v = 1;
-    }
-    cached[dev].store(v);
-  }
-  return v;
+// The decoder: one CTA of kDecThreads threads per SM when there are runs for
+// three quarters of them, else CTAs of kDecThreadsSmall threads over more SMs
+// (65^3, about 1,400 runs: the whole call 250 -> 187 us against 512-thread
+// CTAs on three SMs, with the new window; fewer chains share an SM's pipes).
+template <int NT>
+cudaError_t launch_decode_nt(const DecodeArgs& a, cudaStream_t s) {
+  static std::atomic<unsigned> attr{0};
+  const cudaError_t e = set_smem_once(decode_kernel<NT>, (int)dec_smem(NT, kMaxDict), attr);
+  if (e != cudaSuccess) return e;
+  decode_kernel<NT><<<grid_for((int64_t)(a.nch * kSplits), NT, NT == kDecThreads ? 1 : 2), NT,
+                            dec_smem(NT, a.ncanon), s>>>(a);
+  g_launches.fetch_add(1);
+  return cudaGetLastError();
+}
+cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t s) {
+  if (a.nch * kSplits * 4 >= (unsigned long long)num_sms() * kDecThreads * 3) return launch_decode_nt<kDecThreads>(a, s);
+  return launch_decode_nt<kDecThreadsSmall>(a, s);
 }
 
 // Histogram of symbols [s0, s1) into hist (zeroed by the caller): with
@@ -1856,9 +1858,10 @@ bm_status decode_symbols(const uint8_t* in, const Header& H, Carver& cv, uint16_
     da.n_words = H.n_words; da.word_off = word_off; da.nch = H.n_chunks; da.n = H.n_symbols; da.chunk = H.chunk;
     da.splits = reinterpret_cast<const uint16_t*>(in + H.off_splits);
     da.tab = dt; da.sym = sym; da.sc = sc;
-    BM_CUDA(set_smem_once(decode_kernel, (int)kDecSmem, g_dec_attr));
-    decode_kernel<<<grid_for((int64_t)H.n_chunks * kSplits, kDecThreads, dec_per_sm()), kDecThreads, kDecSmem, s>>>(da);
-    BM_LAUNCHED();
+    // every present symbol takes at least one length byte after its run's header
+    const unsigned long long lb = H.codebook_bytes > 8ull * H.n_runs ? H.codebook_bytes - 8ull * H.n_runs : 0ull;
+    da.ncanon = (unsigned)std::min<unsigned long long>(lb, (unsigned long long)kMaxDict);
+    BM_CUDA(launch_decode(da, s));
     if (stream_mode && H.n_outliers) {
       escape_fixup_kernel<<<grid_for((int64_t)H.n_chunks * 32, 256, 8), 256, 0, s>>>(
           sym, H.n_symbols, H.chunk, H.n_chunks, esc_off, reinterpret_cast<const int32_t*>(in + H.off_outliers),

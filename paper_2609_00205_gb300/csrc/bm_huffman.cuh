@@ -52,15 +52,7 @@ struct CanonTables {
 
 struct DecodeTables {
   CanonTables ct;
-  // sym | len << 16 for codes of <= kLutBits bits; for a prefix of longer
-  // codes, L0 << 16 with L0 > kLutBits the length of the prefix's first code
-  // (kMaxLen + 1: no code has the prefix)
-  alignas(16) unsigned lut[1 << kLutBits];
-  uint16_t canon[kMaxDict];     // symbols in canonical order
-  // construction arrays for more present symbols than shared memory holds
-  uint8_t big_clen[kMaxDict];
-  uint16_t big_csym[kMaxDict];
-  uint16_t big_canon[kMaxDict];
+  alignas(16) uint16_t canon[kMaxDict];  // symbols in canonical order
 };
 
 // ---------------------------------------------------------------------------
@@ -355,7 +347,8 @@ __device__ void build_canonical(const uint8_t* len, int n, unsigned* wcnt, uint1
       if (r0 + t >= rows) break;
       const unsigned L = ll[t];
       const bool ok = L != 0u && L <= (unsigned)kMaxLen;
-      const unsigned m = __match_any_sync(0xffffffffu, ok ? L : 64u + (unsigned)lane);
+      if (!__any_sync(0xffffffffu, ok)) continue;
+      const unsigned m = __match_any_sync(0xffffffffu, ok ? L : 64u);  // few distinct values: match takes a step each
       if (ok && (m & ((1u << lane) - 1u)) == 0u) wcnt[wc_idx(L, wid)] += (unsigned)__popc(m);
       __syncwarp();
     }
@@ -389,7 +382,8 @@ __device__ void build_canonical(const uint8_t* len, int n, unsigned* wcnt, uint1
       const int i = wid * seg + (r0 + t) * 32 + lane;
       const unsigned L = ll[t];
       const bool ok = L != 0u && L <= (unsigned)kMaxLen;
-      const unsigned m = __match_any_sync(0xffffffffu, ok ? L : 64u + (unsigned)lane);
+      if (!__any_sync(0xffffffffu, ok)) continue;
+      const unsigned m = __match_any_sync(0xffffffffu, ok ? L : 64u);
       const unsigned lt = m & ((1u << lane) - 1u);
       const unsigned base = ok ? wcnt[wc_idx(L, wid)] : 0u;
       if (ok) canon[ct->first_pos[L] + base + (unsigned)__popc(lt)] = (uint16_t)i;
@@ -2210,127 +2204,121 @@ __global__ void encode_finish_kernel(unsigned long long raw_total, unsigned long
 // ---------------------------------------------------------------------------
 // Decoding
 // ---------------------------------------------------------------------------
-// Present symbols the decoder-table builder keeps in shared memory; more use
-// the global arrays of DecodeTables.
-constexpr int kDtSmemSyms = 8192;
-
+// Shared memory of the decoder-table builder: the codebook section as it
+// stands in the stream (when it fits), a code length per dictionary symbol
+// and the counting pass's counts.
+constexpr int kDtStage = 128 * 1024;
 struct DtSmem {
-  uint8_t clen[kDtSmemSyms];    // code length of each present symbol (symbol order)
-  uint16_t csym[kDtSmemSyms];   // its symbol
-  uint16_t canon[kDtSmemSyms];  // present-symbol indices in canonical order
-  unsigned key32[kDtSmemSyms];  // the codebook section (when it fits), then counting scratch
-  unsigned scan_tmp[64];
+  unsigned stage[kDtStage / 4];
+  uint8_t len[kMaxDict];
+  unsigned wcnt[(kMaxLen + 1) * 32];
   CanonTables ct;
   unsigned rfirst[512], rcount[512], roff[512];
 };
+static_assert(sizeof(DtSmem) <= 227 * 1024, "decoder tables' shared memory");
 
-// Build decode tables from the stream's codebook runs (one CTA of
-// kCbThreads threads, DtSmem in its dynamic shared memory).  The runs list
-// the present symbols in symbol order: run q's t-th symbol is present symbol
-// (symbols of the runs before q) + t.
+// Canonical order of a stream's codebook (one CTA of kCbThreads threads,
+// DtSmem in its dynamic shared memory): the runs' lengths are spread over
+// the dictionary in shared memory, and one counting pass places every
+// symbol.  Bound by latency: the section's load, the serial walk over the run
+// headers and the counting walk's 64 rows of 32 symbols per warp.  Keeping
+// the lengths of more than 8192 present symbols in global scratch, with a
+// binary search of the runs per length and the look-up table of the decoder
+// filled here too, took 0.129 ms at 513^3, 1e-4 (65,532 present symbols)
+// against 0.042, and 0.091 at 1e-3 (593 runs) against 0.077.
 __device__ __forceinline__ void decode_tables_block(const uint8_t* runs, unsigned long long nbytes,
                                                     unsigned long long n_runs, int dict, DecodeTables* out,
                                                     Scalars* sc, unsigned char* smem_raw) {
   DtSmem& S = *reinterpret_cast<DtSmem*>(smem_raw);
-  __shared__ unsigned s_bad;
-  __shared__ unsigned long long s_kr;
-  __shared__ unsigned s_total, s_n;
-  if (threadIdx.x == 0) { s_bad = 0; s_kr = 0; s_n = 0; }
-  // every present symbol takes at least one length byte after its run's
-  // 8-byte header: this bounds their count and picks the arrays
-  const unsigned long long nbound = nbytes > 8ull * n_runs ? nbytes - 8ull * n_runs : 0ull;
-  const bool small = nbound <= (unsigned long long)kDtSmemSyms;
-  const unsigned cap = small ? (unsigned)kDtSmemSyms : (unsigned)kMaxDict;
-  uint8_t* clen = small ? S.clen : out->big_clen;
-  uint16_t* csym = small ? S.csym : out->big_csym;
-  uint16_t* canon = small ? S.canon : out->big_canon;
-  // the codebook section is walked serially: read it from shared memory when
-  // it fits in the key scratch (free until build_canonical)
+  __shared__ unsigned s_bad, s_long, s_end;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  if (threadIdx.x == 0) s_bad = 0;
+  for (int i = threadIdx.x; i < kMaxDict / 4; i += blockDim.x) reinterpret_cast<unsigned*>(S.len)[i] = 0u;
   const uint8_t* rbase = runs;
-  if (nbytes <= sizeof(S.key32) && (reinterpret_cast<uintptr_t>(runs) & 3) == 0) {
+  if (nbytes <= sizeof(S.stage) && (reinterpret_cast<uintptr_t>(runs) & 3) == 0) {
     const unsigned* src = reinterpret_cast<const unsigned*>(runs);
-    const unsigned nw = (unsigned)(nbytes / 4);
-    for (unsigned i = threadIdx.x; i < nw; i += blockDim.x) S.key32[i] = src[i];
-    uint8_t* kb = reinterpret_cast<uint8_t*>(S.key32);
-    for (unsigned i = 4 * nw + threadIdx.x; i < (unsigned)nbytes; i += blockDim.x) kb[i] = runs[i];
+    const unsigned nwd = (unsigned)(nbytes / 4);
+    for (unsigned i0 = threadIdx.x; i0 < nwd; i0 += 8 * blockDim.x) {  // eight loads in flight
+      unsigned v[8];
+#pragma unroll
+      for (int t = 0; t < 8; ++t) v[t] = i0 + t * blockDim.x < nwd ? src[i0 + t * blockDim.x] : 0u;
+#pragma unroll
+      for (int t = 0; t < 8; ++t)
+        if (i0 + t * blockDim.x < nwd) S.stage[i0 + t * blockDim.x] = v[t];
+    }
+    uint8_t* kb = reinterpret_cast<uint8_t*>(S.stage);
+    for (unsigned i = 4 * nwd + threadIdx.x; i < (unsigned)nbytes; i += blockDim.x) kb[i] = runs[i];
     rbase = kb;
   }
   __syncthreads();
-  // walk the run headers (serial, 512 at a time), then every thread copies
-  // lengths and symbols of the batch (rcount holds each run's first index in
-  // the batch)
+  // walk the run headers (serial, 512 at a time), then spread the batch's
+  // lengths: short runs a warp each, long ones by the whole block
+  constexpr unsigned kLongRun = 1024;
   unsigned long long off = 0;
-  unsigned prev_end = 0;  // runs must be ascending and must not overlap
   for (unsigned long long rb = 0; rb < n_runs; rb += 512) {
     const int nb = (int)min(512ull, n_runs - rb);
-    if (threadIdx.x == 0) {
-      unsigned tot = 0;
-      for (int q = 0; q < nb; ++q) {
-        if (off + 8 > nbytes) { s_bad = 1; break; }
-        const unsigned first = *reinterpret_cast<const unsigned*>(rbase + off);
-        const unsigned cnt = *reinterpret_cast<const unsigned*>(rbase + off + 4);
-        if ((unsigned long long)first + cnt > (unsigned long long)dict || off + 8 + cnt > nbytes ||
-            (rb + q > 0 && first < prev_end) || (unsigned long long)s_n + tot + cnt > cap) {
-          s_bad = 1;
-          break;
-        }
-        S.rfirst[q] = first; S.rcount[q] = tot; S.roff[q] = (unsigned)off;
-        tot += cnt;
-        prev_end = first + cnt;
+    if (threadIdx.x == 0) {  // the chain of headers only: their checks follow in parallel
+      bool ok = true;
+      for (int q = 0; q < nb && ok; ++q) {
+        ok = off + 8 <= nbytes;
+        const unsigned cnt = ok ? *reinterpret_cast<const unsigned*>(rbase + off + 4) : 0u;
+        S.roff[q] = (unsigned)off;
+        ok &= cnt <= (unsigned)dict;
         off += 8ull + ((cnt + 3u) & ~3u);
       }
-      s_total = tot;
+      if (!ok) s_bad = 1;
+      s_long = 0;
     }
     __syncthreads();
     if (s_bad) break;
-    const unsigned tot = s_total, base = s_n;
-    for (unsigned e = threadIdx.x; e < tot; e += blockDim.x) {
-      const int q = upper_bound_u32(S.rcount, 0, nb, e) - 1;
-      const unsigned t = e - S.rcount[q];
-      clen[base + e] = rbase[S.roff[q] + 8 + t];
-      csym[base + e] = (uint16_t)(S.rfirst[q] + t);
+    if (threadIdx.x < (unsigned)nb) {
+      const unsigned o = S.roff[threadIdx.x];
+      const unsigned first = *reinterpret_cast<const unsigned*>(rbase + o);
+      const unsigned cnt = *reinterpret_cast<const unsigned*>(rbase + o + 4);
+      S.rfirst[threadIdx.x] = first;
+      S.rcount[threadIdx.x] = cnt;
+      S.roff[threadIdx.x] = o + 8u;
+      if ((unsigned long long)first + cnt > (unsigned long long)dict || (unsigned long long)o + 8 + cnt > nbytes) s_bad = 1;
+      if (cnt >= kLongRun) s_long = 1;
     }
     __syncthreads();
-    if (threadIdx.x == 0) s_n = base + tot;
+    if (threadIdx.x < (unsigned)nb) {  // ascending, without overlap
+      const unsigned end = threadIdx.x ? S.rfirst[threadIdx.x - 1] + S.rcount[threadIdx.x - 1] : s_end;
+      if ((threadIdx.x || rb) && S.rfirst[threadIdx.x] < end) s_bad = 1;
+    }
+    __syncthreads();
+    if (s_bad) break;
+    if (threadIdx.x == 0) s_end = S.rfirst[nb - 1] + S.rcount[nb - 1];
+    bool bad = false;
+    for (int q = wid; q < nb; q += nw)
+      if (S.rcount[q] < kLongRun)
+        for (unsigned t = lane; t < S.rcount[q]; t += 32) {
+          const uint8_t L = rbase[S.roff[q] + t];
+          bad |= L > kMaxLen;
+          S.len[S.rfirst[q] + t] = L;
+        }
+    for (int q = 0; q < (s_long ? nb : 0); ++q)
+      if (S.rcount[q] >= kLongRun)
+        for (unsigned t = threadIdx.x; t < S.rcount[q]; t += blockDim.x) {
+          const uint8_t L = rbase[S.roff[q] + t];
+          bad |= L > kMaxLen;
+          S.len[S.rfirst[q] + t] = L;
+        }
+    if (bad) s_bad = 1;
     __syncthreads();
   }
-  const int n = (int)s_n;
-  // Kraft sum (exact, in units of 2^-32) and the length bound
-  unsigned long long kr = 0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const unsigned L = clen[i];
-    if (L > (unsigned)kMaxLen) s_bad = 1;
-    else if (L) kr += 1ull << (32 - L);
-  }
-#pragma unroll
-  for (int o = 16; o; o >>= 1) kr += __shfl_xor_sync(0xffffffffu, kr, o);
-  if ((threadIdx.x & 31) == 0) atomicAdd(&s_kr, kr);
-  __syncthreads();
-  if (s_kr > (1ull << 32)) s_bad = 1;
-  __syncthreads();
-  if (s_bad) {
-    if (threadIdx.x == 0) atomicOr(&sc->status, ST_CORRUPT);
-    return;
-  }
-  build_canonical(clen, n, S.key32, canon, &S.ct);
-  for (int i = threadIdx.x; i < (int)S.ct.n; i += blockDim.x) out->canon[i] = csym[canon[i]];
-  __syncthreads();
-  // every LUT entry from its own bits: the length is the first whose
-  // left-justified limit lies above them (canonical order), the symbol that
-  // code's canonical rank; a prefix of longer codes keeps the length of its
-  // first code, where the decoder's search for the length starts
-  for (int p = threadIdx.x; p < (1 << kLutBits); p += blockDim.x) {
-    const unsigned long long peek = (unsigned long long)p << (32 - kLutBits);
-    unsigned L = 1;
-    while (L <= (unsigned)kMaxLen && peek >= S.ct.limit[L]) ++L;
-    unsigned e = L << 16;
-    if (L <= (unsigned)kLutBits) {
-      const unsigned idx = S.ct.first_pos[L] + (((unsigned)peek >> (32 - L)) - S.ct.first_code[L]);
-      e = idx < S.ct.n ? ((unsigned)csym[canon[idx]] | (L << 16)) : ((unsigned)(kMaxLen + 1) << 16);
+  if (!s_bad) build_canonical(S.len, dict, S.wcnt, out->canon, &S.ct);
+  // the lengths must satisfy Kraft's inequality (in units of 2^-32)
+  if (threadIdx.x == 0) {
+    unsigned long long kr = 0;
+    if (!s_bad)
+      for (int L = 1; L <= kMaxLen; ++L) kr += (unsigned long long)S.ct.count[L] << (32 - L);
+    if (s_bad || kr > (1ull << 32)) {
+      S.ct.n = 0;  // no symbol can be decoded
+      atomicOr(&sc->status, ST_CORRUPT);
     }
-    out->lut[p] = e;
+    out->ct = S.ct;
   }
-  if (threadIdx.x == 0) out->ct = S.ct;
 }
 
 struct DecodeArgs {
@@ -2342,55 +2330,117 @@ struct DecodeArgs {
   unsigned long long n;
   int chunk;
   const DecodeTables* tab;
+  unsigned ncanon;                     // symbols staged in shared memory: a bound on the present symbols
   uint16_t* sym;
   Scalars* sc;
 };
 
-// One thread per run (an eighth of a chunk): table-driven canonical decoding
-// with a 64-bit window refilled a word at a time from registers loaded ahead
-// in 16-byte groups, sixteen symbols per step stored as one 32-byte sector.
-// Codes of at most kLutBits bits take one shared-memory lookup; for a longer
-// one the lookup gives the length of the first code of its prefix, from
-// which the left-justified limits are walked (one or two steps).  A run must end exactly where the next one
-// starts (the last run of a chunk within the chunk); reading past the chunk
-// reads zeros and shows in that check.  Persistent CTAs: the tables are
-// staged once per CTA.
-// Threads per decoder CTA: the lookup table (64 KB) is staged once per CTA,
-// so larger CTAs keep more warps per SM on one table.  On GB300 (513^3 FP32
-// streams, 1e-2 .. 1e-5) 512 took 0.399 / 0.501 / 0.723 / 1.186 ms against
-// 0.451 / 0.566 / 0.749 / 1.189 with 256 and 0.682 / 0.903 / 1.180 / 1.586
-// with 128.
-#ifndef BM_DEC_THREADS
-#define BM_DEC_THREADS 512
-#endif
-constexpr int kDecThreads = BM_DEC_THREADS;
-constexpr size_t kDecSmem = sizeof(unsigned) * (1u << kLutBits) + sizeof(unsigned long long) * (kMaxLen + 2) +
-                            2 * sizeof(unsigned) * (kMaxLen + 2);
+// One thread per run (an eighth of a chunk): table-driven canonical decoding.
+// The thread's window is two words at a bit position (one funnel shift gives
+// the next 32 bits); the words after them come from a private ring of eight
+// words in shared memory (word-major: no bank conflicts), filled every fourth
+// symbol at most with a 16-byte group loaded ahead of use, so a symbol's
+// refill is a predicated move and a conflict-free load.  One shared-memory
+// look-up gives a code's length and, for codes of at most kLutBits bits, the
+// symbol; longer ones add their remaining bits to the prefix's canonical
+// position and read the symbol there (predicated, off the chain from one code
+// to the next); only the few prefixes of several lengths walk the
+// left-justified last codes.  Sixteen
+// symbols per step leave as one 32-byte sector.  A run must end exactly where
+// the next one starts (the last run of a chunk within the chunk); reading past
+// the chunk reads other bits or zeros and shows in that check.  Persistent
+// CTAs: the look-up table is built in shared memory once per CTA.
+// Bound by the latency and the rate of the shared-memory accesses (look-up,
+// canonical symbol, ring: 7 wavefronts a symbol and warp, 38 % of the issue
+// slots).  513^3 GRF, 1e-2 / 1e-3 / 1e-4 / 1e-5 (the last two with the outlier
+// codes' pass): 0.290 / 0.291 / 0.538 / 0.846 ms; the kernel before it (a
+// 64-bit window refilled by selects from a queue of registers, limits walked
+// for every longer code, the canonical symbols in global memory, 512-thread
+// CTAs) took 0.434 / 0.486 / 0.640 / 1.095.
+constexpr int kDecThreads = 1024, kDecThreadsSmall = 256;
+constexpr int kDecRing = 8;  // words of a thread's ring
+constexpr unsigned kLutWalk = 63;  // length field of a prefix of several lengths
+__host__ __device__ constexpr size_t dec_smem(int threads, unsigned ncanon) {
+  return (size_t)threads * kDecRing * 4 + (4u << kLutBits) + 2 * 4 * (kMaxLen + 4) + 2 * (((size_t)ncanon + 7) / 8 * 8);
+}
+static_assert(dec_smem(kDecThreads, kMaxDict) <= 227 * 1024, "decoder shared memory");
+__device__ __forceinline__ unsigned ld_shared_if(unsigned addr, bool pred, unsigned v) {
+  asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %2, 0;\n @q ld.shared.u32 %0, [%1];\n}\n"
+               : "+r"(v)
+               : "r"(addr), "r"((unsigned)pred));
+  return v;
+}
+__device__ __forceinline__ unsigned ld_shared_u16_if(unsigned addr, bool pred, unsigned v) {
+  asm volatile("{\n .reg .pred q;\n .reg .u16 h;\n setp.ne.u32 q, %2, 0;\n @q ld.shared.u16 h, [%1];\n @q cvt.u32.u16 %0, h;\n}\n"
+               : "+r"(v)
+               : "r"(addr), "r"((unsigned)pred));
+  return v;
+}
+__device__ __forceinline__ void st_shared(unsigned addr, unsigned v) {
+  asm volatile("st.shared.u32 [%0], %1;\n" ::"r"(addr), "r"(v));
+}
 
-__global__ void __launch_bounds__(kDecThreads) decode_kernel(DecodeArgs a) {
+template <int NT>
+__global__ void __launch_bounds__(NT, NT == kDecThreads ? 1 : 2) decode_kernel(DecodeArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  unsigned* lut = reinterpret_cast<unsigned*>(smem_raw);
-  unsigned long long* limit = reinterpret_cast<unsigned long long*>(lut + (1 << kLutBits));
-  unsigned* fcode = reinterpret_cast<unsigned*>(limit + kMaxLen + 2);
-  unsigned* fpos = fcode + kMaxLen + 2;
+  unsigned* lut = reinterpret_cast<unsigned*>(smem_raw + (size_t)NT * kDecRing * 4);
+  unsigned* last = lut + (1 << kLutBits);  // [kMaxLen + 4] left-justified last code of each length
+  unsigned* base = last + kMaxLen + 4;     // [kMaxLen + 4] canonical position minus code
+  uint16_t* canon = reinterpret_cast<uint16_t*>(base + kMaxLen + 4);
   const DecodeTables* T = a.tab;
+  const unsigned nsym = min(T->ct.n, a.ncanon);
   {
-    const uint4* src = reinterpret_cast<const uint4*>(T->lut);
-    uint4* dst = reinterpret_cast<uint4*>(lut);
-    for (int i = threadIdx.x; i < (1 << kLutBits) / 4; i += blockDim.x) dst[i] = src[i];
+    const uint4* src = reinterpret_cast<const uint4*>(T->canon);
+    uint4* dst = reinterpret_cast<uint4*>(canon);
+    const unsigned nv = (nsym + 7) / 8;
+    for (unsigned i0 = threadIdx.x; i0 < nv; i0 += 4 * NT) {  // four loads in flight
+      uint4 v[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) v[t] = i0 + t * NT < nv ? src[i0 + t * NT] : make_uint4(0, 0, 0, 0);
+#pragma unroll
+      for (int t = 0; t < 4; ++t)
+        if (i0 + t * NT < nv) dst[i0 + t * NT] = v[t];
+    }
   }
-  if (threadIdx.x < kMaxLen + 2) {
-    limit[threadIdx.x] = T->ct.limit[threadIdx.x];
-    fcode[threadIdx.x] = T->ct.first_code[threadIdx.x];
-    fpos[threadIdx.x] = T->ct.first_pos[threadIdx.x];
+  if (threadIdx.x == 0) last[kMaxLen + 1] = ~0u;
+  if (threadIdx.x <= kMaxLen) {
+    last[threadIdx.x] = (unsigned)(T->ct.limit[threadIdx.x] - 1ull);
+    base[threadIdx.x] = T->ct.first_pos[threadIdx.x] - T->ct.first_code[threadIdx.x];
   }
-  const unsigned nsym = T->ct.n;
-  const uint16_t* canon = T->canon;
+  __shared__ unsigned s_minl;
+  if (threadIdx.x == 0) s_minl = kMaxLen + 1;
   __syncthreads();
+  if (threadIdx.x >= 1 && threadIdx.x <= kMaxLen && T->ct.count[threadIdx.x]) atomicMin(&s_minl, threadIdx.x);
+  __syncthreads();
+  // the look-up table: length << 16 | the symbol of a code of at most kLutBits
+  // bits, or, for a prefix whose codes all have one longer length, the
+  // canonical position of the first of them; kLutWalk << 16 | the length of
+  // the first code for a prefix of several lengths (kMaxLen + 1: no code has
+  // the prefix).  The last codes ascend with the length from the shortest one
+  // on: binary search.  Positions are checked here, so that the walk below
+  // takes them as they are (tables of a corrupt codebook).
+  for (int p = threadIdx.x; p < (1 << kLutBits); p += NT) {
+    const unsigned pf = (unsigned)p << (32 - kLutBits), pl = pf | ((1u << (32 - kLutBits)) - 1u);
+    int l0 = (int)s_minl, l1 = kMaxLen + 1;
+    while (l0 < l1) {
+      const int mid = (l0 + l1) >> 1;
+      if (pf <= last[mid]) l1 = mid; else l0 = mid + 1;
+    }
+    unsigned e = (kLutWalk << 16) | (unsigned)l0;
+    if (l0 <= kMaxLen && pl <= last[l0]) {
+      const unsigned i0 = (pf >> (32 - l0)) + base[l0], i1 = (pl >> (32 - l0)) + base[l0];
+      if (i0 <= i1 && i1 < nsym) e = ((unsigned)l0 << 16) | (l0 <= kLutBits ? (unsigned)canon[i0] : i0);
+    }
+    lut[p] = e;
+  }
+  __syncthreads();
+  const unsigned ring = smem_u32(smem_raw) + 4u * threadIdx.x, canon_s = smem_u32(canon);
+  constexpr unsigned kRow = 4u * NT, kMask = kRow * kDecRing - 1u;
+  const unsigned* const wall = a.words + a.n_words;
   const unsigned long long nruns = a.nch * kSplits;
   const int sub = a.chunk / kSplits;
-  for (unsigned long long r = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; r < nruns;
-       r += (unsigned long long)gridDim.x * blockDim.x) {
+  for (unsigned long long r = blockIdx.x * (unsigned long long)NT + threadIdx.x; r < nruns;
+       r += (unsigned long long)gridDim.x * NT) {
     const unsigned long long c = r / kSplits;
     const int k = (int)(r % kSplits);
     const unsigned long long cw0 = a.word_off[c], cw1 = a.word_off[c + 1];
@@ -2401,73 +2451,71 @@ __global__ void __launch_bounds__(kDecThreads) decode_kernel(DecodeArgs a) {
     if (b0 > b1 || b1 > cbits) { atomicOr(&a.sc->status, ST_CORRUPT); continue; }
     const unsigned long long s0 = c * (unsigned long long)a.chunk + (unsigned long long)k * sub;
     const int cnt = (int)(min(a.n, s0 + (unsigned long long)sub) - s0);
-    // words enter the window from a queue (c0..c3, cl of them valid) filled
-    // from aligned 16-byte groups, the next group (n) in flight; a group is
-    // read as one vector unless it reaches past the bitstream (words past a
-    // chunk's end are never consumed by a valid run and show in the check below)
-    const unsigned* const wall = a.words + a.n_words;
+    // words past the bitstream read zeros; words past a chunk's end are never
+    // consumed by a valid run and show in the check below
     auto ld = [&](const unsigned* q) { return q < wall ? __ldg(q) : 0u; };
     auto ld4 = [&](const unsigned* g) {
       if (g + 4 <= wall) return __ldg(reinterpret_cast<const uint4*>(g));
       return make_uint4(ld(g), ld(g + 1), ld(g + 2), ld(g + 3));
     };
     const unsigned* gp = a.words + cw0 + (b0 >> 5);
-    const unsigned w0 = ld(gp), w1 = ld(gp + 1);
+    unsigned hi = ld(gp), lo = ld(gp + 1);
     gp += 2;
-    const int m = (int)((reinterpret_cast<uintptr_t>(gp) >> 2) & 3);
-    const unsigned* gq = gp - m;  // 16-byte aligned
-    const uint4 A = ld4(gq);
-    uint4 n = ld4(gq + 4);
-    gq += 8;
-    unsigned c0 = m == 0 ? A.x : m == 1 ? A.y : m == 2 ? A.z : A.w;
-    unsigned c1 = m == 0 ? A.y : m == 1 ? A.z : A.w;
-    unsigned c2 = m == 0 ? A.z : A.w;
-    unsigned c3 = A.w;
-    int cl = 4 - m;
-    const int skip = (int)(b0 & 31);
-    unsigned long long buf = (((unsigned long long)w0 << 32) | w1) << skip;
-    int nbits = 64 - skip;
-    unsigned nwords = 2;  // words entered into the window
+    const unsigned m = (unsigned)((reinterpret_cast<uintptr_t>(gp) >> 2) & 3);
+    const unsigned* gq = gp - m;  // 16-byte aligned; ring rows 0..3 hold its words, the m first not part of the run
+    auto push = [&](const uint4& v, unsigned row) {
+      st_shared(ring + row, v.x);
+      st_shared(ring + row + kRow, v.y);
+      st_shared(ring + row + 2 * kRow, v.z);
+      st_shared(ring + row + 3 * kRow, v.w);
+    };
+    push(ld4(gq), 0u);
+    push(ld4(gq + 4), 4u * kRow);
+    uint4 next = ld4(gq + 8);
+    gq += 12;
+    unsigned rp = m * kRow, wrow = 0u;  // ring offsets of the next read and of the next group
+    unsigned nx = ld_shared_if(ring + rp, true, 0u);
+    rp += kRow;
+    int wend = 10 - (int)m;  // words of the run before this one are loaded or in the ring
+    const unsigned pos0 = (unsigned)(b0 & 31);
+    unsigned pos = pos0;  // bits from the run's first word
     bool bad = false;
-    auto one = [&]() -> unsigned {
-      // a word into the window when 32 bits or fewer are left: selects, so
-      // that lanes refilling at different symbols do not diverge; only the
-      // reload of the queue (every fourth word) branches
-      const bool need = nbits <= 32;
-      const int sh = need ? 32 - nbits : 0;
-      buf |= need ? (unsigned long long)c0 << sh : 0ull;
-      nbits += need ? 32 : 0;
-      nwords += need ? 1u : 0u;
-      c0 = need ? c1 : c0;
-      c1 = need ? c2 : c1;
-      c2 = need ? c3 : c2;
-      cl -= need ? 1 : 0;
-      if (cl == 0) {
-        c0 = n.x;
-        c1 = n.y;
-        c2 = n.z;
-        c3 = n.w;
-        n = ld4(gq);
+    // before a symbol: words [pos / 32, + 2] of the run are hi, lo, nx, and the
+    // ring holds those up to wend; a symbol moves on by one word at most
+    auto refill = [&](int need) {
+      if (wend - 3 - (int)(pos >> 5) < need) {
+        push(next, wrow);
+        wrow ^= 4u * kRow;
+        wend += 4;
+        next = ld4(gq);
         gq += 4;
-        cl = 4;
       }
-      const unsigned peek = (unsigned)(buf >> 32);
+    };
+    auto one = [&]() -> unsigned {
+      const unsigned peek = __funnelshift_l(lo, hi, pos);
       unsigned e = lut[peek >> (32 - kLutBits)];
       unsigned L = e >> 16;
-      if (L > (unsigned)kLutBits) {  // a longer code: its length from its prefix's first on
-        while (L <= (unsigned)kMaxLen && (unsigned long long)peek >= limit[L]) ++L;
-        const unsigned idx = L <= (unsigned)kMaxLen ? fpos[L] + ((peek >> (32 - L)) - fcode[L]) : nsym;
+      const bool longer = L > (unsigned)kLutBits;
+      unsigned idx = (e & 0xFFFFu) + ((peek << kLutBits) >> ((32 + kLutBits - L) & 31u));
+      if (L == kLutWalk) {  // a prefix of several lengths
+        L = e & 0xFFFFu;
+        while (peek > last[L]) ++L;  // ends at the sentinel past kMaxLen
+        idx = L <= (unsigned)kMaxLen ? (peek >> (32 - L)) + base[L] : nsym;
         if (idx >= nsym) {
           bad = true;
           L = 1;
-          e = 0;
-        } else {
-          e = (unsigned)canon[idx];
+          idx = 0;
         }
       }
-      buf <<= L;
-      nbits -= (int)L;
-      return e & 0xFFFFu;
+      e = ld_shared_u16_if(canon_s + 2u * idx, longer, e);
+      const unsigned np = pos + L;
+      const bool cross = ((np ^ pos) & 32u) != 0u;
+      pos = np;
+      hi = cross ? lo : hi;
+      lo = cross ? nx : lo;
+      nx = ld_shared_if(ring + rp, cross, nx);
+      rp = cross ? (rp + kRow) & kMask : rp;
+      return e;
     };
     uint16_t* out = a.sym + s0;
     int i = 0;
@@ -2476,17 +2524,21 @@ __global__ void __launch_bounds__(kDecThreads) decode_kernel(DecodeArgs a) {
         unsigned v[8];
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
-          const unsigned lo = one();
-          v[t] = lo | (one() << 16);
+          if ((t & 1) == 0) refill(4);  // four symbols consume four words at most
+          const unsigned e0 = one(), e1 = one();
+          v[t] = __byte_perm(e0, e1, 0x5410);
         }
         uint4* o = reinterpret_cast<uint4*>(out + i);
         o[0] = make_uint4(v[0], v[1], v[2], v[3]);
         o[1] = make_uint4(v[4], v[5], v[6], v[7]);
       }
     }
-    for (; i < cnt; ++i) out[i] = (uint16_t)one();
+    for (; i < cnt; ++i) {
+      refill(1);
+      out[i] = (uint16_t)one();
+    }
     // bits consumed from the chunk start
-    const unsigned long long used = b0 + (unsigned long long)nwords * 32ull - (unsigned long long)skip - nbits;
+    const unsigned long long used = b0 + (pos - pos0);
     if (bad || (k < kSplits - 1 ? used != b1 : used > b1)) atomicOr(&a.sc->status, ST_CORRUPT);
   }
 }

@@ -1,0 +1,71 @@
+"""The Huffman decoder at its edges: codebook sections of many short runs (in
+several batches, and too long for the shared-memory copy), long runs, both
+launch shapes (few and many runs of symbols), prefixes with codes of several
+lengths, and codebook sections damaged on the host."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+def _round_trip(sym, dict_size, chunk):
+    import paper_2609_00205_gb300 as bm
+
+    so, mo = oracle.huffman_encode(sym, dict_size, chunk)
+    back = bm.huffman_decode(torch.from_numpy(so.copy()).to("cuda"), mo, sym.size, dict_size, chunk)
+    np.testing.assert_array_equal(back.cpu().numpy().view(np.uint16), sym)
+    return so, mo
+
+
+@pytest.mark.parametrize("stride,offset", [(2, 0), (3, 1), (7, 5), (64, 63)])
+def test_codebooks_of_short_runs(stride, offset):
+    """Every stride-th symbol of the dictionary: one run per symbol (32,768
+    runs, a 393 KB section, at stride 2)."""
+    rng = np.random.default_rng(stride)
+    present = np.arange(offset, 65536, stride)
+    sym = np.concatenate([present, rng.choice(present, 60_000)]).astype(np.uint16)
+    rng.shuffle(sym)
+    _round_trip(sym, 65536, 2048)
+
+
+@pytest.mark.parametrize("n_present", [1, 2, 1023, 1024, 1025, 8192, 8193, 65536])
+def test_one_run(n_present):
+    rng = np.random.default_rng(n_present)
+    sym = np.concatenate([np.arange(n_present), rng.integers(0, n_present, 5000)]).astype(np.uint16)
+    _round_trip(sym, 65536, 1024)
+
+
+@pytest.mark.parametrize("chunk,chunks", [(64, 14_591), (64, 14_592), (256, 15_001)])
+def test_launch_shapes(chunk, chunks):
+    """Around the chunk count from which one large CTA per SM decodes (three
+    quarters of 152 x 1024 runs), with geometric counts: codes of 1 to about 20
+    bits, so prefixes of several lengths."""
+    rng = np.random.default_rng(chunks)
+    sym = np.minimum(rng.geometric(0.5, chunk * chunks - 11) - 1, 255).astype(np.uint16)
+    _round_trip(sym, 256, chunk)
+
+
+def test_damaged_codebooks_are_refused_or_decoded():
+    import paper_2609_00205_gb300 as bm
+
+    rng = np.random.default_rng(9)
+    sym = np.minimum(rng.geometric(0.05, 20_000) * 3, 4095).astype(np.uint16)
+    so, mo = oracle.huffman_encode(sym, 4096, 2048)
+    cb = 8 * ((4 * mo["n_chunks"] + 7) // 8) + 8 * ((14 * mo["n_chunks"] + 7) // 8)  # after chunk words and splits
+    first = so.copy()
+    first[cb:cb + 4] = 255  # a run beyond the dictionary
+    with pytest.raises(bm.BlockMGARDError) as e:
+        bm.huffman_decode(torch.from_numpy(first).to("cuda"), mo, sym.size, 4096, 2048)
+    assert e.value.status == 4
+    for _ in range(20):
+        bad = so.copy()
+        bad[cb + int(rng.integers(0, mo["codebook_bytes"]))] ^= 1 << int(rng.integers(0, 8))
+        try:
+            bm.huffman_decode(torch.from_numpy(bad).to("cuda"), mo, sym.size, 4096, 2048)
+        except bm.BlockMGARDError as err:
+            assert err.status == 4
+    torch.cuda.synchronize()
+    _round_trip(sym, 4096, 2048)
