@@ -1669,8 +1669,8 @@ bm_status compress_t(const T* field, const int64_t* shape, const Params& prm, do
                                             0, s));
         BM_LAUNCHED();
       }
-      BM_CUDA(set_smem_once(codebook_kernel, (int)sizeof(CbSmem), g_cb_attr));
-      codebook_kernel<<<1, kCbThreads, sizeof(CbSmem), s>>>(ca);
+      BM_CUDA(set_smem_once(codebook_kernel, (int)kCbSmemBytes, g_cb_attr));
+      codebook_kernel<<<1, kCbThreads, kCbSmemBytes, s>>>(ca);
       BM_LAUNCHED();
       BM_CUDA(cudaGetLastError());
       if (coop) {  // above 8192 present symbols the codes are emitted on kPreCtas CTAs
@@ -2581,8 +2581,8 @@ bm_status bm_compress_batch(int n, const bm_batch_item* items, size_t* out_bytes
         const size_t dcb = ddesc + (size_t)n * sizeof(BatchField<double>) + groups.size() * 512 + 256;
         CodebookArgs* dc = reinterpret_cast<CodebookArgs*>(ctx->d + dcb);
         BM_CUDA(cudaMemcpyAsync(dc, hc, (size_t)ncb * sizeof(CodebookArgs), cudaMemcpyHostToDevice, q));
-        BM_CUDA(set_smem_once(codebook_batch_kernel, (int)sizeof(CbSmem), g_cbb_attr));
-        codebook_batch_kernel<<<(unsigned)ncb, kCbThreads, sizeof(CbSmem), q>>>(dc);
+        BM_CUDA(set_smem_once(codebook_batch_kernel, (int)kCbSmemBytes, g_cbb_attr));
+        codebook_batch_kernel<<<(unsigned)ncb, kCbThreads, kCbSmemBytes, q>>>(dc);
         BM_LAUNCHED();
         BM_CUDA(cudaGetLastError());
       }
@@ -3049,8 +3049,8 @@ bm_status bm_huffman_encode(const uint16_t* d_symbols, uint64_t n, int dict_size
   {
     Stage st("huffman_codebook");
     CodebookArgs ca{hist, dict_size, lens, codes, out, off_cb, out_capacity, sc, 0, nch, ~0ull, cb_big, packed, first_code};
-    BM_CUDA(set_smem_once(codebook_kernel, (int)sizeof(CbSmem), g_cb_attr));
-    codebook_kernel<<<1, kCbThreads, sizeof(CbSmem), s>>>(ca);
+    BM_CUDA(set_smem_once(codebook_kernel, (int)kCbSmemBytes, g_cb_attr));
+    codebook_kernel<<<1, kCbThreads, kCbSmemBytes, s>>>(ca);
     BM_LAUNCHED();
   }
   {
@@ -3224,8 +3224,8 @@ extern "C" bm_status bm_huffman_encode_noalloc(const uint16_t* d_symbols, uint64
   BM_CUDA(cudaMemsetAsync(out, 0, off_cb, s));
   hist_kernel<<<grid_for((int64_t)n, 256, 4), 256, 0, s>>>(d_symbols, n, dict_size, hist, sc);
   CodebookArgs ca{hist, dict_size, lens, codes, out, off_cb, out_capacity, sc, 0, nch, ~0ull, nullptr, packed, first_code};
-  BM_CUDA(set_smem_once(codebook_kernel, (int)sizeof(CbSmem), g_cb_attr));
-  codebook_kernel<<<1, kCbThreads, sizeof(CbSmem), s>>>(ca);
+  BM_CUDA(set_smem_once(codebook_kernel, (int)kCbSmemBytes, g_cb_attr));
+  codebook_kernel<<<1, kCbThreads, kCbSmemBytes, s>>>(ca);
   FusedEncodeArgs ea{};
   ea.sym = d_symbols; ea.esc = nullptr; ea.n = n; ea.chunk = chunk_symbols; ea.lens = lens; ea.codes = codes;
   ea.dict = dict_size; ea.nch = nch; ea.ticket = reinterpret_cast<unsigned*>(tickets);

@@ -442,44 +442,39 @@ struct CbArrays {
 
 // Shared-memory layout for at most kCbSmemSyms present symbols (16-bit ids).
 struct CbSmem {
-  unsigned ka[kCbSmemSyms];                 // 32 KB  } global-scratch variant: a tile of the
-  unsigned iw[kCbSmemSyms];                 // 32 KB  } two queues (sort: kb; later canon)
+  unsigned scan_tmp[64];
+  CanonTables ct;
+  unsigned ka[kCbSmemSyms];                 // 32 KB
+  unsigned iw[kCbSmemSyms];                 // 32 KB (sort: kb; later canon)
   unsigned wcnt[256 * 32];                  // 32 KB (rounds: round_end u16[N])
   uint16_t parent[2 * kCbSmemSyms];         // 32 KB (sort: sb)
   uint8_t depth[2 * kCbSmemSyms];           // 16 KB
   uint16_t sa[kCbSmemSyms];                 // 16 KB
   uint16_t csym[kCbSmemSyms];               // 16 KB
   uint8_t clen[kCbSmemSyms];                //  8 KB
-  unsigned scan_tmp[64];
-  CanonTables ct;
 };
 static_assert(sizeof(CbSmem) <= 227 * 1024, "codebook shared memory");
 static_assert(256 * 32 >= kCbSmemSyms, "run offsets over the sort counts");
 
-// Shared memory of the global-scratch variant's rounds, in the arrays only
-// the shared-memory variant uses: the samples of its two queues (samp, in
-// parent), and per tile of merged ranks the new parent of each leaf and
-// internal node taken (pa, pb: tile-relative pair index, in depth and sa)
-// and the weights of the new nodes (wk, in csym), so that the global arrays
-// are written with coalesced stores; after the rounds, the leaves' lengths
-// (lens, over all of these arrays), copied out in compact-index order.
-struct CbTileScratch {
-  unsigned* samp;
-  uint16_t* pa;
-  uint16_t* pb;
-  unsigned* wk;
-  uint8_t* lens;
+// Shared memory of the global-scratch variant's tree: a tile of merged ranks
+// (the weights of its leaves, then of its internal nodes), samples of the two
+// queues, and the parent of every internal node.
+// After the rounds the tile holds a depth byte per internal node, and at the
+// end the parents' place the leaves' lengths, gathered there before an
+// in-order copy out.
+constexpr int kCbTile = 20480;  // ranks of a tile (even)
+struct CbBigSmem {
+  unsigned scan_tmp[64];
+  CanonTables ct;
+  alignas(16) unsigned wcnt[256 * 32];  // the sort's counts, before the rounds (then part of the tile)
+  unsigned tile_rest[kCbTile - 256 * 32];
+  unsigned samp[2 * (kMaxDict / 64)];
+  uint16_t par[kMaxDict];
+  __device__ __forceinline__ unsigned* tile() { return wcnt; }
 };
-static_assert(sizeof(CbSmem::parent) >= 2 * (kMaxDict / 64) * sizeof(unsigned), "queue samples");
-static_assert(sizeof(CbSmem::depth) >= kCbSmemSyms * sizeof(uint16_t) && sizeof(CbSmem::sa) >= kCbSmemSyms * 2 &&
-                  sizeof(CbSmem::csym) >= kCbSmemSyms / 2 * sizeof(unsigned),
-              "tile scratch");
-static_assert(offsetof(CbSmem, clen) + sizeof(CbSmem::clen) - offsetof(CbSmem, parent) >= kMaxDict,
-              "a length byte per leaf from parent to clen");
-__device__ __forceinline__ CbTileScratch cb_tile_scratch(CbSmem& S) {
-  return {reinterpret_cast<unsigned*>(S.parent), reinterpret_cast<uint16_t*>(S.depth), S.sa,
-          reinterpret_cast<unsigned*>(S.csym), reinterpret_cast<uint8_t*>(S.parent)};
-}
+static_assert(sizeof(CbBigSmem) <= 227 * 1024, "codebook shared memory");
+static_assert(kCbTile * sizeof(unsigned) >= kMaxDict, "a depth byte per internal node");
+constexpr size_t kCbSmemBytes = sizeof(CbSmem) > sizeof(CbBigSmem) ? sizeof(CbSmem) : sizeof(CbBigSmem);
 
 // Global scratch of the large variant: n <= kMaxDict present symbols, 32-bit ids.
 constexpr int kPreCtas = 64;  // CTAs of cb_presort_kernel
@@ -548,12 +543,6 @@ __device__ __forceinline__ CbPre* cb_pre(unsigned char* g) {
 // V.csym): Huffman lengths into V.clen.  The lengths are those of the
 // sequential two-queue construction; lengths above kMaxLen are avoided by
 // re-running on max(1, f >> t), t = 1, 2, ...
-// Ranks of a round's merged order handled per shared-memory tile by the
-// global-scratch variant.
-constexpr int kCbTile = 8192;
-static_assert(kCbTile == kCbSmemSyms, "a tile of each queue fills ka, then iw (adjacent)");
-static_assert(2 * kCbTile * sizeof(unsigned) >= kMaxDict, "the staging holds a depth byte per internal node");
-
 // Pairs of the ranks [d0, d1) of merge(A[0..na), B[0..nb)) (A first on equal
 // weight), d0 even, whose first i0 = split(d0) ranks came from A: appends
 // the pairs' weights to iw at qe + rank/2 and sets the parents.  Ids: A[i] is
@@ -579,129 +568,98 @@ __device__ __forceinline__ unsigned merge_pairs(const unsigned* A, int na, const
   }
   return leaves;
 }
-// The same pairs within one tile, their results in shared memory: pa[i] /
-// pb[j], the tile-relative index of the new parent of A[i] / B[j]; wk[k], the
-// weight of the tile's k-th new node.
-__device__ __forceinline__ unsigned merge_pairs_tile(const unsigned* A, int na, const unsigned* B, int nb, int d0,
-                                                     int d1, int i, uint16_t* pa, uint16_t* pb, unsigned* wk) {
-  unsigned leaves = 0;
-  int j = d0 - i;
-  for (int d = d0; d < d1; d += 2) {
-    unsigned w[2];
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-      if (i < na && (j >= nb || A[i] <= B[j])) { w[t] = A[i]; pa[i] = (uint16_t)(d >> 1); ++i; ++leaves; }
-      else { w[t] = B[j]; pb[j] = (uint16_t)(d >> 1); ++j; }
-    }
-    wk[d >> 1] = w[0] + w[1];
-  }
-  return leaves;
+// The sum of the two smallest remaining weights of both queues: the first two
+// of each, read together (a weight is below 2^31, so ~0u marks an empty slot).
+__device__ __forceinline__ unsigned two_smallest(const unsigned* lw, unsigned lp, unsigned n, const unsigned* iw,
+                                                 unsigned qp, unsigned qe) {
+  const unsigned c0 = lp < n ? lw[lp] : ~0u, c1 = lp + 1 < n ? lw[lp + 1] : ~0u;
+  const unsigned d0 = qp < qe ? iw[qp] : ~0u, d1 = qp + 1 < qe ? iw[qp + 1] : ~0u;
+  return c0 <= d0 ? c0 + min(c1, d0) : d0 + min(c0, d1);
 }
 
-// stage (global-scratch variant): shared memory for the tiles of the two
-// queues; ts: its other shared memory, the samples of both queues (which turn
-// each bound search into one global round trip) and the tile's results.
+// Leaves by ascending weight (ties in symbol order) into (V.ka, V.sa), for
+// the weights max(1, f >> shift): the whole block.
 template <typename IdT>
-__device__ void codebook_lengths(const CodebookArgs& a, CbArrays<IdT> V, int n, unsigned* scan_tmp,
-                                 unsigned* stage, int pre_passes = -1, const CbTileScratch* ts = nullptr) {
-  unsigned* const samp = ts ? ts->samp : nullptr;
-  __shared__ unsigned s_lp, s_qp, s_qe, s_pl, s_pq, s_leaves, s_rounds, s_maxd, s_maxk;
-  __shared__ int s_split;
+__device__ void codebook_sort(const CodebookArgs& a, const CbArrays<IdT>& V, int n, unsigned* scan_tmp, int shift) {
+  __shared__ unsigned s_maxk;
+  if (threadIdx.x == 0) s_maxk = 0;
+  __syncthreads();
+  unsigned mk = 0;
+  for (int i0 = threadIdx.x; i0 < n; i0 += 8 * blockDim.x) {  // eight loads in flight
+    unsigned sy[8], f[8];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      const int i = i0 + t * (int)blockDim.x;
+      sy[t] = i < n ? (unsigned)V.csym[i] : 0u;
+    }
+#pragma unroll
+    for (int t = 0; t < 8; ++t) f[t] = i0 + t * (int)blockDim.x < n ? a.hist[sy[t]] : 0u;
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      const int i = i0 + t * (int)blockDim.x;
+      if (i < n) {
+        const unsigned fs = shift ? max(1u, f[t] >> shift) : f[t];
+        V.ka[i] = fs;
+        V.sa[i] = (uint16_t)i;
+        V.clen[i] = 0;
+        mk = max(mk, fs);
+      }
+    }
+  }
+#pragma unroll
+  for (int o = 16; o; o >>= 1) mk = max(mk, __shfl_xor_sync(0xffffffffu, mk, o));
+  if ((threadIdx.x & 31) == 0 && mk) atomicMax(&s_maxk, mk);
+  __syncthreads();
+  const int which = radix_sort_pairs(V.ka, V.sa, V.kb, V.sb, V.wcnt, n, s_maxk, scan_tmp);
+  if (which) {
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      V.ka[i] = V.kb[i];
+      V.sa[i] = V.sb[i];
+    }
+  }
+  __syncthreads();
+}
+
+// At most kCbSmemSyms present symbols: every array in shared memory.
+__device__ void codebook_lengths(const CodebookArgs& a, CbArrays<uint16_t> V, int n, unsigned* scan_tmp) {
+  __shared__ unsigned s_lp, s_qp, s_qe, s_pl, s_pq, s_leaves, s_rounds, s_maxd;
   if (n <= 1) {
     if (n == 1 && threadIdx.x == 0) V.clen[0] = 1;
     __syncthreads();
     return;
   }
   for (int shift = 0;; ++shift) {
-    const bool presorted = shift == 0 && pre_passes > 0;  // pairs sorted by cb_presort_kernel
-    if (presorted && (pre_passes & 1)) {  // the sorted pairs are in (kb, sb)
-      unsigned* tk = V.ka;
-      V.ka = V.kb;
-      V.kb = tk;
-      uint16_t* ts = V.sa;
-      V.sa = V.sb;
-      V.sb = ts;
-    }
-    // 1. (freq', compact index) pairs in symbol order
-    if (threadIdx.x == 0) s_maxk = 0;
-    __syncthreads();
-    if (!presorted) {
-    unsigned mk = 0;
-    for (int i0 = threadIdx.x; i0 < n; i0 += 8 * blockDim.x) {  // eight loads in flight
-      unsigned sy[8], f[8];
-#pragma unroll
-      for (int t = 0; t < 8; ++t) {
-        const int i = i0 + t * (int)blockDim.x;
-        sy[t] = i < n ? (unsigned)V.csym[i] : 0u;
-      }
-#pragma unroll
-      for (int t = 0; t < 8; ++t) f[t] = i0 + t * (int)blockDim.x < n ? a.hist[sy[t]] : 0u;
-#pragma unroll
-      for (int t = 0; t < 8; ++t) {
-        const int i = i0 + t * (int)blockDim.x;
-        if (i < n) {
-          const unsigned fs = shift ? max(1u, f[t] >> shift) : f[t];
-          V.ka[i] = fs;
-          V.sa[i] = (uint16_t)i;
-          V.clen[i] = 0;
-          mk = max(mk, fs);
-        }
-      }
-    }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) mk = max(mk, __shfl_xor_sync(0xffffffffu, mk, o));
-    if ((threadIdx.x & 31) == 0 && mk) atomicMax(&s_maxk, mk);
-    __syncthreads();
-    // leaves by ascending weight, ties in symbol order, into (ka, sa) = (lw, ls)
-    const int which = radix_sort_pairs(V.ka, V.sa, V.kb, V.sb, V.wcnt, n, s_maxk, scan_tmp);
-    if (which) {
-      for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        V.ka[i] = V.kb[i];
-        V.sa[i] = V.sb[i];
-      }
-    }
-    }  // !presorted
+    // 1. (freq', compact index) pairs sorted
+    codebook_sort(a, V, n, scan_tmp, shift);
     const unsigned* lw = V.ka;
     const uint16_t* ls = V.sa;
-    unsigned* isamp = samp ? samp + kMaxDict / 64 : nullptr;
-    if (samp) {  // the leaves' samples (the last block's is the last leaf), once the sort's copies are in
-      __syncthreads();
-      for (int k = threadIdx.x; k < (n + 63) >> 6; k += blockDim.x) samp[k] = lw[min(64 * k + 63, n - 1)];
-    }
     if (threadIdx.x == 0) { s_lp = 0; s_qp = 0; s_qe = 0; s_rounds = 0; s_leaves = 0; }
     __syncthreads();
-    // 2. parallel rounds of the two-queue construction.  Warp 0 folds the
-    // previous round into the queue state and picks this round's pairs: all
-    // nodes of weight <= X (X = the two smallest weights summed), found by
-    // warp-wide searches of both sorted queues.
+    // 2. parallel rounds of the two-queue construction: the previous round is
+    // folded into the queue state and this round's pairs picked: all nodes of
+    // weight <= X (X = the two smallest weights summed), found by warp-wide
+    // searches of both sorted queues.
     int np_prev = 0;
     while (true) {
       if (threadIdx.x == 0 && np_prev) {
         s_lp += s_leaves;
         s_qp += 2 * np_prev - s_leaves;
         s_qe += np_prev;
-        V.round_end[s_rounds++] = (IdT)s_qe;
+        V.round_end[s_rounds++] = (uint16_t)s_qe;
         s_leaves = 0;
       }
       __syncthreads();
       // warps 0 and 1 find, side by side, how many leaves and how many
       // internal nodes weigh at most X (both compute X)
       if (threadIdx.x < 64) {
-        unsigned lp = s_lp, qp = s_qp;
-        const unsigned qe = s_qe;
+        const unsigned lp = s_lp, qp = s_qp, qe = s_qe;
         if (qe < (unsigned)(n - 1)) {
-          // the two smallest remaining weights: the first two of each queue,
-          // read together (a weight is below 2^31, so ~0u marks an empty slot)
-          const unsigned c0 = lp < (unsigned)n ? lw[lp] : ~0u, c1 = lp + 1 < (unsigned)n ? lw[lp + 1] : ~0u;
-          const unsigned d0 = qp < qe ? V.iw[qp] : ~0u, d1 = qp + 1 < qe ? V.iw[qp + 1] : ~0u;
-          const unsigned X = c0 <= d0 ? c0 + min(c1, d0) : d0 + min(c0, d1);
+          const unsigned X = two_smallest(lw, lp, (unsigned)n, V.iw, qp, qe);
           if (threadIdx.x < 32) {
-            const int pl = (samp ? warp_upper_bound_sampled(lw, samp, (int)lp, n, (n + 63) >> 6, X)
-                                 : warp_upper_bound_u32(lw, (int)lp, n, X)) - (int)lp;
+            const int pl = warp_upper_bound_u32(lw, (int)lp, n, X) - (int)lp;
             if (threadIdx.x == 0) s_pl = (unsigned)pl;
           } else {
-            const int pq = (samp ? warp_upper_bound_sampled(V.iw, isamp, (int)qp, (int)qe, (int)(qe >> 6), X)
-                                 : warp_upper_bound_u32(V.iw, (int)qp, (int)qe, X)) - (int)qp;
+            const int pq = warp_upper_bound_u32(V.iw, (int)qp, (int)qe, X) - (int)qp;
             if (threadIdx.x == 32) s_pq = (unsigned)pq;
           }
         }
@@ -718,94 +676,25 @@ __device__ void codebook_lengths(const CodebookArgs& a, CbArrays<IdT> V, int n, 
       const unsigned* Bq = V.iw + qp;
       const int T = 2 * npairs;
       unsigned leaves = 0;
-      if (stage == nullptr) {  // arrays in shared memory: one split per thread
-        const int seg = 2 * ((npairs + (int)blockDim.x - 1) / (int)blockDim.x);
-        const int d0 = min(T, (int)threadIdx.x * seg), d1 = min(T, d0 + seg);
-        if (d0 < d1) {
-          int lo = max(0, d0 - pq), hi = min(d0, pl);
-          while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (A[mid] <= Bq[d0 - 1 - mid]) lo = mid + 1; else hi = mid;
-          }
-          leaves = merge_pairs<IdT>(A, pl, Bq, pq, d0, d1, lo, lp, n + qp, qe, 0, V.iw, V.parent, n);
+      const int seg = 2 * ((npairs + (int)blockDim.x - 1) / (int)blockDim.x);
+      const int d0 = min(T, (int)threadIdx.x * seg), d1 = min(T, d0 + seg);
+      if (d0 < d1) {
+        int lo = max(0, d0 - pq), hi = min(d0, pl);
+        while (lo < hi) {
+          const int mid = (lo + hi) >> 1;
+          if (A[mid] <= Bq[d0 - 1 - mid]) lo = mid + 1; else hi = mid;
         }
-      } else {  // arrays in global memory: tiles of kCbTile ranks staged in shared memory
-        unsigned* sA = stage;
-        unsigned* sB = stage + kCbTile;
-        int ia = 0;
-        for (int tb = 0; tb < T; tb += kCbTile) {
-          const int te = min(T, tb + kCbTile);
-          if (te == pl + pq) {  // every node of both queues
-            if (threadIdx.x == 0) s_split = pl;
-          } else if (te == T) {  // all but the last of the merged order (A first on equal weight)
-            if (threadIdx.x == 0) s_split = pq == 0 ? pl - 1 : pl == 0 ? 0 : A[pl - 1] <= Bq[pq - 1] ? pl : pl - 1;
-          } else if (threadIdx.x < 32) {
-            const int ib = warp_merge_split(A, pl, Bq, pq, te);
-            if (threadIdx.x == 0) s_split = ib;
-          }
-          __syncthreads();
-          const int ib = s_split, ja = tb - ia, jb = te - ib;
-          for (int k0 = threadIdx.x; k0 < ib - ia; k0 += 8 * blockDim.x) {  // eight loads in flight
-            unsigned x[8];
-#pragma unroll
-            for (int t = 0; t < 8; ++t) {
-              const int k = k0 + t * (int)blockDim.x;
-              x[t] = k < ib - ia ? A[ia + k] : 0u;
-            }
-#pragma unroll
-            for (int t = 0; t < 8; ++t)
-              if (k0 + t * (int)blockDim.x < ib - ia) sA[k0 + t * blockDim.x] = x[t];
-          }
-          for (int k0 = threadIdx.x; k0 < jb - ja; k0 += 8 * blockDim.x) {
-            unsigned x[8];
-#pragma unroll
-            for (int t = 0; t < 8; ++t) {
-              const int k = k0 + t * (int)blockDim.x;
-              x[t] = k < jb - ja ? Bq[ja + k] : 0u;
-            }
-#pragma unroll
-            for (int t = 0; t < 8; ++t)
-              if (k0 + t * (int)blockDim.x < jb - ja) sB[k0 + t * blockDim.x] = x[t];
-          }
-          __syncthreads();
-          const int tl = te - tb, na = ib - ia, nb = jb - ja;
-          const int seg = 2 * ((tl / 2 + (int)blockDim.x - 1) / (int)blockDim.x);
-          const int d0 = min(tl, (int)threadIdx.x * seg), d1 = min(tl, d0 + seg);
-          if (d0 < d1) {
-            int lo = max(0, d0 - nb), hi = min(d0, na);
-            while (lo < hi) {
-              const int mid = (lo + hi) >> 1;
-              if (sA[mid] <= sB[d0 - 1 - mid]) lo = mid + 1; else hi = mid;
-            }
-            leaves += merge_pairs_tile(sA, na, sB, nb, d0, d1, lo, ts->pa, ts->pb, ts->wk);
-          }
-          __syncthreads();
-          // the tile's parents and new weights, coalesced
-          const int kb0 = qe + (tb >> 1);
-          for (int k = threadIdx.x; k < na; k += blockDim.x) V.parent[lp + ia + k] = (IdT)(n + kb0 + ts->pa[k]);
-          for (int k = threadIdx.x; k < nb; k += blockDim.x) V.parent[n + qp + ja + k] = (IdT)(n + kb0 + ts->pb[k]);
-          for (int k = threadIdx.x; k < (tl >> 1); k += blockDim.x) {
-            const unsigned w = ts->wk[k];
-            V.iw[kb0 + k] = w;
-            if (((kb0 + k) & 63) == 63) isamp[(kb0 + k) >> 6] = w;
-          }
-          ia = ib;
-          __syncthreads();
-        }
+        leaves = merge_pairs<uint16_t>(A, pl, Bq, pq, d0, d1, lo, lp, n + qp, qe, 0, V.iw, V.parent, n);
       }
       if (leaves) atomicAdd(&s_leaves, leaves);
       np_prev = npairs;
       __syncthreads();
     }
     // 3. depths, rounds in reverse (a parent is always created in a later
-    // round).  The global-scratch variant keeps the internal nodes' depths in
-    // the tile staging's shared memory (one byte each: a depth stays below 64
-    // for counts below 2^32), indexed by creation order.
+    // round)
     const int root = 2 * n - 2;
-    uint8_t* const dsh = stage ? reinterpret_cast<uint8_t*>(stage) : nullptr;
     if (threadIdx.x == 0) {
-      if (dsh) dsh[n - 2] = 0;
-      else V.depth[root] = 0;
+      V.depth[root] = 0;
       s_maxd = 0;
     }
     __syncthreads();
@@ -813,41 +702,196 @@ __device__ void codebook_lengths(const CodebookArgs& a, CbArrays<IdT> V, int n, 
       const int jb = r ? (int)V.round_end[r - 1] : 0, je = (int)V.round_end[r];
       for (int j = jb + threadIdx.x; j < je; j += blockDim.x) {
         const int v = n + j;
-        if (v != root) {
-          if (dsh) dsh[j] = (uint8_t)(dsh[(int)V.parent[v] - n] + 1);
-          else V.depth[v] = V.depth[V.parent[v]] + 1;
-        }
+        if (v != root) V.depth[v] = V.depth[V.parent[v]] + 1;
       }
       __syncthreads();
     }
     unsigned md = 0;
-    for (int i0 = threadIdx.x; i0 < n; i0 += 8 * blockDim.x) {  // eight loads in flight
-      unsigned pa[8], li[8], dd[8];
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      const unsigned dd = (unsigned)V.depth[V.parent[i]] + 1u;
+      V.clen[ls[i]] = (uint8_t)min(dd, 255u);
+      md = max(md, dd);
+    }
+    if (md) atomicMax(&s_maxd, md);
+    __syncthreads();
+    if (s_maxd <= (unsigned)kMaxLen) break;
+    __syncthreads();
+  }
+}
+
+// More present symbols: the queues in global scratch, a round's nodes staged
+// in tiles of merged ranks, one pass over a tile: the leaves' parents and the
+// new weights go straight to global memory, the internal nodes' parents stay
+// in shared memory, where the depths follow them.  Bound by the latency of a
+// round's steps (19 to 28 rounds) and one SM's issue rate.  With the results
+// staged per queue and every parent in global memory the tree of 65,468
+// symbols (100x500x500 at 1e-4) took 0.195 ms against 0.153; ranks found by
+// a binary search per node instead of the merge path took 0.211.
+__device__ void codebook_lengths_big(const CodebookArgs& a, CbArrays<unsigned> V, int n, CbBigSmem& S,
+                                     int pre_passes) {
+  __shared__ unsigned s_lp, s_qp, s_qe, s_pl, s_pq, s_rounds, s_maxd;
+  __shared__ int s_split;
+  // a round's X is at least 1.5 times the one before (a node left over by an
+  // odd count weighs at least X / 2): at most 54 rounds
+  __shared__ unsigned s_rend[64];
+  unsigned* const lsamp = S.samp;
+  unsigned* const isamp = S.samp + kMaxDict / 64;
+  unsigned* const tw = S.tile();  // a tile's weights: leaves, then internal nodes
+  uint16_t* const lpar = reinterpret_cast<uint16_t*>(V.parent);  // parents of the leaves
+  for (int shift = 0;; ++shift) {
+    if (shift == 0 && pre_passes > 0) {  // pairs sorted by cb_presort_kernel
+      if (pre_passes & 1) {  // into (kb, sb)
+        unsigned* tk = V.ka;
+        V.ka = V.kb;
+        V.kb = tk;
+        uint16_t* ts = V.sa;
+        V.sa = V.sb;
+        V.sb = ts;
+      }
+    } else {
+      codebook_sort(a, V, n, S.scan_tmp, shift);
+    }
+    const unsigned* lw = V.ka;
+    const uint16_t* ls = V.sa;
+    // the leaves' samples (the last block's is the last leaf)
+    for (int k = threadIdx.x; k < (n + 63) >> 6; k += blockDim.x) lsamp[k] = lw[min(64 * k + 63, n - 1)];
+    if (threadIdx.x == 0) { s_lp = 0; s_qp = 0; s_qe = 0; s_rounds = 0; }
+    __syncthreads();
+    while (true) {
+      if (threadIdx.x < 64) {
+        const unsigned lp = s_lp, qp = s_qp, qe = s_qe;
+        if (qe < (unsigned)(n - 1)) {
+          const unsigned X = two_smallest(lw, lp, (unsigned)n, V.iw, qp, qe);
+          if (threadIdx.x < 32) {
+            const int pl = warp_upper_bound_sampled(lw, lsamp, (int)lp, n, (n + 63) >> 6, X) - (int)lp;
+            if (threadIdx.x == 0) s_pl = (unsigned)pl;
+          } else {
+            const int pq = warp_upper_bound_sampled(V.iw, isamp, (int)qp, (int)qe, (int)(qe >> 6), X) - (int)qp;
+            if (threadIdx.x == 32) s_pq = (unsigned)pq;
+          }
+        }
+      }
+      __syncthreads();
+      if (s_qe >= (unsigned)(n - 1)) break;
+      const int lp = s_lp, qp = s_qp, qe = s_qe, pl = s_pl, pq = s_pq;
+      const int npairs = (pl + pq) >> 1;
+      const unsigned* A = lw + lp;
+      const unsigned* Bq = V.iw + qp;
+      const int T = 2 * npairs;
+      int ia = 0;
+      for (int tb = 0; tb < T; tb += kCbTile) {
+        const int te = min(T, tb + kCbTile);
+        int ib;
+        if (te == pl + pq) {  // every node of both queues
+          ib = pl;
+        } else {
+          if (te == T) {  // all but the last of the merged order (A first on equal weight)
+            if (threadIdx.x == 0) s_split = pq == 0 ? pl - 1 : pl == 0 ? 0 : A[pl - 1] <= Bq[pq - 1] ? pl : pl - 1;
+          } else if (threadIdx.x < 32) {
+            const int sp = warp_merge_split(A, pl, Bq, pq, te);
+            if (threadIdx.x == 0) s_split = sp;
+          }
+          __syncthreads();
+          ib = s_split;
+        }
+        const int ja = tb - ia, na = ib - ia, tl = te - tb, nb = tl - na;
+        for (int k0 = threadIdx.x; k0 < tl; k0 += 10 * blockDim.x) {  // ten loads in flight
+          unsigned x[10];
+#pragma unroll
+          for (int t = 0; t < 10; ++t) {
+            const int k = k0 + t * (int)blockDim.x;
+            x[t] = k < na ? A[ia + k] : k < tl ? Bq[ja + k - na] : 0u;
+          }
+#pragma unroll
+          for (int t = 0; t < 10; ++t)
+            if (k0 + t * (int)blockDim.x < tl) tw[k0 + t * blockDim.x] = x[t];
+        }
+        __syncthreads();
+        // merge path: thread t takes the tile's ranks [d0, d1) (d0 even), finds
+        // how many of the first d0 are leaves by one binary search, then walks
+        // its ranks, one look-up each (~0u past a queue's end)
+        const int kb0 = qe + (tb >> 1);
+        const int seg = 2 * ((tl / 2 + (int)blockDim.x - 1) / (int)blockDim.x);
+        const int d0 = min(tl, (int)threadIdx.x * seg), d1 = min(tl, d0 + seg);
+        if (d0 < d1) {
+          const unsigned* sB = tw + na;
+          int lo = max(0, d0 - nb), hi = min(d0, na);
+          while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (tw[mid] <= sB[d0 - 1 - mid]) lo = mid + 1; else hi = mid;
+          }
+          int i = lo, j = na + d0 - lo;  // next leaf, next internal node (indices into tw)
+          unsigned x = i < na ? tw[i] : ~0u, y = j < tl ? tw[j] : ~0u;
+          for (int d = d0; d < d1; d += 2) {
+            unsigned w = 0;
+            const uint16_t parent = (uint16_t)(kb0 + (d >> 1));
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+              const bool leaf = x <= y;
+              w += leaf ? x : y;
+              if (leaf) lpar[lp + ia + i] = parent;
+              else S.par[qp + ja + j - na] = parent;
+              const int nx = leaf ? ++i : ++j;
+              const unsigned v = nx < (leaf ? na : tl) ? tw[nx] : ~0u;
+              x = leaf ? v : x;
+              y = leaf ? y : v;
+            }
+            V.iw[parent] = w;
+            if ((parent & 63) == 63) isamp[parent >> 6] = w;
+          }
+        }
+        ia = ib;
+        if (te < T) __syncthreads();
+      }
+      if (threadIdx.x == 0) {
+        s_lp = lp + ia;
+        s_qp = qp + T - ia;
+        s_qe = qe + npairs;
+        s_rend[s_rounds++] = (unsigned)(qe + npairs);
+      }
+      __syncthreads();
+    }
+    // depths, rounds in reverse (a parent is always created in a later round),
+    // one byte each in the tile's place (a depth stays below 64 for counts
+    // below 2^32), indexed by creation order
+    uint8_t* const dsh = reinterpret_cast<uint8_t*>(S.tile());
+    if (threadIdx.x == 0) {
+      dsh[n - 2] = 0;
+      s_maxd = 0;
+    }
+    __syncthreads();
+    for (int r = (int)s_rounds - 1; r >= 0; --r) {
+      const int jb = r ? (int)s_rend[r - 1] : 0, je = (int)s_rend[r];
+      for (int j = jb + threadIdx.x; j < je; j += blockDim.x)
+        if (j != n - 2) dsh[j] = (uint8_t)(dsh[S.par[j]] + 1);
+      __syncthreads();
+    }
+    // the leaves' lengths, gathered over the parents (scattered byte stores),
+    // then copied out in compact-index order
+    uint8_t* const lens = reinterpret_cast<uint8_t*>(S.par);
+    unsigned md = 0;
+    for (int i0 = threadIdx.x; i0 < n; i0 += 8 * blockDim.x) {  // sixteen loads in flight
+      unsigned pa[8], li[8];
 #pragma unroll
       for (int t = 0; t < 8; ++t) {
         const int i = i0 + t * (int)blockDim.x;
-        pa[t] = i < n ? (unsigned)V.parent[i] : 0u;
+        pa[t] = i < n ? (unsigned)lpar[i] : 0u;
         li[t] = i < n ? (unsigned)ls[i] : 0u;
       }
 #pragma unroll
       for (int t = 0; t < 8; ++t)
-        dd[t] = i0 + t * (int)blockDim.x < n ? (unsigned)(dsh ? dsh[pa[t] - (unsigned)n] : V.depth[pa[t]]) + 1u : 0u;
-#pragma unroll
-      for (int t = 0; t < 8; ++t)
         if (i0 + t * (int)blockDim.x < n) {
-          // the global-scratch variant gathers the lengths in shared memory
-          // (scattered byte stores), then copies them out in order
-          if (ts) ts->lens[li[t]] = (uint8_t)min(dd[t], 255u);
-          else V.clen[li[t]] = (uint8_t)min(dd[t], 255u);
-          md = max(md, dd[t]);
+          const unsigned dd = (unsigned)dsh[pa[t]] + 1u;
+          lens[li[t]] = (uint8_t)min(dd, 255u);
+          md = max(md, dd);
         }
     }
     if (md) atomicMax(&s_maxd, md);
     __syncthreads();
-    if (ts) {
-      for (int i = threadIdx.x; i < n; i += blockDim.x) V.clen[i] = ts->lens[i];
-      __syncthreads();
-    }
+    for (int i = threadIdx.x; i < n / 4; i += blockDim.x)
+      reinterpret_cast<unsigned*>(V.clen)[i] = reinterpret_cast<const unsigned*>(lens)[i];
+    if (threadIdx.x < (unsigned)(n & 3)) V.clen[(n & ~3) + threadIdx.x] = lens[(n & ~3) + threadIdx.x];
+    __syncthreads();
     if (s_maxd <= (unsigned)kMaxLen) break;
     __syncthreads();
   }
@@ -1065,15 +1109,17 @@ __device__ void codebook_emit(const CodebookArgs& a, CbArrays<IdT> V, int n, uns
 // order) into the global arrays with their frequencies as keys, the compact
 // index as payload and zero lengths, and, when more than kCbSmemSyms symbols
 // are present, sorts the pairs by key, stably, with 8-bit LSD passes: each
-// CTA owns a contiguous segment of the pairs; a pass counts the segment's
-// digits, and after the barrier thread d of each CTA walks its segment (staged
-// in shared memory) in order and places the keys of digit d at the digit's
-// global offset (all keys of smaller digits, then those of digit d in the
-// CTAs before), so equal keys keep their order.  The sorted pairs are in
+// CTA owns a contiguous segment of the pairs; in a pass its warps rank their
+// rows by digit, and after the barrier every pair goes to the digit's global
+// offset (all keys of smaller digits, then those of digit d in the CTAs and
+// the warps before) plus its rank, so equal keys keep their order.  One
+// thread per digit walking the segment instead took 26 us a pass (65,468
+// pairs: the launch 91 us against 31).  The sorted pairs are in
 // (ka, sa) after an even number of passes and in (kb, sb) after an odd one
 // (CbPre::passes; 0 when the codebook kernel sorts in shared memory itself).
 constexpr int kPreThreads = 256;
 constexpr int kPreSeg = kMaxDict / kPreCtas;  // pairs per CTA at most
+constexpr int kPreWarps = kPreThreads / 32, kPreRows = kPreSeg / kPreThreads;  // rows of 32 pairs per warp
 __global__ void __launch_bounds__(kPreThreads) cb_presort_kernel(CodebookArgs a) {
   cooperative_groups::grid_group grid = cooperative_groups::this_grid();
   CbPre* pre = cb_pre(a.big);
@@ -1081,10 +1127,8 @@ __global__ void __launch_bounds__(kPreThreads) cb_presort_kernel(CodebookArgs a)
   const int dict = a.dict, c = blockIdx.x, G = gridDim.x;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   __shared__ unsigned s_red[kPreThreads / 32];
-  __shared__ unsigned s_scan[kPreThreads];
-  __shared__ unsigned s_dc[256];
-  __shared__ unsigned s_key[kPreSeg];
-  __shared__ uint16_t s_val[kPreSeg];
+  __shared__ unsigned s_scan[32], s_tot;
+  __shared__ unsigned s_wc[kPreWarps * 256];
   __shared__ unsigned s_base, s_n, s_maxk;
   auto block_sum = [&](unsigned v) {
 #pragma unroll
@@ -1096,20 +1140,7 @@ __global__ void __launch_bounds__(kPreThreads) cb_presort_kernel(CodebookArgs a)
     for (int w = 0; w < kPreThreads / 32; ++w) t += s_red[w];
     return t;
   };
-  auto block_excl = [&](unsigned v, unsigned* total) {  // exclusive scan over the block's threads
-    s_scan[threadIdx.x] = v;
-    __syncthreads();
-    for (int o = 1; o < kPreThreads; o <<= 1) {
-      const unsigned y = threadIdx.x >= (unsigned)o ? s_scan[threadIdx.x - o] : 0u;
-      __syncthreads();
-      s_scan[threadIdx.x] += y;
-      __syncthreads();
-    }
-    const unsigned incl = s_scan[threadIdx.x];
-    if (total) *total = s_scan[kPreThreads - 1];
-    __syncthreads();
-    return incl - v;
-  };
+  auto block_excl = [&](unsigned v, unsigned* total) { return block_excl_scan(v, s_scan, total); };
   // 0. tables cleared; present symbols of this CTA's dictionary segment counted
   for (int s = c * kPreThreads + threadIdx.x; s < dict; s += G * kPreThreads) {
     a.lens[s] = 0;
@@ -1144,8 +1175,7 @@ __global__ void __launch_bounds__(kPreThreads) cb_presort_kernel(CodebookArgs a)
   for (int s0 = d0; s0 < d1; s0 += kPreThreads) {
     const int s = s0 + threadIdx.x;
     const unsigned f = s < d1 ? a.hist[s] : 0u;
-    unsigned tot = 0;
-    const unsigned r = block_excl(f != 0u ? 1u : 0u, &tot);
+    const unsigned r = block_excl(f != 0u ? 1u : 0u, &s_tot);
     if (f) {
       const unsigned i = pos + r;
       V.csym[i] = (uint16_t)s;
@@ -1154,7 +1184,8 @@ __global__ void __launch_bounds__(kPreThreads) cb_presort_kernel(CodebookArgs a)
       V.sa[i] = (uint16_t)i;
       mk = max(mk, f);
     }
-    pos += tot;
+    pos += s_tot;
+    __syncthreads();
   }
 #pragma unroll
   for (int o = 16; o; o >>= 1) mk = max(mk, __shfl_xor_sync(0xffffffffu, mk, o));
@@ -1177,36 +1208,62 @@ __global__ void __launch_bounds__(kPreThreads) cb_presort_kernel(CodebookArgs a)
     const uint16_t* sin = (p & 1) ? V.sb : V.sa;
     unsigned* kout = (p & 1) ? V.ka : V.kb;
     uint16_t* sout = (p & 1) ? V.sa : V.sb;
-    // the segment staged, its digits counted
-    s_dc[threadIdx.x] = 0u;
+    // every warp ranks its four rows of 32 pairs by digit (match), with a
+    // running count per (warp, digit): the pair's rank among the warp's
+    for (int i = threadIdx.x; i < kPreWarps * 256; i += kPreThreads) s_wc[i] = 0u;
     __syncthreads();
-    for (int i = p0 + threadIdx.x; i < p1; i += kPreThreads) {
-      const unsigned k = kin[i];
-      s_key[i - p0] = k;
-      s_val[i - p0] = sin[i];
-      atomicAdd(&s_dc[(k >> shift) & 255u], 1u);
+    unsigned key[kPreRows], rank[kPreRows];
+    uint16_t val[kPreRows];
+#pragma unroll
+    for (int t = 0; t < kPreRows; ++t) {
+      const int i = p0 + (wid * kPreRows + t) * 32 + lane;
+      key[t] = i < p1 ? kin[i] : 0u;
+      val[t] = i < p1 ? sin[i] : (uint16_t)0;
+    }
+#pragma unroll
+    for (int t = 0; t < kPreRows; ++t) {
+      const bool ok = p0 + (wid * kPreRows + t) * 32 + lane < p1;
+      const unsigned d = (key[t] >> shift) & 255u;
+      const unsigned m = __match_any_sync(0xffffffffu, ok ? d : 256u);
+      const unsigned lt = m & ((1u << lane) - 1u), seen = ok ? s_wc[wid * 256 + d] : 0u;
+      rank[t] = seen + (unsigned)__popc(lt);
+      __syncwarp();
+      if (ok && lt == 0u) s_wc[wid * 256 + d] = seen + (unsigned)__popc(m);
+      __syncwarp();
     }
     __syncthreads();
-    pre->dcnt[c * 256 + threadIdx.x] = s_dc[threadIdx.x];
+    {  // thread d: the digit's count over the warps, and each warp's offset in it
+      unsigned t = 0;
+#pragma unroll
+      for (int w = 0; w < kPreWarps; ++w) {
+        const unsigned v = s_wc[w * 256 + threadIdx.x];
+        s_wc[w * 256 + threadIdx.x] = t;
+        t += v;
+      }
+      pre->dcnt[c * 256 + threadIdx.x] = t;
+    }
     grid.sync();
     // offsets of digit d (thread d): keys of smaller digits, then of digit d
     // in the CTAs before this one
     const unsigned d = threadIdx.x;
     unsigned col = 0, part = 0;
+#pragma unroll 16
     for (int k = 0; k < G; ++k) {
       const unsigned v = pre->dcnt[k * 256 + d];
       if (k < c) part += v;
       col += v;
     }
-    unsigned off = block_excl(col, nullptr) + part;
-    for (int i = 0; i < p1 - p0; ++i) {
-      const unsigned k = s_key[i];
-      if (((k >> shift) & 255u) == d) {
-        kout[off] = k;
-        sout[off] = s_val[i];
-        ++off;
+    const unsigned off = block_excl(col, nullptr) + part;
+#pragma unroll
+    for (int w = 0; w < kPreWarps; ++w) s_wc[w * 256 + d] += off;
+    __syncthreads();
+#pragma unroll
+    for (int t = 0; t < kPreRows; ++t)
+      if (p0 + (wid * kPreRows + t) * 32 + lane < p1) {
+        const unsigned o = s_wc[wid * 256 + ((key[t] >> shift) & 255u)] + rank[t];
+        kout[o] = key[t];
+        sout[o] = val[t];
       }
-    }
     grid.sync();
   }
 }
@@ -1214,9 +1271,10 @@ __global__ void __launch_bounds__(kPreThreads) cb_presort_kernel(CodebookArgs a)
 // Multi-CTA end of the codebook for wide code distributions (after the one-CTA
 // tree, above kCbSmemSyms present symbols; cooperative launch of kPreCtas
 // CTAs, grid-wide barriers between the phases): what codebook_emit does, each
-// CTA over its segment of compact indices.  Canonical order: per-(CTA,
-// length) counts, then thread L of each CTA places its segment's indices of
-// length L in order (symbol order within a length).  Runs of consecutive
+// CTA over its segment of compact indices.  Codes: per-(CTA, length) counts
+// and the warps' ranks by length (symbol order within a length), as in the
+// presort (one thread per length walking the segment: the launch 45 us
+// against 29).  Runs of consecutive
 // present symbols: per-CTA start counts give each start's run index; the
 // runs' section bytes are summed per CTA for their offsets.  The sums of the
 // size bound and of the encoder's window go to global atomics; CTA 0 makes
@@ -1230,29 +1288,16 @@ __global__ void __launch_bounds__(kPreThreads) cb_emit_kernel(CodebookArgs a) {
   const int c = blockIdx.x, G = gridDim.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   __shared__ uint8_t s_len[kPreSeg];
   __shared__ uint16_t s_sym[kPreSeg];
-  __shared__ unsigned s_lc[kMaxLen + 2];
-  __shared__ unsigned s_scan[kPreThreads];
+  __shared__ unsigned s_wl[kPreWarps * 64];  // per (warp, length): codes, then offsets
+  __shared__ unsigned s_scan[32], s_tot;
   __shared__ unsigned s_red[kPreThreads / 32];
   __shared__ unsigned long long s_r64[kPreThreads / 32];
   __shared__ CanonTables s_ct;
   __shared__ unsigned s_prev, s_rbase, s_nruns, s_boff, s_total;
-  auto block_excl = [&](unsigned v, unsigned* total) {
-    s_scan[tid] = v;
-    __syncthreads();
-    for (int o = 1; o < kPreThreads; o <<= 1) {
-      const unsigned y = tid >= o ? s_scan[tid - o] : 0u;
-      __syncthreads();
-      s_scan[tid] += y;
-      __syncthreads();
-    }
-    const unsigned incl = s_scan[tid];
-    if (total) *total = s_scan[kPreThreads - 1];
-    __syncthreads();
-    return incl - v;
-  };
+  auto block_excl = [&](unsigned v, unsigned* total) { return block_excl_scan(v, s_scan, total); };
   const int pseg = (n + G - 1) / G, e0 = min(n, c * pseg), e1 = min(n, e0 + pseg), m = e1 - e0;
   // E0: the segment staged; its length counts, run starts and size sums
-  if (tid < kMaxLen + 2) s_lc[tid] = 0u;
+  for (int i = tid; i < kPreWarps * 64; i += kPreThreads) s_wl[i] = 0u;
   if (tid == 0) s_prev = e0 > 0 ? (unsigned)V.csym[e0 - 1] : 0u;
   __syncthreads();
   unsigned long long my_bits = 0;
@@ -1260,7 +1305,6 @@ __global__ void __launch_bounds__(kPreThreads) cb_emit_kernel(CodebookArgs a) {
     const unsigned L = V.clen[e0 + i], sy = V.csym[e0 + i];
     s_len[i] = (uint8_t)L;
     s_sym[i] = (uint16_t)sy;
-    if (L >= 1u && L <= (unsigned)kMaxLen) atomicAdd(&s_lc[L], 1u);
     my_bits += (unsigned long long)a.hist[sy] * L;
   }
   __syncthreads();
@@ -1289,15 +1333,39 @@ __global__ void __launch_bounds__(kPreThreads) cb_emit_kernel(CodebookArgs a) {
     atomicAdd(&pre->bits, b);
     pre->rcnt[c] = st;
   }
-  if (tid < kMaxLen + 2) pre->dcnt[c * 256 + tid] = s_lc[tid];
+  // ranks by length: every warp's rows in order, as in the presort
+  unsigned rank[kPreRows];
+#pragma unroll
+  for (int t = 0; t < kPreRows; ++t) {
+    const int i = (wid * kPreRows + t) * 32 + lane;
+    const bool ok = i < m && s_len[i] >= 1 && s_len[i] <= kMaxLen;
+    const unsigned L = ok ? (unsigned)s_len[i] : 0u;
+    const unsigned mm = __match_any_sync(0xffffffffu, L);
+    const unsigned lt = mm & ((1u << lane) - 1u), seen = s_wl[wid * 64 + L];
+    rank[t] = seen + (unsigned)__popc(lt);
+    __syncwarp();
+    if (lt == 0u) s_wl[wid * 64 + L] = seen + (unsigned)__popc(mm);
+    __syncwarp();
+  }
+  __syncthreads();
+  if (tid <= kMaxLen) {
+    unsigned t = 0;
+    for (int w = 0; w < kPreWarps; ++w) {
+      const unsigned v = s_wl[w * 64 + tid];
+      s_wl[w * 64 + tid] = t;
+      t += v;
+    }
+    pre->dcnt[c * 256 + tid] = tid ? t : 0u;
+  }
   grid.sync();
   // E1: canonical tables (every CTA, the same), this segment's canonical
   // positions; run bases
   unsigned part = 0;
   if (tid <= kMaxLen + 1) {
     unsigned tot = 0;
+#pragma unroll 16
     for (int k = 0; k < G; ++k) {
-      const unsigned v = pre->dcnt[k * 256 + tid];
+      const unsigned v = tid <= kMaxLen ? pre->dcnt[k * 256 + tid] : 0u;
       if (k < c) part += v;
       tot += v;
     }
@@ -1316,10 +1384,20 @@ __global__ void __launch_bounds__(kPreThreads) cb_emit_kernel(CodebookArgs a) {
   __syncthreads();
   if (tid == 0) canon_from_counts(&s_ct);
   __syncthreads();
-  if (tid >= 1 && tid <= kMaxLen) {
-    unsigned pos = s_ct.first_pos[tid] + part;
-    for (int i = 0; i < m; ++i)
-      if (s_len[i] == (unsigned)tid) V.canon[pos++] = (uint16_t)(e0 + i);
+  if (tid <= kMaxLen)
+    for (int w = 0; w < kPreWarps; ++w) s_wl[w * 64 + tid] += part;
+  if (c == 0 && tid <= kMaxLen) a.first_code[tid] = s_ct.first_code[tid];
+  __syncthreads();
+#pragma unroll
+  for (int t = 0; t < kPreRows; ++t) {  // a symbol's code: its length's first one plus its rank
+    const int i = (wid * kPreRows + t) * 32 + lane;
+    const unsigned L = i < m ? (unsigned)s_len[i] : 0u;
+    if (L >= 1u && L <= (unsigned)kMaxLen) {
+      const unsigned cd = s_ct.first_code[L] + s_wl[wid * 64 + L] + rank[t], sy = s_sym[i];
+      a.codes[sy] = cd;
+      a.packed[sy] = enc_entry(cd, L);
+      a.lens[sy] = (uint8_t)L;
+    }
   }
   const int nruns = (int)s_nruns;
   {  // run starts of the segment at their run indices
@@ -1327,24 +1405,14 @@ __global__ void __launch_bounds__(kPreThreads) cb_emit_kernel(CodebookArgs a) {
     for (int i0 = 0; i0 < m; i0 += kPreThreads) {
       const int i = i0 + tid;
       const bool st = i < m && is_start(i);
-      unsigned tot = 0;
-      const unsigned r = block_excl(st ? 1u : 0u, &tot);
+      const unsigned r = block_excl(st ? 1u : 0u, &s_tot);
       if (st) V.run_start[q + r] = (unsigned)(e0 + i);
-      q += tot;
+      q += s_tot;
+      __syncthreads();
     }
   }
   grid.sync();
-  // E2: code tables over the canonical order; section bytes of this CTA's runs
-  if (c == 0 && tid <= kMaxLen) a.first_code[tid] = s_ct.first_code[tid];
-  for (int i = c * kPreThreads + tid; i < n; i += G * kPreThreads) {
-    const unsigned ci = V.canon[i];
-    const unsigned L = V.clen[ci];
-    const unsigned cd = s_ct.first_code[L] + (unsigned)(i - (int)s_ct.first_pos[L]);
-    const unsigned sy = V.csym[ci];
-    a.codes[sy] = cd;
-    a.packed[sy] = enc_entry(cd, L);
-    a.lens[sy] = (uint8_t)L;
-  }
+  // E2: section bytes of this CTA's runs
   const int rq = (nruns + G - 1) / G, q0 = min(nruns, c * rq), q1 = min(nruns, q0 + rq);
   unsigned my_b = 0;
   for (int q = q0 + tid; q < q1; q += kPreThreads) {
@@ -1382,8 +1450,7 @@ __global__ void __launch_bounds__(kPreThreads) cb_emit_kernel(CodebookArgs a) {
       const int q = qb + tid;
       const unsigned st = q < q1 ? V.run_start[q] : 0u, en = q < q1 ? V.run_end[q] : 0u;
       const unsigned bq = q < q1 ? 8u + (((en - st) + 3u) & ~3u) : 0u;
-      unsigned tot = 0;
-      const unsigned r = block_excl(bq, &tot);
+      const unsigned r = block_excl(bq, &s_tot);
       if (q < q1) {
         V.run_off[q] = off + r;
         if (fits) {
@@ -1393,7 +1460,8 @@ __global__ void __launch_bounds__(kPreThreads) cb_emit_kernel(CodebookArgs a) {
           for (unsigned t = en - st; t < (((en - st) + 3u) & ~3u); ++t) p[8 + t] = 0;
         }
       }
-      off += tot;
+      off += s_tot;
+      __syncthreads();
     }
   }
   grid.sync();
@@ -1403,13 +1471,13 @@ __global__ void __launch_bounds__(kPreThreads) cb_emit_kernel(CodebookArgs a) {
     for (int i0 = 0; i0 < m; i0 += kPreThreads) {
       const int i = i0 + tid;
       const bool st = i < m && is_start(i);
-      unsigned tot = 0;
-      const unsigned r = block_excl(st ? 1u : 0u, &tot);
+      const unsigned r = block_excl(st ? 1u : 0u, &s_tot);
       if (i < m) {
         const unsigned qi = q + r + (st ? 1u : 0u) - 1u;  // starts up to and including i, minus one
         a.out[a.off + V.run_off[qi] + 8 + ((unsigned)(e0 + i) - V.run_start[qi])] = s_len[i];
       }
-      q += tot;
+      q += s_tot;
+      __syncthreads();
     }
     if (c == 0 && tid == 0)
       for (unsigned long long t = total; t < pad8(total); ++t) a.out[a.off + t] = 0;
@@ -1433,12 +1501,11 @@ __device__ void codebook_block(const CodebookArgs& a) {
       for (int i = threadIdx.x; i < n; i += blockDim.x) S.csym[i] = gsym[i];
       __syncthreads();
       const CbArrays<uint16_t> V = cb_small(S);
-      codebook_lengths<uint16_t>(a, V, n, S.scan_tmp, nullptr);
+      codebook_lengths(a, V, n, S.scan_tmp);
       codebook_emit<uint16_t>(a, V, n, S.scan_tmp, &S.ct);
     } else {  // the tree here; cb_emit_kernel emits the codes on many CTAs afterwards
-      const CbArrays<unsigned> V = cb_big(a.big, S.wcnt);
-      const CbTileScratch ts = cb_tile_scratch(S);
-      codebook_lengths<unsigned>(a, V, n, S.scan_tmp, S.ka, passes, &ts);
+      CbBigSmem& L = *reinterpret_cast<CbBigSmem*>(smem_raw);
+      codebook_lengths_big(a, cb_big(a.big, L.wcnt), n, L, passes);
     }
     return;
   }
@@ -1501,14 +1568,13 @@ __device__ void codebook_block(const CodebookArgs& a) {
   __syncthreads();
   if (small) {
     const CbArrays<uint16_t> V = cb_small(S);
-    codebook_lengths<uint16_t>(a, V, n, S.scan_tmp, nullptr);
+    codebook_lengths(a, V, n, S.scan_tmp);
     codebook_emit<uint16_t>(a, V, n, S.scan_tmp, &S.ct);
   } else {
-    const CbArrays<unsigned> V = cb_big(a.big, S.wcnt);
-    // S.ka and S.iw (adjacent) stage the tiles
-    const CbTileScratch ts = cb_tile_scratch(S);
-    codebook_lengths<unsigned>(a, V, n, S.scan_tmp, S.ka, -1, &ts);
-    codebook_emit<unsigned>(a, V, n, S.scan_tmp, &S.ct);
+    CbBigSmem& L = *reinterpret_cast<CbBigSmem*>(smem_raw);
+    const CbArrays<unsigned> V = cb_big(a.big, L.wcnt);
+    codebook_lengths_big(a, V, n, L, -1);
+    codebook_emit<unsigned>(a, V, n, L.scan_tmp, &L.ct);
   }
 }
 
