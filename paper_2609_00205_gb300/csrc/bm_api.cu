@@ -2231,7 +2231,8 @@ bm_status launch_group(const BatchGroup& g, std::vector<BatchSlot>& slot, const 
   }
   for (size_t j = 0; j < nf; ++j) {
     hf[j].blk0 = nmax + nblk;
-    nblk += (unsigned long long)hf[j].a.nblocks;
+    const int nbg = sizeof(T) == 8 ? block_group(g.B) : 1;  // a ticket per group of blocks
+    nblk += (unsigned long long)((hf[j].a.nblocks + nbg - 1) / nbg);
   }
   BatchQueue q{};
   q.ticket = dticket;

@@ -665,12 +665,49 @@ __global__ void __launch_bounds__(BlockCfg<T, B, K>::NT_FWD, BlockCfg<T, B, K>::
   }
 }
 
+// Symbols and escapes of a block -> int32 codes in shared memory (the inverse
+// of store_codes): consecutive threads take consecutive groups of four, and a
+// group with an escape symbol loads its four escape-array entries as one
+// coalesced 16-byte load.
+template <int PB>
+__device__ __forceinline__ void load_codes(const uint16_t* __restrict__ sym, const int32_t* __restrict__ esc,
+                                           int32_t* __restrict__ st, const int radius) {
+  bool vec = false;
+  if constexpr (PB % 4 == 0)
+    vec = ((reinterpret_cast<uintptr_t>(sym) & 7) | (reinterpret_cast<uintptr_t>(esc) & 15)) == 0;
+  if (vec) {
+    const uint2* s2 = reinterpret_cast<const uint2*>(sym);
+    const int4* e4 = reinterpret_cast<const int4*>(esc);
+    int4* d4 = reinterpret_cast<int4*>(st);
+    for (int i = threadIdx.x; i < PB / 4; i += blockDim.x) {
+      const uint2 w = __ldg(s2 + i);
+      const int a0 = (int)(w.x & 0xFFFFu), a1 = (int)(w.x >> 16), a2 = (int)(w.y & 0xFFFFu), a3 = (int)(w.y >> 16);
+      int4 c = make_int4(0, 0, 0, 0);
+      if (!(a0 && a1 && a2 && a3)) c = __ldg(e4 + i);
+      d4[i] = make_int4(a0 ? a0 - radius : c.x, a1 ? a1 - radius : c.y, a2 ? a2 - radius : c.z,
+                        a3 ? a3 - radius : c.w);
+    }
+  } else {
+    for (int i = threadIdx.x; i < PB; i += blockDim.x) {
+      const int a = (int)sym[i];
+      st[i] = a ? a - radius : esc[i];
+    }
+  }
+}
+
+}  // namespace bm
+
+#include "bm_block_class.cuh"  // coded double fields
+
+namespace bm {
+
 // ---------------------------------------------------------------------------
 // Batched forward (Sec. III-B / III-D: many fields per launch): one persistent
 // launch drains a device-side queue of work items spanning every field of a
 // batch that shares (dtype, B, K).  Items are taken in ticket order from one
 // global counter: first the max|u| items of every field (a slice of
-// kBatchMaxChunk elements each), then one item per block.  The CTA that
+// kBatchMaxChunk elements each), then one item per block (double fields: per
+// group of block_group blocks).  The CTA that
 // finishes a field's last max|u| item computes that field's quantiser table
 // and raises its ready flag; a CTA taking a block of the field waits for the
 // flag (bounded, acquire).  Every max|u| item holds a lower ticket than every
@@ -684,7 +721,7 @@ struct BatchField {
   QtabArgs qa;                // its quantiser table (qa.sc: the field's scalars)
   int64_t nel;                // elements of the field
   unsigned long long max0;    // first max|u| ticket
-  unsigned long long blk0;    // first block ticket
+  unsigned long long blk0;    // first block (or group) ticket
 };
 
 struct BatchQueue {
@@ -726,8 +763,20 @@ __device__ __forceinline__ void maxabs_slice(const T* __restrict__ u, int64_t lo
   for (int64_t i = lo + h + nv * V + threadIdx.x; i < hi; i += blockDim.x) maxabs_acc(u[i], m, bad);
 }
 
+// Launch shape of the batched kernel and blocks per item.
 template <typename T, int B, int K>
-__global__ void __launch_bounds__(BlockCfg<T, B, K>::NT_FWD, BlockCfg<T, B, K>::FWD_MIN_CTAS)
+struct BatchCfg {
+  static constexpr int NB = 1, NT = BlockCfg<T, B, K>::NT_FWD, MIN_CTAS = BlockCfg<T, B, K>::FWD_MIN_CTAS;
+  static constexpr size_t smem = BlockCfg<T, B, K>::fwd_smem;
+};
+template <int B, int K>
+struct BatchCfg<double, B, K> {
+  static constexpr int NB = block_group(B), NT = GroupCfg<B, K>::NT_FWD, MIN_CTAS = GroupCfg<B, K>::FWD_MIN_CTAS;
+  static constexpr size_t smem = GroupCfg<B, K>::fwd_smem;
+};
+
+template <typename T, int B, int K>
+__global__ void __launch_bounds__(BatchCfg<T, B, K>::NT, BatchCfg<T, B, K>::MIN_CTAS)
     block_fwd_batch_kernel(const BatchField<T>* __restrict__ fields, BatchQueue q) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const FwdSmem<T, B, K> S(smem_raw);
@@ -735,7 +784,7 @@ __global__ void __launch_bounds__(BlockCfg<T, B, K>::NT_FWD, BlockCfg<T, B, K>::
   __shared__ int s_ok;
   __shared__ T s_m[32];
   __shared__ int s_bad;
-  fwd_init(S);
+  if constexpr (sizeof(T) == 4) fwd_init(S);
   unsigned phase = 0, centre = 0;
   while (true) {
     if (threadIdx.x == 0) s_t = atomicAdd(q.ticket, 1ull);
@@ -779,7 +828,7 @@ __global__ void __launch_bounds__(BlockCfg<T, B, K>::NT_FWD, BlockCfg<T, B, K>::
         }
       }
       __syncthreads();
-    } else {  // one block
+    } else {  // one block, or one group of blocks
       const int f = batch_field_of(fields, q.nfields, t, true);
       const BatchField<T>& F = fields[f];
       if (threadIdx.x == 0) {
@@ -799,38 +848,14 @@ __global__ void __launch_bounds__(BlockCfg<T, B, K>::NT_FWD, BlockCfg<T, B, K>::
       __syncthreads();
       if (!s_ok) continue;  // the field's table never came: reported, block skipped
       bool ovf = false;
-      if (!fwd_block<T, B, K, 0>(F.a, (int64_t)(t - F.blk0), S, phase, ovf, centre)) return;
+      if constexpr (sizeof(T) == 8) {
+        constexpr int NB = block_group(B);
+        const int64_t b = (int64_t)(t - F.blk0) * NB;
+        fwd_group<B, K>(F.a, b, (int)(F.a.nblocks - b < NB ? F.a.nblocks - b : NB), smem_raw, ovf);
+      } else {
+        if (!fwd_block<T, B, K, 0>(F.a, (int64_t)(t - F.blk0), S, phase, ovf, centre)) return;
+      }
       if (ovf) atomicOr(&F.a.sc->status, ST_OVERFLOW);
-    }
-  }
-}
-
-// Symbols and escapes of a block -> int32 codes in shared memory (the inverse
-// of store_codes): consecutive threads take consecutive groups of four, and a
-// group with an escape symbol loads its four escape-array entries as one
-// coalesced 16-byte load.
-template <int PB>
-__device__ __forceinline__ void load_codes(const uint16_t* __restrict__ sym, const int32_t* __restrict__ esc,
-                                           int32_t* __restrict__ st, const int radius) {
-  bool vec = false;
-  if constexpr (PB % 4 == 0)
-    vec = ((reinterpret_cast<uintptr_t>(sym) & 7) | (reinterpret_cast<uintptr_t>(esc) & 15)) == 0;
-  if (vec) {
-    const uint2* s2 = reinterpret_cast<const uint2*>(sym);
-    const int4* e4 = reinterpret_cast<const int4*>(esc);
-    int4* d4 = reinterpret_cast<int4*>(st);
-    for (int i = threadIdx.x; i < PB / 4; i += blockDim.x) {
-      const uint2 w = __ldg(s2 + i);
-      const int a0 = (int)(w.x & 0xFFFFu), a1 = (int)(w.x >> 16), a2 = (int)(w.y & 0xFFFFu), a3 = (int)(w.y >> 16);
-      int4 c = make_int4(0, 0, 0, 0);
-      if (!(a0 && a1 && a2 && a3)) c = __ldg(e4 + i);
-      d4[i] = make_int4(a0 ? a0 - radius : c.x, a1 ? a1 - radius : c.y, a2 ? a2 - radius : c.z,
-                        a3 ? a3 - radius : c.w);
-    }
-  } else {
-    for (int i = threadIdx.x; i < PB; i += blockDim.x) {
-      const int a = (int)sym[i];
-      st[i] = a ? a - radius : esc[i];
     }
   }
 }

@@ -121,7 +121,8 @@ constexpr BlockLevel<T, N> make_block_level() {
 
 // Restriction + tridiagonal solve of one line held in registers:
 // z = M_c^{-1} (I^T M_f d), all coefficients compile-time constants.
-template <typename T, int N, class Tab>
+// ODD: the even nodes' values are zero (all-coarse lines) and left out.
+template <typename T, int N, bool ODD = false, class Tab>
 __device__ __forceinline__ void restrict_solve(const Tab& tb, const T (&d)[N], T (&z)[(N + 1) / 2]) {
   constexpr int C = (N + 1) / 2;
   T r[C];
@@ -131,7 +132,7 @@ __device__ __forceinline__ void restrict_solve(const Tab& tb, const T (&d)[N], T
 #pragma unroll
     for (int m = 0; m < 5; ++m) {
       const int col = 2 * J - 2 + m;
-      if (col >= 0 && col < N) s = fma(tb.rs[J][m], d[col], s);
+      if (col >= 0 && col < N && (!ODD || (col & 1))) s = fma(tb.rs[J][m], d[col], s);
     }
     r[J] = s;
   }
@@ -151,13 +152,30 @@ __device__ __forceinline__ int quantize(float c, float rq, bool& ovf) {
   if (!(fabsf(y) < 1073741824.0f)) { ovf = true; return 0; }
   return __float2int_rd(y);
 }
+// Double precision on this GPU runs at two lanes a clock and SM, comparisons
+// and conversions included (16 to 19 cycles a warp instruction), so only the
+// multiply-add is taken there: the range check and the floor work on y's bits
+// (y is never -0: an exact zero sum of the multiply-add is +0).
 __device__ __forceinline__ int quantize(double c, double rq, bool& ovf) {
   const double y = __fma_rn(c, rq, 0.5);
-  if (!(fabs(y) < 1073741824.0)) { ovf = true; return 0; }
-  return __double2int_rd(y);
+  const unsigned hi = (unsigned)__double2hiint(y), lo = (unsigned)__double2loint(y);
+  const unsigned ex = (hi >> 20) & 0x7FFu;
+  if (ex >= 1023u + 30u) { ovf = true; return 0; }  // |y| >= 2^30, an infinity or NaN
+  const unsigned top = (hi << 11) | (lo >> 21) | 0x80000000u;  // the mantissa's first 32 bits
+  const unsigned sh = 1023u + 31u - ex;                         // at least 2
+  const unsigned ip = __funnelshift_rc(top, 0u, sh);            // integer part of |y| (0 from a shift of 32 on)
+  const bool frac = ((__funnelshift_lc(0u, ip, sh) ^ top) | (lo << 11)) != 0u;
+  return (int)hi < 0 ? (int)~(frac ? ip : ip - 1u) : (int)ip;
 }
 __device__ __forceinline__ float dequant(int code, float q) { return __int2float_rn(code) * q; }
-__device__ __forceinline__ double dequant(int code, double q) { return __int2double_rn(code) * q; }
+// The code's double built from its bits (exact: 32 bits fit the mantissa).
+__device__ __forceinline__ double dequant(int code, double q) {
+  const unsigned m = code < 0 ? 0u - (unsigned)code : (unsigned)code;
+  const int lz = __clz((int)m);
+  const unsigned n = m << (lz & 31);  // leading one at bit 31
+  const unsigned hi = ((unsigned)code & 0x80000000u) | (((unsigned)(1023 + 31 - lz) << 20) + ((n << 1) >> 12));
+  return (m ? __hiloint2double((int)hi, (int)(n << 21)) : 0.0) * q;
+}
 
 // Asynchronous global->shared copy of one element with zero fill
 // (cp.async; src_bytes = 0 fills zeros without reading).
