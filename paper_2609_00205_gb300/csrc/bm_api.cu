@@ -22,6 +22,7 @@
 #include "bm_huffman.cuh"
 #include "bm_internal.h"
 #include "bm_plan.h"
+#include "bm_plane.h"
 #include "bm_qtab.cuh"
 
 #ifndef BM_FWD_HIST
@@ -1004,6 +1005,27 @@ std::vector<T*> round_grids(const PlanHost& h, Carver& cv, T* last) {
   return g;
 }
 
+// The fused 2-D kernels' arguments that both directions share.
+template <typename T>
+PlaneArgs<T> plane_args(PlanDev& P, T* field, T* G) {
+  const PlanHost& h = P.h;
+  PlaneArgs<T> a{};
+  a.field = field;
+  a.G = G;
+  const int64_t fs[3] = {h.shape[1] * h.shape[2], h.shape[2], 1}, gs[3] = {h.gshape[1] * h.gshape[2], h.gshape[2], 1};
+  const int x0 = h.ax[0], x1 = h.ax[1];
+  a.e0 = h.shape[x0]; a.e1 = h.shape[x1]; a.st0 = fs[x0]; a.st1 = fs[x1];
+  a.gs0 = gs[x0]; a.gs1 = gs[x1];
+  a.nb1 = h.nb[x1];
+  a.nblocks = h.nblocks;
+  auto& RL = rlevels<T>(P);
+  for (int l = 0; l < h.K && l < 4; ++l) {
+    const GDim<T>& D = RL[(size_t)l].d[2];
+    a.lev[l] = {D.band, D.tm, D.tib, D.tsup};
+  }
+  return a;
+}
+
 // What run_decompose does with the fused In-cache Block stage: launch it,
 // only record its arguments (and return before any launch), or skip it (the
 // batched forward kernel ran it).
@@ -1022,7 +1044,13 @@ bm_status run_decompose(PlanDev& P, const T* field, int mode, const FwdOut<T>& o
   T* W1 = cv.take<T>((size_t)std::max<int64_t>(gs.W1, 1));
   T* W2 = cv.take<T>((size_t)std::max<int64_t>(gs.W2, 1));
   std::vector<T*> Gr = round_grids<T>(h, cv, U[0]);
-  if (h.reduced) {  // a field with an extent of 1: in-cache levels on the block-major grid
+  if (h.reduced && mode == 0 && plane_fused(h.ax[0] >= 0, h.B, h.K)) {  // 2-D: fused blocks
+    Stage st("incache_decompose");
+    PlaneArgs<T> a = plane_args<T>(P, const_cast<T*>(field), Gr[0]);
+    a.sym = o.sym; a.esc = o.esc; a.tier = o.tier; a.rq = o.rq; a.radius = o.radius; a.ntiers = o.ntiers; a.sc = o.sc;
+    BM_CUDA(launch_plane(0, h.B, h.K, a, s, num_sms()));
+    BM_LAUNCHED();
+  } else if (h.reduced) {  // a field with an extent of 1: in-cache levels on the block-major grid
     Stage st("incache_decompose");
     std::vector<T*> RB;
     for (int64_t n : gs.RB) RB.push_back(cv.take<T>((size_t)n));
@@ -1192,7 +1220,14 @@ bm_status run_recompose(PlanDev& P, T* field, int mode, const InvIn<T>& in, Carv
     g_launches.fetch_add(5);
     BM_CUDA(cudaGetLastError());
   }
-  if (h.reduced) {
+  if (h.reduced && mode == 0 && plane_fused(h.ax[0] >= 0, h.B, h.K)) {
+    Stage st("incache_recompose");
+    PlaneArgs<T> a = plane_args<T>(P, field, Gr[0]);
+    a.sym = const_cast<uint16_t*>(in.sym); a.esc = const_cast<int32_t*>(in.esc); a.tier = in.tier; a.q = in.q;
+    a.radius = in.radius; a.ntiers = in.ntiers; a.sc = in.sc;
+    BM_CUDA(launch_plane(1, h.B, h.K, a, s, num_sms()));
+    BM_LAUNCHED();
+  } else if (h.reduced) {
     Stage st("incache_recompose");
     std::vector<T*> RB;
     for (int64_t n : gs.RB) RB.push_back(cv.take<T>((size_t)n));
