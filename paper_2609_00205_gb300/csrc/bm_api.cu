@@ -705,6 +705,7 @@ struct HeaderArgs {
   unsigned long long n_symbols, n_chunks, off_tiers, off_qtab, off_btier, off_chunks, off_splits, off_codebook;
   unsigned long long raw_total, capacity;
   Scalars* sc;
+  Scalars* host;  // device-side address of the call's pinned copy of the scalars
 };
 
 template <typename V>
@@ -712,8 +713,7 @@ __device__ __forceinline__ void put(uint8_t* p, size_t off, V v) { *reinterpret_
 
 // Header of a coded stream; also zeroes the padding after the bitstream and
 // the outlier section.
-__global__ void header_kernel(HeaderArgs a) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+__device__ __forceinline__ void write_header(const HeaderArgs& a) {
   Scalars* sc = a.sc;
   encode_finish(a.raw_total, a.capacity, sc);
   if (sc->status & ST_RAW) return;
@@ -759,6 +759,16 @@ __global__ void header_kernel(HeaderArgs a) {
   for (unsigned long long i = oend; i < sc->off_bits; ++i) o[i] = 0;
   const unsigned long long wend = sc->off_bits + 4ull * sc->n_words;
   for (unsigned long long i = wend; i < sc->total; ++i) o[i] = 0;
+}
+
+// One warp; the scalars, final with the header, go to the host's copy.
+__global__ void header_kernel(HeaderArgs a) {
+  if (threadIdx.x == 0) write_header(a);
+  __syncwarp();
+  static_assert(sizeof(Scalars) % 8 == 0, "the scalars are copied in 8-byte words");
+  const volatile unsigned long long* src = reinterpret_cast<const volatile unsigned long long*>(a.sc);
+  unsigned long long* dst = reinterpret_cast<unsigned long long*>(a.host);
+  for (int i = threadIdx.x; i < (int)(sizeof(Scalars) / 8); i += 32) dst[i] = src[i];
 }
 
 __global__ void raw_header_kernel(uint8_t* o, int f64, int B, int64_t s0, int64_t s1, int64_t s2, int rel, double tol,
@@ -1725,24 +1735,29 @@ bm_status compress_t(const T* field, const int64_t* shape, const Params& prm, do
     ea.chunk_words = reinterpret_cast<unsigned*>(out + L.off_chunks);
     ea.splits = reinterpret_cast<uint16_t*>(out + L.off_splits);
     ea.out = out; ea.capacity = cap; ea.sc = sc;
-    // the codebook picked one of three variants (the others return at once):
-    // every symbol in a small window, two CTAs of eight warps per SM; every
-    // symbol in the large window, or the split table of the whole dictionary,
-    // one CTA of kEncWarps warps per SM
-    constexpr int ew = kEncWarps * 32;
-    const int eg = grid_for((int64_t)L.nch * 32, ew, 1);
-    const size_t m0 = enc_smem<0>(8, kEncWinSmall, dict), m3 = enc_smem<3>(kEncWarps, kEncWin, dict),
-                 m2 = enc_smem<2>(kEncWarps, 0, dict);
-    BM_CUDA(set_smem_once(encode_fused_kernel<8, false, 0>, (int)m0, g_enc0_attr));
-    BM_CUDA(set_smem_once(encode_fused_kernel<kEncWarps, false, 3>, (int)m3, g_enc3_attr));
-    BM_CUDA(set_smem_once(encode_fused_kernel<kEncWarps, false, 2>, (int)enc_smem<2>(kEncWarps, 0, kMaxDict), g_enc2_attr));
-    FusedEncodeArgs e0 = ea, e3 = ea;
-    e0.win = kEncWinSmall;
-    e3.win = kEncWin;
-    encode_fused_kernel<8, false, 0><<<grid_for((int64_t)L.nch * 32, 256, 4), 256, m0, s>>>(e0);
-    encode_fused_kernel<kEncWarps, false, 3><<<eg, ew, m3, s>>>(e3);
-    encode_fused_kernel<kEncWarps, false, 2><<<eg, ew, m2, s>>>(ea);
-    g_launches.fetch_add(3);
+    if (L.nch <= (unsigned long long)kEncSmallChunks * num_sms()) {
+      encode_small_kernel<<<grid_for((int64_t)L.nch * 32, 256, 1), 256, kEncSmallSmem, s>>>(ea);
+      g_launches.fetch_add(1);
+    } else {
+      // the codebook picked one of three variants (the others return at once):
+      // every symbol in a small window, two CTAs of eight warps per SM; every
+      // symbol in the large window, or the split table of the whole dictionary,
+      // one CTA of kEncWarps warps per SM
+      constexpr int ew = kEncWarps * 32;
+      const int eg = grid_for((int64_t)L.nch * 32, ew, 1);
+      const size_t m0 = enc_smem<0>(8, kEncWinSmall, dict), m3 = enc_smem<3>(kEncWarps, kEncWin, dict),
+                   m2 = enc_smem<2>(kEncWarps, 0, dict);
+      BM_CUDA(set_smem_once(encode_fused_kernel<8, false, 0>, (int)m0, g_enc0_attr));
+      BM_CUDA(set_smem_once(encode_fused_kernel<kEncWarps, false, 3>, (int)m3, g_enc3_attr));
+      BM_CUDA(set_smem_once(encode_fused_kernel<kEncWarps, false, 2>, (int)enc_smem<2>(kEncWarps, 0, kMaxDict), g_enc2_attr));
+      FusedEncodeArgs e0 = ea, e3 = ea;
+      e0.win = kEncWinSmall;
+      e3.win = kEncWin;
+      encode_fused_kernel<8, false, 0><<<grid_for((int64_t)L.nch * 32, 256, 4), 256, m0, s>>>(e0);
+      encode_fused_kernel<kEncWarps, false, 3><<<eg, ew, m3, s>>>(e3);
+      encode_fused_kernel<kEncWarps, false, 2><<<eg, ew, m2, s>>>(ea);
+      g_launches.fetch_add(3);
+    }
   }
   {
     Stage st("finish");
@@ -1754,15 +1769,13 @@ bm_status compress_t(const T* field, const int64_t* shape, const Params& prm, do
     ha.tol = tol; ha.n_symbols = (unsigned long long)h.n_coeffs; ha.n_chunks = L.nch;
     ha.off_tiers = L.off_tiers; ha.off_qtab = L.off_qtab; ha.off_btier = ntiers > 1 ? L.off_btier : L.off_chunks;
     ha.off_chunks = L.off_chunks; ha.off_splits = L.off_splits; ha.off_codebook = L.off_codebook; ha.sc = sc;
+    ha.host = reinterpret_cast<Scalars*>(hpd);
     header_kernel<<<1, 32, 0, s>>>(ha);
     // a raw fallback is written on the device in the same pass (no second host round trip)
     raw_stream_kernel<T><<<mgrid, 256, 0, s>>>(out, field, nel, f64, h.B, shape[0], shape[1], shape[2], rel, tol,
                                                raw_total, sc, prm.ndim);
     g_launches.fetch_add(2);
     BM_CUDA(cudaGetLastError());
-    Spans back;
-    back.add(hpd, sc, sizeof(Scalars));
-    BM_CUDA(back.launch(s));
   }
   if (bs) {  // the batch reads the result after its single synchronisation
     bs->raw_now = false;

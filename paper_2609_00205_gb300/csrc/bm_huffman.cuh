@@ -1823,29 +1823,41 @@ constexpr int enc_group(int warps) { return warps > 8 ? 4 : 8; }
 //   2     the whole dictionary split into the symbol's rank among the codes of
 //         its length (u16, `low`) and the length (u8, `len`): any code is
 //         first_code[len] + rank, with the left-justified first codes in `fc`.
+// and, left in global memory (encode_small_kernel):
+//   4     the whole dictionary, one enc_entry per symbol, as in 0 and 3;
+//   5     its lengths and codes, split as in 2 at the look-up.
+constexpr bool enc_split(int mode) { return mode == 2 || mode == 5; }
 template <int MODE, bool CLAMP>
 struct EncTab {
   const unsigned* ent;
   const uint16_t* low;
   const uint8_t* len;
   const unsigned* fc;  // [kMaxLen + 1] first codes, left-justified
+  const unsigned* codes;       // mode 5
+  const unsigned* first_code;
   unsigned lo;
   // What a symbol's look-up keeps in a register: the window's entry, or
   // rank | len << 16.
   __device__ __forceinline__ unsigned entry(unsigned s) const {
     if (MODE == 2) return (unsigned)low[s] | ((unsigned)len[s] << 16);
+    if (MODE == 5) {
+      const unsigned L = len[s];
+      return ((codes[s] - first_code[L]) & 0xFFFFu) | (L << 16);
+    }
     return ent[s - lo];
   }
-  __device__ __forceinline__ unsigned length(unsigned s) const { return MODE == 2 ? (unsigned)len[s] : ent[s - lo] & 31u; }
+  __device__ __forceinline__ unsigned length(unsigned s) const {
+    return enc_split(MODE) ? (unsigned)len[s] : ent[s - lo] & 31u;
+  }
   // Symbol i of a lane's eight.
   __device__ __forceinline__ static unsigned symbol(const unsigned (&w)[4], int i, unsigned dmax) {
     const unsigned s = (i & 1) ? w[i >> 1] >> 16 : w[i >> 1] & 0xFFFFu;
     return CLAMP ? min(s, dmax) : s;
   }
-  __device__ __forceinline__ static unsigned bits(unsigned e) { return MODE == 2 ? e >> 16 : e & 31u; }
+  __device__ __forceinline__ static unsigned bits(unsigned e) { return enc_split(MODE) ? e >> 16 : e & 31u; }
   // The code left-justified in 32 bits.
   __device__ __forceinline__ unsigned code(unsigned e, unsigned L) const {
-    if (MODE == 2) return fc[L] + ((e & 0xFFFFu) << (32u - L));
+    if (enc_split(MODE)) return fc[L] + ((e & 0xFFFFu) << (32u - L));
     return e & ~31u;
   }
 };
@@ -1854,7 +1866,10 @@ struct EncTab {
 constexpr int kEncStage = 260;
 template <int MODE>
 __host__ __device__ constexpr size_t enc_table_bytes(int win, int dict) {
-  return MODE == 2 ? (size_t)(dict + 7) / 8 * 8 * 3 + 4 * (kMaxLen + 4) : 4 * (size_t)win;
+  return MODE == 2 ? (size_t)(dict + 7) / 8 * 8 * 3 + 4 * (kMaxLen + 4)
+         : MODE == 5 ? 4 * (kMaxLen + 4)
+         : MODE == 4 ? 0
+                     : 4 * (size_t)win;
 }
 template <int MODE>
 __host__ __device__ constexpr size_t enc_smem(int warps, int win, int dict) {
@@ -2005,18 +2020,12 @@ __device__ __forceinline__ void enc_outliers(const int32_t* __restrict__ esc, in
 // 1e-3 / 1e-4 / 1e-5: 0.33 / 0.377 / 0.53 / 0.95 ms before, 0.26 / 0.284 /
 // 0.397 / 0.502 now.
 template <int WARPS, bool CLAMP, int MODE>
-__global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) encode_fused_kernel(FusedEncodeArgs a) {
+__device__ __forceinline__ void encode_tiles(const FusedEncodeArgs& a) {
   extern __shared__ __align__(16) unsigned char enc_smem_raw[];
   constexpr int kEncGroup = enc_group(WARPS), NG = WARPS / kEncGroup;
   __shared__ unsigned s_tile[NG], s_w[NG][kEncGroup], s_e[NG][kEncGroup], s_ok[NG];
   __shared__ unsigned long long s_base[NG][2];
   Scalars* sc = a.sc;
-  if (sc->skip) return;  // the stream is already known to be a raw copy
-  if (CLAMP) {
-    if ((a.dict <= kEncWinSmall && sc->max_len <= kPackLen) != (MODE == 0)) return;
-  } else if ((unsigned)MODE != sc->enc_mode) {
-    return;
-  }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   EncTab<MODE, CLAMP> tab{};
   if (MODE == 2) {
@@ -2033,6 +2042,16 @@ __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) encode_fused_kernel(Fu
     tab.low = low;
     tab.len = len;
     tab.fc = fc;
+  } else if (MODE == 5) {
+    unsigned* fc = reinterpret_cast<unsigned*>(enc_smem_raw);
+    if (threadIdx.x <= kMaxLen) fc[threadIdx.x] = threadIdx.x ? a.first_code[threadIdx.x] << (32 - threadIdx.x) : 0u;
+    tab.len = a.lens;
+    tab.codes = a.codes;
+    tab.first_code = a.first_code;
+    tab.fc = fc;
+  } else if (MODE == 4) {
+    tab.ent = a.packed;
+    tab.lo = 0;
   } else {
     unsigned* ent = reinterpret_cast<unsigned*>(enc_smem_raw);
     const unsigned wlo = CLAMP ? 0u : sc->enc_lo;
@@ -2255,7 +2274,34 @@ __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) encode_fused_kernel(Fu
   }
 }
 
-// After the fused encoder (one thread): stream length and the raw decision.
+// One table: returns at once unless the codebook picked it.
+template <int WARPS, bool CLAMP, int MODE>
+__global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) encode_fused_kernel(FusedEncodeArgs a) {
+  const Scalars* sc = a.sc;
+  if (sc->skip) return;  // the stream is already known to be a raw copy
+  if (CLAMP) {
+    if ((a.dict <= kEncWinSmall && sc->max_len <= kPackLen) != (MODE == 0)) return;
+  } else if ((unsigned)MODE != sc->enc_mode) {
+    return;
+  }
+  encode_tiles<WARPS, CLAMP, MODE>(a);
+}
+
+// Any codebook, a stream of at most kEncSmallChunks chunks per SM: the table
+// stays in global memory (and what the symbols meet of it in L1), as a CTA
+// codes too few symbols to pay for a copy of it, and a CTA of eight warps
+// takes 8.5 KB of shared memory, so that the items of a batch share an
+// SM.  In place of the three launches above, two of which return at once (but
+// wait for an SM with 200 KB of free shared memory to do so): 64 fields of up
+// to 64^3 in a batch 4.60 ms against 4.45, 65^3 0.195 ms against 0.176; with the
+// tables copied by one kernel of any mode 5.57 and 0.181.
+constexpr int kEncSmallChunks = 8;
+constexpr size_t kEncSmallSmem = enc_smem<5>(8, 0, 0);
+__global__ void __launch_bounds__(256) encode_small_kernel(FusedEncodeArgs a) {
+  if (a.sc->skip) return;  // the stream is already known to be a raw copy
+  if (a.sc->max_len <= kPackLen) encode_tiles<8, false, 4>(a);
+  else encode_tiles<8, false, 5>(a);
+}
 __device__ __forceinline__ void encode_finish(unsigned long long raw_total, unsigned long long capacity, Scalars* sc) {
   if (sc->skip) return;  // already raw
   const unsigned long long total = sc->off_bits + pad8(4ull * sc->n_words);

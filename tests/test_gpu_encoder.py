@@ -49,3 +49,39 @@ def test_codes_longer_than_a_window_entry(dict_size):
     sym = np.repeat(np.arange(3, 3 + len(f)), f).astype(np.uint16)
     rng.shuffle(sym)
     _check(sym, dict_size, 2048)
+
+
+def test_short_stream_with_codes_too_long_for_an_entry():
+    """A stream short enough for the encoder without a table of its own, whose
+    codes are up to 28 bits: 29 values with Fibonacci counts."""
+    import paper_2609_00205_gb300 as bm
+
+    shape, B, K, M = (119, 119, 119), 17, 2, 1
+    n = bm.coeff_count(shape, B, K, M)
+    fib = [1, 1]
+    while len(fib) < 29:
+        fib.append(fib[-1] + fib[-2])
+    values = np.repeat(np.arange(29) - 14, fib)
+    codes = np.full(n, 14, np.int64)  # the most frequent
+    codes[: values.size] = values
+    codes = np.random.default_rng(0).permutation(codes)
+    # the bin widths of the levels, from a stream of the same shape and tolerance
+    probe = bm.compress(torch.from_numpy(np.random.default_rng(1).normal(size=shape)).to("cuda"), 1.0, mode="abs",
+                        block=B, levels=K, global_levels=M).cpu().numpy()
+    h = oracle.stream_header(probe)
+    q = probe[h["off_qtab"]:][: 8 * (K + M + 1)].view("<f8")
+    per = [B ** 3 - 9 ** 3, 9 ** 3 - 5 ** 3]
+    nb = 7 ** 3
+    width = np.tile(np.repeat(q[:K], per), nb)
+    gcount = 35 ** 3 - 18 ** 3
+    width = np.concatenate([width, np.full(gcount, q[K]), np.full(n - width.size - gcount, q[K + 1])])
+    u = bm.recompose(torch.from_numpy(codes * width).to("cuda"), shape, B, K, M)
+    s = bm.compress(u, 1.0, mode="abs", block=B, levels=K, global_levels=M)
+    got = bm.stream_codes(s).cpu().numpy()
+    np.testing.assert_array_equal(got, codes)  # the bins are far wider than the roundings
+    hs = oracle.stream_header(s.cpu().numpy())
+    so, mo = oracle.huffman_encode((codes + 32768).astype(np.uint16), 65536, 2048)
+    assert mo["n_words"] == hs["n_words"] and mo["n_runs"] == hs["n_runs"]
+    words = s.cpu().numpy()[hs["off_bits"]:][: 4 * hs["n_words"]]
+    off = sum(-(-b // 8) * 8 for b in (4 * mo["n_chunks"], 14 * mo["n_chunks"], mo["codebook_bytes"]))
+    np.testing.assert_array_equal(words, so[off:][: 4 * mo["n_words"]])
