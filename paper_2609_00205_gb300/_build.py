@@ -25,6 +25,8 @@ CU_SOURCES = [
     "bm_block_f64_b17.cu",
     "bm_adjoint_f32.cu",
     "bm_adjoint_f64.cu",
+    "bm_levels_f32.cu",
+    "bm_levels_f64.cu",
     "bm_plane.cu",
 ]
 CPP_SOURCES = ["bm_plan.cpp"]

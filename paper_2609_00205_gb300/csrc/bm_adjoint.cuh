@@ -266,7 +266,7 @@ cudaError_t launch_adj_one(int dir, const BlockArgs<T>& a, cudaStream_t s, int n
 }
 
 // ---------------------------------------------------------------------------
-// Global levels (physical coordinates, plan tables), one thread per line
+// Global levels (physical coordinates, plan tables)
 // ---------------------------------------------------------------------------
 
 // A line pass along one dimension between a grid with n nodes on it (fine
@@ -285,24 +285,212 @@ LineShape line_shape(const GLevel<T>& L, int dim) {
   return LineShape{A.nb, A.ncol, A.in_b, A.in_i, A.in_c, A.out_b, A.out_j, A.out_c};
 }
 
-// fine line = M_f I M_c^-1 (coarse line): Thomas sweeps with the coarse
-// values kept in the fine line's coarse slots, then the fine slots by
-// interpolation, then the mass matrix with a rolling window (in place).
+// What an expansion does with t = (M_f I M_c^-1 x) at a fine node: EXP_STORE
+// stores it; the last (dim 2) pass of the transposed decomposition writes
+// v = S_F^T g_D + t (EXP_ADD), that of the transposed recomposition the
+// coefficient gradient g_u - t (EXP_COEF).
+enum { EXP_STORE = 0, EXP_ADD = 1, EXP_COEF = 2 };
+
+template <typename T, int FIN>
+__device__ __forceinline__ void expand_emit(const GLevel<T>& L, const LineShape& S, T* fine, const T* g, T* coef,
+                                            int64_t b, int64_t col, int i, T t) {
+  const int64_t o = b * S.f_b + (int64_t)i * S.f_i + col * S.f_c;
+  if (FIN == EXP_STORE) {
+    fine[o] = t;
+    return;
+  }
+  const int n1 = L.d[1].n, i0 = (int)(col / n1), i1 = (int)(col - (int64_t)i0 * n1);
+  const bool cc = all_coarse(L, i0, i1, i);
+  const int64_t pos = cc ? 0 : nc_pos(L, i0, i1, i, o);
+  if (FIN == EXP_ADD) fine[o] = (cc ? T(0) : coef[pos]) + t;
+  else if (!cc) coef[pos] = g[o] - t;
+}
+
+__device__ __forceinline__ float rn_mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double rn_mul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float rn_add(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double rn_add(double a, double b) { return __dadd_rn(a, b); }
+
+// A value with its rounding error, hi + lo (error-free sum and product as in
+// T. J. Dekker, "A floating-point technique for extending the available
+// precision", 1971, and D. E. Knuth's two-sum).
 template <typename T>
-__global__ void __launch_bounds__(256) gl_expand(GDim<T> D, LineShape S, const T* __restrict__ coarse,
-                                                  T* __restrict__ fine) {
+struct HiLo {
+  T hi, lo;
+};
+// m * a + b
+template <typename T>
+__device__ __forceinline__ HiLo<T> hl_affine(T m, HiLo<T> a, HiLo<T> b) {
+  const T p = rn_mul(m, a.hi), pe = fma(m, a.hi, -p);
+  const T s = rn_add(p, b.hi), v = rn_add(s, -p);
+  const T e = rn_add(rn_add(p, -rn_add(s, -v)), rn_add(b.hi, -v));
+  return {s, fma(m, a.lo, rn_add(rn_add(pe, e), b.lo))};
+}
+
+// z = M_c^-1 r of one line in shared memory, in place, by a warp: the scans
+// of line_scan_solve with the value part of the maps carried with its rounding
+// error, so that every lane replays its rows from a rounded exact input.  The
+// plain scan's error against wider arithmetic is up to 3% larger than that of
+// the serial recurrences (4.49e-8 against 4.35e-8 relative at 32 rows in FP32,
+// 8.61e-17 against 8.37e-17 in FP64); this one's is not larger (4.31e-8,
+// 8.27e-17).
+template <typename T, int E>
+__device__ __forceinline__ void line_scan_solve_hl(const GDim<T>& D, T* r, const int lane) {
+  const int c = D.c;
+  const int j0 = lane * E;
+  T y[E];
+  HiLo<T> a{T(0), T(0)};
+  T m = T(1);
+#pragma unroll
+  for (int k = 0; k < E; ++k) {
+    const int J = j0 + k;
+    if (J < c) {
+      const T t = -D.tm[J];
+      a = hl_affine(t, a, HiLo<T>{r[J], T(0)});
+      m = t * m;
+    }
+  }
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const HiLo<T> pa{__shfl_up_sync(0xffffffffu, a.hi, off), __shfl_up_sync(0xffffffffu, a.lo, off)};
+    const T pm = __shfl_up_sync(0xffffffffu, m, off);
+    if (lane >= off) {
+      a = hl_affine(m, pa, a);
+      m *= pm;
+    }
+  }
+  T prev = __shfl_up_sync(0xffffffffu, rn_add(a.hi, a.lo), 1);
+  if (lane == 0) prev = T(0);
+#pragma unroll
+  for (int k = 0; k < E; ++k) {
+    const int J = j0 + k;
+    if (J < c) {
+      y[k] = fma(-D.tm[J], prev, r[J]);
+      prev = y[k];
+    }
+  }
+  a = {T(0), T(0)};
+  m = T(1);
+#pragma unroll
+  for (int k = E - 1; k >= 0; --k) {
+    const int J = j0 + k;
+    if (J < c) {
+      const T ib = D.tib[J], t = -D.tsup[J];
+      const HiLo<T> v = hl_affine(t, a, HiLo<T>{y[k], T(0)});
+      a.hi = rn_mul(v.hi, ib);
+      a.lo = fma(v.lo, ib, fma(v.hi, ib, -a.hi));
+      m = t * ib * m;
+    }
+  }
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const HiLo<T> pa{__shfl_down_sync(0xffffffffu, a.hi, off), __shfl_down_sync(0xffffffffu, a.lo, off)};
+    const T pm = __shfl_down_sync(0xffffffffu, m, off);
+    if (lane + off < 32) {
+      a = hl_affine(m, pa, a);
+      m *= pm;
+    }
+  }
+  T next = __shfl_down_sync(0xffffffffu, rn_add(a.hi, a.lo), 1);
+  if (lane == 31) next = T(0);
+  __syncwarp();  // every lane has read its r before any z overwrites it
+#pragma unroll
+  for (int k = E - 1; k >= 0; --k) {
+    const int J = j0 + k;
+    if (J < c) {
+      next = fma(-D.tsup[J], next, y[k]) * D.tib[J];
+      r[J] = next;
+    }
+  }
+}
+
+// fine line = M_f I M_c^-1 (coarse line), line by line along dimension DIM.
+// A CTA stages 2^lsh coarse lines in shared memory (shared memory and line
+// counts as for gl_line); a warp solves a line with the scans of
+// line_scan_solve_hl and interpolates it to the fine nodes, and the mass matrix
+// is applied as the lines are written.  Bound by latency: the chain of a line
+// is O(log) steps instead of the 2 c of a Thomas sweep, and a line is a warp's
+// work instead of a thread's.  (With a thread per line, 2 to 25 CTAs, the six
+// expansions of a 257^3 field's two levels took 194 us; now 56.)
+template <typename T, int DIM, int FIN, int E>
+__global__ void __launch_bounds__(256) gl_expand(GLevel<T> L, LineShape S, const T* __restrict__ coarse,
+                                                 T* __restrict__ fine, const T* __restrict__ g, T* __restrict__ coef,
+                                                 const int lsh) {
+  const int LT = 1 << lsh;  // lines of the CTA
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const GDim<T>& D = L.d[DIM];
+  const int n = D.n, c = D.c, sn = n | 1, sc = c | 1;
+  T* s_f = reinterpret_cast<T*>(smem_raw);  // [LT][sn] I M_c^-1 x
+  T* s_c = s_f + LT * sn;                   // [LT][sc] x, then M_c^-1 x
+  const int64_t tiles = (S.ncol + LT - 1) / LT;
+  const int64_t b = blockIdx.x / tiles;
+  const int64_t col0 = (blockIdx.x - b * tiles) * LT;
+  const int nl = (int)(S.ncol - col0 < LT ? S.ncol - col0 : LT);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const T* x = coarse + b * S.c_b;
+  if (S.c_i == 1) {
+    for (int w = warp; w < nl; w += 8)
+      for (int J = lane; J < c; J += 32) s_c[w * sc + J] = x[(col0 + w) * S.c_c + J];
+  } else {
+    for (int e = threadIdx.x; e < c * LT; e += 256) {
+      const int J = e >> lsh, w = e - (J << lsh);
+      if (w < nl) s_c[w * sc + J] = x[(int64_t)J * S.c_i + (col0 + w) * S.c_c];
+    }
+  }
+  __syncthreads();
+  const bool same = c == n;  // a dimension of at most two nodes is not coarsened
+  if (!same) {
+    for (int w = warp; w < nl; w += 8) {
+      T* z = s_c + w * sc;
+      line_scan_solve_hl<T, E>(D, z, lane);
+      __syncwarp();
+      for (int i = lane; i < n; i += 32) {
+        const T zl = z[D.jlo[i]], zr = z[D.jhi[i]];
+        s_f[w * sn + i] = D.isc[i] ? zl : fma(D.wl[i], zl, D.wr[i] * zr);
+      }
+    }
+    __syncthreads();
+  }
+  auto emit = [&](int i, int w) {
+    T t;
+    if (same) {
+      t = s_c[w * sc + i];
+    } else {
+      const T* y = s_f + w * sn;
+      t = D.md[i] * y[i];
+      if (i > 0) t = fma(D.mo[i - 1], y[i - 1], t);
+      if (i + 1 < n) t = fma(D.mo[i], y[i + 1], t);
+    }
+    expand_emit<T, FIN>(L, S, fine, g, coef, b, col0 + w, i, t);
+  };
+  if (S.f_i == 1) {
+    for (int w = warp; w < nl; w += 8)
+      for (int i = lane; i < n; i += 32) emit(i, w);
+  } else {
+    for (int e = threadIdx.x; e < n * LT; e += 256) {
+      const int i = e >> lsh, w = e - (i << lsh);
+      if (w < nl) emit(i, w);
+    }
+  }
+}
+
+// The expansion of lines too long for gl_expand's segments and shared memory
+// (more than 544 coarse nodes), one thread per line: Thomas sweeps with the
+// coarse values kept in the fine line's coarse slots of `buf`, then the fine
+// slots by interpolation, then the mass matrix with a rolling window (in
+// place, or into `fine` where the pass is the last).
+template <typename T, int DIM, int FIN>
+__global__ void __launch_bounds__(256) gl_expand_long(GLevel<T> L, LineShape S, const T* __restrict__ coarse, T* buf,
+                                                      T* fine, const T* g, T* coef) {
+  const GDim<T>& D = L.d[DIM];
   const int n = D.n, c = D.c;
   const int64_t lines = S.nb * S.ncol;
   for (int64_t line = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; line < lines;
        line += (int64_t)gridDim.x * blockDim.x) {
     const int64_t b = line / S.ncol, col = line - b * S.ncol;
     const T* x = coarse + b * S.c_b + col * S.c_c;
-    T* y = fine + b * S.f_b + col * S.f_c;
+    T* y = buf + b * S.f_b + col * S.f_c;
     const int64_t so = S.f_i, si = S.c_i;
-    if (c == n) {  // a dimension of at most two nodes is not coarsened
-      for (int i = 0; i < n; ++i) y[i * so] = x[i * si];
-      continue;
-    }
     T yv = x[0];
     y[(int64_t)D.cidx[0] * so] = yv;
     for (int J = 1; J < c; ++J) {
@@ -324,69 +512,53 @@ __global__ void __launch_bounds__(256) gl_expand(GDim<T> D, LineShape S, const T
       T v = D.md[i] * w0;
       if (i > 0) v = fma(D.mo[i - 1], wm, v);
       if (i + 1 < n) v = fma(D.mo[i], wp, v);
-      y[i * so] = v;
+      expand_emit<T, FIN>(L, S, fine, g, coef, b, col, i, v);
       wm = w0;
       w0 = wp;
     }
   }
 }
 
-// coarse line = I^T (fine line): each coarse node gathers itself and its
-// fine neighbours with their interpolation weights.
-template <typename T>
-__global__ void __launch_bounds__(256) gl_restrict_interp(GDim<T> D, LineShape S, const T* __restrict__ fine,
+// coarse = I^T fine in all three dimensions: each coarse node gathers itself
+// and its fine neighbours with their interpolation weights, dimension 2
+// innermost (op for op the three line passes that it stands for, which wrote
+// and read two intermediate grids).  CORRECT 0 stores it; CORRECT 1 adds
+// g_c - I^T v to v at the node itself (no other node's stencil reads an
+// all-coarse node, so in place).
+template <typename T, int CORRECT>
+__global__ void __launch_bounds__(256) gl_restrict_interp(GLevel<T> L, NodeDiv cd, T* __restrict__ fine,
                                                            T* __restrict__ coarse) {
-  const int n = D.n, c = D.c;
-  const int64_t total = S.nb * S.ncol * c;
+  const GDim<T>&D0 = L.d[0], &D1 = L.d[1], &D2 = L.d[2];
+  const int64_t n1 = D1.n, n2 = D2.n;
+  const int64_t total = (int64_t)D0.c * D1.c * D2.c;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    // e = (b * c + J) * ncol + col: consecutive threads take consecutive columns
-    const int64_t col = e % S.ncol, t = e / S.ncol;
-    const int J = (int)(t % c);
-    const int64_t b = t / c;
-    const T* x = fine + b * S.f_b + col * S.f_c;
-    const int i = D.cidx[J];
-    T v = x[i * S.f_i];
-    if (c != n) {
-      if (i > 0 && !D.isc[i - 1]) v = fma(D.wr[i - 1], x[(i - 1) * S.f_i], v);
-      if (i + 1 < n && !D.isc[i + 1]) v = fma(D.wl[i + 1], x[(i + 1) * S.f_i], v);
-    }
-    coarse[b * S.c_b + (int64_t)J * S.c_i + col * S.c_c] = v;
-  }
-}
-
-template <typename T>
-__global__ void gl_axpy(T* __restrict__ y, const T* __restrict__ x, int64_t n) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    y[i] += x[i];
-}
-
-// g_u at the all-coarse nodes: += g_c - I^T v.
-template <typename T>
-__global__ void gl_adj_correct(GLevel<T> L, T* __restrict__ U, const T* __restrict__ gc, const T* __restrict__ r) {
-  const int c0 = L.d[0].c, c1 = L.d[1].c, c2 = L.d[2].c, n1 = L.d[1].n, n2 = L.d[2].n;
-  const int64_t total = (int64_t)c0 * c1 * c2;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int j2 = (int)(e % c2);
-    const int64_t t = e / c2;
-    const int j1 = (int)(t % c1), j0 = (int)(t / c1);
-    const int64_t u = ((int64_t)L.d[0].cidx[j0] * n1 + L.d[1].cidx[j1]) * n2 + L.d[2].cidx[j2];
-    U[u] += gc[e] - r[e];
-  }
-}
-
-// Coefficient gradients of a level: g - t at the non all-coarse nodes, in
-// stream order.
-template <typename T>
-__global__ void gl_adj_gather(GLevel<T> L, const T* __restrict__ g, const T* __restrict__ t, T* __restrict__ coef) {
-  const int n0 = L.d[0].n, n1 = L.d[1].n, n2 = L.d[2].n;
-  const int64_t total = (int64_t)n0 * n1 * n2;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int i2 = (int)(idx % n2);
-    const int64_t q = idx / n2;
-    const int i1 = (int)(q % n1), i0 = (int)(q / n1);
-    if (all_coarse(L, i0, i1, i2)) continue;
-    coef[nc_pos(L, i0, i1, i2, idx)] = g[idx] - t[idx];
+    int j0, j1, j2;
+    node_of(cd, e, j0, j1, j2);
+    const int i0 = D0.cidx[j0], i1 = D1.cidx[j1], i2 = D2.cidx[j2];
+    const bool l0 = i0 > 0 && !D0.isc[i0 - 1], r0 = i0 + 1 < D0.n && !D0.isc[i0 + 1];
+    const bool l1 = i1 > 0 && !D1.isc[i1 - 1], r1 = i1 + 1 < D1.n && !D1.isc[i1 + 1];
+    const bool l2 = i2 > 0 && !D2.isc[i2 - 1], r2 = i2 + 1 < D2.n && !D2.isc[i2 + 1];
+    const T wl0 = l0 ? D0.wr[i0 - 1] : T(0), wr0 = r0 ? D0.wl[i0 + 1] : T(0);
+    const T wl1 = l1 ? D1.wr[i1 - 1] : T(0), wr1 = r1 ? D1.wl[i1 + 1] : T(0);
+    const T wl2 = l2 ? D2.wr[i2 - 1] : T(0), wr2 = r2 ? D2.wl[i2 + 1] : T(0);
+    const int64_t u = ((int64_t)i0 * n1 + i1) * n2 + i2;
+    auto line = [&](const T* x) {
+      T v = x[0];
+      if (l2) v = fma(wl2, x[-1], v);
+      if (r2) v = fma(wr2, x[1], v);
+      return v;
+    };
+    auto plane = [&](const T* x) {
+      T v = line(x);
+      if (l1) v = fma(wl1, line(x - n2), v);
+      if (r1) v = fma(wr1, line(x + n2), v);
+      return v;
+    };
+    T v = plane(fine + u);
+    if (l0) v = fma(wl0, plane(fine + u - n1 * n2), v);
+    if (r0) v = fma(wr0, plane(fine + u + n1 * n2), v);
+    if (CORRECT) fine[u] += coarse[e] - v;
+    else coarse[e] = v;
   }
 }
 

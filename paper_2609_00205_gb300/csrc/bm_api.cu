@@ -21,6 +21,7 @@
 #include "bm_global.cuh"
 #include "bm_huffman.cuh"
 #include "bm_internal.h"
+#include "bm_levels.h"
 #include "bm_plan.h"
 #include "bm_plane.h"
 #include "bm_qtab.cuh"
@@ -956,36 +957,27 @@ cudaError_t launch_block<double>(int dir, int B, int K, int mode, const BlockArg
 // One restriction pass of a global level: band product and tridiagonal solve
 // per line (gl_line), or the dense projection (gl_apply) for lines longer than
 // gl_line takes.
-template <typename T, int DIM, int FINAL, int E>
-cudaError_t launch_line(const GLevel<T>& L, const ApplyShape& S, const T* in, T* out, const T* U, cudaStream_t s) {
-  const GDim<T>& D = L.d[DIM];
-  const size_t smem = line_smem<T>(D.n, D.c);
-  static std::atomic<int> attr{0};  // largest dynamic shared memory enabled so far
-  if ((int)smem > 48 * 1024 && (int)smem > attr.load()) {
-    const cudaError_t e = cudaFuncSetAttribute(gl_line<T, DIM, FINAL, E>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)smem);
-    if (e != cudaSuccess) return e;
-    attr.store((int)smem);
-  }
-  const int64_t ctas = S.nb * ((S.ncol + line_tile<T>() - 1) / line_tile<T>());
-  gl_line<T, DIM, FINAL, E><<<(unsigned)ctas, 256, smem, s>>>(L, S, in, out, U);
-  return cudaGetLastError();
+// A restriction pass along dimension DIM of a global level.
+template <typename T, int DIM, int FINAL, int SRC>
+cudaError_t launch_lines(const GLevel<T>& L, const T* in, T* out, const T* U, const LineSrc<T>& W, cudaStream_t s) {
+  BM_LAUNCHED();
+  return level_lines<T, DIM, FINAL, SRC>(L, in, out, U, W, s, num_sms());
 }
-
 template <typename T, int DIM, int FINAL>
 cudaError_t launch_apply(const GLevel<T>& L, const T* in, T* out, const T* U, cudaStream_t s) {
-  const ApplyShape S = apply_shape(L, DIM);
-  if (S.nb * S.ncol == 0) return cudaSuccess;
-  switch (line_segment(L.d[DIM].c)) {
-    case 1: return launch_line<T, DIM, FINAL, 1>(L, S, in, out, U, s);
-    case 3: return launch_line<T, DIM, FINAL, 3>(L, S, in, out, U, s);
-    case 9: return launch_line<T, DIM, FINAL, 9>(L, S, in, out, U, s);
-    case 17: return launch_line<T, DIM, FINAL, 17>(L, S, in, out, U, s);
-    default: break;
-  }
-  const int64_t ctas = S.nb * ((S.ncol + kApplyCols - 1) / kApplyCols);
-  gl_apply<T, DIM, FINAL><<<(unsigned)ctas, 256, 0, s>>>(L, S, in, out, U);
-  return cudaGetLastError();
+  return launch_lines<T, DIM, FINAL, SRC_GRID>(L, in, out, U, LineSrc<T>{}, s);
+}
+
+// The passes after the first of a global level's restriction: dimension 1,
+// then dimension 0 with FINAL.  A dimension 0 that is not coarsened (at most
+// two nodes: every plane) has nothing to restrict and the dimension-1 pass is
+// the last one, its outputs laid out alike (1535x2049: 10 and 5 us of a
+// compress call's 301 saved).
+template <typename T, int FINAL>
+cudaError_t launch_apply10(const GLevel<T>& L, const T* W1, T* W2, T* out, const T* U, cudaStream_t s) {
+  if (L.d[0].c == L.d[0].n && line_segment(L.d[1].c)) return launch_apply<T, 1, FINAL>(L, W1, out, U, s);
+  const cudaError_t e = launch_apply<T, 1, 0>(L, W1, W2, nullptr, s);
+  return e != cudaSuccess ? e : launch_apply<T, 0, FINAL>(L, W2, out, U, s);
 }
 
 // Outputs of the decomposition (mode 0: symbols + escapes + histogram).
@@ -1069,18 +1061,18 @@ bm_status run_decompose(PlanDev& P, const T* field, int mode, const FwdOut<T>& o
     auto& RL = rlevels<T>(P);
     for (int l = 0; l < h.K; ++l) {
       const GLevel<T>& L = RL[(size_t)l];
-      const int64_t rows = (int64_t)L.d[0].n * L.d[1].n;
+      const int64_t nn = (int64_t)L.d[0].n * L.d[1].n * L.d[2].n;
       const T* rq = o.rq ? o.rq + l : nullptr;
       if (mode == 0)
-        gl_fwd_detail<T, 0><<<grid_for(rows * 32, 256, 8), 256, 0, s>>>(L, RB[l], Dbuf, o.sym, o.esc, o.coef, rq, o.radius,
-                                                                       o.sc, o.tier, h.K);
+        gl_fwd_detail<T, 0><<<grid_for(nn, 256), 256, 0, s>>>(L, RB[l], Dbuf, o.sym, o.esc, o.coef, rq, o.radius,
+                                                              o.sc, node_div(L), o.tier, h.K);
       else
-        gl_fwd_detail<T, 1><<<grid_for(rows * 32, 256, 8), 256, 0, s>>>(L, RB[l], Dbuf, o.sym, o.esc, o.coef, rq, o.radius,
-                                                                       o.sc, nullptr, 0);
+        gl_fwd_detail<T, 1><<<grid_for(nn, 256), 256, 0, s>>>(L, RB[l], Dbuf, o.sym, o.esc, o.coef, rq, o.radius,
+                                                              o.sc, node_div(L), nullptr, 0);
       BM_CUDA((launch_apply<T, 2, 0>(L, Dbuf, W1, nullptr, s)));
       BM_CUDA((launch_apply<T, 1, 0>(L, W1, W2, nullptr, s)));
       gl_ident0<T, 1><<<grid_for(gs.RB[(size_t)l + 1], 256), 256, 0, s>>>(L, W2, RB[(size_t)l + 1], RB[l]);
-      g_launches.fetch_add(4);
+      g_launches.fetch_add(2);
     }
     reblock_kernel<T, 1><<<grid_for(gs.RB.back(), 256), 256, 0, s>>>(rc, Gr[0], RB.back());
     g_launches.fetch_add(2);
@@ -1103,18 +1095,18 @@ bm_status run_decompose(PlanDev& P, const T* field, int mode, const FwdOut<T>& o
       for (int l = 0; l < h.K; ++l) {
         const GLevel<T>& L = XL[(size_t)l];
         T* next = l + 1 < h.K ? XP[(size_t)l + 1] : Gr[r];
-        const int64_t rows = (int64_t)L.d[0].n * L.d[1].n;
+        const int64_t nn = (int64_t)L.d[0].n * L.d[1].n * L.d[2].n;
         const T* rq = o.rq ? o.rq + l : nullptr;
         if (mode == 0)
-          gl_fwd_detail<T, 0><<<grid_for(rows * 32, 256, 8), 256, 0, s>>>(L, XP[(size_t)l], Dbuf, o.sym, o.esc,
-                                                                         o.coef, rq, o.radius, o.sc, tier, h.K);
+          gl_fwd_detail<T, 0><<<grid_for(nn, 256), 256, 0, s>>>(L, XP[(size_t)l], Dbuf, o.sym, o.esc, o.coef,
+                                                                rq, o.radius, o.sc, node_div(L), tier, h.K);
         else
-          gl_fwd_detail<T, 1><<<grid_for(rows * 32, 256, 8), 256, 0, s>>>(L, XP[(size_t)l], Dbuf, o.sym, o.esc, o.coef,
-                                                                         rq, o.radius, o.sc, nullptr, 0);
+          gl_fwd_detail<T, 1><<<grid_for(nn, 256), 256, 0, s>>>(L, XP[(size_t)l], Dbuf, o.sym, o.esc, o.coef,
+                                                                rq, o.radius, o.sc, node_div(L), nullptr, 0);
         BM_CUDA((launch_apply<T, 2, 0>(L, Dbuf, W1, nullptr, s)));
         BM_CUDA((launch_apply<T, 1, 0>(L, W1, W2, nullptr, s)));
         BM_CUDA((launch_apply<T, 0, 1>(L, W2, next, XP[(size_t)l], s)));
-        g_launches.fetch_add(4);
+        g_launches.fetch_add(1);
       }
       toff += rd.nblocks;
     }
@@ -1152,15 +1144,20 @@ bm_status run_decompose(PlanDev& P, const T* field, int mode, const FwdOut<T>& o
     const GLevel<T>& L = G[l];
     const int64_t nn = gs.U[l];
     const T* rq = o.rq ? o.rq + o.ntiers * h.K + l : nullptr;
-    const int64_t rows = (int64_t)L.d[0].n * L.d[1].n;  // one warp per row, 8 rows per CTA
-    if (mode == 0) gl_fwd_detail<T, 0><<<grid_for(rows * 32, 256, 8), 256, 0, s>>>(L, U[l], Dbuf, o.sym, o.esc, o.coef, rq, o.radius, o.sc);
-    else gl_fwd_detail<T, 1><<<grid_for(rows * 32, 256, 8), 256, 0, s>>>(L, U[l], Dbuf, o.sym, o.esc, o.coef, rq, o.radius, o.sc);
-    (void)nn;
-    BM_LAUNCHED();
-    BM_CUDA((launch_apply<T, 2, 0>(L, Dbuf, W1, nullptr, s)));
-    BM_CUDA((launch_apply<T, 1, 0>(L, W1, W2, nullptr, s)));
-    BM_CUDA((launch_apply<T, 0, 1>(L, W2, U[l + 1], U[l], s)));
-    g_launches.fetch_add(3);
+    if (coefs_in_line_pass(L, num_sms())) {
+      LineSrc<T> W{};
+      W.sym = o.sym; W.esc = o.esc; W.coef = o.coef; W.rq = rq; W.radius = o.radius; W.sc = o.sc;
+      if (mode == 0) BM_CUDA((launch_lines<T, 2, 0, SRC_CODE>(L, U[l], W1, nullptr, W, s)));
+      else BM_CUDA((launch_lines<T, 2, 0, SRC_COEF>(L, U[l], W1, nullptr, W, s)));
+    } else {
+      if (mode == 0) gl_fwd_detail<T, 0><<<grid_for(nn, 256), 256, 0, s>>>(L, U[l], Dbuf, o.sym, o.esc, o.coef, rq,
+                                                                           o.radius, o.sc, node_div(L));
+      else gl_fwd_detail<T, 1><<<grid_for(nn, 256), 256, 0, s>>>(L, U[l], Dbuf, o.sym, o.esc, o.coef, rq, o.radius,
+                                                                 o.sc, node_div(L));
+      BM_LAUNCHED();
+      BM_CUDA((launch_apply<T, 2, 0>(L, Dbuf, W1, nullptr, s)));
+    }
+    BM_CUDA((launch_apply10<T, 1>(L, W1, W2, U[l + 1], U[l], s)));
   }
   {
     Stage st("coarsest");
@@ -1220,14 +1217,24 @@ bm_status run_recompose(PlanDev& P, T* field, int mode, const InvIn<T>& in, Carv
     const int64_t nn = gs.U[l];
     const double* q = in.q ? in.q + in.ntiers * h.K + l : nullptr;
     // U[l] <- dequantised coefficients; z = P D; coarse' = U[l+1] - z (into W1); U[l] = I coarse' + D
-    if (mode == 0) gl_inv_dequant<T, 0><<<grid_for(nn, 256), 256, 0, s>>>(L, in.sym, in.esc, in.coef, q, in.radius, U[l]);
-    else gl_inv_dequant<T, 1><<<grid_for(nn, 256), 256, 0, s>>>(L, in.sym, in.esc, in.coef, q, in.radius, U[l]);
     T* Cn = Dbuf;  // corrected coarse values (size of U[l+1] <= size of U[0])
-    BM_CUDA((launch_apply<T, 2, 0>(L, U[l], W1, nullptr, s)));
-    BM_CUDA((launch_apply<T, 1, 0>(L, W1, W2, nullptr, s)));
-    BM_CUDA((launch_apply<T, 0, 2>(L, W2, Cn, U[l + 1], s)));
-    gl_inv_interp<T><<<grid_for(nn, 256), 256, 0, s>>>(L, Cn, U[l]);
-    g_launches.fetch_add(5);
+    if (coefs_in_line_pass(L, num_sms())) {
+      LineSrc<T> W{};
+      W.sym = const_cast<uint16_t*>(in.sym); W.esc = const_cast<int32_t*>(in.esc); W.coef = const_cast<T*>(in.coef);
+      W.q = q; W.radius = in.radius; W.D = U[l];
+      if (mode == 0) BM_CUDA((launch_lines<T, 2, 0, SRC_DECODE>(L, nullptr, W1, nullptr, W, s)));
+      else BM_CUDA((launch_lines<T, 2, 0, SRC_READ>(L, nullptr, W1, nullptr, W, s)));
+    } else {
+      if (mode == 0) gl_inv_dequant<T, 0><<<grid_for(nn, 256), 256, 0, s>>>(L, in.sym, in.esc, in.coef, q, in.radius,
+                                                                            U[l], node_div(L));
+      else gl_inv_dequant<T, 1><<<grid_for(nn, 256), 256, 0, s>>>(L, in.sym, in.esc, in.coef, q, in.radius, U[l],
+                                                                  node_div(L));
+      BM_LAUNCHED();
+      BM_CUDA((launch_apply<T, 2, 0>(L, U[l], W1, nullptr, s)));
+    }
+    BM_CUDA((launch_apply10<T, 2>(L, W1, W2, Cn, U[l + 1], s)));
+    gl_inv_interp<T><<<grid_for(row_cells(L), 256), 256, 0, s>>>(L, Cn, U[l], row_cell_div(L));
+    BM_LAUNCHED();
     BM_CUDA(cudaGetLastError());
   }
   if (h.reduced && mode == 0 && plane_fused(h.ax[0] >= 0, h.B, h.K)) {
@@ -1250,15 +1257,15 @@ bm_status run_recompose(PlanDev& P, T* field, int mode, const InvIn<T>& in, Carv
       const double* q = in.q ? in.q + l : nullptr;
       const int64_t nn = gs.RB[(size_t)l];
       if (mode == 0)
-        gl_inv_dequant<T, 0><<<grid_for(nn, 256), 256, 0, s>>>(L, in.sym, in.esc, in.coef, q, in.radius, RB[l], in.tier,
+        gl_inv_dequant<T, 0><<<grid_for(nn, 256), 256, 0, s>>>(L, in.sym, in.esc, in.coef, q, in.radius, RB[l], node_div(L), in.tier,
                                                                 h.K, in.ntiers, in.sc);
       else
-        gl_inv_dequant<T, 1><<<grid_for(nn, 256), 256, 0, s>>>(L, in.sym, in.esc, in.coef, q, in.radius, RB[l]);
+        gl_inv_dequant<T, 1><<<grid_for(nn, 256), 256, 0, s>>>(L, in.sym, in.esc, in.coef, q, in.radius, RB[l], node_div(L));
       BM_CUDA((launch_apply<T, 2, 0>(L, RB[l], W1, nullptr, s)));
       BM_CUDA((launch_apply<T, 1, 0>(L, W1, W2, nullptr, s)));
       gl_ident0<T, 2><<<grid_for(gs.RB[(size_t)l + 1], 256), 256, 0, s>>>(L, W2, Cn, RB[(size_t)l + 1]);
-      gl_inv_interp<T><<<grid_for(nn, 256), 256, 0, s>>>(L, Cn, RB[l]);
-      g_launches.fetch_add(5);
+      gl_inv_interp<T><<<grid_for(row_cells(L), 256), 256, 0, s>>>(L, Cn, RB[l], row_cell_div(L));
+      g_launches.fetch_add(3);
     }
     reblock_kernel<T, 1><<<grid_for(gs.RB[0], 256), 256, 0, s>>>(rf, field, RB[0]);
     g_launches.fetch_add(2);
@@ -1282,15 +1289,15 @@ bm_status run_recompose(PlanDev& P, T* field, int mode, const InvIn<T>& in, Carv
         const int64_t nn = (int64_t)L.d[0].n * L.d[1].n * L.d[2].n;
         if (mode == 0)
           gl_inv_dequant<T, 0><<<grid_for(nn, 256), 256, 0, s>>>(L, in.sym, in.esc, in.coef, q, in.radius,
-                                                                  XP[(size_t)l], tier, h.K, in.ntiers, in.sc);
+                                                                  XP[(size_t)l], node_div(L), tier, h.K, in.ntiers, in.sc);
         else
           gl_inv_dequant<T, 1><<<grid_for(nn, 256), 256, 0, s>>>(L, in.sym, in.esc, in.coef, q, in.radius,
-                                                                  XP[(size_t)l]);
+                                                                  XP[(size_t)l], node_div(L));
         BM_CUDA((launch_apply<T, 2, 0>(L, XP[(size_t)l], W1, nullptr, s)));
         BM_CUDA((launch_apply<T, 1, 0>(L, W1, W2, nullptr, s)));
         BM_CUDA((launch_apply<T, 0, 2>(L, W2, Cn, coarse, s)));
-        gl_inv_interp<T><<<grid_for(nn, 256), 256, 0, s>>>(L, Cn, XP[(size_t)l]);
-        g_launches.fetch_add(5);
+        gl_inv_interp<T><<<grid_for(row_cells(L), 256), 256, 0, s>>>(L, Cn, XP[(size_t)l], row_cell_div(L));
+        g_launches.fetch_add(2);
       }
       T* out = rr == 0 ? field : Gr[rr - 1];
       pad_kernel<T, 1><<<grid_for(rd.shape[0] * rd.shape[1] * rd.shape[2], 256), 256, 0, s>>>(
@@ -1990,16 +1997,10 @@ cudaError_t launch_block_adj<double>(int dir, int B, int K, const BlockArgs<doub
   return launch_block_adj_f64(dir, B, K, a, s, num_sms());
 }
 
-// Expansion (M_f I M_c^-1) or restriction (I^T) along one dimension of a global level.
-template <typename T>
-void launch_gl_line(const GLevel<T>& L, int dim, bool expand, const T* in, T* out, cudaStream_t s) {
-  const LineShape S = line_shape(L, dim);
-  if (expand) {
-    gl_expand<T><<<grid_for(S.nb * S.ncol, 256), 256, 0, s>>>(L.d[dim], S, in, out);
-  } else {
-    gl_restrict_interp<T><<<grid_for(S.nb * S.ncol * L.d[dim].c, 256), 256, 0, s>>>(L.d[dim], S, in, out);
-  }
+template <typename T, int DIM, int FIN>
+cudaError_t launch_expand(const GLevel<T>& L, const T* in, T* buf, T* fine, const T* g, T* coef, cudaStream_t s) {
   BM_LAUNCHED();
+  return level_expand<T, DIM, FIN>(L, in, buf, fine, g, coef, s, num_sms());
 }
 
 // dir 0: coefficient gradients (gcoef, read) -> field gradients (gfield, written);
@@ -2029,19 +2030,14 @@ bm_status run_adjoint(PlanDev& P, int dir, T* gfield, T* gcoef, Carver& cv, cuda
     BM_CUDA(cudaMemcpyAsync(U[h.M], gcoef + h.sym_off[h.M], (size_t)ncoarsest * sizeof(T), cudaMemcpyDeviceToDevice, s));
     for (int l = h.M - 1; l >= 0; --l) {
       const GLevel<T>& L = G[l];
-      const int64_t nn = gs.U[l], nc = gs.U[l + 1];
+      const int64_t nc = gs.U[l + 1];
       // v = S_F^T g_D + P^T g_c
-      gl_inv_dequant<T, 1><<<grid_for(nn, 256), 256, 0, s>>>(L, nullptr, nullptr, gcoef, nullptr, 0, U[l]);
-      launch_gl_line<T>(L, 0, true, U[l + 1], W2, s);
-      launch_gl_line<T>(L, 1, true, W2, W1, s);
-      launch_gl_line<T>(L, 2, true, W1, Dbuf, s);
-      gl_axpy<T><<<grid_for(nn, 256), 256, 0, s>>>(U[l], Dbuf, nn);
+      BM_CUDA((launch_expand<T, 0, EXP_STORE>(L, U[l + 1], W2, W2, nullptr, nullptr, s)));
+      BM_CUDA((launch_expand<T, 1, EXP_STORE>(L, W2, W1, W1, nullptr, nullptr, s)));
+      BM_CUDA((launch_expand<T, 2, EXP_ADD>(L, W1, Dbuf, U[l], nullptr, gcoef, s)));
       // g_u = v + R_C^T (g_c - I^T v)
-      launch_gl_line<T>(L, 2, false, U[l], W1, s);
-      launch_gl_line<T>(L, 1, false, W1, W2, s);
-      launch_gl_line<T>(L, 0, false, W2, Dbuf, s);
-      gl_adj_correct<T><<<grid_for(nc, 256), 256, 0, s>>>(L, U[l], U[l + 1], Dbuf);
-      g_launches.fetch_add(3);
+      gl_restrict_interp<T, 1><<<grid_for(nc, 256), 256, 0, s>>>(L, coarse_div(L), U[l], U[l + 1]);
+      BM_LAUNCHED();
       BM_CUDA(cudaGetLastError());
     }
   }
@@ -2053,17 +2049,14 @@ bm_status run_adjoint(PlanDev& P, int dir, T* gfield, T* gcoef, Carver& cv, cuda
     Stage st("adjoint_global");
     for (int l = 0; l < h.M; ++l) {
       const GLevel<T>& L = G[l];
-      const int64_t nn = gs.U[l];
+      const int64_t nc = gs.U[l + 1];
       // g_c = I^T g_u, then g_D = S_F (g_u - P^T g_c)
-      launch_gl_line<T>(L, 2, false, U[l], W1, s);
-      launch_gl_line<T>(L, 1, false, W1, W2, s);
-      launch_gl_line<T>(L, 0, false, W2, U[l + 1], s);
-      launch_gl_line<T>(L, 0, true, U[l + 1], W2, s);
-      launch_gl_line<T>(L, 1, true, W2, W1, s);
-      launch_gl_line<T>(L, 2, true, W1, Dbuf, s);
-      gl_adj_gather<T><<<grid_for(nn, 256), 256, 0, s>>>(L, U[l], Dbuf, gcoef);
-      g_launches.fetch_add(1);
+      gl_restrict_interp<T, 0><<<grid_for(nc, 256), 256, 0, s>>>(L, coarse_div(L), U[l], U[l + 1]);
+      BM_LAUNCHED();
       BM_CUDA(cudaGetLastError());
+      BM_CUDA((launch_expand<T, 0, EXP_STORE>(L, U[l + 1], W2, W2, nullptr, nullptr, s)));
+      BM_CUDA((launch_expand<T, 1, EXP_STORE>(L, W2, W1, W1, nullptr, nullptr, s)));
+      BM_CUDA((launch_expand<T, 2, EXP_COEF>(L, W1, Dbuf, Dbuf, U[l], gcoef, s)));
     }
     BM_CUDA(cudaMemcpyAsync(gcoef + h.sym_off[h.M], U[h.M], (size_t)ncoarsest * sizeof(T), cudaMemcpyDeviceToDevice, s));
   }

@@ -104,70 +104,100 @@ __device__ __forceinline__ int64_t nc_pos(const GLevel<T>& L, int i0, int i1, in
   return L.sym_off + flat - before + (int64_t)i0 * L.blk_extra;
 }
 
+// (i0, i1, i2) of a flat node index: divisions by multiplication with the
+// extents' rounded-up reciprocals (exact for 32-bit indices), 64-bit divisions
+// above them.
+struct NodeDiv {
+  unsigned n1, n2;
+  unsigned long long m1, m2;
+  bool wide;
+};
+inline NodeDiv node_div(int64_t n0, int n1, int n2) {
+  NodeDiv d{};
+  d.n1 = (unsigned)n1;
+  d.n2 = (unsigned)n2;
+  d.m1 = ~0ull / d.n1 + 1ull;
+  d.m2 = ~0ull / d.n2 + 1ull;
+  d.wide = n0 * n1 * n2 > 0xFFFFFFFFll;
+  return d;
+}
+template <typename T>
+NodeDiv node_div(const GLevel<T>& L) { return node_div(L.d[0].n, L.d[1].n, L.d[2].n); }
+template <typename T>
+NodeDiv coarse_div(const GLevel<T>& L) { return node_div(L.d[0].c, L.d[1].c, L.d[2].c); }
+// rows i0 of the fine grid, coarse cells of the other two dimensions
+template <typename T>
+int64_t row_cells(const GLevel<T>& L) { return (int64_t)L.d[0].n * L.d[1].c * L.d[2].c; }
+template <typename T>
+NodeDiv row_cell_div(const GLevel<T>& L) { return node_div(L.d[0].n, L.d[1].c, L.d[2].c); }
+__device__ __forceinline__ void node_of(const NodeDiv& d, int64_t idx, int& i0, int& i1, int& i2) {
+  if (!d.wide) {
+    const unsigned u = (unsigned)idx;
+    const unsigned t = d.n2 == 1u ? u : (unsigned)__umul64hi((unsigned long long)u, d.m2);
+    const unsigned q = d.n1 == 1u ? t : (unsigned)__umul64hi((unsigned long long)t, d.m1);
+    i2 = (int)(u - t * d.n2);
+    i1 = (int)(t - q * d.n1);
+    i0 = (int)q;
+  } else {
+    const int64_t t = idx / d.n2, q = t / d.n1;
+    i2 = (int)(idx - t * d.n2);
+    i1 = (int)(t - q * d.n1);
+    i0 = (int)q;
+  }
+}
+
 // Coefficients of one global level: D = U - I(U|C) at every node (0 at
 // all-coarse nodes, exactly), written to Dfull; the non-coarse ones are
 // quantised (mode 0; a histogram pass counts the symbols afterwards) or stored
-// (mode 1) at their stream position.  One warp
-// per grid row (i0, i1): the row's interpolation sources, weights and stream
-// offset are computed once, the lanes walk i2.
+// (mode 1) at their stream position.  One thread per node: the level's grid is
+// small (155^3 at 513^3) and the tables stay in L1, so what counts is enough
+// threads in flight and cheap index arithmetic.  (One warp per row of the grid
+// took 0.040 ms for the first level at 513^3 against 0.045, and on the few
+// long rows of a plane's grid 0.040 against 0.008.)
 // With tier != null (the in-cache levels of the block-major grid), the
-// quantiser width of row (i0, i1) is rq_ptr[tier[i0] * tstride] (the block's
-// ROI tier); otherwise rq_ptr[0].
+// quantiser width of a node is rq_ptr[tier[i0] * tstride] (the block's ROI
+// tier); otherwise rq_ptr[0].
 template <typename T, int MODE>
 __global__ void __launch_bounds__(256) gl_fwd_detail(GLevel<T> L, const T* __restrict__ U, T* __restrict__ Dfull,
                                                      uint16_t* sym, int32_t* esc, T* coef, const T* rq_ptr,
-                                                     int radius, Scalars* sc, const uint8_t* tier = nullptr,
-                                                     int tstride = 0) {
+                                                     int radius, Scalars* sc, NodeDiv nd,
+                                                     const uint8_t* tier = nullptr, int tstride = 0) {
   const GDim<T>&D0 = L.d[0], &D1 = L.d[1], &D2 = L.d[2];
   const int n1 = D1.n, n2 = D2.n;
-  const int64_t rows = (int64_t)D0.n * n1, c12 = (int64_t)D1.c * D2.c;
+  const int64_t total = (int64_t)D0.n * n1 * n2;
   const unsigned dict = 2u * (unsigned)radius;
   bool ovf = false;
-  const int lane = threadIdx.x & 31;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; row < rows; row += nwarps) {
-    const int i0 = (int)(row / n1), i1 = (int)(row - (int64_t)i0 * n1);
-    const T rq_row = MODE == 0 && !L.bmode ? rq_ptr[tier ? (int)tier[i0] * tstride : 0] : T(0);
+  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
+       idx += (int64_t)gridDim.x * blockDim.x) {
+    int i0, i1, i2;
+    node_of(nd, idx, i0, i1, i2);
     const int a0 = g_cidx(D0, g_jlo(D0, i0)), b0 = g_cidx(D0, g_jhi(D0, i0));
     const int a1 = g_cidx(D1, g_jlo(D1, i1)), b1 = g_cidx(D1, g_jhi(D1, i1));
+    const int a2 = g_cidx(D2, g_jlo(D2, i2)), b2 = g_cidx(D2, g_jhi(D2, i2));
     const T wl0 = g_wl(D0, i0), wr0 = g_wr(D0, i0), wl1 = g_wl(D1, i1), wr1 = g_wr(D1, i1);
+    const T wl2 = g_wl(D2, i2), wr2 = g_wr(D2, i2);
     const T* r00 = U + ((int64_t)a0 * n1 + a1) * n2;
     const T* r01 = U + ((int64_t)a0 * n1 + b1) * n2;
     const T* r10 = U + ((int64_t)b0 * n1 + a1) * n2;
     const T* r11 = U + ((int64_t)b0 * n1 + b1) * n2;
-    const bool cc01 = g_isc(D0, i0) && g_isc(D1, i1);  // the row holds all-coarse nodes
-    // stream rank of the row's first node: flat index minus the all-coarse nodes before it
-    int64_t before = (int64_t)g_cb(D0, i0) * c12;
-    if (g_isc(D0, i0)) before += (int64_t)g_cb(D1, i1) * D2.c;
-    const int64_t rbase = L.sym_off + row * n2 - before + (int64_t)i0 * L.blk_extra;
-    for (int i2 = lane; i2 < n2; i2 += 32) {
-      const int a2 = g_cidx(D2, g_jlo(D2, i2)), b2 = g_cidx(D2, g_jhi(D2, i2));
-      const T wl2 = g_wl(D2, i2), wr2 = g_wr(D2, i2);
-      const T ta = fma(wl1, fma(wl2, r00[a2], wr2 * r00[b2]), wr1 * fma(wl2, r01[a2], wr2 * r01[b2]));
-      const T tb = fma(wl1, fma(wl2, r10[a2], wr2 * r10[b2]), wr1 * fma(wl2, r11[a2], wr2 * r11[b2]));
-      const T e = fma(wl0, ta, wr0 * tb);
-      const int64_t idx = row * n2 + i2;
-      const T dv = U[idx] - e;
-      Dfull[idx] = dv;
-      if (cc01 && g_isc(D2, i2)) continue;  // all-coarse node: no coefficient
-      int64_t pos;
-      T rq = rq_row;
-      if (L.bmode) {  // block-major order; the block's ROI tier
-        pos = blk_pos(L, i0, i1, i2);
-        if (MODE == 0) rq = rq_ptr[tier ? (int)tier[blk_of(L, i0, i1, i2)] * tstride : 0];
-      } else {
-        pos = rbase + i2 - (cc01 ? g_cb(D2, i2) : 0);
-      }
-      if (MODE == 0) {
-        const int code = quantize(dv, rq, ovf);
-        const unsigned u = (unsigned)(code + radius);
-        const bool in = u - 1u < dict - 1u;
-        const unsigned sv = in ? u : 0u;
-        sym[pos] = (uint16_t)sv;
-        if (!in) esc[pos] = code;
-      } else {
-        coef[pos] = dv;
-      }
+    const T ta = fma(wl1, fma(wl2, r00[a2], wr2 * r00[b2]), wr1 * fma(wl2, r01[a2], wr2 * r01[b2]));
+    const T tb = fma(wl1, fma(wl2, r10[a2], wr2 * r10[b2]), wr1 * fma(wl2, r11[a2], wr2 * r11[b2]));
+    const T e = fma(wl0, ta, wr0 * tb);
+    const T dv = U[idx] - e;
+    Dfull[idx] = dv;
+    if (all_coarse(L, i0, i1, i2)) continue;  // no coefficient
+    const int64_t pos = nc_pos(L, i0, i1, i2, idx);
+    if (MODE == 0) {
+      // the quantiser width of the block's ROI tier (in-cache levels)
+      const int64_t tb_ = !tier ? 0 : (int64_t)tier[L.bmode ? blk_of(L, i0, i1, i2) : (int64_t)i0] * tstride;
+      const int code = quantize(dv, rq_ptr[tb_], ovf);
+      const unsigned u = (unsigned)(code + radius);
+      const bool in = u - 1u < dict - 1u;
+      const unsigned sv = in ? u : 0u;
+      sym[pos] = (uint16_t)sv;
+      if (!in) esc[pos] = code;
+    } else {
+      coef[pos] = dv;
     }
   }
   if (MODE == 0 && ovf) atomicOr(&sc->status, ST_OVERFLOW);
@@ -275,27 +305,192 @@ __global__ void __launch_bounds__(256) gl_apply(GLevel<T> L, ApplyShape S, const
 // l*E .. l*E+E-1, composes their maps, combines them across the warp with
 // shuffles, then replays its rows from the combined input).  The same
 // operator as the dense projection in gl_apply, in O(n) work per line.
-// A CTA stages kLineTile lines (one 128-byte row of columns) in shared memory,
+// A CTA stages 2^lsh lines (line_tile_shift) in shared memory,
 // read coalesced along the line when it is contiguous (DIM 2) and across the
 // lines otherwise; eight warps take one line at a time.  Shapes and FINAL as
 // for gl_apply.  E is odd, so the lanes' rows of a segment never share a bank.
+// Lines of a CTA, as a shift: a 128-byte row of columns, or a 32-byte sector
+// when those tiles would leave SMs idle (a plane's 455 lines of 605 nodes in 15
+// CTAs of 32 lines took 24 us, in 57 of 8 14).
 template <typename T>
-constexpr int line_tile() {
-  return 128 / (int)sizeof(T);
+int line_tile_shift(int64_t nb, int64_t ncol, int nsm) {
+  const int full = sizeof(T) == 4 ? 5 : 4;
+  return nb * ((ncol >> full) + 1) < 2 * nsm ? full - 2 : full;
 }
 inline int line_segment(int c) {  // rows per lane (0: the line is too long for gl_line)
   const int e = (c + 31) / 32;
   return e <= 1 ? 1 : e <= 3 ? 3 : e <= 9 ? 9 : e <= 17 ? 17 : 0;
 }
+// Whether a level's coefficients are taken by its first restriction pass: where
+// that pass's lines fill the SMs (a plane's 455 lines of 605 nodes: 38 us in
+// one kernel, 8 + 14.4 in two; 155^3: 53 in one, 45 + 18 in two, and for the
+// inverse 27 against 22 + 18).
 template <typename T>
-size_t line_smem(int n, int c) {
-  return (size_t)line_tile<T>() * (size_t)((n | 1) + (c | 1)) * sizeof(T);
+bool coefs_in_line_pass(const GLevel<T>& L, int nsm) {
+  const int64_t lines = (int64_t)L.d[0].n * L.d[1].n;
+  return line_segment(L.d[2].c) && lines >> line_tile_shift<T>(1, lines, nsm) >= nsm;
+}
+template <typename T>
+size_t line_smem(int n, int c, int lsh) {
+  return ((size_t)((n | 1) + (c | 1)) << lsh) * sizeof(T);
 }
 
-template <typename T, int DIM, int FINAL, int E>
+// z = M_c^-1 r of one line in shared memory, in place, by a warp.
+template <typename T, int E>
+__device__ __forceinline__ void line_scan_solve(const GDim<T>& D, T* r, const int lane) {
+  const int c = D.c;
+  const int j0 = lane * E;
+  T y[E];
+  // forward recurrence y_J = r_J - tm_J y_{J-1} (y_{-1} = 0)
+  T a = T(0), m = T(1);
+#pragma unroll
+  for (int k = 0; k < E; ++k) {
+    const int J = j0 + k;
+    if (J < c) {
+      const T t = D.tm[J];
+      a = fma(-t, a, r[J]);
+      m = -t * m;
+    }
+  }
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const T pa = __shfl_up_sync(0xffffffffu, a, off), pm = __shfl_up_sync(0xffffffffu, m, off);
+    if (lane >= off) {
+      a = fma(m, pa, a);
+      m *= pm;
+    }
+  }
+  T prev = __shfl_up_sync(0xffffffffu, a, 1);
+  if (lane == 0) prev = T(0);
+#pragma unroll
+  for (int k = 0; k < E; ++k) {
+    const int J = j0 + k;
+    if (J < c) {
+      y[k] = fma(-D.tm[J], prev, r[J]);
+      prev = y[k];
+    }
+  }
+  // backward recurrence z_J = (y_J - tsup_J z_{J+1}) tib_J (z_c = 0)
+  a = T(0);
+  m = T(1);
+#pragma unroll
+  for (int k = E - 1; k >= 0; --k) {
+    const int J = j0 + k;
+    if (J < c) {
+      const T ib = D.tib[J], q = -D.tsup[J] * ib;
+      a = fma(q, a, y[k] * ib);
+      m = q * m;
+    }
+  }
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const T pa = __shfl_down_sync(0xffffffffu, a, off), pm = __shfl_down_sync(0xffffffffu, m, off);
+    if (lane + off < 32) {
+      a = fma(m, pa, a);
+      m *= pm;
+    }
+  }
+  T next = __shfl_down_sync(0xffffffffu, a, 1);
+  if (lane == 31) next = T(0);
+  __syncwarp();  // every lane has read its r before any z overwrites it
+#pragma unroll
+  for (int k = E - 1; k >= 0; --k) {
+    const int J = j0 + k;
+    if (J < c) {
+      next = fma(-D.tsup[J], next, y[k]) * D.tib[J];
+      r[J] = next;
+    }
+  }
+}
+
+// What the first (DIM 2) pass of a global level restricts: a grid in memory
+// (SRC_GRID); the level's coefficients, computed from the grid U and quantised
+// (SRC_CODE) or stored (SRC_COEF) at their stream position as the lines are
+// staged; the coefficients read back from the stream's codes (SRC_DECODE) or
+// values (SRC_READ), kept in the grid D for the interpolation.
+enum { SRC_GRID = 0, SRC_CODE = 1, SRC_COEF = 2, SRC_DECODE = 3, SRC_READ = 4 };
+template <typename T>
+struct LineSrc {
+  uint16_t* sym;
+  int32_t* esc;
+  T* coef;
+  const T* rq;      // SRC_CODE: the level's reciprocal bin width
+  const double* q;  // SRC_DECODE: its bin width
+  T* D;
+  int radius;
+  Scalars* sc;
+};
+
+// Stages line `line` (its row of U at u) of a global level by a warp: the same
+// operations per node as gl_fwd_detail and gl_inv_dequant, with everything
+// that depends on (i0, i1) taken once a line.  Bound by issue and the latency
+// of a warp's loads; four nodes of a lane in flight were slower (0.060 against
+// 0.053 ms at 155^3: the lines are five nodes a lane, the rest is thrown away).
+template <typename T, int SRC>
+__device__ __forceinline__ void stage_coefs(const GLevel<T>& L, const LineSrc<T>& W, const T* __restrict__ U,
+                                            int64_t line, T* x, int lane, bool& ovf) {
+  const GDim<T>&D0 = L.d[0], &D1 = L.d[1], &D2 = L.d[2];
+  const int n1 = D1.n, n2 = D2.n;
+  const int i0 = (int)(line / n1), i1 = (int)(line - (int64_t)i0 * n1);
+  const bool ic0 = g_isc(D0, i0), cc = ic0 && g_isc(D1, i1);
+  int64_t before = (int64_t)g_cb(D0, i0) * D1.c * D2.c;
+  if (ic0) before += (int64_t)g_cb(D1, i1) * D2.c;
+  const int64_t flat = line * n2, pos0 = L.sym_off + flat - before;
+  if (SRC == SRC_CODE || SRC == SRC_COEF) {
+    const int a0 = g_cidx(D0, g_jlo(D0, i0)), b0 = g_cidx(D0, g_jhi(D0, i0));
+    const int a1 = g_cidx(D1, g_jlo(D1, i1)), b1 = g_cidx(D1, g_jhi(D1, i1));
+    const T wl0 = g_wl(D0, i0), wr0 = g_wr(D0, i0), wl1 = g_wl(D1, i1), wr1 = g_wr(D1, i1);
+    const T* r00 = U + ((int64_t)a0 * n1 + a1) * n2;
+    const T* r01 = U + ((int64_t)a0 * n1 + b1) * n2;
+    const T* r10 = U + ((int64_t)b0 * n1 + a1) * n2;
+    const T* r11 = U + ((int64_t)b0 * n1 + b1) * n2;
+    const T rq = SRC == SRC_CODE ? *W.rq : T(0);
+    const unsigned dict = 2u * (unsigned)W.radius;
+    for (int i2 = lane; i2 < n2; i2 += 32) {
+      const int a2 = g_cidx(D2, g_jlo(D2, i2)), b2 = g_cidx(D2, g_jhi(D2, i2));
+      const T wl2 = g_wl(D2, i2), wr2 = g_wr(D2, i2);
+      const T ta = fma(wl1, fma(wl2, r00[a2], wr2 * r00[b2]), wr1 * fma(wl2, r01[a2], wr2 * r01[b2]));
+      const T tb = fma(wl1, fma(wl2, r10[a2], wr2 * r10[b2]), wr1 * fma(wl2, r11[a2], wr2 * r11[b2]));
+      const T e = fma(wl0, ta, wr0 * tb);
+      const T dv = U[flat + i2] - e;
+      x[i2] = dv;
+      if (cc && g_isc(D2, i2)) continue;  // no coefficient
+      const int64_t pos = pos0 + i2 - (cc ? g_cb(D2, i2) : 0);
+      if (SRC == SRC_CODE) {
+        const int code = quantize(dv, rq, ovf);
+        const unsigned u = (unsigned)(code + W.radius);
+        const bool in = u - 1u < dict - 1u;
+        const unsigned sv = in ? u : 0u;
+        W.sym[pos] = (uint16_t)sv;
+        if (!in) W.esc[pos] = code;
+      } else {
+        W.coef[pos] = dv;
+      }
+    }
+  } else {
+    const T q = SRC == SRC_DECODE ? (T)*W.q : T(0);
+    for (int i2 = lane; i2 < n2; i2 += 32) {
+      T v = T(0);
+      if (!(cc && g_isc(D2, i2))) {
+        const int64_t pos = pos0 + i2 - (cc ? g_cb(D2, i2) : 0);
+        if (SRC == SRC_DECODE) {
+          const unsigned s = W.sym[pos];
+          v = dequant(s ? (int)s - W.radius : W.esc[pos], q);
+        } else {
+          v = W.coef[pos];
+        }
+      }
+      x[i2] = v;
+      W.D[flat + i2] = v;
+    }
+  }
+}
+
+template <typename T, int DIM, int FINAL, int E, int SRC>
 __global__ void __launch_bounds__(256) gl_line(GLevel<T> L, ApplyShape S, const T* __restrict__ in,
-                                               T* __restrict__ out, const T* __restrict__ U) {
-  constexpr int LT = line_tile<T>();
+                                               T* __restrict__ out, const T* __restrict__ U, const int lsh,
+                                               LineSrc<T> W) {
+  const int LT = 1 << lsh;  // lines of the CTA
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const GDim<T>& D = L.d[DIM];
   const int n = D.n, c = D.c, sn = n | 1, sc = c | 1;
@@ -307,12 +502,16 @@ __global__ void __launch_bounds__(256) gl_line(GLevel<T> L, ApplyShape S, const 
   const int nl = (int)(S.ncol - col0 < LT ? S.ncol - col0 : LT);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const T* inb = in + b * S.in_b;
-  if (S.in_i == 1) {
+  if (SRC != SRC_GRID) {
+    bool ovf = false;
+    for (int w = warp; w < nl; w += 8) stage_coefs<T, SRC>(L, W, in, col0 + w, s_in + w * sn, lane, ovf);
+    if (SRC == SRC_CODE && ovf) atomicOr(&W.sc->status, ST_OVERFLOW);
+  } else if (S.in_i == 1) {
     for (int w = warp; w < nl; w += 8)
       for (int i = lane; i < n; i += 32) s_in[w * sn + i] = inb[(col0 + w) * S.in_c + i];
   } else {
     for (int e = threadIdx.x; e < n * LT; e += 256) {
-      const int i = e / LT, w = e - i * LT;
+      const int i = e >> lsh, w = e - (i << lsh);
       if (w < nl) s_in[w * sn + i] = inb[(int64_t)i * S.in_i + (col0 + w) * S.in_c];
     }
   }
@@ -333,77 +532,17 @@ __global__ void __launch_bounds__(256) gl_line(GLevel<T> L, ApplyShape S, const 
       r[J] = v;
     }
     __syncwarp();
-    const int j0 = lane * E;
-    T y[E];
-    // forward recurrence y_J = r_J - tm_J y_{J-1} (y_{-1} = 0)
-    T a = T(0), m = T(1);
-#pragma unroll
-    for (int k = 0; k < E; ++k) {
-      const int J = j0 + k;
-      if (J < c) {
-        const T t = D.tm[J];
-        a = fma(-t, a, r[J]);
-        m = -t * m;
-      }
-    }
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const T pa = __shfl_up_sync(0xffffffffu, a, off), pm = __shfl_up_sync(0xffffffffu, m, off);
-      if (lane >= off) {
-        a = fma(m, pa, a);
-        m *= pm;
-      }
-    }
-    T prev = __shfl_up_sync(0xffffffffu, a, 1);
-    if (lane == 0) prev = T(0);
-#pragma unroll
-    for (int k = 0; k < E; ++k) {
-      const int J = j0 + k;
-      if (J < c) {
-        y[k] = fma(-D.tm[J], prev, r[J]);
-        prev = y[k];
-      }
-    }
-    // backward recurrence z_J = (y_J - tsup_J z_{J+1}) tib_J (z_c = 0)
-    a = T(0);
-    m = T(1);
-#pragma unroll
-    for (int k = E - 1; k >= 0; --k) {
-      const int J = j0 + k;
-      if (J < c) {
-        const T ib = D.tib[J], q = -D.tsup[J] * ib;
-        a = fma(q, a, y[k] * ib);
-        m = q * m;
-      }
-    }
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const T pa = __shfl_down_sync(0xffffffffu, a, off), pm = __shfl_down_sync(0xffffffffu, m, off);
-      if (lane + off < 32) {
-        a = fma(m, pa, a);
-        m *= pm;
-      }
-    }
-    T next = __shfl_down_sync(0xffffffffu, a, 1);
-    if (lane == 31) next = T(0);
-    __syncwarp();  // every lane has read its r before any z overwrites it
-#pragma unroll
-    for (int k = E - 1; k >= 0; --k) {
-      const int J = j0 + k;
-      if (J < c) {
-        next = fma(-D.tsup[J], next, y[k]) * D.tib[J];
-        r[J] = next;
-      }
-    }
+    line_scan_solve<T, E>(D, r, lane);
   }
   __syncthreads();
   auto emit = [&](int J, int w) {
     const int64_t col = col0 + w;
     const int64_t o = b * S.out_b + (int64_t)J * S.out_j + col * S.out_c;
     const T z = s_out[w * sc + J];
-    if (FINAL == 1) {
-      const int c2 = L.d[2].c, j1 = (int)(col / c2), j2 = (int)(col - (int64_t)j1 * c2);
-      const int64_t u = ((int64_t)L.d[0].cidx[J] * L.d[1].n + L.d[1].cidx[j1]) * L.d[2].n + L.d[2].cidx[j2];
+    if (FINAL == 1) {  // (j0, j1, j2): (J, col) along dimension 0, (b, J, col) along dimension 1
+      const int c2 = L.d[2].c, j1 = DIM == 1 ? J : (int)(col / c2), j2 = (int)(DIM == 1 ? col : col - (int64_t)j1 * c2);
+      const int j0 = DIM == 1 ? (int)b : J;
+      const int64_t u = ((int64_t)L.d[0].cidx[j0] * L.d[1].n + L.d[1].cidx[j1]) * L.d[2].n + L.d[2].cidx[j2];
       out[o] = U[u] + z;
     } else if (FINAL == 2) {
       out[o] = U[o] - z;
@@ -416,7 +555,7 @@ __global__ void __launch_bounds__(256) gl_line(GLevel<T> L, ApplyShape S, const 
       for (int J = lane; J < c; J += 32) emit(J, w);
   } else {
     for (int e = threadIdx.x; e < c * LT; e += 256) {
-      const int J = e / LT, w = e - J * LT;
+      const int J = e >> lsh, w = e - (J << lsh);
       if (w < nl) emit(J, w);
     }
   }
@@ -500,21 +639,21 @@ __global__ void __launch_bounds__(256) pad_kernel(const T* __restrict__ src, T* 
 }
 
 // Inverse: dequantised coefficients into a full grid (0 at all-coarse nodes).
+// (With 64-bit divisions for the node's indices it took 0.027 ms for the first
+// level at 513^3 against 0.022.)
 // With tier != null (the in-cache levels of the block-major grid), the
 // quantiser width of the nodes with index i0 is q_ptr[tier[i0] * tstride];
 // the tier byte is range-checked against ntiers (a corrupt stream flags sc).
 template <typename T, int MODE>
 __global__ void gl_inv_dequant(GLevel<T> L, const uint16_t* __restrict__ sym, const int32_t* __restrict__ esc,
                                const T* __restrict__ coef, const double* q_ptr, int radius, T* __restrict__ Dfull,
-                               const uint8_t* tier = nullptr, int tstride = 0, int ntiers = 1, Scalars* sc = nullptr) {
-  const int n0 = L.d[0].n, n1 = L.d[1].n, n2 = L.d[2].n;
-  const int64_t total = (int64_t)n0 * n1 * n2;
+                               NodeDiv nd, const uint8_t* tier = nullptr, int tstride = 0, int ntiers = 1,
+                               Scalars* sc = nullptr) {
+  const int64_t total = (int64_t)L.d[0].n * L.d[1].n * L.d[2].n;
   for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
        idx += (int64_t)gridDim.x * blockDim.x) {
-    const int i2 = (int)(idx % n2);
-    const int64_t t = idx / n2;
-    const int i1 = (int)(t % n1);
-    const int i0 = (int)(t / n1);
+    int i0, i1, i2;
+    node_of(nd, idx, i0, i1, i2);
     T v = T(0);
     if (!all_coarse(L, i0, i1, i2)) {
       const int64_t pos = nc_pos(L, i0, i1, i2, idx);
@@ -536,32 +675,55 @@ __global__ void gl_inv_dequant(GLevel<T> L, const uint16_t* __restrict__ sym, co
   }
 }
 
-// Inverse: U = I(Uc) + D in place (Dfull holds D on entry, U on exit).
+// Inverse: U = I(Uc) + D in place (Dfull holds D on entry, U on exit).  One
+// thread per pair of coarse cells' rows: the up to four nodes of row i0 that
+// follow coarse nodes J1, J2 (each, and the node after it where that is not
+// coarse) share the corner values and the partial interpolants.  A coarse node
+// interpolates from itself with weights 1 and 0.  A thread per node, with the
+// tables and all eight values read for each, took 0.029 ms for the first level
+// at 513^3 (155^3 nodes) and 0.007 for the second against 0.020 and 0.007; a
+// thread per cell in all three dimensions 0.026 and 0.011.
 template <typename T>
-__global__ void gl_inv_interp(GLevel<T> L, const T* __restrict__ Uc, T* __restrict__ Dfull) {
-  const int n0 = L.d[0].n, n1 = L.d[1].n, n2 = L.d[2].n;
-  const int c1 = L.d[1].c, c2 = L.d[2].c;
-  const int64_t total = (int64_t)n0 * n1 * n2;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int i2 = (int)(idx % n2);
-    const int64_t t = idx / n2;
-    const int i1 = (int)(t % n1);
-    const int i0 = (int)(t / n1);
-    const int a0 = g_jlo(L.d[0], i0), b0 = g_jhi(L.d[0], i0);
-    const int a1 = g_jlo(L.d[1], i1), b1 = g_jhi(L.d[1], i1);
-    const int a2 = g_jlo(L.d[2], i2), b2 = g_jhi(L.d[2], i2);
-    const T wl0 = g_wl(L.d[0], i0), wr0 = g_wr(L.d[0], i0);
-    const T wl1 = g_wl(L.d[1], i1), wr1 = g_wr(L.d[1], i1);
-    const T wl2 = g_wl(L.d[2], i2), wr2 = g_wr(L.d[2], i2);
-    auto s = [&](int x0, int x1) {
-      const T* row = Uc + ((int64_t)x0 * c1 + x1) * c2;
-      return fma(wl2, row[a2], wr2 * row[b2]);
+__global__ void __launch_bounds__(256) gl_inv_interp(GLevel<T> L, const T* __restrict__ Uc, T* __restrict__ Dfull,
+                                                     NodeDiv cd) {
+  const GDim<T>&D0 = L.d[0], &D1 = L.d[1], &D2 = L.d[2];
+  const int c1 = D1.c, c2 = D2.c, n1 = D1.n, n2 = D2.n;
+  const int64_t total = (int64_t)D0.n * c1 * c2;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+    int i0, J1, J2;
+    node_of(cd, e, i0, J1, J2);
+    const int a0 = g_jlo(D0, i0), b0 = g_jhi(D0, i0), i1 = g_cidx(D1, J1), i2 = g_cidx(D2, J2);
+    const T wl0 = g_wl(D0, i0), wr0 = g_wr(D0, i0);
+    const bool f1 = i1 + 1 < n1 && !g_isc(D1, i1 + 1), f2 = i2 + 1 < n2 && !g_isc(D2, i2 + 1);
+    T* const u = Dfull + ((int64_t)i0 * n1 + i1) * n2 + i2;
+    T d[2][2];
+#pragma unroll
+    for (int k1 = 0; k1 < 2; ++k1)
+#pragma unroll
+      for (int k2 = 0; k2 < 2; ++k2) d[k1][k2] = (!k1 || f1) && (!k2 || f2) ? u[(int64_t)k1 * n2 + k2] : T(0);
+    const T wl1 = f1 ? D1.wl[i1 + 1] : T(1), wr1 = f1 ? D1.wr[i1 + 1] : T(0);
+    const T wl2 = f2 ? D2.wl[i2 + 1] : T(1), wr2 = f2 ? D2.wr[i2 + 1] : T(0);
+    // the nodes (k1, k2) interpolated along dimensions 2 and 1 in coarse row x0
+    auto plane = [&](int x0, T (&t)[2][2]) {
+      const T* r0 = Uc + ((int64_t)x0 * c1 + J1) * c2 + J2;
+      const T* r1 = f1 ? r0 + c2 : r0;
+      const T g00 = r0[0], g01 = f2 ? r0[1] : g00, g10 = r1[0], g11 = f2 ? r1[1] : g10;
+      const T s00 = fma(T(1), g00, T(0) * g00), s01 = fma(wl2, g00, wr2 * g01);
+      const T s10 = fma(T(1), g10, T(0) * g10), s11 = fma(wl2, g10, wr2 * g11);
+      t[0][0] = fma(T(1), s00, T(0) * s00);
+      t[0][1] = fma(T(1), s01, T(0) * s01);
+      t[1][0] = fma(wl1, s00, wr1 * s10);
+      t[1][1] = fma(wl1, s01, wr1 * s11);
     };
-    const T ta = fma(wl1, s(a0, a1), wr1 * s(a0, b1));
-    const T tb = fma(wl1, s(b0, a1), wr1 * s(b0, b1));
-    const T e = fma(wl0, ta, wr0 * tb);
-    Dfull[idx] = e + Dfull[idx];
+    T ta[2][2], tb[2][2];
+    plane(a0, ta);
+    plane(b0, tb);
+#pragma unroll
+    for (int k1 = 0; k1 < 2; ++k1)
+#pragma unroll
+      for (int k2 = 0; k2 < 2; ++k2)
+        if ((!k1 || f1) && (!k2 || f2))
+          u[(int64_t)k1 * n2 + k2] = fma(wl0, ta[k1][k2], wr0 * tb[k1][k2]) + d[k1][k2];
   }
 }
 

@@ -88,3 +88,26 @@ def test_loss_gradient_central_differences(bm):
     ad = torch.dot(grad, d)
     # the loss is quadratic in c: central differences are exact up to rounding
     assert abs(fd.item() - ad.item()) <= 1e-6 * abs(ad.item())
+
+
+# Global grids whose lines take every segment length of the scans (up to 32,
+# 96, 288 and 544 coarse nodes) and the sweep of longer ones, along each
+# dimension, with a few lines (tiles of 8 or 4) and with many (32 or 16).
+LINES = [(300, 20, 19), (19, 1000, 20), (20, 18, 3000), (4100, 18, 19), (18, 4100, 19), (18, 19, 4100),
+         (330, 340, 40), (3000, 40, 70)]
+
+
+@pytest.mark.parametrize("shape", LINES)
+def test_global_lines_of_every_length(bm, shape):
+    g = torch.Generator(device="cpu").manual_seed(sum(shape))
+    x = torch.randn(shape, generator=g, dtype=torch.float64).to(DEV)
+    y = torch.randn(bm.coeff_count(shape, 17, 2, 2), generator=g, dtype=torch.float64).to(DEV)
+    dec, rec = bm.decompose(x, 17, 2, 2), bm.recompose(y, shape, 17, 2, 2)
+    gu, gc = bm.decompose_adjoint(y, shape, 17, 2, 2), bm.recompose_adjoint(x, 17, 2, 2)
+    # a sum of n products of unit variance each rounds to about sqrt(n) eps of its terms' size
+    bound = 64 * 2.0 ** -53 * x.numel() ** 0.5 * 64
+    assert abs((torch.dot(dec, y) - torch.dot(x.ravel(), gu.ravel())).item()) <= bound
+    assert abs((torch.dot(rec.ravel(), x.ravel()) - torch.dot(y, gc)).item()) <= bound
+    # FP32 against FP64: a level's few dozen roundings of 2^-24 of the values' size
+    for a, b in ((bm.decompose_adjoint(y.float(), shape, 17, 2, 2), gu), (bm.recompose_adjoint(x.float(), 17, 2, 2), gc)):
+        assert (a.double() - b).abs().max().item() <= 64 * 2.0 ** -24 * b.abs().max().item()
