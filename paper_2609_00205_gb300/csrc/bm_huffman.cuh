@@ -209,6 +209,78 @@ __device__ int radix_sort_pairs(unsigned* ka, uint16_t* sa, unsigned* kb, uint16
   }
   return cur;
 }
+// The same sort of at most 8 kCbThreads pairs, whose keys, payloads and ranks
+// within (digit, warp) stay in registers between the counting and the scatter:
+// one walk instead of two.
+__device__ int radix_sort_pairs_small(unsigned* ka, uint16_t* sa, unsigned* kb, uint16_t* sb, unsigned* wcnt, int n,
+                                      unsigned maxkey, unsigned* scan_tmp) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int rows = (n + kCbThreads - 1) / kCbThreads;  // at most 8
+  const int base_i = wid * rows * 32 + lane;
+  int passes = 1;
+  while (passes < 4 && (maxkey >> (8 * passes)) != 0u) ++passes;
+  int cur = 0;
+  for (int p = 0; p < passes; ++p) {
+    const int shift = 8 * p;
+    const unsigned* kin = cur ? kb : ka;
+    const uint16_t* sin = cur ? sb : sa;
+    unsigned* kout = cur ? ka : kb;
+    uint16_t* sout = cur ? sa : sb;
+    unsigned kk[8], rk[8];
+    uint16_t pp[8];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      const int i = base_i + 32 * t;
+      const bool ok = t < rows && i < n;
+      kk[t] = ok ? kin[i] : 0u;
+      pp[t] = ok ? sin[i] : (uint16_t)0;
+    }
+    for (int i = threadIdx.x; i < 256 * 32; i += blockDim.x) wcnt[i] = 0u;
+    __syncthreads();
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      if (t < rows) {
+        const bool ok = base_i + 32 * t < n;
+        const unsigned d = (kk[t] >> shift) & 255u;
+        const unsigned m = __match_any_sync(0xffffffffu, ok ? d : 256u);
+        const unsigned lt = m & ((1u << lane) - 1u);
+        const unsigned before = ok ? wcnt[wc_idx(d, wid)] : 0u;
+        __syncwarp();
+        if (ok && lt == 0u) wcnt[wc_idx(d, wid)] = before + (unsigned)__popc(m);
+        rk[t] = before + (unsigned)__popc(lt);
+        __syncwarp();
+      }
+    }
+    __syncthreads();
+    // exclusive scan in (digit, warp) order: thread t owns entries 8t .. 8t+7
+    unsigned v[8], sum = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int k = threadIdx.x * 8 + j;
+      v[j] = wcnt[wc_idx((unsigned)k >> 5, k & 31)];
+      sum += v[j];
+    }
+    unsigned pre = block_excl_scan(sum, scan_tmp, nullptr);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int k = threadIdx.x * 8 + j;
+      wcnt[wc_idx((unsigned)k >> 5, k & 31)] = pre;
+      pre += v[j];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      if (t < rows && base_i + 32 * t < n) {
+        const unsigned dst = wcnt[wc_idx((kk[t] >> shift) & 255u, wid)] + rk[t];
+        kout[dst] = kk[t];
+        sout[dst] = pp[t];
+      }
+    }
+    __syncthreads();
+    cur ^= 1;
+  }
+  return cur;
+}
 
 __device__ __forceinline__ int upper_bound_u32(const unsigned* a, int lo, int hi, unsigned v) {
   while (lo < hi) {
@@ -223,7 +295,7 @@ __device__ __forceinline__ int upper_bound_u32(const unsigned* a, int lo, int hi
 __device__ __forceinline__ int warp_upper_bound_u32(const unsigned* a, int lo, int hi, unsigned v) {
   const int lane = threadIdx.x & 31;
   while (hi - lo > 32) {
-    const int step = (hi - lo + 31) / 32;
+    const int step = (hi - lo + 31) >> 5;
     const int p = min(lo + (lane + 1) * step, hi) - 1;
     const unsigned m = __ballot_sync(0xffffffffu, a[p] > v);
     if (m == 0u) return hi;
@@ -554,17 +626,22 @@ __device__ __forceinline__ unsigned merge_pairs(const unsigned* A, int na, const
   unsigned leaves = 0;
   int j = d0 - i;
   for (int d = d0; d < d1; d += 2) {
-    int id[2];
-    unsigned w[2];
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-      if (i < na && (j >= nb || A[i] <= B[j])) { w[t] = A[i]; id[t] = aid0 + i; ++i; ++leaves; }
-      else { w[t] = B[j]; id[t] = bid0 + j; ++j; }
-    }
+    // both queues' next two read together (~0u past a queue's end: a weight is
+    // below 2^31, and a pair's two nodes exist)
+    const unsigned a0 = i < na ? A[i] : ~0u, a1 = i + 1 < na ? A[i + 1] : ~0u;
+    const unsigned b0 = j < nb ? B[j] : ~0u, b1 = j + 1 < nb ? B[j + 1] : ~0u;
+    const bool f = a0 <= b0;                    // the first is a leaf
+    const bool s = f ? a1 <= b0 : a0 <= b1;     // the second is a leaf
+    const int i2 = i + (f ? 1 : 0), j2 = j + (f ? 0 : 1);
+    const int id0 = f ? aid0 + i : bid0 + j, id1 = s ? aid0 + i2 : bid0 + j2;
+    const unsigned w = (f ? a0 : b0) + (s ? (f ? a1 : a0) : (f ? b0 : b1));
+    i = i2 + (s ? 1 : 0);
+    j = j2 + (s ? 0 : 1);
+    leaves += (f ? 1u : 0u) + (s ? 1u : 0u);
     const int k = (rank0 + d) >> 1;
-    iw[qe + k] = w[0] + w[1];
-    parent[id[0]] = (IdT)(n + qe + k);
-    parent[id[1]] = (IdT)(n + qe + k);
+    iw[qe + k] = w;
+    parent[id0] = (IdT)(n + qe + k);
+    parent[id1] = (IdT)(n + qe + k);
   }
   return leaves;
 }
@@ -610,7 +687,8 @@ __device__ void codebook_sort(const CodebookArgs& a, const CbArrays<IdT>& V, int
   for (int o = 16; o; o >>= 1) mk = max(mk, __shfl_xor_sync(0xffffffffu, mk, o));
   if ((threadIdx.x & 31) == 0 && mk) atomicMax(&s_maxk, mk);
   __syncthreads();
-  const int which = radix_sort_pairs(V.ka, V.sa, V.kb, V.sb, V.wcnt, n, s_maxk, scan_tmp);
+  const int which = n <= 8 * kCbThreads ? radix_sort_pairs_small(V.ka, V.sa, V.kb, V.sb, V.wcnt, n, s_maxk, scan_tmp)
+                                        : radix_sort_pairs(V.ka, V.sa, V.kb, V.sb, V.wcnt, n, s_maxk, scan_tmp);
   if (which) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
       V.ka[i] = V.kb[i];
@@ -622,7 +700,7 @@ __device__ void codebook_sort(const CodebookArgs& a, const CbArrays<IdT>& V, int
 
 // At most kCbSmemSyms present symbols: every array in shared memory.
 __device__ void codebook_lengths(const CodebookArgs& a, CbArrays<uint16_t> V, int n, unsigned* scan_tmp) {
-  __shared__ unsigned s_lp, s_qp, s_qe, s_pl, s_pq, s_leaves, s_rounds, s_maxd;
+  __shared__ unsigned s_p[2], s_leaves, s_maxd;
   if (n <= 1) {
     if (n == 1 && threadIdx.x == 0) V.clen[0] = 1;
     __syncthreads();
@@ -633,40 +711,28 @@ __device__ void codebook_lengths(const CodebookArgs& a, CbArrays<uint16_t> V, in
     codebook_sort(a, V, n, scan_tmp, shift);
     const unsigned* lw = V.ka;
     const uint16_t* ls = V.sa;
-    if (threadIdx.x == 0) { s_lp = 0; s_qp = 0; s_qe = 0; s_rounds = 0; s_leaves = 0; }
-    __syncthreads();
-    // 2. parallel rounds of the two-queue construction: the previous round is
-    // folded into the queue state and this round's pairs picked: all nodes of
-    // weight <= X (X = the two smallest weights summed), found by warp-wide
-    // searches of both sorted queues.
-    int np_prev = 0;
-    while (true) {
-      if (threadIdx.x == 0 && np_prev) {
-        s_lp += s_leaves;
-        s_qp += 2 * np_prev - s_leaves;
-        s_qe += np_prev;
-        V.round_end[s_rounds++] = (uint16_t)s_qe;
-        s_leaves = 0;
+    // 2. parallel rounds of the two-queue construction: a round pairs all nodes
+    // of weight <= X (X = the two smallest weights summed), found by warp-wide
+    // searches of both sorted queues.  Every thread keeps the queues' state; the
+    // leaves a round takes come from the thread that owns the round's last rank.
+    // Bound by the latency of a round's steps (about 1,900 cycles, 18 rounds for
+    // 1,749 symbols).  With the leaves counted by atomics and folded into a
+    // shared state behind a third barrier, and the sort in two walks, the whole
+    // codebook of 65^3 at 1e-3 took 63 us against 57 (1535x2049, 3,660 symbols:
+    // 75 against 67); every warp making the searches for itself, one barrier a
+    // round, was no faster than that (the tree 25 us against 22).
+    unsigned lp = 0, qp = 0, qe = 0;
+    int rounds = 0;
+    while (qe < (unsigned)(n - 1)) {
+      if (threadIdx.x < 64) {  // warps 0 and 1: the leaves and the internal nodes that weigh at most X
+        const unsigned X = two_smallest(lw, lp, (unsigned)n, V.iw, qp, qe);
+        const bool first = threadIdx.x < 32;
+        const int from = (int)(first ? lp : qp);
+        const int cnt = warp_upper_bound_u32(first ? lw : V.iw, from, first ? n : (int)qe, X) - from;
+        if ((threadIdx.x & 31) == 0) s_p[first ? 0 : 1] = (unsigned)cnt;
       }
       __syncthreads();
-      // warps 0 and 1 find, side by side, how many leaves and how many
-      // internal nodes weigh at most X (both compute X)
-      if (threadIdx.x < 64) {
-        const unsigned lp = s_lp, qp = s_qp, qe = s_qe;
-        if (qe < (unsigned)(n - 1)) {
-          const unsigned X = two_smallest(lw, lp, (unsigned)n, V.iw, qp, qe);
-          if (threadIdx.x < 32) {
-            const int pl = warp_upper_bound_u32(lw, (int)lp, n, X) - (int)lp;
-            if (threadIdx.x == 0) s_pl = (unsigned)pl;
-          } else {
-            const int pq = warp_upper_bound_u32(V.iw, (int)qp, (int)qe, X) - (int)qp;
-            if (threadIdx.x == 32) s_pq = (unsigned)pq;
-          }
-        }
-      }
-      __syncthreads();
-      if (s_qe >= (unsigned)(n - 1)) break;
-      const int lp = s_lp, qp = s_qp, qe = s_qe, pl = s_pl, pq = s_pq;
+      const int pl = (int)s_p[0], pq = (int)s_p[1];
       const int npairs = (pl + pq) >> 1;
       // the first 2*npairs nodes of the merged order (leaf first on equal
       // weight) pair up in order.  Merge path: thread t takes the ranks
@@ -675,7 +741,6 @@ __device__ void codebook_lengths(const CodebookArgs& a, CbArrays<uint16_t> V, in
       const unsigned* A = lw + lp;
       const unsigned* Bq = V.iw + qp;
       const int T = 2 * npairs;
-      unsigned leaves = 0;
       const int seg = 2 * ((npairs + (int)blockDim.x - 1) / (int)blockDim.x);
       const int d0 = min(T, (int)threadIdx.x * seg), d1 = min(T, d0 + seg);
       if (d0 < d1) {
@@ -684,11 +749,17 @@ __device__ void codebook_lengths(const CodebookArgs& a, CbArrays<uint16_t> V, in
           const int mid = (lo + hi) >> 1;
           if (A[mid] <= Bq[d0 - 1 - mid]) lo = mid + 1; else hi = mid;
         }
-        leaves = merge_pairs<uint16_t>(A, pl, Bq, pq, d0, d1, lo, lp, n + qp, qe, 0, V.iw, V.parent, n);
+        const unsigned leaves = merge_pairs<uint16_t>(A, pl, Bq, pq, d0, d1, lo, (int)lp, n + (int)qp, (int)qe, 0, V.iw,
+                                                      V.parent, n);
+        if (d1 == T) s_leaves = (unsigned)lo + leaves;
       }
-      if (leaves) atomicAdd(&s_leaves, leaves);
-      np_prev = npairs;
+      if (threadIdx.x == 0) V.round_end[rounds] = (uint16_t)(qe + npairs);
       __syncthreads();
+      const unsigned taken = s_leaves;  // written again after the next barrier
+      lp += taken;
+      qp += (unsigned)T - taken;
+      qe += (unsigned)npairs;
+      ++rounds;
     }
     // 3. depths, rounds in reverse (a parent is always created in a later
     // round)
@@ -698,7 +769,7 @@ __device__ void codebook_lengths(const CodebookArgs& a, CbArrays<uint16_t> V, in
       s_maxd = 0;
     }
     __syncthreads();
-    for (int r = (int)s_rounds - 1; r >= 0; --r) {
+    for (int r = rounds - 1; r >= 0; --r) {
       const int jb = r ? (int)V.round_end[r - 1] : 0, je = (int)V.round_end[r];
       for (int j = jb + threadIdx.x; j < je; j += blockDim.x) {
         const int v = n + j;

@@ -62,3 +62,27 @@ def test_many_cta_codebook_of_a_compress_call(scale):
     np.testing.assert_array_equal(got, sec[off:off + meta["codebook_bytes"]])
     d = bm.decompress(torch.from_numpy(sg.copy()).to("cuda")).cpu().numpy()
     assert np.abs(d.astype(np.float64) - u).max() <= tol
+
+
+@pytest.mark.parametrize("kind", ["equal", "ramp", "skewed", "ties", "doubling"])
+@pytest.mark.parametrize("n", [1, 2, 3, 31, 33, 64, 1023, 1024, 1025, 2049, 7169, 8191, 8192])
+def test_lengths_in_shared_memory(n, kind):
+    """The tree of one block: rows of the sort, a thread's ranks of a round, and
+    rounds of a single pair (counts that double)."""
+    import paper_2609_00205_gb300 as bm
+
+    rng = np.random.default_rng(n)
+    present = np.sort(rng.choice(65536, n, replace=False))
+    if kind == "doubling":
+        counts = 2 ** np.minimum(np.arange(n), 19)[rng.permutation(n)] if n <= 64 else 1 + (np.arange(n) % 20 == 0) * 300
+        counts = np.minimum(counts, 2 ** 19)
+    elif kind == "skewed" and n < 64:
+        counts = 2 ** rng.integers(0, 18, n)
+    else:
+        counts = _counts(kind, n, rng)
+    sym = np.repeat(present, counts).astype(np.uint16)
+    rng.shuffle(sym)
+    so, mo = oracle.huffman_encode(sym, 65536, 2048)
+    sg, mg = bm.huffman_encode(torch.from_numpy(sym.view(np.int16)).to("cuda"), 65536, 2048)
+    assert mg == mo
+    np.testing.assert_array_equal(sg.cpu().numpy(), so)
