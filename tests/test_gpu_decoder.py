@@ -69,3 +69,54 @@ def test_damaged_codebooks_are_refused_or_decoded():
             assert err.status == 4
     torch.cuda.synchronize()
     _round_trip(sym, 4096, 2048)
+
+
+def _present(kind, n_runs, rng):
+    """Symbols of n_runs runs: of one symbol, of a few, or with long ones among
+    them (255 to 700 symbols, around the limit of a thread's own copy)."""
+    if kind == "ones":
+        return np.arange(n_runs) * 2
+    lens = rng.integers(1, 5, n_runs)
+    if kind == "long":
+        at = rng.choice(n_runs, 24, replace=False)
+        lens[at] = rng.integers(255, 700, 24)
+        lens[at[:3]] = (255, 256, 257)
+    gaps = 1 + rng.integers(0, 3, n_runs)
+    first = np.cumsum(np.concatenate([[0], lens[:-1] + gaps[:-1]]))
+    return np.concatenate([np.arange(f, f + c) for f, c in zip(first, lens) if f + c <= 65536])
+
+
+@pytest.mark.parametrize("kind", ["ones", "few", "long"])
+@pytest.mark.parametrize("n_runs", [512, 513, 514, 1000, 2731, 8000, 10922, 10923])
+def test_run_headers_side_by_side(kind, n_runs):
+    """Around the run count from which the headers are walked in segments, and
+    the section size (10,922 runs of one symbol) up to which they are."""
+    rng = np.random.default_rng(n_runs)
+    present = _present(kind, n_runs, rng)
+    sym = np.concatenate([present, rng.choice(present, 9000)]).astype(np.uint16)
+    rng.shuffle(sym)
+    _round_trip(sym, 65536, 512)
+
+
+@pytest.mark.parametrize("word,value", [(0, 60000), (1, 65537), (1, 0xFFFFFFFF), (1, 40000), (3 * 777, 0), (3 * 777, 65536),
+                                        (3 * 777 + 1, 4), (3 * 777 + 1, 0), (3 * 1999 + 1, 0xFFFFFFF0), (3 * 777 + 2, 33)])
+def test_damaged_headers_of_many_runs(word, value):
+    """One word of a section of 2,000 runs of one symbol changed on the host: an
+    error, and the context stays usable.  (The symbols are three apart: a count
+    of 3 takes the padding as lengths of 0 and overlaps nothing, which is a
+    valid section; 4 is the least that is not.)"""
+    import paper_2609_00205_gb300 as bm
+
+    rng = np.random.default_rng(word)
+    present = np.arange(2000) * 3 + 100
+    sym = np.concatenate([present, rng.choice(present, 9000)]).astype(np.uint16)
+    so, mo = oracle.huffman_encode(sym, 65536, 512)
+    assert mo["n_runs"] == 2000 and mo["codebook_bytes"] == 24000
+    off = (4 * mo["n_chunks"] + 7) // 8 * 8 + (14 * mo["n_chunks"] + 7) // 8 * 8
+    bad = so.copy()
+    bad[off:off + 24000].view(np.uint32)[word] = value
+    with pytest.raises(Exception):
+        bm.huffman_decode(torch.from_numpy(bad).to("cuda"), mo, sym.size, 65536, 512)
+        torch.cuda.synchronize()
+    back = bm.huffman_decode(torch.from_numpy(so).to("cuda"), mo, sym.size, 65536, 512)
+    np.testing.assert_array_equal(back.cpu().numpy().view(np.uint16), sym)
