@@ -971,8 +971,8 @@ cudaError_t launch_apply(const GLevel<T>& L, const T* in, T* out, const T* U, cu
 // The passes after the first of a global level's restriction: dimension 1,
 // then dimension 0 with FINAL.  A dimension 0 that is not coarsened (at most
 // two nodes: every plane) has nothing to restrict and the dimension-1 pass is
-// the last one, its outputs laid out alike (1535x2049: 10 and 5 us of a
-// compress call's 301 saved).
+// the last one, its outputs laid out alike (1535x2049: the passes took 13 + 10
+// and 9 + 5 us, in one 19 and 14, and a launch less each).
 template <typename T, int FINAL>
 cudaError_t launch_apply10(const GLevel<T>& L, const T* W1, T* W2, T* out, const T* U, cudaStream_t s) {
   if (L.d[0].c == L.d[0].n && line_segment(L.d[1].c)) return launch_apply<T, 1, FINAL>(L, W1, out, U, s);

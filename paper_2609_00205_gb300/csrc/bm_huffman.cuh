@@ -2363,8 +2363,8 @@ __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) encode_fused_kernel(Fu
 // codes too few symbols to pay for a copy of it, and a CTA of eight warps
 // takes 8.5 KB of shared memory, so that the items of a batch share an
 // SM.  In place of the three launches above, two of which return at once (but
-// wait for an SM with 200 KB of free shared memory to do so): 64 fields of up
-// to 64^3 in a batch 4.60 ms against 4.45, 65^3 0.195 ms against 0.176; with the
+// wait for an SM with 200 KB of free shared memory to do so): 64 uneven fields
+// in a batch 4.60 ms against 4.45, 65^3 0.195 ms against 0.176; with the
 // tables copied by one kernel of any mode 5.57 and 0.181.
 constexpr int kEncSmallChunks = 8;
 constexpr size_t kEncSmallSmem = enc_smem<5>(8, 0, 0);
@@ -2510,7 +2510,7 @@ __device__ __forceinline__ void walk_runs_parallel(DtSmem& S, unsigned long long
 // the lengths of more than 8192 present symbols in global scratch, with a
 // binary search of the runs per length and the look-up table of the decoder
 // filled here too, took 0.129 ms at 513^3, 1e-4 (65,532 present symbols)
-// against 0.042, and 0.091 at 1e-3 (593 runs) against 0.077.
+// against 0.042, and 0.091 at 1e-3 (593 runs) against 0.050.
 __device__ __forceinline__ void decode_tables_block(const uint8_t* runs, unsigned long long nbytes,
                                                     unsigned long long n_runs, int dict, DecodeTables* out,
                                                     Scalars* sc, unsigned char* smem_raw) {
