@@ -327,6 +327,12 @@ __device__ __forceinline__ HiLo<T> hl_affine(T m, HiLo<T> a, HiLo<T> b) {
   return {s, fma(m, a.lo, rn_add(rn_add(pe, e), b.lo))};
 }
 
+// The value (an infinity has no rounding error: NaN in lo).
+template <typename T>
+__device__ __forceinline__ T hl_value(HiLo<T> a) {
+  return rn_add(a.lo, -a.lo) == T(0) ? rn_add(a.hi, a.lo) : a.hi;
+}
+
 // z = M_c^-1 r of one line in shared memory, in place, by a warp: the scans
 // of line_scan_solve with the value part of the maps carried with its rounding
 // error, so that every lane replays its rows from a rounded exact input.  The
@@ -359,7 +365,7 @@ __device__ __forceinline__ void line_scan_solve_hl(const GDim<T>& D, T* r, const
       m *= pm;
     }
   }
-  T prev = __shfl_up_sync(0xffffffffu, rn_add(a.hi, a.lo), 1);
+  T prev = __shfl_up_sync(0xffffffffu, hl_value(a), 1);
   if (lane == 0) prev = T(0);
 #pragma unroll
   for (int k = 0; k < E; ++k) {
@@ -391,7 +397,7 @@ __device__ __forceinline__ void line_scan_solve_hl(const GDim<T>& D, T* r, const
       m *= pm;
     }
   }
-  T next = __shfl_down_sync(0xffffffffu, rn_add(a.hi, a.lo), 1);
+  T next = __shfl_down_sync(0xffffffffu, hl_value(a), 1);
   if (lane == 31) next = T(0);
   __syncwarp();  // every lane has read its r before any z overwrites it
 #pragma unroll

@@ -282,13 +282,6 @@ __device__ int radix_sort_pairs_small(unsigned* ka, uint16_t* sa, unsigned* kb, 
   return cur;
 }
 
-__device__ __forceinline__ int upper_bound_u32(const unsigned* a, int lo, int hi, unsigned v) {
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (a[mid] <= v) lo = mid + 1; else hi = mid;
-  }
-  return lo;
-}
 // upper_bound by the 32 lanes of a warp (all lanes call it with the same
 // arguments and get the same result): each step probes the last element of 32
 // equal segments and keeps the first segment whose last element exceeds v.
@@ -363,14 +356,6 @@ __device__ __forceinline__ int warp_merge_split(const unsigned* A, int na, const
   }
   const unsigned m = __ballot_sync(0xffffffffu, lane < hi - lo && after(lo + lane));
   return m ? lo + __ffs(m) - 1 : hi;
-}
-
-__device__ __forceinline__ int lower_bound_u32(const unsigned* a, int lo, int hi, unsigned v) {
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (a[mid] < v) lo = mid + 1; else hi = mid;
-  }
-  return lo;
 }
 
 // First codes, first positions, left-justified limits, the symbol count and
