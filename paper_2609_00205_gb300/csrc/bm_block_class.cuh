@@ -131,8 +131,8 @@ __device__ __forceinline__ void coarse_sums(const T* r00, const T* r01, const T*
 
 // One line of the first forward pass: coefficients d = u - I(u|C), staged,
 // then the restriction and solve along the line into T1.  The values are those
-// of the general expression of level_fwd (for fields below a quarter of the
-// largest number).
+// of the general expression of level_fwd (field_huge excludes the fields whose
+// sums could overflow here first).
 template <typename T, int N, int CLS>
 __device__ __forceinline__ void fwd_line(const T* X, T* T1, T* out, const int i0,
                                          const int i1, const int lvl_off, const T rq, uint16_t* stage,
@@ -206,12 +206,14 @@ constexpr int lvl_stride(int j) {
   return j == 0 ? cube(B) : (j & 1) ? cube((B + 1) / 2) : cube(((B + 1) / 2 + 1) / 2);
 }
 
-// Whether a field holds values from which a sum of four can overflow: its
-// lines then take the general expression (its infinities make the stream raw).
-template <typename T>
+// Whether a field holds values of 2^960 or more: its lines then take the
+// general expression, whose infinities make the stream raw.  A both-odd line
+// adds eight values before it scales them, the general expression four, so the
+// two part ways from values of 2^1021 on; a level's coarse values are at most
+// 55 times its input's largest one (|z| <= 3^3 times the coefficients, which are
+// at most twice the values), so no level of a smaller field comes near.
 __device__ __forceinline__ bool field_huge(const Scalars* sc) {
-  const unsigned long long m = __ldcg(&sc->maxabs_bits);
-  return sizeof(T) == 4 ? (unsigned)m >= 0x7E800000u : m >= 0x7FD0000000000000ull;  // 2^126, 2^1022
+  return __ldcg(&sc->maxabs_bits) >= 0x7BF0000000000000ull;  // 2^960
 }
 
 // ---------------------------------------------------------------------------
@@ -327,7 +329,7 @@ __device__ __forceinline__ void fwd_group(const BlockArgs<double>& a, const int6
   const int64_t sbase = b * (int64_t)Cfg::PB;
   const LevelBufs<double> bufs{A, cb0, cb1};
   const bool full = a.radius == (1 << 15) && !BM_FWD_HIST;
-  GroupFwdLevels<B, 0, K, B>::run(bufs, T1, s_rq, stage, a.esc + sbase, ovf, full, field_huge<double>(a.sc), nv);
+  GroupFwdLevels<B, 0, K, B>::run(bufs, T1, s_rq, stage, a.esc + sbase, ovf, full, field_huge(a.sc), nv);
   for (int blk = 0; blk < nv; ++blk) {  // block coarse values -> gathered grid G
     constexpr int M = Cfg::M;
     const BlockCoord bc(b + blk, a.nb1, a.nb2);
@@ -381,7 +383,13 @@ __device__ __forceinline__ void inv_line(T* X, T* T1, const int i0, const int i1
   for (int j = 0; j < C; ++j) T1[(i0 * C + j) * N + i1] = z[j];
 }
 
-// One line of the last inverse pass: u = I(u|C) + d in X.
+// Whether a value is 2^1023 or more in magnitude, an infinity or NaN (on its
+// bits: integer work, not the double unit's).
+__device__ __forceinline__ bool top_binade(double v) { return ((unsigned)__double2hiint(v) << 1) >= 0xFFC00000u; }
+
+// One line of the last inverse pass: u = I(u|C) + d in X.  A both-odd line adds
+// two sums of four: where one lies in the top binade the sums are scaled first
+// (exact), so that only the sum of four itself can overflow.
 template <typename T, int N, int CLS>
 __device__ __forceinline__ void interp_line(T* X, const T* cin, const int i0, const int i1) {
   constexpr int C = (N + 1) / 2;
@@ -389,11 +397,22 @@ __device__ __forceinline__ void interp_line(T* X, const T* cin, const int i0, co
   T v[C];
   coarse_sums<T, C, CLS>(cin + (a0 * C + a1) * C, cin + (a0 * C + b1) * C, cin + (b0 * C + a1) * C,
                          cin + (b0 * C + b1) * C, 1, v);
-  constexpr T se = CLS == 2 ? T(0.25) : CLS == 1 ? T(0.5) : T(1);
+  T se = CLS == 2 ? T(0.25) : CLS == 1 ? T(0.5) : T(1), ho = T(0.5) * se;
+  if (CLS == 2) {
+    bool top = false;
+#pragma unroll
+    for (int J = 0; J < C; ++J) top |= top_binade(v[J]);
+    if (top) {
+#pragma unroll
+      for (int J = 0; J < C; ++J) v[J] *= T(0.25);
+      se = T(1);
+      ho = T(0.5);
+    }
+  }
   T* x = X + (i0 * N + i1) * N;
 #pragma unroll
   for (int k = 0; k < N; ++k) {
-    if (k & 1) x[k] = fma(T(0.5) * se, v[k / 2] + v[k / 2 + 1], x[k]);
+    if (k & 1) x[k] = fma(ho, v[k / 2] + v[k / 2 + 1], x[k]);
     else if (CLS) x[k] = fma(se, v[k / 2], x[k]);
     else x[k] = v[k / 2];
   }

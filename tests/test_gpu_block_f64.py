@@ -1,7 +1,7 @@
 """The coded double kernels (groups of four 9-node blocks, lines by parity
 class): block counts of every remainder modulo four, every level count, ROI
-tiers per block of a group, coefficients at the range check's edge, and fields
-so large that sums of four values overflow."""
+tiers per block of a group, and fields so large that sums of four values, or of
+eight, overflow."""
 import numpy as np
 import pytest
 import torch
@@ -54,3 +54,27 @@ def test_sums_that_overflow_give_the_oracles_raw_copy(B, K):
     assert oracle.stream_header(so)["raw"]
     s = bm.compress(torch.from_numpy(u).to("cuda"), 1e-3, block=B, levels=K, global_levels=1).cpu().numpy()
     np.testing.assert_array_equal(s, so)
+
+
+def _huge_field(kind, shape):
+    p = 2.0 ** 1022
+    u = np.full(shape, 0.6 * p)  # a sum of four is finite, one of eight is not
+    if kind == "peak":  # the largest value above 2^1022, alone
+        u[:] = 0.9 * p
+        u[3, 5, 7] = 1.05 * p
+    return u
+
+
+@pytest.mark.parametrize("B,K", [(9, 1), (9, 3), (17, 1), (17, 4)])
+@pytest.mark.parametrize("kind", ["flat", "peak"])
+def test_fields_whose_sums_of_eight_overflow(kind, B, K):
+    """The oracle codes these fields, and so must the kernels, in both
+    directions (check_stream_parity decodes and checks the bound)."""
+    import paper_2609_00205_gb300 as bm
+
+    # whole blocks for several levels: the zeros around a field make its coarse
+    # values overshoot, and a sum of four of them must stay finite
+    u = _huge_field(kind, (20, 19, 21) if K == 1 else (2 * B, B, 3 * B))
+    s = bm.compress(torch.from_numpy(u).to("cuda"), 1e-3, block=B, levels=K, global_levels=1).cpu().numpy()
+    assert not oracle.stream_header(s)["raw"]
+    check_stream_parity(bm, u, s, 1e-3, "rel", B, K, 1, label=f"f64_huge_{kind}_{B}_{K}")
