@@ -2522,13 +2522,16 @@ __device__ __forceinline__ void decode_tables_block(const uint8_t* runs, unsigne
   }
   __syncthreads();
   // walk the run headers (serial, 512 at a time), then spread the batch's
-  // lengths: short runs a warp each, long ones by the whole block
+  // lengths: short runs a warp each, long ones by the whole block.  A fault is
+  // collected in registers and the barrier's OR decides, so that all threads
+  // leave the loop together.
   constexpr unsigned kLongRun = 1024;
   unsigned long long off = 0;
   const bool parallel = rbase != runs && n_runs > kDtWalkRuns;
   if (parallel) walk_runs_parallel(S, nbytes, n_runs, (unsigned)dict, &s_bad, &s_long);
   for (unsigned long long rb = 0; rb < (parallel ? 0ull : n_runs); rb += 512) {
     const int nb = (int)min(512ull, n_runs - rb);
+    bool bad = false;
     if (threadIdx.x == 0) {  // the chain of headers only: their checks follow in parallel
       bool ok = true;
       for (int q = 0; q < nb && ok; ++q) {
@@ -2538,11 +2541,13 @@ __device__ __forceinline__ void decode_tables_block(const uint8_t* runs, unsigne
         ok &= cnt <= (unsigned)dict;
         off += 8ull + ((cnt + 3u) & ~3u);
       }
-      if (!ok) s_bad = 1;
+      bad = !ok;
       s_long = 0;
     }
-    __syncthreads();
-    if (s_bad) break;
+    if (__syncthreads_or(bad)) {
+      s_bad = 1;
+      break;
+    }
     if (threadIdx.x < (unsigned)nb) {
       const unsigned o = S.roff[threadIdx.x];
       const unsigned first = *reinterpret_cast<const unsigned*>(rbase + o);
@@ -2550,18 +2555,19 @@ __device__ __forceinline__ void decode_tables_block(const uint8_t* runs, unsigne
       S.rfirst[threadIdx.x] = first;
       S.rcount[threadIdx.x] = cnt;
       S.roff[threadIdx.x] = o + 8u;
-      if ((unsigned long long)first + cnt > (unsigned long long)dict || (unsigned long long)o + 8 + cnt > nbytes) s_bad = 1;
+      if ((unsigned long long)first + cnt > (unsigned long long)dict || (unsigned long long)o + 8 + cnt > nbytes) bad = true;
       if (cnt >= kLongRun) s_long = 1;
     }
     __syncthreads();
     if (threadIdx.x < (unsigned)nb) {  // ascending, without overlap
       const unsigned end = threadIdx.x ? S.rfirst[threadIdx.x - 1] + S.rcount[threadIdx.x - 1] : s_end;
-      if ((threadIdx.x || rb) && S.rfirst[threadIdx.x] < end) s_bad = 1;
+      if ((threadIdx.x || rb) && S.rfirst[threadIdx.x] < end) bad = true;
     }
-    __syncthreads();
-    if (s_bad) break;
+    if (__syncthreads_or(bad)) {
+      s_bad = 1;
+      break;
+    }
     if (threadIdx.x == 0) s_end = S.rfirst[nb - 1] + S.rcount[nb - 1];
-    bool bad = false;
     for (int q = wid; q < nb; q += nw)
       if (S.rcount[q] < kLongRun)
         for (unsigned t = lane; t < S.rcount[q]; t += 32) {
@@ -2576,9 +2582,12 @@ __device__ __forceinline__ void decode_tables_block(const uint8_t* runs, unsigne
           bad |= L > kMaxLen;
           S.len[S.rfirst[q] + t] = L;
         }
-    if (bad) s_bad = 1;
-    __syncthreads();
+    if (__syncthreads_or(bad)) {
+      s_bad = 1;
+      break;
+    }
   }
+  __syncthreads();
   if (!s_bad) build_canonical(S.len, dict, S.wcnt, out->canon, &S.ct);
   // the lengths must satisfy Kraft's inequality (in units of 2^-32)
   if (threadIdx.x == 0) {

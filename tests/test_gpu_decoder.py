@@ -120,3 +120,41 @@ def test_damaged_headers_of_many_runs(word, value):
         torch.cuda.synchronize()
     back = bm.huffman_decode(torch.from_numpy(so).to("cuda"), mo, sym.size, 65536, 512)
     np.testing.assert_array_equal(back.cpu().numpy().view(np.uint16), sym)
+
+
+@pytest.mark.parametrize("n_runs,step", [(40, 1400), (600, 100), (11_000, 5)])
+@pytest.mark.parametrize("what", ["first", "count", "order", "length", "long length"])
+def test_damaged_sections_walked_in_batches(n_runs, step, what):
+    """Few runs, and a section too long for the shared-memory copy (several
+    batches of headers): every check of a batch refuses the stream."""
+    import paper_2609_00205_gb300 as bm
+
+    lens = np.ones(n_runs, np.int64)
+    if what == "long length":
+        lens[1] = 1200  # a run that the whole block copies
+    first = np.concatenate([[0], np.cumsum(np.maximum(lens, step - 3)[:-1] + 3)])
+    keep = first + lens <= 65536
+    n_runs, first, lens = int(keep.sum()), first[keep], lens[keep]
+    present = np.concatenate([np.arange(f, f + c) for f, c in zip(first, lens)])
+    rng = np.random.default_rng(n_runs)
+    sym = np.concatenate([present, rng.choice(present, 9000)]).astype(np.uint16)
+    so, mo = oracle.huffman_encode(sym, 65536, 512)
+    assert mo["n_runs"] == n_runs and (n_runs <= 600 or mo["codebook_bytes"] > 128 * 1024)
+    cb = (4 * mo["n_chunks"] + 7) // 8 * 8 + (14 * mo["n_chunks"] + 7) // 8 * 8
+    run = 1 if what == "long length" else n_runs - 2
+    at = cb + int((8 + (lens[:run] + 3) // 4 * 4).sum())
+    bad = so.copy()
+    h = bad[at:at + 8].view(np.uint32)
+    if what == "first":
+        h[0] = 65536
+    elif what == "count":
+        h[1] = 65537
+    elif what == "order":
+        h[0] = first[run - 1]
+    else:
+        bad[at + 8 + int(lens[run]) - 1] = 33
+    with pytest.raises(bm.BlockMGARDError) as e:
+        bm.huffman_decode(torch.from_numpy(bad).to("cuda"), mo, sym.size, 65536, 512)
+    assert e.value.status == 4
+    back = bm.huffman_decode(torch.from_numpy(so).to("cuda"), mo, sym.size, 65536, 512)
+    np.testing.assert_array_equal(back.cpu().numpy().view(np.uint16), sym)
