@@ -26,9 +26,6 @@
 #include "bm_plane.h"
 #include "bm_qtab.cuh"
 
-#ifndef BM_FWD_HIST
-#define BM_FWD_HIST 0
-#endif
 // The block region's histogram: on a second stream beside the global levels
 // (BM_HIST_OVERLAP) with BM_HIST_CTAS CTAs per SM.
 // BM_CB_PRESORT: a compress call's codebook starts with the multi-CTA
@@ -1127,7 +1124,7 @@ bm_status run_decompose(PlanDev& P, const T* field, int mode, const FwdOut<T>& o
       a.esc = o.esc ? o.esc + rd.off : nullptr;
       a.coef = o.coef ? o.coef + rd.off : nullptr;
       a.tier = o.tier ? o.tier + toff : nullptr;
-      a.rq = o.rq; a.hist = o.hist; a.radius = o.radius; a.sc = o.sc;
+      a.rq = o.rq; a.radius = o.radius; a.sc = o.sc;
       if (ic == Incache::Record) {
         if (rec) *rec = a;
         return BM_OK;
@@ -1667,7 +1664,6 @@ bm_status compress_t(const T* field, const int64_t* shape, const Params& prm, do
   // (the batched kernel never counts: its items take the separate pass on
   // the item's own stream)
   auto block_hist = [&]() -> bm_status {
-    if (BM_FWD_HIST && phase == kWhole) return BM_OK;
     cudaStream_t hs = s;
     const bool overlap = BM_HIST_OVERLAP && phase == kWhole;
     if (overlap) {
@@ -1696,7 +1692,7 @@ bm_status compress_t(const T* field, const int64_t* shape, const Params& prm, do
                                           phase == kFinishA ? Incache::Skip : Incache::Run);
     // join the second stream before anything else (also on errors: no work
     // of this call may outlive it)
-    if (phase == kWhole && !BM_FWD_HIST && BM_HIST_OVERLAP && ws->aux) BM_CUDA(cudaStreamWaitEvent(s, ws->ev_join, 0));
+    if (phase == kWhole && BM_HIST_OVERLAP && ws->aux) BM_CUDA(cudaStreamWaitEvent(s, ws->ev_join, 0));
     if (st) return st;
   }
   {

@@ -21,20 +21,15 @@
 #include "bm_internal.h"
 #include "bm_qtab.cuh"
 
-// Build-time choices of the forward kernel: whether it keeps the symbol
-// histogram itself (BM_FWD_HIST; otherwise a separate pass counts the
-// symbols), its threads per CTA (BM_FWD_THREADS; 0 = one per
-// line of the first pass, B^2 rounded up to whole warps) and the CTAs per SM
-// it is compiled for (BM_FWD_MIN_CTAS, capped by what shared memory holds);
-// BM_INV_THREADS and BM_INV_MIN_CTAS are the last two for the inverse.  The
-// defaults are the fastest measured on GB300 for the 513^3 FP32 workload: the
-// in-kernel histogram's shared atomics and its 32 KB cost more than a separate
-// pass, prefetching costs more than it hides, and five-warp CTAs (two lines of
-// the first pass per thread, four or more CTAs per SM) let one CTA's barrier
-// waits overlap the others' work.
-#ifndef BM_FWD_HIST
-#define BM_FWD_HIST 0
-#endif
+// Build-time choices of the forward kernel: its threads per CTA
+// (BM_FWD_THREADS; 0 = one per line of the first pass, B^2 rounded up to whole
+// warps) and the CTAs per SM it is compiled for (BM_FWD_MIN_CTAS, capped by what
+// shared memory holds); BM_INV_THREADS and BM_INV_MIN_CTAS are the same for the
+// inverse.  The defaults are the fastest measured on GB300 for the 513^3 FP32
+// workload: prefetching costs more than it hides, and five-warp CTAs (two lines
+// of the first pass per thread, four or more CTAs per SM) let one CTA's barrier
+// waits overlap the others' work.  (A histogram kept in the kernel cost more,
+// by its shared atomics and its 32 KB, than the separate pass.)
 #ifndef BM_FWD_MIN_CTAS
 #define BM_FWD_MIN_CTAS 4
 #endif
@@ -129,27 +124,25 @@ struct BlockCfg {
   static constexpr int CB1 = C2 * C2 * C2;
   static constexpr int PB = per_block_count(B, K);
   static constexpr int M = lvl_n(B, K);
-  // byte offsets: the symbol staging area and the histogram start on 16-byte
-  // boundaries (the staging area is copied out with 8-byte vectors)
+  // byte offsets: the symbol staging area starts on a 16-byte boundary (it is
+  // copied out with 8-byte vectors)
   static constexpr size_t up16(size_t x) { return (x + 15) / 16 * 16; }
   static constexpr size_t fwd_stage_off = up16(sizeof(T) * (A + T1 + CB0 + CB1));  // T2 overlays A
-  static constexpr size_t fwd_hist_off = up16(fwd_stage_off + 2 * PB);
-  static constexpr size_t fwd_hist_end = fwd_hist_off + (BM_FWD_HIST ? 4 * kHistWin : 0);
+  static constexpr size_t fwd_end = up16(fwd_stage_off + 2 * PB);
   // bulk staging: B^2 row slots of RP bytes (a row of B elements starting
   // anywhere on an element boundary, rounded out to 16-byte boundaries) from
   // the end of the block array on (over T1, the coarse buffers and the symbol
-  // staging area; after the histogram when the kernel keeps one), then the
-  // copies' mbarrier
+  // staging area), then the copies' mbarrier
   static constexpr int RP = (int)((B * sizeof(T) + 16 - sizeof(T) + 15) / 16 * 16);
-  static constexpr size_t fwd_stg_off = BM_FWD_HIST ? up16(fwd_hist_end) : up16(sizeof(T) * A);
+  static constexpr size_t fwd_stg_off = up16(sizeof(T) * A);
   // used unless the slots would cut the CTAs an SM holds (228 KB, 1 KB
   // reserved per CTA) below 16: FP64 with B = 17 keeps the element-wise copy
   static constexpr size_t fwd_stg_end = fwd_stg_off + (size_t)B * B * RP;
-  static constexpr size_t fwd_bar_off = up16(fwd_stg_end > fwd_hist_end ? fwd_stg_end : fwd_hist_end);
+  static constexpr size_t fwd_bar_off = up16(fwd_stg_end > fwd_end ? fwd_stg_end : fwd_end);
   static constexpr int fit_of(size_t bytes) { return (int)((228u * 1024u) / (bytes + 1024u)); }
   static constexpr bool BULK = BM_FWD_BULK &&
-                               (fit_of(fwd_bar_off + 16) >= fit_of(fwd_hist_end) || fit_of(fwd_bar_off + 16) >= 16);
-  static constexpr size_t fwd_smem = BULK ? fwd_bar_off + 16 : fwd_hist_end;
+                               (fit_of(fwd_bar_off + 16) >= fit_of(fwd_end) || fit_of(fwd_bar_off + 16) >= 16);
+  static constexpr size_t fwd_smem = BULK ? fwd_bar_off + 16 : fwd_end;
   static constexpr size_t inv_stage_off = up16(sizeof(T) * (A + T1 + T2 + CB0 + CB1));
   static constexpr size_t inv_smem(int mode) {
     return inv_stage_off + up16((mode ? sizeof(T) : (BM_INV_CODES ? 4 : 2)) * PB);
@@ -162,20 +155,6 @@ struct BlockCfg {
   static constexpr int inv_fit = (int)((228u * 1024u) / (inv_smem(1) + 1024u));
   static constexpr int INV_MIN_CTAS = inv_fit < 1 ? 1 : (inv_fit < BM_INV_MIN_CTAS ? inv_fit : BM_INV_MIN_CTAS);
 };
-
-// Histogram of one CTA: a window of kHistWin symbols around the centre in
-// shared memory, global atomics outside it; the centre symbol (code 0, most
-// of the symbols at loose tolerances) is counted in a register per thread and
-// added once at the end.
-__device__ __forceinline__ void hist_count(unsigned* hloc, unsigned* hglob, int radius, unsigned s, unsigned& centre) {
-  if (s == (unsigned)radius) {
-    ++centre;
-    return;
-  }
-  const int bin = (int)s - (radius - kHistWin / 2);
-  if (bin >= 0 && bin < kHistWin) atomicAdd(hloc + bin, 1u);
-  else atomicAdd(hglob + s, 1u);
-}
 
 // ---------------------------------------------------------------------------
 // Forward level
@@ -480,8 +459,7 @@ __device__ __forceinline__ void store_block(const BlockSpan<T, B>& sp, const T* 
 // the escape array) stores its other escapes one by one.
 template <int PB>
 __device__ __forceinline__ void store_codes(uint16_t* __restrict__ sym, int32_t* __restrict__ esc,
-                                            const uint16_t* __restrict__ st, const int radius, unsigned* hloc,
-                                            unsigned* hglob, unsigned& centre) {
+                                            const uint16_t* __restrict__ st, const int radius) {
   const unsigned span = (unsigned)(2 * radius - 1);
   auto to_sym = [&](unsigned b) {  // b: staged value; wide codes always escape
     const unsigned u = (unsigned)((int)b - kStageBias + radius);
@@ -516,9 +494,6 @@ __device__ __forceinline__ void store_codes(uint16_t* __restrict__ sym, int32_t*
             if (a[j] == 0u && b[j] != kStageWide) esc[4 * i + j] = (int)b[j] - kStageBias;
         }
       }
-      if (BM_FWD_HIST)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) hist_count(hloc, hglob, radius, a[j], centre);
     }
   } else {
     for (int i = threadIdx.x; i < PB; i += blockDim.x) {
@@ -526,7 +501,6 @@ __device__ __forceinline__ void store_codes(uint16_t* __restrict__ sym, int32_t*
       const unsigned a = to_sym(b);
       sym[i] = (uint16_t)a;
       if (!a && b != kStageWide) esc[i] = (int)b - kStageBias;
-      if (BM_FWD_HIST) hist_count(hloc, hglob, radius, a, centre);
     }
   }
 }
@@ -553,7 +527,6 @@ struct FwdSmem {
   T* cb0;          // coarse values of odd levels (C^3)
   T* cb1;          // coarse values of even levels
   uint16_t* stage;  // the block's staged codes
-  unsigned* hloc;  // histogram window (BM_FWD_HIST)
   uint64_t* bar;   // bulk-copy barrier (BM_FWD_BULK)
   unsigned char* stg;  // bulk-copy row slots
   __device__ __forceinline__ explicit FwdSmem(unsigned char* raw) {
@@ -563,7 +536,6 @@ struct FwdSmem {
     cb0 = T1 + Cfg::T1;
     cb1 = cb0 + Cfg::CB0;
     stage = reinterpret_cast<uint16_t*>(raw + Cfg::fwd_stage_off);
-    hloc = reinterpret_cast<unsigned*>(raw + Cfg::fwd_hist_off);
     bar = reinterpret_cast<uint64_t*>(raw + Cfg::fwd_bar_off);
     stg = raw + Cfg::fwd_stg_off;
   }
@@ -588,7 +560,7 @@ __device__ __forceinline__ void fwd_init(const FwdSmem<T, B, K>& S) {
 // the status is set and the CTA must stop.
 template <typename T, int B, int K, int MODE>
 __device__ __forceinline__ bool fwd_block(const BlockArgs<T>& a, int64_t b, const FwdSmem<T, B, K>& S,
-                                          unsigned& phase, bool& ovf, unsigned& centre) {
+                                          unsigned& phase, bool& ovf) {
   using Cfg = BlockCfg<T, B, K>;
   const BlockCoord bc(b, a.nb1, a.nb2);
   const BlockSpan<const T, B> sp(a.field, a.n0, a.n1, a.n2, bc);
@@ -615,7 +587,7 @@ __device__ __forceinline__ bool fwd_block(const BlockArgs<T>& a, int64_t b, cons
   for (int l = 0; l < K; ++l) rq[l] = MODE == 0 ? __ldcg(a.rq + tier * K + l) : T(0);
   const int64_t sbase = b * (int64_t)Cfg::PB;
   const LevelBufs<T> bufs{S.A, S.cb0, S.cb1};
-  const bool full = MODE == 0 && a.radius == (1 << 15) && !BM_FWD_HIST;
+  const bool full = MODE == 0 && a.radius == (1 << 15);
   FwdLevels<T, B, 0, K, B, MODE>::run(bufs, S.T1, rq, S.stage, a.esc + (MODE == 0 ? sbase : 0),
                                       a.coef + (MODE == 1 ? sbase : 0), ovf, full);
   {  // block coarse values -> gathered grid G
@@ -629,7 +601,7 @@ __device__ __forceinline__ bool fwd_block(const BlockArgs<T>& a, int64_t b, cons
   }
   if (MODE == 0) {
     if (full) copy_symbols<Cfg::PB>(a.sym + sbase, S.stage);
-    else store_codes<Cfg::PB>(a.sym + sbase, a.esc + sbase, S.stage, a.radius, S.hloc, a.hist, centre);
+    else store_codes<Cfg::PB>(a.sym + sbase, a.esc + sbase, S.stage, a.radius);
   }
   if (Cfg::BULK) fence_proxy_async_smem();  // the next block's bulk copies overwrite what was read here
   __syncthreads();
@@ -644,25 +616,12 @@ __global__ void __launch_bounds__(BlockCfg<T, B, K>::NT_FWD, BlockCfg<T, B, K>::
     block_fwd_kernel(BlockArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const FwdSmem<T, B, K> S(smem_raw);
-  if (MODE == 0 && BM_FWD_HIST)
-    for (int i = threadIdx.x; i < kHistWin; i += blockDim.x) S.hloc[i] = 0;
   fwd_init(S);
   bool ovf = false;
-  unsigned centre = 0, phase = 0;
+  unsigned phase = 0;
   for (int64_t b = blockIdx.x; b < a.nblocks; b += gridDim.x)
-    if (!fwd_block<T, B, K, MODE>(a, b, S, phase, ovf, centre)) return;
+    if (!fwd_block<T, B, K, MODE>(a, b, S, phase, ovf)) return;
   if (MODE == 0 && ovf) atomicOr(&a.sc->status, ST_OVERFLOW);
-  if (MODE == 0 && BM_FWD_HIST) {
-#pragma unroll
-    for (int o = 16; o; o >>= 1) centre += __shfl_xor_sync(0xffffffffu, centre, o);
-    if ((threadIdx.x & 31) == 0 && centre) atomicAdd(S.hloc + (kHistWin / 2), centre);
-    __syncthreads();
-    const int lo = a.radius - kHistWin / 2;
-    for (int i = threadIdx.x; i < kHistWin; i += blockDim.x) {
-      const unsigned v = S.hloc[i];
-      if (v && lo + i >= 0 && lo + i < 2 * a.radius) atomicAdd(a.hist + lo + i, v);
-    }
-  }
 }
 
 // Symbols and escapes of a block -> int32 codes in shared memory (the inverse
@@ -785,7 +744,7 @@ __global__ void __launch_bounds__(BatchCfg<T, B, K>::NT, BatchCfg<T, B, K>::MIN_
   __shared__ T s_m[32];
   __shared__ int s_bad;
   if constexpr (sizeof(T) == 4) fwd_init(S);
-  unsigned phase = 0, centre = 0;
+  unsigned phase = 0;
   while (true) {
     if (threadIdx.x == 0) s_t = atomicAdd(q.ticket, 1ull);
     __syncthreads();
@@ -853,7 +812,7 @@ __global__ void __launch_bounds__(BatchCfg<T, B, K>::NT, BatchCfg<T, B, K>::MIN_
         const int64_t b = (int64_t)(t - F.blk0) * NB;
         fwd_group<B, K>(F.a, b, (int)(F.a.nblocks - b < NB ? F.a.nblocks - b : NB), smem_raw, ovf);
       } else {
-        if (!fwd_block<T, B, K, 0>(F.a, (int64_t)(t - F.blk0), S, phase, ovf, centre)) return;
+        if (!fwd_block<T, B, K, 0>(F.a, (int64_t)(t - F.blk0), S, phase, ovf)) return;
       }
       if (ovf) atomicOr(&F.a.sc->status, ST_OVERFLOW);
     }

@@ -328,7 +328,7 @@ __device__ __forceinline__ void fwd_group(const BlockArgs<double>& a, const int6
   __syncthreads();
   const int64_t sbase = b * (int64_t)Cfg::PB;
   const LevelBufs<double> bufs{A, cb0, cb1};
-  const bool full = a.radius == (1 << 15) && !BM_FWD_HIST;
+  const bool full = a.radius == (1 << 15);
   GroupFwdLevels<B, 0, K, B>::run(bufs, T1, s_rq, stage, a.esc + sbase, ovf, full, field_huge(a.sc), nv);
   for (int blk = 0; blk < nv; ++blk) {  // block coarse values -> gathered grid G
     constexpr int M = Cfg::M;
@@ -340,11 +340,10 @@ __device__ __forceinline__ void fwd_group(const BlockArgs<double>& a, const int6
       g[((int64_t)j0 * a.g1 + j1) * a.g2 + j2] = cf[e];
     }
   }
-  unsigned centre = 0;
   for (int blk = 0; blk < nv; ++blk) {
     const int64_t o = sbase + (int64_t)blk * Cfg::PB;
     if (full) copy_symbols<Cfg::PB>(a.sym + o, stage + blk * Cfg::PB);
-    else store_codes<Cfg::PB>(a.sym + o, a.esc + o, stage + blk * Cfg::PB, a.radius, nullptr, a.hist, centre);
+    else store_codes<Cfg::PB>(a.sym + o, a.esc + o, stage + blk * Cfg::PB, a.radius);
   }
   __syncthreads();
 }

@@ -21,7 +21,6 @@ struct BlockArgs {
   const uint8_t* tier;  // per block tier or null
   const T* rq;          // fwd: 1/q per [tier*K + level]
   const double* q;      // inv: q per [tier*K + level]
-  unsigned* hist;       // global histogram [2*radius]
   int radius;
   Scalars* sc;
   int ntiers;           // inv: tiers in the q table (a block tier at or above it is corrupt)
