@@ -25,6 +25,7 @@
 #include "bm_plan.h"
 #include "bm_plane.h"
 #include "bm_qtab.cuh"
+#include "bm_smem.h"
 
 // The block region's histogram: on a second stream beside the global levels
 // (BM_HIST_OVERLAP) with BM_HIST_CTAS CTAs per SM.
@@ -529,20 +530,9 @@ Reblock reblock_of(const PlanHost& h, bool coarse) {
   return R;
 }
 
-// cudaFuncAttributeMaxDynamicSharedMemorySize set once per device for a kernel.
+// The devices on which each kernel's dynamic shared memory is allowed (set_smem_once).
 std::atomic<unsigned> g_cb_attr{0}, g_dt_attr{0}, g_cbb_attr{0};
 std::atomic<unsigned> g_enc0_attr{0}, g_enc2_attr{0}, g_enc3_attr{0}, g_encc0_attr{0}, g_encc2_attr{0};
-template <class F>
-cudaError_t set_smem_once(F* fn, int bytes, std::atomic<unsigned>& done) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  const unsigned bit = 1u << (dev & 31);
-  if (done.load() & bit) return cudaSuccess;
-  e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e == cudaSuccess) done.fetch_or(bit);
-  return e;
-}
 
 int grid_for(int64_t work, int threads, int per_sm = 8) {
   int64_t g = (work + threads - 1) / threads;

@@ -10,8 +10,13 @@
 #include "bm_adjoint.cuh"
 #include "bm_global.cuh"
 #include "bm_levels.h"
+#include "bm_smem.h"
 
 namespace bm {
+
+// The most shared memory that lines of at most E coarse nodes a lane take: a
+// full tile (128 bytes across the lines) of 2 * 32 E - 1 and 32 E nodes.
+constexpr int line_smem_max(int E) { return 128 * 96 * E; }
 
 template <typename T, int DIM, int FINAL, int SRC, int E>
 cudaError_t launch_line(const GLevel<T>& L, const ApplyShape& S, const T* in, T* out, const T* U, const LineSrc<T>& W,
@@ -19,12 +24,10 @@ cudaError_t launch_line(const GLevel<T>& L, const ApplyShape& S, const T* in, T*
   const GDim<T>& D = L.d[DIM];
   const int lsh = line_tile_shift<T>(S.nb, S.ncol, nsm);
   const size_t smem = line_smem<T>(D.n, D.c, lsh);
-  static std::atomic<int> attr{0};  // largest dynamic shared memory enabled so far
-  if ((int)smem > 48 * 1024 && (int)smem > attr.load()) {
-    const cudaError_t e = cudaFuncSetAttribute(gl_line<T, DIM, FINAL, E, SRC>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (line_smem_max(E) > 48 * 1024) {
+    static std::atomic<unsigned> allowed{0};
+    const cudaError_t e = set_smem_once(gl_line<T, DIM, FINAL, E, SRC>, line_smem_max(E), allowed);
     if (e != cudaSuccess) return e;
-    attr.store((int)smem);
   }
   const int64_t ctas = S.nb * ((S.ncol + (1 << lsh) - 1) >> lsh);
   gl_line<T, DIM, FINAL, E, SRC><<<(unsigned)ctas, 256, smem, s>>>(L, S, in, out, U, lsh, W);
@@ -54,12 +57,10 @@ cudaError_t launch_expand_line(const GLevel<T>& L, const LineShape& S, const T* 
   const GDim<T>& D = L.d[DIM];
   const int lsh = line_tile_shift<T>(S.nb, S.ncol, nsm);
   const size_t smem = line_smem<T>(D.n, D.c, lsh);
-  static std::atomic<int> attr{0};  // largest dynamic shared memory enabled so far
-  if ((int)smem > 48 * 1024 && (int)smem > attr.load()) {
-    const cudaError_t e = cudaFuncSetAttribute(gl_expand<T, DIM, FIN, E>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)smem);
+  if (line_smem_max(E) > 48 * 1024) {
+    static std::atomic<unsigned> allowed{0};
+    const cudaError_t e = set_smem_once(gl_expand<T, DIM, FIN, E>, line_smem_max(E), allowed);
     if (e != cudaSuccess) return e;
-    attr.store((int)smem);
   }
   const int64_t ctas = S.nb * ((S.ncol + (1 << lsh) - 1) >> lsh);
   gl_expand<T, DIM, FIN, E><<<(unsigned)ctas, 256, smem, s>>>(L, S, in, fine, g, coef, lsh);
