@@ -1781,7 +1781,9 @@ __global__ void __launch_bounds__(kHistWideThreads)
     else if (s < (unsigned)dict) atomicAdd(hist + s, 1u);
     else bad = true;
   };
-  const unsigned long long a0 = min(s1, (s0 + 7) & ~7ull);  // 16-byte aligned start
+  // the 16-byte aligned start (a caller's symbols may begin at any address)
+  const unsigned head = (unsigned)((16u - (reinterpret_cast<uintptr_t>(sym + s0) & 15u)) & 15u) / 2u;
+  const unsigned long long a0 = min(s1, s0 + head);
   const unsigned long long tid = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x;
   const unsigned long long nth = (unsigned long long)gridDim.x * blockDim.x;
   for (unsigned long long i = s0 + tid; i < a0; i += nth) count(sym[i]);

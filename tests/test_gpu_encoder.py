@@ -85,3 +85,22 @@ def test_short_stream_with_codes_too_long_for_an_entry():
     words = s.cpu().numpy()[hs["off_bits"]:][: 4 * hs["n_words"]]
     off = sum(-(-b // 8) * 8 for b in (4 * mo["n_chunks"], 14 * mo["n_chunks"], mo["codebook_bytes"]))
     np.testing.assert_array_equal(words, so[off:][: 4 * mo["n_words"]])
+
+
+@pytest.mark.parametrize("dict_size", [8192, 8194, 65536])
+@pytest.mark.parametrize("off", [1, 3, 7])
+def test_symbols_at_any_address(off, dict_size):
+    """Symbols that start between 16-byte boundaries, fewer and more of them
+    than reach the first boundary."""
+    import paper_2609_00205_gb300 as bm
+
+    rng = np.random.default_rng(off)
+    for n in (1, 8 - off, 9, 5003):
+        sym = rng.integers(0, dict_size, n).astype(np.uint16)
+        so, mo = oracle.huffman_encode(sym, dict_size, 2048)
+        buf = torch.empty(n + 8, dtype=torch.int16, device="cuda")
+        d = buf[off:off + n]
+        d.copy_(torch.from_numpy(sym.view(np.int16)))
+        sg, mg = bm.huffman_encode(d, dict_size, 2048)
+        assert mg == mo
+        np.testing.assert_array_equal(sg.cpu().numpy(), so)
