@@ -94,8 +94,8 @@ size_t bm_compress_bound(int ndim, const int64_t* shape, bm_dtype dtype);
  *               ceil(shape[d]/B); same mode as tol.  Block i's tolerance is min(tol, h_roi_tol[i]) (Sec. III-C
  *               block-wise tolerance assignment).  NULL = uniform.  At most 255
  *               distinct values.
- *   d_out       device buffer for the stream; out_capacity bytes (use
- *               bm_compress_bound()).
+ *   d_out       device buffer for the stream, 8-byte aligned; out_capacity
+ *               bytes (use bm_compress_bound()).
  *   out_bytes   receives the stream length (host pointer).
  * Guarantee: decompression reproduces every node of block i within its
  * tolerance (L-inf), including floating-point round-off, or the stream is a

@@ -2162,6 +2162,7 @@ bm_status batch_ctx(size_t hbytes, BatchCtx** out) {
 
 bm_status check_item(const bm_batch_item& it, Params& prm, int64_t s3[3]) {
   if (!it.d_field || !it.d_out) return fail(BM_ERR_ARG, "NULL pointer in a batch item");
+  if (reinterpret_cast<uintptr_t>(it.d_out) % 8) return fail(BM_ERR_ARG, "output pointer must be 8-byte aligned");
   if (bm_status st = norm_shape(it.ndim, it.shape, s3)) return st;
   if (it.dtype != BM_F32 && it.dtype != BM_F64) return fail(BM_ERR_ARG, "dtype");
   if (!(it.tol > 0.0) || !std::isfinite(it.tol)) return fail(BM_ERR_ARG, "tolerance must be finite and > 0");
@@ -2384,6 +2385,7 @@ bm_status bm_compress(const void* d_field, int ndim, const int64_t* shape, bm_dt
                       bm_tol_mode tol_mode, const double* h_roi_tol, const bm_params* params, void* d_out,
                       size_t out_capacity, size_t* out_bytes, void* stream) {
   if (!d_field || !d_out || !out_bytes) return fail(BM_ERR_ARG, "NULL pointer argument");
+  if (reinterpret_cast<uintptr_t>(d_out) % 8) return fail(BM_ERR_ARG, "output pointer must be 8-byte aligned");
   int64_t s3_[3];
   if (bm_status st = norm_shape(ndim, shape, s3_)) return st;
   shape = s3_;

@@ -100,3 +100,14 @@ def test_stream_info_on_2d_header(lib):
     assert lib.bm_stream_info(s.ctypes.data, s.size, 0, ctypes.byref(nd), shp, ctypes.byref(dt), ctypes.byref(nc)) == 0
     assert nd.value == 2 and list(shp) == [40, 23, 0] and dt.value == 0
     assert nc.value == oracle.plan((40, 23), 9, 2, 1)["n_coeffs"]
+
+
+def test_unaligned_output_is_refused_before_any_launch(lib):
+    """The stream's words are stored at 8-byte boundaries of the output."""
+    shape = (ctypes.c_int64 * 3)(65, 65, 65)
+    cap, size = ctypes.c_size_t(1 << 22), (ctypes.c_size_t * 1)()
+    lib.bm_last_error_detail.restype = ctypes.c_char_p
+    for off in (1, 4):
+        st = lib.bm_compress(ctypes.c_void_p(1 << 20), 3, shape, 0, ctypes.c_double(1e-3), 1, None, None,
+                             ctypes.c_void_p((1 << 24) + off), cap, size, None)
+        assert st == 1 and b"aligned" in lib.bm_last_error_detail()
