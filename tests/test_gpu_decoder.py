@@ -38,6 +38,18 @@ def test_one_run(n_present):
     _round_trip(sym, 65536, 1024)
 
 
+@pytest.mark.parametrize("first,last", [(0, 0), (1, 40), (30_000, 30_700), (65_535, 65_535), (40_000, 65_535)])
+@pytest.mark.parametrize("step", [1, 3])
+def test_codebooks_anywhere_in_the_dictionary(first, last, step):
+    """The canonical order is counted between the first and the last present
+    symbol only."""
+    present = np.unique(np.append(np.arange(first, last + 1, step), last))
+    rng = np.random.default_rng(first)
+    p = 0.7 ** np.minimum(np.arange(present.size), 60)
+    sym = np.concatenate([present, rng.choice(present, 5000, p=p / p.sum())]).astype(np.uint16)
+    _round_trip(sym, 65536, 2048)
+
+
 @pytest.mark.parametrize("chunk,chunks", [(64, 14_591), (64, 14_592), (256, 15_001)])
 def test_launch_shapes(chunk, chunks):
     """Around the chunk count from which one large CTA per SM decodes (three
