@@ -541,11 +541,17 @@ int grid_for(int64_t work, int threads, int per_sm = 8) {
   return (int)std::max<int64_t>(g, 1);
 }
 
-// The encoder over caller-supplied symbols: the window of a dictionary of at
-// most kEncWinSmall symbols unless a code is too long for its entries, else
-// the split table (the variant that does not apply returns at once).
+// The encoder over caller-supplied symbols: few chunks with the table left in
+// global memory; else the window of a dictionary of at most kEncWinSmall
+// symbols unless a code is too long for its entries, else the split table (the
+// variant that does not apply returns at once).
 cudaError_t launch_encode_clamped(FusedEncodeArgs a, unsigned long long nch, cudaStream_t s) {
   cudaError_t e = cudaSuccess;
+  if (nch <= (unsigned long long)kEncSmallChunks * num_sms()) {
+    encode_small_kernel<true><<<grid_for((int64_t)nch * 32, 256, 1), 256, kEncSmallSmem, s>>>(a);
+    g_launches.fetch_add(1);
+    return cudaGetLastError();
+  }
   if (a.dict <= kEncWinSmall) {
     a.win = kEncWinSmall;
     const size_t m0 = enc_smem<0>(8, kEncWinSmall, a.dict);
@@ -1729,7 +1735,7 @@ bm_status compress_t(const T* field, const int64_t* shape, const Params& prm, do
     ea.splits = reinterpret_cast<uint16_t*>(out + L.off_splits);
     ea.out = out; ea.capacity = cap; ea.sc = sc;
     if (L.nch <= (unsigned long long)kEncSmallChunks * num_sms()) {
-      encode_small_kernel<<<grid_for((int64_t)L.nch * 32, 256, 1), 256, kEncSmallSmem, s>>>(ea);
+      encode_small_kernel<false><<<grid_for((int64_t)L.nch * 32, 256, 1), 256, kEncSmallSmem, s>>>(ea);
       g_launches.fetch_add(1);
     } else {
       // the codebook picked one of three variants (the others return at once):

@@ -2354,13 +2354,16 @@ __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) encode_fused_kernel(Fu
 // SM.  In place of the three launches above, two of which return at once (but
 // wait for an SM with 200 KB of free shared memory to do so): 64 uneven fields
 // in a batch 4.60 ms against 4.45, 65^3 0.195 ms against 0.176; with the
-// tables copied by one kernel of any mode 5.57 and 0.181.
+// tables copied by one kernel of any mode 5.57 and 0.181.  (CLAMP: Huffman
+// encoding of 65,536 caller's symbols with a dictionary of 65,536 took 162 us
+// with the two launches of launch_encode_clamped.)
 constexpr int kEncSmallChunks = 8;
 constexpr size_t kEncSmallSmem = enc_smem<5>(8, 0, 0);
+template <bool CLAMP>
 __global__ void __launch_bounds__(256) encode_small_kernel(FusedEncodeArgs a) {
   if (a.sc->skip) return;  // the stream is already known to be a raw copy
-  if (a.sc->max_len <= kPackLen) encode_tiles<8, false, 4>(a);
-  else encode_tiles<8, false, 5>(a);
+  if (a.sc->max_len <= kPackLen) encode_tiles<8, CLAMP, 4>(a);
+  else encode_tiles<8, CLAMP, 5>(a);
 }
 __device__ __forceinline__ void encode_finish(unsigned long long raw_total, unsigned long long capacity, Scalars* sc) {
   if (sc->skip) return;  // already raw

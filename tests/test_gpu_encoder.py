@@ -37,6 +37,25 @@ def test_symbol_counts_around_tiles(n, dict_size, scale):
     _check(fields.laplace_symbols(n, dict_size // 2, scale, seed=n), dict_size, 2048)
 
 
+@pytest.mark.parametrize("dict_size,scale", [(4096, 1.0), (4096, 300.0), (65536, 9000.0)])
+@pytest.mark.parametrize("chunk,over", [(64, 0), (64, 1), (512, 1)])
+def test_short_and_long_streams(chunk, over, dict_size, scale):
+    """At and above the chunk count (eight per SM of 152) up to which one
+    launch codes with the table left in global memory."""
+    n = 8 * 152 * chunk + over
+    _check(fields.laplace_symbols(n, dict_size // 2, scale, seed=n), dict_size, chunk)
+
+
+def test_short_stream_of_long_codes():
+    """29 symbols with Fibonacci counts: codes of up to 28 bits."""
+    f = [1, 1]
+    while len(f) < 29:
+        f.append(f[-1] + f[-2])
+    sym = np.repeat(np.arange(3, 3 + len(f)), f).astype(np.uint16)
+    np.random.default_rng(6).shuffle(sym)
+    _check(sym, 4096, 2048)
+
+
 @pytest.mark.parametrize("dict_size", [128, 16384])
 def test_codes_longer_than_a_window_entry(dict_size):
     """Fibonacci counts (36 symbols, 39 M in all) give codes of 1 to 35 bits,
