@@ -2141,7 +2141,21 @@ __device__ __forceinline__ void encode_tiles(const FusedEncodeArgs& a) {
   // an eighth of a chunk is 32 ns symbols, 4 ns lanes of the steps; the
   // reciprocal divides lane indices below 256 exactly
   const unsigned lpe = 4u * ns, lpe_inv = lpe ? (65536u + lpe - 1u) / lpe : 0u;
-  const bool steps_ok = (a.chunk & 255) == 0 && (reinterpret_cast<uintptr_t>(a.sym) & 15) == 0;
+  const bool steps_ok = (a.chunk & 255) == 0 && (CLAMP || (reinterpret_cast<uintptr_t>(a.sym) & 15) == 0);
+  // a lane's eight symbols (at p, from symbol i0 of the array): one load, or,
+  // where a caller's array starts between 16-byte boundaries, eight
+  auto eight = [&](const uint4* p, unsigned long long i0) {
+    if constexpr (CLAMP) {
+      if (reinterpret_cast<uintptr_t>(a.sym) & 15) {
+        const uint16_t* h = a.sym + i0;
+        unsigned w[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[i] = (unsigned)__ldg(h + 2 * i) | ((unsigned)__ldg(h + 2 * i + 1) << 16);
+        return make_uint4(w[0], w[1], w[2], w[3]);
+      }
+    }
+    return __ldg(p);
+  };
   const int grp = warp / kEncGroup, gw = warp % kEncGroup;  // tile group, warp of the group
   const unsigned long long ntiles = (a.nch + kEncGroup - 1) / kEncGroup;
   auto group_sync = [&] { asm volatile("bar.sync %0, %1;\n" ::"r"(grp + 1), "n"(kEncGroup * 32) : "memory"); };
@@ -2163,7 +2177,7 @@ __device__ __forceinline__ void encode_tiles(const FusedEncodeArgs& a) {
       const uint4* p = reinterpret_cast<const uint4*>(a.sym + cb) + lane;
       uint4 q[kEncSteps];
 #pragma unroll
-      for (int k = 0; k < kEncSteps; ++k) q[k] = k < ns ? __ldg(p + 32 * k) : make_uint4(0, 0, 0, 0);
+      for (int k = 0; k < kEncSteps; ++k) q[k] = k < ns ? eight(p + 32 * k, cb + 256 * k + 8 * lane) : make_uint4(0, 0, 0, 0);
       unsigned sum = 0;  // bits | escapes << 17
 #pragma unroll
       for (int k = 0; k < kEncSteps; ++k) {
@@ -2236,12 +2250,12 @@ __device__ __forceinline__ void encode_tiles(const FusedEncodeArgs& a) {
     unsigned* const gw = words + pw;
     if (steps) {
       const uint4* p = reinterpret_cast<const uint4*>(a.sym + cb) + lane;
-      uint4 qn = __ldg(p);
+      uint4 qn = eight(p, cb + 8 * lane);
       unsigned b0 = 0, carry = 0;  // the step's first bit in the chunk; the bits before it in its word
 #pragma unroll 1
       for (int k = 0; k < ns; ++k) {
         const unsigned w[4] = {qn.x, qn.y, qn.z, qn.w};
-        if (k + 1 < ns) qn = __ldg(p + 32 * (k + 1));
+        if (k + 1 < ns) qn = eight(p + 32 * (k + 1), cb + 256 * (k + 1) + 8 * lane);
         unsigned e[8], v = 0;  // v: this lane's bits | escapes << 16
 #pragma unroll
         for (int i = 0; i < 8; ++i) e[i] = tab.entry(tab.symbol(w, i, dmax));
@@ -2356,7 +2370,7 @@ __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) encode_fused_kernel(Fu
 // in a batch 4.60 ms against 4.45, 65^3 0.195 ms against 0.176; with the
 // tables copied by one kernel of any mode 5.57 and 0.181.  (CLAMP: Huffman
 // encoding of 65,536 caller's symbols with a dictionary of 65,536 took 162 us
-// with the two launches of launch_encode_clamped.)
+// with the two launches of launch_encode_clamped against 137.)
 constexpr int kEncSmallChunks = 8;
 constexpr size_t kEncSmallSmem = enc_smem<5>(8, 0, 0);
 template <bool CLAMP>

@@ -114,7 +114,7 @@ def test_symbols_at_any_address(off, dict_size):
     import paper_2609_00205_gb300 as bm
 
     rng = np.random.default_rng(off)
-    for n in (1, 8 - off, 9, 5003):
+    for n in (1, 8 - off, 9, 5003, 8 * 2048):
         sym = rng.integers(0, dict_size, n).astype(np.uint16)
         so, mo = oracle.huffman_encode(sym, dict_size, 2048)
         buf = torch.empty(n + 8, dtype=torch.int16, device="cuda")
