@@ -292,6 +292,14 @@ LineShape line_shape(const GLevel<T>& L, int dim) {
 enum { EXP_STORE = 0, EXP_ADD = 1, EXP_COEF = 2 };
 
 template <typename T, int FIN>
+__device__ __forceinline__ void expand_emit_at(const GLevel<T>& L, T* fine, const T* g, T* coef, int i0, int i1, int i2,
+                                               int64_t o, T t) {
+  const bool cc = all_coarse(L, i0, i1, i2);
+  const int64_t pos = cc ? 0 : nc_pos(L, i0, i1, i2, o);
+  if (FIN == EXP_ADD) fine[o] = (cc ? T(0) : coef[pos]) + t;
+  else if (!cc) coef[pos] = g[o] - t;
+}
+template <typename T, int FIN>
 __device__ __forceinline__ void expand_emit(const GLevel<T>& L, const LineShape& S, T* fine, const T* g, T* coef,
                                             int64_t b, int64_t col, int i, T t) {
   const int64_t o = b * S.f_b + (int64_t)i * S.f_i + col * S.f_c;
@@ -300,10 +308,7 @@ __device__ __forceinline__ void expand_emit(const GLevel<T>& L, const LineShape&
     return;
   }
   const int n1 = L.d[1].n, i0 = (int)(col / n1), i1 = (int)(col - (int64_t)i0 * n1);
-  const bool cc = all_coarse(L, i0, i1, i);
-  const int64_t pos = cc ? 0 : nc_pos(L, i0, i1, i, o);
-  if (FIN == EXP_ADD) fine[o] = (cc ? T(0) : coef[pos]) + t;
-  else if (!cc) coef[pos] = g[o] - t;
+  expand_emit_at<T, FIN>(L, fine, g, coef, i0, i1, i, o, t);
 }
 
 __device__ __forceinline__ float rn_mul(float a, float b) { return __fmul_rn(a, b); }
@@ -480,23 +485,24 @@ __global__ void __launch_bounds__(256) gl_expand(GLevel<T> L, LineShape S, const
   }
 }
 
-// The expansion of lines too long for gl_expand's segments and shared memory
-// (more than 544 coarse nodes), one thread per line: Thomas sweeps with the
-// coarse values kept in the fine line's coarse slots of `buf`, then the fine
-// slots by interpolation, then the mass matrix with a rolling window (in
-// place, or into `fine` where the pass is the last).
-template <typename T, int DIM, int FIN>
-__global__ void __launch_bounds__(256) gl_expand_long(GLevel<T> L, LineShape S, const T* __restrict__ coarse, T* buf,
-                                                      T* fine, const T* g, T* coef) {
-  const GDim<T>& D = L.d[DIM];
+// The expansion by one thread per line (expand_serial): Thomas sweeps with the
+// coarse values kept in the fine line's coarse slots, then the fine slots by
+// interpolation, then the mass matrix with a rolling window, in place.
+template <typename T>
+__global__ void __launch_bounds__(256) gl_expand_serial(GDim<T> D, LineShape S, const T* __restrict__ coarse,
+                                                         T* __restrict__ fine) {
   const int n = D.n, c = D.c;
   const int64_t lines = S.nb * S.ncol;
   for (int64_t line = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; line < lines;
        line += (int64_t)gridDim.x * blockDim.x) {
     const int64_t b = line / S.ncol, col = line - b * S.ncol;
     const T* x = coarse + b * S.c_b + col * S.c_c;
-    T* y = buf + b * S.f_b + col * S.f_c;
+    T* y = fine + b * S.f_b + col * S.f_c;
     const int64_t so = S.f_i, si = S.c_i;
+    if (c == n) {  // a dimension of at most two nodes is not coarsened
+      for (int i = 0; i < n; ++i) y[i * so] = x[i * si];
+      continue;
+    }
     T yv = x[0];
     y[(int64_t)D.cidx[0] * so] = yv;
     for (int J = 1; J < c; ++J) {
@@ -518,10 +524,26 @@ __global__ void __launch_bounds__(256) gl_expand_long(GLevel<T> L, LineShape S, 
       T v = D.md[i] * w0;
       if (i > 0) v = fma(D.mo[i - 1], wm, v);
       if (i + 1 < n) v = fma(D.mo[i], wp, v);
-      expand_emit<T, FIN>(L, S, fine, g, coef, b, col, i, v);
+      y[i * so] = v;
       wm = w0;
       w0 = wp;
     }
+  }
+}
+
+// What gl_expand's last pass does with t as it emits it, over a grid of t: a
+// thread a node, so that the grids and the coefficients are walked in order (a
+// thread per line wrote and read them a line apart: 2100x30x2100 doubles, B = 9,
+// K = 1, the whole gradient 15.5 ms).
+template <typename T, int FIN>
+__global__ void __launch_bounds__(256) gl_expand_finish(GLevel<T> L, NodeDiv nd, const T* __restrict__ t,
+                                                         T* __restrict__ fine, const T* __restrict__ g,
+                                                         T* __restrict__ coef) {
+  const int64_t total = (int64_t)L.d[0].n * L.d[1].n * L.d[2].n;
+  for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < total; o += (int64_t)gridDim.x * blockDim.x) {
+    int i0, i1, i2;
+    node_of(nd, o, i0, i1, i2);
+    expand_emit_at<T, FIN>(L, fine, g, coef, i0, i1, i2, o, t[o]);
   }
 }
 

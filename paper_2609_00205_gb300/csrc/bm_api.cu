@@ -1991,7 +1991,7 @@ cudaError_t launch_block_adj<double>(int dir, int B, int K, const BlockArgs<doub
 
 template <typename T, int DIM, int FIN>
 cudaError_t launch_expand(const GLevel<T>& L, const T* in, T* buf, T* fine, const T* g, T* coef, cudaStream_t s) {
-  BM_LAUNCHED();
+  g_launches.fetch_add(FIN != EXP_STORE && expand_serial(L, DIM, num_sms()) ? 2 : 1);
   return level_expand<T, DIM, FIN>(L, in, buf, fine, g, coef, s, num_sms());
 }
 

@@ -71,15 +71,23 @@ template <typename T, int DIM, int FIN>
 cudaError_t level_expand(const GLevel<T>& L, const T* in, T* buf, T* fine, const T* g, T* coef, cudaStream_t s,
                          int nsm) {
   const LineShape S = line_shape(L, DIM);
-  switch (line_segment(L.d[DIM].c)) {
-    case 1: return launch_expand_line<T, DIM, FIN, 1>(L, S, in, fine, g, coef, s, nsm);
-    case 3: return launch_expand_line<T, DIM, FIN, 3>(L, S, in, fine, g, coef, s, nsm);
-    case 9: return launch_expand_line<T, DIM, FIN, 9>(L, S, in, fine, g, coef, s, nsm);
-    case 17: return launch_expand_line<T, DIM, FIN, 17>(L, S, in, fine, g, coef, s, nsm);
-    default: break;
+  if (!expand_serial(L, DIM, nsm)) {
+    switch (line_segment(L.d[DIM].c)) {
+      case 1: return launch_expand_line<T, DIM, FIN, 1>(L, S, in, fine, g, coef, s, nsm);
+      case 3: return launch_expand_line<T, DIM, FIN, 3>(L, S, in, fine, g, coef, s, nsm);
+      case 9: return launch_expand_line<T, DIM, FIN, 9>(L, S, in, fine, g, coef, s, nsm);
+      case 17: return launch_expand_line<T, DIM, FIN, 17>(L, S, in, fine, g, coef, s, nsm);
+      default: return cudaErrorInvalidValue;  // the rule
+    }
   }
-  const int64_t grid = std::min<int64_t>((S.nb * S.ncol + 255) / 256, 8ll * nsm);
-  gl_expand_long<T, DIM, FIN><<<(unsigned)grid, 256, 0, s>>>(L, S, in, buf, fine, g, coef);
+  const int64_t cap = 8ll * nsm;
+  gl_expand_serial<T><<<(unsigned)std::min<int64_t>((S.nb * S.ncol + 255) / 256, cap), 256, 0, s>>>(
+      L.d[DIM], S, in, FIN == EXP_STORE ? fine : buf);
+  if constexpr (FIN != EXP_STORE) {
+    const int64_t nn = (int64_t)L.d[0].n * L.d[1].n * L.d[2].n;
+    gl_expand_finish<T, FIN><<<(unsigned)std::min<int64_t>((nn + 255) / 256, cap), 256, 0, s>>>(L, node_div(L), buf,
+                                                                                               fine, g, coef);
+  }
   return cudaGetLastError();
 }
 

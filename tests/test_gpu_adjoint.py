@@ -91,8 +91,9 @@ def test_loss_gradient_central_differences(bm):
 
 
 # Global grids whose lines take every segment length of the scans (up to 32,
-# 96, 288 and 544 coarse nodes) and the sweep of longer ones, along each
-# dimension, with a few lines (tiles of 8 or 4) and with many (32 or 16).
+# 96, 288 and 544 coarse nodes) and the sweeps of longer ones and of many short
+# ones, along each dimension, with a few lines (tiles of 8 or 4) and with many
+# (32 or 16).
 LINES = [(300, 20, 19), (19, 1000, 20), (20, 18, 3000), (4100, 18, 19), (18, 4100, 19), (18, 19, 4100),
          (330, 340, 40), (3000, 40, 70)]
 
