@@ -311,118 +311,19 @@ __device__ __forceinline__ void expand_emit(const GLevel<T>& L, const LineShape&
   expand_emit_at<T, FIN>(L, fine, g, coef, i0, i1, i, o, t);
 }
 
-__device__ __forceinline__ float rn_mul(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double rn_mul(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ float rn_add(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ double rn_add(double a, double b) { return __dadd_rn(a, b); }
-
-// A value with its rounding error, hi + lo (error-free sum and product as in
-// T. J. Dekker, "A floating-point technique for extending the available
-// precision", 1971, and D. E. Knuth's two-sum).
-template <typename T>
-struct HiLo {
-  T hi, lo;
-};
-// m * a + b
-template <typename T>
-__device__ __forceinline__ HiLo<T> hl_affine(T m, HiLo<T> a, HiLo<T> b) {
-  const T p = rn_mul(m, a.hi), pe = fma(m, a.hi, -p);
-  const T s = rn_add(p, b.hi), v = rn_add(s, -p);
-  const T e = rn_add(rn_add(p, -rn_add(s, -v)), rn_add(b.hi, -v));
-  return {s, fma(m, a.lo, rn_add(rn_add(pe, e), b.lo))};
-}
-
-// The value (an infinity has no rounding error: NaN in lo).
-template <typename T>
-__device__ __forceinline__ T hl_value(HiLo<T> a) {
-  return rn_add(a.lo, -a.lo) == T(0) ? rn_add(a.hi, a.lo) : a.hi;
-}
-
-// z = M_c^-1 r of one line in shared memory, in place, by a warp: the scans
-// of line_scan_solve with the value part of the maps carried with its rounding
-// error, so that every lane replays its rows from a rounded exact input.  The
-// plain scan's error against wider arithmetic is up to 3% larger than that of
-// the serial recurrences (4.49e-8 against 4.35e-8 relative at 32 rows in FP32,
-// 8.61e-17 against 8.37e-17 in FP64); this one's is not larger (4.31e-8,
-// 8.27e-17).
-template <typename T, int E>
-__device__ __forceinline__ void line_scan_solve_hl(const GDim<T>& D, T* r, const int lane) {
-  const int c = D.c;
-  const int j0 = lane * E;
-  T y[E];
-  HiLo<T> a{T(0), T(0)};
-  T m = T(1);
-#pragma unroll
-  for (int k = 0; k < E; ++k) {
-    const int J = j0 + k;
-    if (J < c) {
-      const T t = -D.tm[J];
-      a = hl_affine(t, a, HiLo<T>{r[J], T(0)});
-      m = t * m;
-    }
-  }
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const HiLo<T> pa{__shfl_up_sync(0xffffffffu, a.hi, off), __shfl_up_sync(0xffffffffu, a.lo, off)};
-    const T pm = __shfl_up_sync(0xffffffffu, m, off);
-    if (lane >= off) {
-      a = hl_affine(m, pa, a);
-      m *= pm;
-    }
-  }
-  T prev = __shfl_up_sync(0xffffffffu, hl_value(a), 1);
-  if (lane == 0) prev = T(0);
-#pragma unroll
-  for (int k = 0; k < E; ++k) {
-    const int J = j0 + k;
-    if (J < c) {
-      y[k] = fma(-D.tm[J], prev, r[J]);
-      prev = y[k];
-    }
-  }
-  a = {T(0), T(0)};
-  m = T(1);
-#pragma unroll
-  for (int k = E - 1; k >= 0; --k) {
-    const int J = j0 + k;
-    if (J < c) {
-      const T ib = D.tib[J], t = -D.tsup[J];
-      const HiLo<T> v = hl_affine(t, a, HiLo<T>{y[k], T(0)});
-      a.hi = rn_mul(v.hi, ib);
-      a.lo = fma(v.lo, ib, fma(v.hi, ib, -a.hi));
-      m = t * ib * m;
-    }
-  }
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const HiLo<T> pa{__shfl_down_sync(0xffffffffu, a.hi, off), __shfl_down_sync(0xffffffffu, a.lo, off)};
-    const T pm = __shfl_down_sync(0xffffffffu, m, off);
-    if (lane + off < 32) {
-      a = hl_affine(m, pa, a);
-      m *= pm;
-    }
-  }
-  T next = __shfl_down_sync(0xffffffffu, hl_value(a), 1);
-  if (lane == 31) next = T(0);
-  __syncwarp();  // every lane has read its r before any z overwrites it
-#pragma unroll
-  for (int k = E - 1; k >= 0; --k) {
-    const int J = j0 + k;
-    if (J < c) {
-      next = fma(-D.tsup[J], next, y[k]) * D.tib[J];
-      r[J] = next;
-    }
-  }
-}
-
 // fine line = M_f I M_c^-1 (coarse line), line by line along dimension DIM.
 // A CTA stages 2^lsh coarse lines in shared memory (shared memory and line
 // counts as for gl_line); a warp solves a line with the scans of
-// line_scan_solve_hl and interpolates it to the fine nodes, and the mass matrix
-// is applied as the lines are written.  Bound by latency: the chain of a line
+// line_scan_solve and interpolates it to the fine nodes, and the mass matrix is
+// applied as the lines are written.  The mass matrix smooths: neighbouring
+// rows' roundings that alternate, as the sweeps leave them, cancel in it, and
+// the scan's independent ones do not (FP32, 21 rows: the fine line's error
+// 6.77e-8 of its norm against the sweeps' 6.30e-8), so the lanes replay their
+// rows from each other's results until a lane's chain of own roundings is seven
+// rows or more (6.30e-8).  Bound by latency: the chain of a line
 // is O(log) steps instead of the 2 c of a Thomas sweep, and a line is a warp's
-// work instead of a thread's.  (With a thread per line, 2 to 25 CTAs, the six
-// expansions of a 257^3 field's two levels took 194 us; now 56.)
+// work instead of a thread's.  (Global levels of the transposed decomposition of
+// 257^3 floats, B = 17, K = 2: 215 us with a thread per line, 77 with the scans.)
 template <typename T, int DIM, int FIN, int E>
 __global__ void __launch_bounds__(256) gl_expand(GLevel<T> L, LineShape S, const T* __restrict__ coarse,
                                                  T* __restrict__ fine, const T* __restrict__ g, T* __restrict__ coef,
@@ -453,7 +354,7 @@ __global__ void __launch_bounds__(256) gl_expand(GLevel<T> L, LineShape S, const
   if (!same) {
     for (int w = warp; w < nl; w += 8) {
       T* z = s_c + w * sc;
-      line_scan_solve_hl<T, E>(D, z, lane);
+      line_scan_solve<T, E, E == 1 ? 6 : E == 3 ? 2 : 1>(D, z, lane);
       __syncwarp();
       for (int i = lane; i < n; i += 32) {
         const T zl = z[D.jlo[i]], zr = z[D.jhi[i]];

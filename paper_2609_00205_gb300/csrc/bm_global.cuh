@@ -335,8 +335,11 @@ size_t line_smem(int n, int c, int lsh) {
   return ((size_t)((n | 1) + (c | 1)) << lsh) * sizeof(T);
 }
 
-// z = M_c^-1 r of one line in shared memory, in place, by a warp.
-template <typename T, int E>
+// z = M_c^-1 r of one line in shared memory, in place, by a warp.  AGAIN: times
+// that the lanes replay their rows once more, from the value their neighbour
+// computed; each time a value's roundings are those of the serial recurrence
+// E rows further back.
+template <typename T, int E, int AGAIN = 0>
 __device__ __forceinline__ void line_scan_solve(const GDim<T>& D, T* r, const int lane) {
   const int c = D.c;
   const int j0 = lane * E;
@@ -363,11 +366,18 @@ __device__ __forceinline__ void line_scan_solve(const GDim<T>& D, T* r, const in
   T prev = __shfl_up_sync(0xffffffffu, a, 1);
   if (lane == 0) prev = T(0);
 #pragma unroll
-  for (int k = 0; k < E; ++k) {
-    const int J = j0 + k;
-    if (J < c) {
-      y[k] = fma(-D.tm[J], prev, r[J]);
-      prev = y[k];
+  for (int p = 0; p <= AGAIN; ++p) {
+#pragma unroll
+    for (int k = 0; k < E; ++k) {
+      const int J = j0 + k;
+      if (J < c) {
+        y[k] = fma(-D.tm[J], prev, r[J]);
+        prev = y[k];
+      }
+    }
+    if (p < AGAIN) {
+      prev = __shfl_up_sync(0xffffffffu, prev, 1);
+      if (lane == 0) prev = T(0);
     }
   }
   // backward recurrence z_J = (y_J - tsup_J z_{J+1}) tib_J (z_c = 0)
@@ -394,11 +404,18 @@ __device__ __forceinline__ void line_scan_solve(const GDim<T>& D, T* r, const in
   if (lane == 31) next = T(0);
   __syncwarp();  // every lane has read its r before any z overwrites it
 #pragma unroll
-  for (int k = E - 1; k >= 0; --k) {
-    const int J = j0 + k;
-    if (J < c) {
-      next = fma(-D.tsup[J], next, y[k]) * D.tib[J];
-      r[J] = next;
+  for (int p = 0; p <= AGAIN; ++p) {
+#pragma unroll
+    for (int k = E - 1; k >= 0; --k) {
+      const int J = j0 + k;
+      if (J < c) {
+        next = fma(-D.tsup[J], next, y[k]) * D.tib[J];
+        if (p == AGAIN) r[J] = next;
+      }
+    }
+    if (p < AGAIN) {  // (a lane without rows holds 0)
+      next = __shfl_down_sync(0xffffffffu, next, 1);
+      if (lane == 31) next = T(0);
     }
   }
 }

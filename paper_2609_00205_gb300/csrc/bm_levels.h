@@ -15,25 +15,25 @@ cudaError_t level_lines(const GLevel<T>& L, const T* in, T* out, const T* U, con
 
 // Whether the expansion along dimension dim takes a thread per line
 // (gl_expand_serial) instead of a warp per line (gl_expand): lines too long for
-// the scans' segments and shared memory, or so many, or so short, that the
-// scans' work costs more than the sweeps' latency.  The scans are bound by
-// issue: a line takes about 1700 + 600 E cycles of an SM in double precision
-// (whose unit runs two lanes a clock) and 100 + 40 E in single, beside a
-// launch's chain of about 7,600; the sweeps by latency, about 1,350 cycles per
-// coarse node along dimensions 0 and 1 and 2,500 along dimension 2, where a
-// thread's neighbours are a line apart.  Global levels of a transposed
-// decomposition with the scans alone (but for long lines) / the sweeps alone /
-// this rule, in us: doubles, B = 9, K = 1: 257^3 657 / 444 / 445, 2100x30x2100 (lines
-// of 11 coarse nodes among longer ones) 9110 / 2807 / 2805; doubles, B = 9, K = 2:
-// 1800x64x64 397 / 724 / 170; floats, B = 17, K = 2: 257^3 79 / 215 / 79; floats, B =
-// 9, K = 1: 2100x30x2100 2353 / 2113 / 2109.
+// the scans' segments and shared memory, or so many and so short that the
+// scans' work costs more than the sweeps.  The scans are bound by issue: a line
+// takes about 450 + 350 E cycles of an SM in double precision (whose unit runs
+// two lanes a clock) and 100 + 40 E in single, beside a launch's chain of about
+// 7,600; the sweeps by latency, about 1,350 cycles per coarse node along
+// dimensions 0 and 1 and 2,500 along dimension 2, where a thread's neighbours
+// are a line apart, and by 8 per line and coarse node.  Global levels of a
+// transposed decomposition with the scans (but for long lines) / the sweeps /
+// this rule, in us: doubles, B = 9, K = 1: 257^3 271 / 444 / 270, 2100x30x2100
+// (lines of 11 coarse nodes among longer ones) 4540 / 2806 / 2808; doubles, B = 9,
+// K = 2: 1800x64x64 187 / 714 / 151; floats, B = 17, K = 2: 257^3 80 / 215 / 77;
+// floats, B = 9, K = 1: 2100x30x2100 2279 / 2087 / 2098.
 template <typename T>
 bool expand_serial(const GLevel<T>& L, int dim, int nsm) {
   const int E = line_segment(L.d[dim].c);
   if (E == 0) return true;
   const LineShape S = line_shape(L, dim);
-  const int64_t line = sizeof(T) == 8 ? 1700 + 600 * E : 100 + 40 * E;
-  return 7600 + S.nb * S.ncol * line / nsm > (int64_t)L.d[dim].c * (dim == 2 ? 2500 : 1350);
+  const int64_t lines = S.nb * S.ncol, c = L.d[dim].c, line = sizeof(T) == 8 ? 450 + 350 * E : 100 + 40 * E;
+  return 7600 + lines * line / nsm > c * (dim == 2 ? 2500 : 1350) + lines * c * 8 / nsm;
 }
 
 // Expansion (M_f I M_c^-1) along dimension DIM, FIN as in expand_emit.  buf:

@@ -101,14 +101,18 @@ LINES = [(300, 20, 19), (19, 1000, 20), (20, 18, 3000), (4100, 18, 19), (18, 410
 @pytest.mark.parametrize("shape", LINES)
 def test_global_lines_of_every_length(bm, shape):
     g = torch.Generator(device="cpu").manual_seed(sum(shape))
-    x = torch.randn(shape, generator=g, dtype=torch.float64).to(DEV)
-    y = torch.randn(bm.coeff_count(shape, 17, 2, 2), generator=g, dtype=torch.float64).to(DEV)
+    x = torch.randn(shape, generator=g, dtype=torch.float32).double().to(DEV)  # the same values in both types
+    y = torch.randn(bm.coeff_count(shape, 17, 2, 2), generator=g, dtype=torch.float32).double().to(DEV)
     dec, rec = bm.decompose(x, 17, 2, 2), bm.recompose(y, shape, 17, 2, 2)
     gu, gc = bm.decompose_adjoint(y, shape, 17, 2, 2), bm.recompose_adjoint(x, 17, 2, 2)
-    # a sum of n products of unit variance each rounds to about sqrt(n) eps of its terms' size
-    bound = 64 * 2.0 ** -53 * x.numel() ** 0.5 * 64
+    # sums of n products of unit variance, each term with a few dozen roundings
+    # of 2^-53 of its size, which add as independent ones do
+    bound = 64 * 2.0 ** -53 * x.numel() ** 0.5
     assert abs((torch.dot(dec, y) - torch.dot(x.ravel(), gu.ravel())).item()) <= bound
     assert abs((torch.dot(rec.ravel(), x.ravel()) - torch.dot(y, gc)).item()) <= bound
-    # FP32 against FP64: a level's few dozen roundings of 2^-24 of the values' size
+    # FP32 against FP64: no value off by more than a level's few dozen roundings
+    # of 2^-24 of the largest, and twenty of them in all (each 0.41 * 2^-24 of a
+    # value's size, root mean square; independent ones add in quadrature)
     for a, b in ((bm.decompose_adjoint(y.float(), shape, 17, 2, 2), gu), (bm.recompose_adjoint(x.float(), 17, 2, 2), gc)):
         assert (a.double() - b).abs().max().item() <= 64 * 2.0 ** -24 * b.abs().max().item()
+        assert (a.double() - b).norm().item() <= 20 ** 0.5 * 0.41 * 2.0 ** -24 * b.norm().item()
