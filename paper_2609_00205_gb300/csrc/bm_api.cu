@@ -987,6 +987,23 @@ struct FwdOut {
   Scalars* sc = nullptr;
 };
 
+// The coefficients of a level that its first line pass does not take.
+template <typename T>
+void launch_detail(const GLevel<T>& L, const T* U, T* D, const FwdOut<T>& o, int mode, const T* rq, const uint8_t* tier,
+                   int tstride, cudaStream_t s) {
+  const int64_t rows = (int64_t)L.d[0].n * L.d[1].n, nn = rows * L.d[2].n;
+  if (detail_by_rows(L, num_sms())) {
+    const int g = grid_for(rows * 32, 256);
+    if (mode == 0) gl_fwd_detail_rows<T, 0><<<g, 256, 0, s>>>(L, U, D, o.sym, o.esc, o.coef, rq, o.radius, o.sc, tier, tstride);
+    else gl_fwd_detail_rows<T, 1><<<g, 256, 0, s>>>(L, U, D, o.sym, o.esc, o.coef, rq, o.radius, o.sc, nullptr, 0);
+  } else {
+    const int g = grid_for(nn, 256);
+    const NodeDiv nd = node_div(L);
+    if (mode == 0) gl_fwd_detail<T, 0><<<g, 256, 0, s>>>(L, U, D, o.sym, o.esc, o.coef, rq, o.radius, o.sc, nd, tier, tstride);
+    else gl_fwd_detail<T, 1><<<g, 256, 0, s>>>(L, U, D, o.sym, o.esc, o.coef, rq, o.radius, o.sc, nd, nullptr, 0);
+  }
+}
+
 // Gathered grids of the re-blocking rounds: every round but the last writes
 // its own (carved from the workspace); the last writes the global levels'
 // input.
@@ -1054,14 +1071,8 @@ bm_status run_decompose(PlanDev& P, const T* field, int mode, const FwdOut<T>& o
     auto& RL = rlevels<T>(P);
     for (int l = 0; l < h.K; ++l) {
       const GLevel<T>& L = RL[(size_t)l];
-      const int64_t nn = (int64_t)L.d[0].n * L.d[1].n * L.d[2].n;
       const T* rq = o.rq ? o.rq + l : nullptr;
-      if (mode == 0)
-        gl_fwd_detail<T, 0><<<grid_for(nn, 256), 256, 0, s>>>(L, RB[l], Dbuf, o.sym, o.esc, o.coef, rq, o.radius,
-                                                              o.sc, node_div(L), o.tier, h.K);
-      else
-        gl_fwd_detail<T, 1><<<grid_for(nn, 256), 256, 0, s>>>(L, RB[l], Dbuf, o.sym, o.esc, o.coef, rq, o.radius,
-                                                              o.sc, node_div(L), nullptr, 0);
+      launch_detail(L, RB[l], Dbuf, o, mode, rq, o.tier, h.K, s);
       BM_CUDA((launch_apply<T, 2, 0>(L, Dbuf, W1, nullptr, s)));
       BM_CUDA((launch_apply<T, 1, 0>(L, W1, W2, nullptr, s)));
       gl_ident0<T, 1><<<grid_for(gs.RB[(size_t)l + 1], 256), 256, 0, s>>>(L, W2, RB[(size_t)l + 1], RB[l]);
@@ -1088,14 +1099,8 @@ bm_status run_decompose(PlanDev& P, const T* field, int mode, const FwdOut<T>& o
       for (int l = 0; l < h.K; ++l) {
         const GLevel<T>& L = XL[(size_t)l];
         T* next = l + 1 < h.K ? XP[(size_t)l + 1] : Gr[r];
-        const int64_t nn = (int64_t)L.d[0].n * L.d[1].n * L.d[2].n;
         const T* rq = o.rq ? o.rq + l : nullptr;
-        if (mode == 0)
-          gl_fwd_detail<T, 0><<<grid_for(nn, 256), 256, 0, s>>>(L, XP[(size_t)l], Dbuf, o.sym, o.esc, o.coef,
-                                                                rq, o.radius, o.sc, node_div(L), tier, h.K);
-        else
-          gl_fwd_detail<T, 1><<<grid_for(nn, 256), 256, 0, s>>>(L, XP[(size_t)l], Dbuf, o.sym, o.esc, o.coef,
-                                                                rq, o.radius, o.sc, node_div(L), nullptr, 0);
+        launch_detail(L, XP[(size_t)l], Dbuf, o, mode, rq, tier, h.K, s);
         BM_CUDA((launch_apply<T, 2, 0>(L, Dbuf, W1, nullptr, s)));
         BM_CUDA((launch_apply<T, 1, 0>(L, W1, W2, nullptr, s)));
         BM_CUDA((launch_apply<T, 0, 1>(L, W2, next, XP[(size_t)l], s)));
@@ -1143,10 +1148,7 @@ bm_status run_decompose(PlanDev& P, const T* field, int mode, const FwdOut<T>& o
       if (mode == 0) BM_CUDA((launch_lines<T, 2, 0, SRC_CODE>(L, U[l], W1, nullptr, W, s)));
       else BM_CUDA((launch_lines<T, 2, 0, SRC_COEF>(L, U[l], W1, nullptr, W, s)));
     } else {
-      if (mode == 0) gl_fwd_detail<T, 0><<<grid_for(nn, 256), 256, 0, s>>>(L, U[l], Dbuf, o.sym, o.esc, o.coef, rq,
-                                                                           o.radius, o.sc, node_div(L));
-      else gl_fwd_detail<T, 1><<<grid_for(nn, 256), 256, 0, s>>>(L, U[l], Dbuf, o.sym, o.esc, o.coef, rq, o.radius,
-                                                                 o.sc, node_div(L));
+      launch_detail(L, U[l], Dbuf, o, mode, rq, nullptr, 0, s);
       BM_LAUNCHED();
       BM_CUDA((launch_apply<T, 2, 0>(L, Dbuf, W1, nullptr, s)));
     }

@@ -203,6 +203,77 @@ __global__ void __launch_bounds__(256) gl_fwd_detail(GLevel<T> L, const T* __res
   if (MODE == 0 && ovf) atomicOr(&sc->status, ST_OVERFLOW);
 }
 
+// The same with a warp per grid row (i0, i1), whose interpolation sources,
+// weights and stream offset are taken once, the lanes walking i2.
+template <typename T, int MODE>
+__global__ void __launch_bounds__(256) gl_fwd_detail_rows(GLevel<T> L, const T* __restrict__ U,
+                                                          T* __restrict__ Dfull, uint16_t* sym, int32_t* esc, T* coef,
+                                                          const T* rq_ptr, int radius, Scalars* sc,
+                                                          const uint8_t* tier, int tstride) {
+  const GDim<T>&D0 = L.d[0], &D1 = L.d[1], &D2 = L.d[2];
+  const int n1 = D1.n, n2 = D2.n;
+  const int64_t rows = (int64_t)D0.n * n1, c12 = (int64_t)D1.c * D2.c;
+  const unsigned dict = 2u * (unsigned)radius;
+  bool ovf = false;
+  const int lane = threadIdx.x & 31;
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; row < rows; row += nwarps) {
+    const int i0 = (int)(row / n1), i1 = (int)(row - (int64_t)i0 * n1);
+    const T rq_row = MODE == 0 && !L.bmode ? rq_ptr[tier ? (int)tier[i0] * tstride : 0] : T(0);
+    const int a0 = g_cidx(D0, g_jlo(D0, i0)), b0 = g_cidx(D0, g_jhi(D0, i0));
+    const int a1 = g_cidx(D1, g_jlo(D1, i1)), b1 = g_cidx(D1, g_jhi(D1, i1));
+    const T wl0 = g_wl(D0, i0), wr0 = g_wr(D0, i0), wl1 = g_wl(D1, i1), wr1 = g_wr(D1, i1);
+    const T* r00 = U + ((int64_t)a0 * n1 + a1) * n2;
+    const T* r01 = U + ((int64_t)a0 * n1 + b1) * n2;
+    const T* r10 = U + ((int64_t)b0 * n1 + a1) * n2;
+    const T* r11 = U + ((int64_t)b0 * n1 + b1) * n2;
+    const bool cc01 = g_isc(D0, i0) && g_isc(D1, i1);  // the row holds all-coarse nodes
+    // stream rank of the row's first node: flat index minus the all-coarse nodes before it
+    int64_t before = (int64_t)g_cb(D0, i0) * c12;
+    if (g_isc(D0, i0)) before += (int64_t)g_cb(D1, i1) * D2.c;
+    const int64_t rbase = L.sym_off + row * n2 - before + (int64_t)i0 * L.blk_extra;
+    for (int i2 = lane; i2 < n2; i2 += 32) {
+      const int a2 = g_cidx(D2, g_jlo(D2, i2)), b2 = g_cidx(D2, g_jhi(D2, i2));
+      const T wl2 = g_wl(D2, i2), wr2 = g_wr(D2, i2);
+      const T ta = fma(wl1, fma(wl2, r00[a2], wr2 * r00[b2]), wr1 * fma(wl2, r01[a2], wr2 * r01[b2]));
+      const T tb = fma(wl1, fma(wl2, r10[a2], wr2 * r10[b2]), wr1 * fma(wl2, r11[a2], wr2 * r11[b2]));
+      const T e = fma(wl0, ta, wr0 * tb);
+      const int64_t idx = row * n2 + i2;
+      const T dv = U[idx] - e;
+      Dfull[idx] = dv;
+      if (cc01 && g_isc(D2, i2)) continue;  // all-coarse node: no coefficient
+      int64_t pos;
+      T rq = rq_row;
+      if (L.bmode) {  // block-major order; the block's ROI tier
+        pos = blk_pos(L, i0, i1, i2);
+        if (MODE == 0) rq = rq_ptr[tier ? (int)tier[blk_of(L, i0, i1, i2)] * tstride : 0];
+      } else {
+        pos = rbase + i2 - (cc01 ? g_cb(D2, i2) : 0);
+      }
+      if (MODE == 0) {
+        const int code = quantize(dv, rq, ovf);
+        const unsigned u = (unsigned)(code + radius);
+        const bool in = u - 1u < dict - 1u;
+        const unsigned sv = in ? u : 0u;
+        sym[pos] = (uint16_t)sv;
+        if (!in) esc[pos] = code;
+      } else {
+        coef[pos] = dv;
+      }
+    }
+  }
+  if (MODE == 0 && ovf) atomicOr(&sc->status, ST_OVERFLOW);
+}
+
+// Whether a warp a row pays: single precision, long rows, and enough of them for
+// many steps of every warp (the two levels of 400x410x390, B = 8, with the line
+// passes: 2350 us against 2595; of 100x90x80 85 against 82, of 300x290x310 doubles
+// 3334 against 3226).
+template <typename T>
+bool detail_by_rows(const GLevel<T>& L, int nsm) {
+  return sizeof(T) == 4 && L.d[2].n >= 64 && (int64_t)L.d[0].n * L.d[1].n >= 256ll * nsm;
+}
+
 // One restriction pass of a global level as a dense contraction with the
 // level's projection P = M_c^{-1} I^T M_f (c x n) along dimension DIM:
 //   out[b][J][col] = sum_i P[J][i] in[b][i][col]

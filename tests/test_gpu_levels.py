@@ -6,6 +6,7 @@ import numpy as np
 import pytest
 import torch
 
+import fields
 import oracle
 from _util import check_stream_parity
 
@@ -32,3 +33,14 @@ def test_streams_and_fields(shape, B, K, dt):
     bound = 64 * eps * np.abs(u).max()
     assert np.abs(c.cpu().numpy() - want).max() <= bound
     assert (bm.recompose(c, shape, B, K, 3).cpu() - torch.from_numpy(u)).abs().max().item() <= bound
+
+
+@pytest.mark.parametrize("shape", [(198, 200, 66), (198, 190, 70)])
+def test_coefficients_by_rows_and_by_nodes(shape):
+    """Whole-grid in-cache levels (8-node blocks) of 200 x 200 rows, where a warp
+    takes a row's coefficients, and of 200 x 192, where a thread takes a node's."""
+    import paper_2609_00205_gb300 as bm
+
+    u = fields.power_law_grf(shape, exponent=-3.0, seed=8, dtype=torch.float64).float().numpy()
+    s = bm.compress(torch.from_numpy(u).to("cuda"), 1e-3, block=8, levels=2, global_levels=1).cpu().numpy()
+    check_stream_parity(bm, u, s, 1e-3, "rel", 8, 2, 1, label=f"rows_{shape}")
