@@ -376,7 +376,7 @@ __global__ void __launch_bounds__(256) gl_apply(GLevel<T> L, ApplyShape S, const
 // l*E .. l*E+E-1, composes their maps, combines them across the warp with
 // shuffles, then replays its rows from the combined input).  The same
 // operator as the dense projection in gl_apply, in O(n) work per line.
-// A CTA stages 2^lsh lines (line_tile_shift) in shared memory,
+// A CTA stages 2^LSH lines (line_tile_shift) in shared memory,
 // read coalesced along the line when it is contiguous (DIM 2) and across the
 // lines otherwise; eight warps take one line at a time.  Shapes and FINAL as
 // for gl_apply.  E is odd, so the lanes' rows of a segment never share a bank.
@@ -384,8 +384,10 @@ __global__ void __launch_bounds__(256) gl_apply(GLevel<T> L, ApplyShape S, const
 // when those tiles would leave SMs idle (a plane's 455 lines of 605 nodes in 15
 // CTAs of 32 lines took 24 us, in 57 of 8 14).
 template <typename T>
+constexpr int line_full_shift() { return sizeof(T) == 4 ? 5 : 4; }
+template <typename T>
 int line_tile_shift(int64_t nb, int64_t ncol, int nsm) {
-  const int full = sizeof(T) == 4 ? 5 : 4;
+  constexpr int full = line_full_shift<T>();
   return nb * ((ncol >> full) + 1) < 2 * nsm ? full - 2 : full;
 }
 inline int line_segment(int c) {  // rows per lane (0: the line is too long for gl_line)
@@ -574,11 +576,12 @@ __device__ __forceinline__ void stage_coefs(const GLevel<T>& L, const LineSrc<T>
   }
 }
 
-template <typename T, int DIM, int FINAL, int E, int SRC>
+template <typename T, int DIM, int FINAL, int E, int SRC, int LSH>
 __global__ void __launch_bounds__(256) gl_line(GLevel<T> L, ApplyShape S, const T* __restrict__ in,
-                                               T* __restrict__ out, const T* __restrict__ U, const int lsh,
-                                               LineSrc<T> W) {
-  const int LT = 1 << lsh;  // lines of the CTA
+                                               T* __restrict__ out, const T* __restrict__ U, LineSrc<T> W) {
+  // lines of the CTA (with the shift an argument, the short lines of a block-major
+  // grid, 8 nodes and 5 columns of 47,000 blocks, took 93 us against 75)
+  constexpr int lsh = LSH, LT = 1 << LSH;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const GDim<T>& D = L.d[DIM];
   const int n = D.n, c = D.c, sn = n | 1, sc = c | 1;

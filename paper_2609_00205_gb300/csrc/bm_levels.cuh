@@ -18,20 +18,27 @@ namespace bm {
 // full tile (128 bytes across the lines) of 2 * 32 E - 1 and 32 E nodes.
 constexpr int line_smem_max(int E) { return 128 * 96 * E; }
 
+template <typename T, int DIM, int FINAL, int SRC, int E, int LSH>
+cudaError_t launch_line_tile(const GLevel<T>& L, const ApplyShape& S, const T* in, T* out, const T* U,
+                             const LineSrc<T>& W, cudaStream_t s) {
+  const GDim<T>& D = L.d[DIM];
+  const size_t smem = line_smem<T>(D.n, D.c, LSH);
+  if (line_smem_max(E) > 48 * 1024) {
+    static std::atomic<unsigned> allowed{0};
+    const cudaError_t e = set_smem_once(gl_line<T, DIM, FINAL, E, SRC, LSH>, line_smem_max(E), allowed);
+    if (e != cudaSuccess) return e;
+  }
+  const int64_t ctas = S.nb * ((S.ncol + (1 << LSH) - 1) >> LSH);
+  gl_line<T, DIM, FINAL, E, SRC, LSH><<<(unsigned)ctas, 256, smem, s>>>(L, S, in, out, U, W);
+  return cudaGetLastError();
+}
 template <typename T, int DIM, int FINAL, int SRC, int E>
 cudaError_t launch_line(const GLevel<T>& L, const ApplyShape& S, const T* in, T* out, const T* U, const LineSrc<T>& W,
                         cudaStream_t s, int nsm) {
-  const GDim<T>& D = L.d[DIM];
-  const int lsh = line_tile_shift<T>(S.nb, S.ncol, nsm);
-  const size_t smem = line_smem<T>(D.n, D.c, lsh);
-  if (line_smem_max(E) > 48 * 1024) {
-    static std::atomic<unsigned> allowed{0};
-    const cudaError_t e = set_smem_once(gl_line<T, DIM, FINAL, E, SRC>, line_smem_max(E), allowed);
-    if (e != cudaSuccess) return e;
-  }
-  const int64_t ctas = S.nb * ((S.ncol + (1 << lsh) - 1) >> lsh);
-  gl_line<T, DIM, FINAL, E, SRC><<<(unsigned)ctas, 256, smem, s>>>(L, S, in, out, U, lsh, W);
-  return cudaGetLastError();
+  constexpr int full = line_full_shift<T>();
+  if (line_tile_shift<T>(S.nb, S.ncol, nsm) == full)
+    return launch_line_tile<T, DIM, FINAL, SRC, E, full>(L, S, in, out, U, W, s);
+  return launch_line_tile<T, DIM, FINAL, SRC, E, full - 2>(L, S, in, out, U, W, s);
 }
 
 template <typename T, int DIM, int FINAL, int SRC>
