@@ -84,8 +84,8 @@ struct Lines {
 };
 // The quantisation codes of a line (all its nodes, or the odd ones of an
 // all-coarse line), staged as in level_fwd.
-template <typename T, int N, bool CC>
-__device__ __forceinline__ void stage_line(const T (&d)[N], const T rq, const int base, uint16_t* stage,
+template <int N, bool CC>
+__device__ __forceinline__ void stage_line(const double (&d)[N], const double rq, const int base, uint16_t* stage,
                                            int32_t* esc_blk, bool& ovf, const bool full) {
   const unsigned sadd = full ? 1u : 0u, swide = full ? 0u : kStageWide;
   int codes[N];
@@ -118,9 +118,9 @@ __device__ __forceinline__ int line_base(int i0, int i1) {
 // 1/4 for a both-odd one: scalings by powers of two, folded exactly into the
 // multiply-adds that use them).  row: distance of neighbouring lines, st:
 // distance of coarse nodes in a line.
-template <typename T, int C, int CLS>
-__device__ __forceinline__ void coarse_sums(const T* r00, const T* r01, const T* r10, const T* r11, const int st,
-                                            T (&v)[C]) {
+template <int C, int CLS>
+__device__ __forceinline__ void coarse_sums(const double* r00, const double* r01, const double* r10, const double* r11,
+                                            const int st, double (&v)[C]) {
 #pragma unroll
   for (int J = 0; J < C; ++J) {
     if (CLS == 2) v[J] = (r00[st * J] + r01[st * J]) + (r10[st * J] + r11[st * J]);
@@ -133,32 +133,32 @@ __device__ __forceinline__ void coarse_sums(const T* r00, const T* r01, const T*
 // then the restriction and solve along the line into T1.  The values are those
 // of the general expression of level_fwd (field_huge excludes the fields whose
 // sums could overflow here first).
-template <typename T, int N, int CLS>
-__device__ __forceinline__ void fwd_line(const T* X, T* T1, T* out, const int i0,
-                                         const int i1, const int lvl_off, const T rq, uint16_t* stage,
+template <int N, int CLS>
+__device__ __forceinline__ void fwd_line(const double* X, double* T1, double* out, const int i0,
+                                         const int i1, const int lvl_off, const double rq, uint16_t* stage,
                                          int32_t* esc_blk, bool& ovf, const bool full) {
   constexpr int C = (N + 1) / 2;
-  const T* x = X + (i0 * N + i1) * N;
+  const double* x = X + (i0 * N + i1) * N;
   const int lo0 = CLS && (i0 & 1) ? i0 - 1 : i0, hi0 = CLS && (i0 & 1) ? i0 + 1 : i0;
   const int lo1 = CLS && (i1 & 1) ? i1 - 1 : i1, hi1 = CLS && (i1 & 1) ? i1 + 1 : i1;
-  T v[C];
-  coarse_sums<T, C, CLS>(X + (lo0 * N + lo1) * N, X + (lo0 * N + hi1) * N, X + (hi0 * N + lo1) * N,
+  double v[C];
+  coarse_sums<C, CLS>(X + (lo0 * N + lo1) * N, X + (lo0 * N + hi1) * N, X + (hi0 * N + lo1) * N,
                          X + (hi0 * N + hi1) * N, 2, v);
-  constexpr T se = CLS == 2 ? T(0.25) : CLS == 1 ? T(0.5) : T(1);
-  T d[N];
+  constexpr double se = CLS == 2 ? 0.25 : CLS == 1 ? 0.5 : 1.0;
+  double d[N];
 #pragma unroll
   for (int k = 0; k < N; ++k) {
-    if (k & 1) d[k] = fma(T(-0.5) * se, v[k / 2] + v[k / 2 + 1], x[k]);
+    if (k & 1) d[k] = fma(-0.5 * se, v[k / 2] + v[k / 2 + 1], x[k]);
     else if (CLS) d[k] = fma(-se, v[k / 2], x[k]);
-    else d[k] = T(0);
+    else d[k] = 0.0;
   }
   if (CLS == 0) {  // u|C of this line: the start of the coarse values (the third pass adds z)
 #pragma unroll
     for (int J = 0; J < C; ++J) out[((i0 / 2) * C + i1 / 2) * C + J] = v[J];
   }
-  stage_line<T, N, CLS == 0>(d, rq, lvl_off + line_base<N>(i0, i1), stage, esc_blk, ovf, full);
-  T z[C];
-  restrict_solve<T, N, CLS == 0>(block_tab<T, N>(), d, z);
+  stage_line<N, CLS == 0>(d, rq, lvl_off + line_base<N>(i0, i1), stage, esc_blk, ovf, full);
+  double z[C];
+  restrict_solve<double, N, CLS == 0>(block_tab<double, N>(), d, z);
 #pragma unroll
   for (int j = 0; j < C; ++j) T1[(i0 * C + j) * N + i1] = z[j];
 }
@@ -166,19 +166,19 @@ __device__ __forceinline__ void fwd_line(const T* X, T* T1, T* out, const int i0
 // Second and third restriction passes of a level over NB blocks (array
 // strides t1s, t2s, os): T1 -> T2 along dimension 1, T2 along dimension 0 added
 // to (SIGN 1) or subtracted from (SIGN -1) the coarse values.
-template <typename T, int N, int NB, int SIGN>
-__device__ __forceinline__ void restrict_passes(const T* T1, const int t1s, T* T2,
-                                                const int t2s, T* out, const int os) {
+template <int N, int NB, int SIGN>
+__device__ __forceinline__ void restrict_passes(const double* T1, const int t1s, double* T2,
+                                                const int t2s, double* out, const int os) {
   constexpr int C = (N + 1) / 2;
-  const auto& tb = block_tab<T, N>();
+  const auto& tb = block_tab<double, N>();
   for (int I = threadIdx.x; I < NB * N * C; I += blockDim.x) {
     const int blk = NB > 1 ? I / (N * C) : 0, L = I - blk * (N * C);  // L = i0*C + j2
     const int i0 = L / C, j2 = L - i0 * C;
-    T d[N];
+    double d[N];
 #pragma unroll
     for (int i = 0; i < N; ++i) d[i] = T1[blk * t1s + L * N + i];
-    T z[C];
-    restrict_solve<T, N>(tb, d, z);
+    double z[C];
+    restrict_solve<double, N>(tb, d, z);
 #pragma unroll
     for (int j = 0; j < C; ++j) T2[blk * t2s + (j * C + j2) * N + i0] = z[j];
   }
@@ -186,14 +186,14 @@ __device__ __forceinline__ void restrict_passes(const T* T1, const int t1s, T* T
   for (int I = threadIdx.x; I < NB * C * C; I += blockDim.x) {
     const int blk = NB > 1 ? I / (C * C) : 0, L = I - blk * (C * C);  // L = j1*C + j2
     const int j1 = L / C, j2 = L - j1 * C;
-    T d[N];
+    double d[N];
 #pragma unroll
     for (int i = 0; i < N; ++i) d[i] = T2[blk * t2s + L * N + i];
-    T z[C];
-    restrict_solve<T, N>(tb, d, z);
+    double z[C];
+    restrict_solve<double, N>(tb, d, z);
 #pragma unroll
     for (int J = 0; J < C; ++J) {
-      T* o = out + blk * os + (J * C + j1) * C + j2;
+      double* o = out + blk * os + (J * C + j1) * C + j2;
       *o = SIGN > 0 ? *o + z[J] : *o - z[J];
     }
   }
@@ -222,9 +222,9 @@ __device__ __forceinline__ bool field_huge(const Scalars* sc) {
 // per class to fill warps, and a field of huge values takes the general
 // expression for its overflows: there every line computes it.
 // ---------------------------------------------------------------------------
-template <typename T, int N, int NB>
-__device__ __forceinline__ void group_level_fwd(T* X, const int xs, T* T1, const int t1s, T* out, const int os,
-                                                const int lvl_off, const T* rq, const int rqs, uint16_t* stage,
+template <int N, int NB>
+__device__ __forceinline__ void group_level_fwd(double* X, const int xs, double* T1, const int t1s, double* out,
+                                                const int os, const int lvl_off, const double* rq, const int rqs, uint16_t* stage,
                                                 const int ps, int32_t* esc_blk, bool& ovf, const bool full,
                                                 const bool huge, const int nv) {
   constexpr int C = (N + 1) / 2;
@@ -234,35 +234,35 @@ __device__ __forceinline__ void group_level_fwd(T* X, const int xs, T* T1, const
       int blk, i0, i1;
       const int cls = LN::of(it, blk, i0, i1);
       if (cls < 0 || blk >= nv) continue;
-      T* x = X + blk * xs;
-      T* t1 = T1 + blk * t1s;
-      T* o = out + blk * os;
-      const T q = rq[blk * rqs];
-      if (cls == 2) fwd_line<T, N, 2>(x, t1, o, i0, i1, lvl_off, q, stage + blk * ps, esc_blk + blk * ps, ovf, full);
-      else if (cls == 1) fwd_line<T, N, 1>(x, t1, o, i0, i1, lvl_off, q, stage + blk * ps, esc_blk + blk * ps, ovf, full);
-      else fwd_line<T, N, 0>(x, t1, o, i0, i1, lvl_off, q, stage + blk * ps, esc_blk + blk * ps, ovf, full);
+      double* x = X + blk * xs;
+      double* t1 = T1 + blk * t1s;
+      double* o = out + blk * os;
+      const double q = rq[blk * rqs];
+      if (cls == 2) fwd_line<N, 2>(x, t1, o, i0, i1, lvl_off, q, stage + blk * ps, esc_blk + blk * ps, ovf, full);
+      else if (cls == 1) fwd_line<N, 1>(x, t1, o, i0, i1, lvl_off, q, stage + blk * ps, esc_blk + blk * ps, ovf, full);
+      else fwd_line<N, 0>(x, t1, o, i0, i1, lvl_off, q, stage + blk * ps, esc_blk + blk * ps, ovf, full);
     }
   } else {
 #pragma unroll 1
     for (int I = threadIdx.x; I < NB * N * N; I += blockDim.x) {
       const int blk = I / (N * N), L = I - blk * (N * N);
       if (blk >= nv) continue;
-      const T* x = X + blk * xs;
+      const double* x = X + blk * xs;
       const int i0 = L / N, i1 = L - i0 * N;
       const bool f0 = i0 & 1, f1 = i1 & 1;
       const int lo0 = f0 ? i0 - 1 : i0, hi0 = f0 ? i0 + 1 : i0;
       const int lo1 = f1 ? i1 - 1 : i1, hi1 = f1 ? i1 + 1 : i1;
-      const T* r00 = x + (lo0 * N + lo1) * N;
-      const T* r01 = x + (lo0 * N + hi1) * N;
-      const T* r10 = x + (hi0 * N + lo1) * N;
-      const T* r11 = x + (hi0 * N + hi1) * N;
-      T w[C];
+      const double* r00 = x + (lo0 * N + lo1) * N;
+      const double* r01 = x + (lo0 * N + hi1) * N;
+      const double* r10 = x + (hi0 * N + lo1) * N;
+      const double* r11 = x + (hi0 * N + hi1) * N;
+      double w[C];
 #pragma unroll
-      for (int J = 0; J < C; ++J) w[J] = T(0.25) * ((r00[2 * J] + r01[2 * J]) + (r10[2 * J] + r11[2 * J]));
-      T d[N];
+      for (int J = 0; J < C; ++J) w[J] = 0.25 * ((r00[2 * J] + r01[2 * J]) + (r10[2 * J] + r11[2 * J]));
+      double d[N];
 #pragma unroll
       for (int k = 0; k < N; ++k) {
-        const T e = (k & 1) ? T(0.5) * (w[k / 2] + w[k / 2 + 1]) : w[k / 2];
+        const double e = (k & 1) ? 0.5 * (w[k / 2] + w[k / 2 + 1]) : w[k / 2];
         d[k] = x[L * N + k] - e;
       }
       const bool cc = !f0 && !f1;
@@ -271,16 +271,16 @@ __device__ __forceinline__ void group_level_fwd(T* X, const int xs, T* T1, const
         for (int J = 0; J < C; ++J) out[blk * os + ((i0 / 2) * C + i1 / 2) * C + J] = x[L * N + 2 * J];
       }
       const int base = lvl_off + line_base<N>(i0, i1);
-      if (cc) stage_line<T, N, true>(d, rq[blk * rqs], base, stage + blk * ps, esc_blk + blk * ps, ovf, full);
-      else stage_line<T, N, false>(d, rq[blk * rqs], base, stage + blk * ps, esc_blk + blk * ps, ovf, full);
-      T z[C];
-      restrict_solve<T, N>(block_tab<T, N>(), d, z);
+      if (cc) stage_line<N, true>(d, rq[blk * rqs], base, stage + blk * ps, esc_blk + blk * ps, ovf, full);
+      else stage_line<N, false>(d, rq[blk * rqs], base, stage + blk * ps, esc_blk + blk * ps, ovf, full);
+      double z[C];
+      restrict_solve<double, N>(block_tab<double, N>(), d, z);
 #pragma unroll
       for (int j = 0; j < C; ++j) T1[blk * t1s + (i0 * C + j) * N + i1] = z[j];
     }
   }
   __syncthreads();
-  restrict_passes<T, N, NB, 1>(T1, t1s, X, xs, out, os);  // T2 takes the place of the level's input
+  restrict_passes<N, NB, 1>(T1, t1s, X, xs, out, os);  // T2 takes the place of the level's input
 }
 
 template <int N, int L, int K, int B>
@@ -289,7 +289,7 @@ struct GroupFwdLevels {
                                              uint16_t* stage, int32_t* esc_blk, bool& ovf, const bool full,
                                              const bool huge, const int nv) {
     using Cfg = BlockCfg<double, B, K>;
-    group_level_fwd<double, N, block_group(B)>(bufs(L), lvl_stride<B>(L), T1, Cfg::T1, bufs(L + 1),
+    group_level_fwd<N, block_group(B)>(bufs(L), lvl_stride<B>(L), T1, Cfg::T1, bufs(L + 1),
                                                lvl_stride<B>(L + 1), lvl_offset(B, L), rq + L, K, stage, Cfg::PB,
                                                esc_blk, ovf, full, huge, nv);
     if constexpr (L + 1 < K)
@@ -361,23 +361,23 @@ __global__ void __launch_bounds__(GroupCfg<B, K>::NT_FWD, GroupCfg<B, K>::FWD_MI
 
 // One line of the first inverse pass: its coefficients into X (all-coarse
 // nodes have none), restriction and solve along the line into T1.
-template <typename T, int N, bool CC>
-__device__ __forceinline__ void inv_line(T* X, T* T1, const int i0, const int i1, const int lvl_off, const T q,
-                                         const int32_t* codes) {
+template <int N, bool CC>
+__device__ __forceinline__ void inv_line(double* X, double* T1, const int i0, const int i1, const int lvl_off,
+                                         const double q, const int32_t* codes) {
   constexpr int C = (N + 1) / 2;
-  T* x = X + (i0 * N + i1) * N;
+  double* x = X + (i0 * N + i1) * N;
   const int base = lvl_off + line_base<N>(i0, i1);
-  T d[N];
+  double d[N];
 #pragma unroll
   for (int k = 0; k < N; ++k) {
-    d[k] = T(0);
+    d[k] = 0.0;
     if (!CC || (k & 1)) {
       d[k] = dequant(codes[base + (CC ? k / 2 : k)], q);
       x[k] = d[k];
     }
   }
-  T z[C];
-  restrict_solve<T, N, CC>(block_tab<T, N>(), d, z);
+  double z[C];
+  restrict_solve<double, N, CC>(block_tab<double, N>(), d, z);
 #pragma unroll
   for (int j = 0; j < C; ++j) T1[(i0 * C + j) * N + i1] = z[j];
 }
@@ -389,26 +389,26 @@ __device__ __forceinline__ bool top_binade(double v) { return ((unsigned)__doubl
 // One line of the last inverse pass: u = I(u|C) + d in X.  A both-odd line adds
 // two sums of four: where one lies in the top binade the sums are scaled first
 // (exact), so that only the sum of four itself can overflow.
-template <typename T, int N, int CLS>
-__device__ __forceinline__ void interp_line(T* X, const T* cin, const int i0, const int i1) {
+template <int N, int CLS>
+__device__ __forceinline__ void interp_line(double* X, const double* cin, const int i0, const int i1) {
   constexpr int C = (N + 1) / 2;
   const int a0 = i0 >> 1, b0 = (i0 + 1) >> 1, a1 = i1 >> 1, b1 = (i1 + 1) >> 1;
-  T v[C];
-  coarse_sums<T, C, CLS>(cin + (a0 * C + a1) * C, cin + (a0 * C + b1) * C, cin + (b0 * C + a1) * C,
+  double v[C];
+  coarse_sums<C, CLS>(cin + (a0 * C + a1) * C, cin + (a0 * C + b1) * C, cin + (b0 * C + a1) * C,
                          cin + (b0 * C + b1) * C, 1, v);
-  T se = CLS == 2 ? T(0.25) : CLS == 1 ? T(0.5) : T(1), ho = T(0.5) * se;
+  double se = CLS == 2 ? 0.25 : CLS == 1 ? 0.5 : 1.0, ho = 0.5 * se;
   if (CLS == 2) {
     bool top = false;
 #pragma unroll
     for (int J = 0; J < C; ++J) top |= top_binade(v[J]);
     if (top) {
 #pragma unroll
-      for (int J = 0; J < C; ++J) v[J] *= T(0.25);
-      se = T(1);
-      ho = T(0.5);
+      for (int J = 0; J < C; ++J) v[J] *= 0.25;
+      se = 1.0;
+      ho = 0.5;
     }
   }
-  T* x = X + (i0 * N + i1) * N;
+  double* x = X + (i0 * N + i1) * N;
 #pragma unroll
   for (int k = 0; k < N; ++k) {
     if (k & 1) x[k] = fma(ho, v[k / 2] + v[k / 2 + 1], x[k]);
@@ -420,9 +420,9 @@ __device__ __forceinline__ void interp_line(T* X, const T* cin, const int i0, co
 // Inverse level of the first nv of NB blocks: coarse values `cin` (C^3) and the
 // level's codes give the N^3 values in X.  z = P D (three passes), u|C = c - z,
 // u = I u|C + D.
-template <typename T, int N, int NB>
-__device__ __forceinline__ void group_level_inv(T* X, const int xs, T* T1, const int t1s, T* T2, const int t2s, T* cin,
-                                                const int cs, const int lvl_off, const T* q, const int qs,
+template <int N, int NB>
+__device__ __forceinline__ void group_level_inv(double* X, const int xs, double* T1, const int t1s, double* T2,
+                                                const int t2s, double* cin, const int cs, const int lvl_off, const double* q, const int qs,
                                                 const int32_t* codes, const int ps, const int nv) {
   constexpr int C = (N + 1) / 2;
   // the classes of a level of fewer than nine nodes share warps (they diverge)
@@ -440,18 +440,18 @@ __device__ __forceinline__ void group_level_inv(T* X, const int xs, T* T1, const
     int blk, i0, i1;
     const int cls = line_of(it, blk, i0, i1);
     if (cls < 0 || blk >= nv) continue;
-    if (cls) inv_line<T, N, false>(X + blk * xs, T1 + blk * t1s, i0, i1, lvl_off, q[blk * qs], codes + blk * ps);
-    else inv_line<T, N, true>(X + blk * xs, T1 + blk * t1s, i0, i1, lvl_off, q[blk * qs], codes + blk * ps);
+    if (cls) inv_line<N, false>(X + blk * xs, T1 + blk * t1s, i0, i1, lvl_off, q[blk * qs], codes + blk * ps);
+    else inv_line<N, true>(X + blk * xs, T1 + blk * t1s, i0, i1, lvl_off, q[blk * qs], codes + blk * ps);
   }
   __syncthreads();
-  restrict_passes<T, N, NB, -1>(T1, t1s, T2, t2s, cin, cs);
+  restrict_passes<N, NB, -1>(T1, t1s, T2, t2s, cin, cs);
   for (int it = threadIdx.x; it < total; it += blockDim.x) {
     int blk, i0, i1;
     const int cls = line_of(it, blk, i0, i1);
     if (cls < 0 || blk >= nv) continue;
-    if (cls == 2) interp_line<T, N, 2>(X + blk * xs, cin + blk * cs, i0, i1);
-    else if (cls == 1) interp_line<T, N, 1>(X + blk * xs, cin + blk * cs, i0, i1);
-    else interp_line<T, N, 0>(X + blk * xs, cin + blk * cs, i0, i1);
+    if (cls == 2) interp_line<N, 2>(X + blk * xs, cin + blk * cs, i0, i1);
+    else if (cls == 1) interp_line<N, 1>(X + blk * xs, cin + blk * cs, i0, i1);
+    else interp_line<N, 0>(X + blk * xs, cin + blk * cs, i0, i1);
   }
   __syncthreads();
 }
@@ -461,7 +461,7 @@ struct GroupInvLevels {  // recompose levels L, L-1, ..., 0 (level L has N nodes
   __device__ __forceinline__ static void run(const LevelBufs<double>& bufs, double* T1, double* T2, const double* q,
                                              const int32_t* codes, const int nv) {
     using Cfg = BlockCfg<double, B, K>;
-    group_level_inv<double, N, block_group(B)>(bufs(L), lvl_stride<B>(L), T1, Cfg::T1, T2, Cfg::T2, bufs(L + 1),
+    group_level_inv<N, block_group(B)>(bufs(L), lvl_stride<B>(L), T1, Cfg::T1, T2, Cfg::T2, bufs(L + 1),
                                                lvl_stride<B>(L + 1), lvl_offset(B, L), q + L, K, codes, Cfg::PB, nv);
     if constexpr (L > 0) GroupInvLevels<2 * N - 1, L - 1, K, B>::run(bufs, T1, T2, q, codes, nv);
   }

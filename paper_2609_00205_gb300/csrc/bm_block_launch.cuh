@@ -110,9 +110,12 @@ cudaError_t launch_group_one(int dir, const BlockArgs<double>& a, cudaStream_t s
 
 template <typename T, int B, int K>
 cudaError_t launch_mode(int dir, int mode, const BlockArgs<T>& a, cudaStream_t s, int nsm, int max_grid) {
-  if constexpr (sizeof(T) == 8)
+  if constexpr (sizeof(T) == 8) {
     if (mode == 0) return launch_group_one<B, K>(dir, a, s, nsm, max_grid);
-  return mode == 0 ? launch_one<T, B, K, 0>(dir, a, s, nsm, max_grid) : launch_one<T, B, K, 1>(dir, a, s, nsm, max_grid);
+    return launch_one<T, B, K, 1>(dir, a, s, nsm, max_grid);
+  } else {
+    return mode == 0 ? launch_one<T, B, K, 0>(dir, a, s, nsm, max_grid) : launch_one<T, B, K, 1>(dir, a, s, nsm, max_grid);
+  }
 }
 
 }  // namespace bm
