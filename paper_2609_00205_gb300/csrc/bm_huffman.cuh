@@ -480,7 +480,6 @@ constexpr int kCbSmemSyms = 8192;
 // Arrays of the codebook construction over the n present symbols, indexed by
 // their rank in symbol order ("compact index"); node ids of the Huffman tree
 // are leaves 0..n-1 (sorted order) and internal nodes n.. (creation order).
-template <typename IdT>
 struct CbArrays {
   uint16_t* csym;      // [n] symbol of compact index
   uint8_t* clen;       // [n] code length of compact index
@@ -489,10 +488,10 @@ struct CbArrays {
   unsigned* kb;        // [n] sort buffer (aliases iw in shared memory)
   uint16_t* sb;        // [n] sort buffer (aliases parent in shared memory)
   unsigned* iw;        // [n] internal weights
-  IdT* parent;         // [2n]
-  uint8_t* depth;      // [2n]
+  uint16_t* parent;    // [2n]; more symbols than shared memory holds: [n], the leaves' (internal node by creation)
+  uint8_t* depth;      // [2n] (in shared memory only, as round_end)
   unsigned* wcnt;      // [256*32] sort counts (aliases round_end in shared memory)
-  IdT* round_end;      // [n] internal nodes created up to the end of each round
+  uint16_t* round_end; // [n] internal nodes created up to the end of each round
   uint16_t* canon;     // [n] compact indices in canonical order (aliases iw)
   unsigned* run_start; // [n] compact index of each run's first symbol (aliases ka)
   unsigned* run_end;   // [n] one past its last (aliases iw, after the canonical codes are out)
@@ -547,12 +546,12 @@ struct CbPre {
   unsigned long long bits;         // sum of f len
 };
 __host__ __device__ constexpr size_t cb_big_bytes() {
-  return (size_t)kMaxDict * (2 + 1 + 4 + 2 + 4 + 2 + 4 + 4 * 2 + 2 + 4 + 2) + 3 * 4 * (size_t)kMaxDict + 16 * 256 +
+  return (size_t)kMaxDict * (2 + 1 + 4 + 2 + 4 + 2 + 4 + 2 + 2) + 3 * 4 * (size_t)kMaxDict + 16 * 256 +
          sizeof(CbPre) + 256;
 }
 
-__device__ __forceinline__ CbArrays<uint16_t> cb_small(CbSmem& S) {
-  CbArrays<uint16_t> v;
+__device__ __forceinline__ CbArrays cb_small(CbSmem& S) {
+  CbArrays v;
   v.csym = S.csym; v.clen = S.clen; v.ka = S.ka; v.sa = S.sa;
   v.kb = S.iw; v.sb = S.parent; v.iw = S.iw; v.parent = S.parent; v.depth = S.depth;
   v.wcnt = S.wcnt;
@@ -564,14 +563,14 @@ __device__ __forceinline__ CbArrays<uint16_t> cb_small(CbSmem& S) {
   return v;
 }
 
-__device__ __forceinline__ CbArrays<unsigned> cb_big(unsigned char* g, unsigned* smem_wcnt) {
+__device__ __forceinline__ CbArrays cb_big(unsigned char* g, unsigned* smem_wcnt) {
   auto take = [&](size_t bytes) {
     unsigned char* p = g;
     g += (bytes + 255) & ~size_t(255);
     return p;
   };
   const size_t N = kMaxDict;
-  CbArrays<unsigned> v;
+  CbArrays v;
   v.csym = reinterpret_cast<uint16_t*>(take(2 * N));
   v.clen = take(N);
   v.ka = reinterpret_cast<unsigned*>(take(4 * N));
@@ -579,9 +578,9 @@ __device__ __forceinline__ CbArrays<unsigned> cb_big(unsigned char* g, unsigned*
   v.kb = reinterpret_cast<unsigned*>(take(4 * N));
   v.sb = reinterpret_cast<uint16_t*>(take(2 * N));
   v.iw = reinterpret_cast<unsigned*>(take(4 * N));
-  v.parent = reinterpret_cast<unsigned*>(take(4 * 2 * N));
-  v.depth = take(2 * N);
-  v.round_end = reinterpret_cast<unsigned*>(take(4 * N));
+  v.parent = reinterpret_cast<uint16_t*>(take(2 * N));
+  v.depth = nullptr;
+  v.round_end = nullptr;
   v.canon = reinterpret_cast<uint16_t*>(take(2 * N));
   v.run_start = reinterpret_cast<unsigned*>(take(4 * N));
   v.run_end = reinterpret_cast<unsigned*>(take(4 * N));
@@ -593,23 +592,18 @@ __device__ __forceinline__ CbArrays<unsigned> cb_big(unsigned char* g, unsigned*
 __device__ __forceinline__ CbPre* cb_pre(unsigned char* g) {
   const size_t N = kMaxDict;
   size_t off = 0;
-  const size_t parts[] = {2 * N, N, 4 * N, 2 * N, 4 * N, 2 * N, 4 * N, 8 * N, 2 * N, 4 * N, 2 * N, 4 * N, 4 * N, 4 * N};
+  const size_t parts[] = {2 * N, N, 4 * N, 2 * N, 4 * N, 2 * N, 4 * N, 2 * N, 2 * N, 4 * N, 4 * N, 4 * N};
   for (size_t b : parts) off += (b + 255) & ~size_t(255);
   return reinterpret_cast<CbPre*>(g + off);
 }
 
-// The codebook over the compact arrays V (n present symbols, already in
-// V.csym): Huffman lengths into V.clen.  The lengths are those of the
-// sequential two-queue construction; lengths above kMaxLen are avoided by
-// re-running on max(1, f >> t), t = 1, 2, ...
 // Pairs of the ranks [d0, d1) of merge(A[0..na), B[0..nb)) (A first on equal
 // weight), d0 even, whose first i0 = split(d0) ranks came from A: appends
-// the pairs' weights to iw at qe + rank/2 and sets the parents.  Ids: A[i] is
+// the pairs' weights to iw at qe + d/2 and sets the parents.  Ids: A[i] is
 // node aid0 + i, B[j] is node bid0 + j.
-template <typename IdT>
 __device__ __forceinline__ unsigned merge_pairs(const unsigned* A, int na, const unsigned* B, int nb, int d0, int d1,
-                                                int i, int aid0, int bid0, int qe, int rank0, unsigned* iw,
-                                                IdT* parent, int n) {
+                                                int i, int aid0, int bid0, int qe, unsigned* iw, uint16_t* parent,
+                                                int n) {
   unsigned leaves = 0;
   int j = d0 - i;
   for (int d = d0; d < d1; d += 2) {
@@ -625,10 +619,10 @@ __device__ __forceinline__ unsigned merge_pairs(const unsigned* A, int na, const
     i = i2 + (s ? 1 : 0);
     j = j2 + (s ? 0 : 1);
     leaves += (f ? 1u : 0u) + (s ? 1u : 0u);
-    const int k = (rank0 + d) >> 1;
+    const int k = d >> 1;
     iw[qe + k] = w;
-    parent[id0] = (IdT)(n + qe + k);
-    parent[id1] = (IdT)(n + qe + k);
+    parent[id0] = (uint16_t)(n + qe + k);
+    parent[id1] = (uint16_t)(n + qe + k);
   }
   return leaves;
 }
@@ -643,8 +637,7 @@ __device__ __forceinline__ unsigned two_smallest(const unsigned* lw, unsigned lp
 
 // Leaves by ascending weight (ties in symbol order) into (V.ka, V.sa), for
 // the weights max(1, f >> shift): the whole block.
-template <typename IdT>
-__device__ void codebook_sort(const CodebookArgs& a, const CbArrays<IdT>& V, int n, unsigned* scan_tmp, int shift) {
+__device__ void codebook_sort(const CodebookArgs& a, const CbArrays& V, int n, unsigned* scan_tmp, int shift) {
   __shared__ unsigned s_maxk;
   if (threadIdx.x == 0) s_maxk = 0;
   __syncthreads();
@@ -685,8 +678,12 @@ __device__ void codebook_sort(const CodebookArgs& a, const CbArrays<IdT>& V, int
   __syncthreads();
 }
 
+// The codebook over the compact arrays V (n present symbols, already in
+// V.csym): Huffman lengths into V.clen.  The lengths are those of the
+// sequential two-queue construction; lengths above kMaxLen are avoided by
+// re-running on max(1, f >> t), t = 1, 2, ...
 // At most kCbSmemSyms present symbols: every array in shared memory.
-__device__ void codebook_lengths(const CodebookArgs& a, CbArrays<uint16_t> V, int n, unsigned* scan_tmp) {
+__device__ void codebook_lengths(const CodebookArgs& a, CbArrays V, int n, unsigned* scan_tmp) {
   __shared__ unsigned s_p[2], s_leaves, s_maxd;
   if (n <= 1) {
     if (n == 1 && threadIdx.x == 0) V.clen[0] = 1;
@@ -736,8 +733,7 @@ __device__ void codebook_lengths(const CodebookArgs& a, CbArrays<uint16_t> V, in
           const int mid = (lo + hi) >> 1;
           if (A[mid] <= Bq[d0 - 1 - mid]) lo = mid + 1; else hi = mid;
         }
-        const unsigned leaves = merge_pairs<uint16_t>(A, pl, Bq, pq, d0, d1, lo, (int)lp, n + (int)qp, (int)qe, 0, V.iw,
-                                                      V.parent, n);
+        const unsigned leaves = merge_pairs(A, pl, Bq, pq, d0, d1, lo, (int)lp, n + (int)qp, (int)qe, V.iw, V.parent, n);
         if (d1 == T) s_leaves = (unsigned)lo + leaves;
       }
       if (threadIdx.x == 0) V.round_end[rounds] = (uint16_t)(qe + npairs);
@@ -785,7 +781,7 @@ __device__ void codebook_lengths(const CodebookArgs& a, CbArrays<uint16_t> V, in
 // staged per queue and every parent in global memory the tree of 65,468
 // symbols (100x500x500 at 1e-4) took 0.195 ms against 0.153; ranks found by
 // a binary search per node instead of the merge path took 0.211.
-__device__ void codebook_lengths_big(const CodebookArgs& a, CbArrays<unsigned> V, int n, CbBigSmem& S,
+__device__ void codebook_lengths_big(const CodebookArgs& a, CbArrays V, int n, CbBigSmem& S,
                                      int pre_passes) {
   __shared__ unsigned s_lp, s_qp, s_qe, s_pl, s_pq, s_rounds, s_maxd;
   __shared__ int s_split;
@@ -795,7 +791,7 @@ __device__ void codebook_lengths_big(const CodebookArgs& a, CbArrays<unsigned> V
   unsigned* const lsamp = S.samp;
   unsigned* const isamp = S.samp + kMaxDict / 64;
   unsigned* const tw = S.tile();  // a tile's weights: leaves, then internal nodes
-  uint16_t* const lpar = reinterpret_cast<uint16_t*>(V.parent);  // parents of the leaves
+  uint16_t* const lpar = V.parent;  // of the leaves
   for (int shift = 0;; ++shift) {
     if (shift == 0 && pre_passes > 0) {  // pairs sorted by cb_presort_kernel
       if (pre_passes & 1) {  // into (kb, sb)
@@ -1003,8 +999,7 @@ __device__ inline void codebook_decide(const CodebookArgs& a, unsigned smin, uns
 
 // Canonical codes, the lookup tables of the encoder, the codebook section of
 // the stream and the offsets of the sections after it, from the lengths.
-template <typename IdT>
-__device__ void codebook_emit(const CodebookArgs& a, CbArrays<IdT> V, int n, unsigned* scan_tmp, CanonTables* ct) {
+__device__ void codebook_emit(const CodebookArgs& a, CbArrays V, int n, unsigned* scan_tmp, CanonTables* ct) {
   __shared__ unsigned s_total, s_nruns;
   __shared__ unsigned long long s_bits;
   if (threadIdx.x == 0) s_bits = 0;
@@ -1181,7 +1176,7 @@ constexpr int kPreWarps = kPreThreads / 32, kPreRows = kPreSeg / kPreThreads;  /
 __global__ void __launch_bounds__(kPreThreads) cb_presort_kernel(CodebookArgs a) {
   cooperative_groups::grid_group grid = cooperative_groups::this_grid();
   CbPre* pre = cb_pre(a.big);
-  const CbArrays<unsigned> V = cb_big(a.big, nullptr);
+  const CbArrays V = cb_big(a.big, nullptr);
   const int dict = a.dict, c = blockIdx.x, G = gridDim.x;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   __shared__ unsigned s_red[kPreThreads / 32];
@@ -1340,7 +1335,7 @@ __global__ void __launch_bounds__(kPreThreads) cb_presort_kernel(CodebookArgs a)
 __global__ void __launch_bounds__(kPreThreads) cb_emit_kernel(CodebookArgs a) {
   cooperative_groups::grid_group grid = cooperative_groups::this_grid();
   CbPre* pre = cb_pre(a.big);
-  const CbArrays<unsigned> V = cb_big(a.big, nullptr);
+  const CbArrays V = cb_big(a.big, nullptr);
   const int n = (int)pre->n;
   if (n <= kCbSmemSyms) return;  // the one-CTA kernel emitted everything (the same for every CTA)
   const int c = blockIdx.x, G = gridDim.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -1558,9 +1553,9 @@ __device__ void codebook_block(const CodebookArgs& a) {
       const uint16_t* gsym = cb_big(a.big, S.wcnt).csym;
       for (int i = threadIdx.x; i < n; i += blockDim.x) S.csym[i] = gsym[i];
       __syncthreads();
-      const CbArrays<uint16_t> V = cb_small(S);
+      const CbArrays V = cb_small(S);
       codebook_lengths(a, V, n, S.scan_tmp);
-      codebook_emit<uint16_t>(a, V, n, S.scan_tmp, &S.ct);
+      codebook_emit(a, V, n, S.scan_tmp, &S.ct);
     } else {  // the tree here; cb_emit_kernel emits the codes on many CTAs afterwards
       CbBigSmem& L = *reinterpret_cast<CbBigSmem*>(smem_raw);
       codebook_lengths_big(a, cb_big(a.big, L.wcnt), n, L, passes);
@@ -1625,14 +1620,14 @@ __device__ void codebook_block(const CodebookArgs& a) {
   }
   __syncthreads();
   if (small) {
-    const CbArrays<uint16_t> V = cb_small(S);
+    const CbArrays V = cb_small(S);
     codebook_lengths(a, V, n, S.scan_tmp);
-    codebook_emit<uint16_t>(a, V, n, S.scan_tmp, &S.ct);
+    codebook_emit(a, V, n, S.scan_tmp, &S.ct);
   } else {
     CbBigSmem& L = *reinterpret_cast<CbBigSmem*>(smem_raw);
-    const CbArrays<unsigned> V = cb_big(a.big, L.wcnt);
+    const CbArrays V = cb_big(a.big, L.wcnt);
     codebook_lengths_big(a, V, n, L, -1);
-    codebook_emit<unsigned>(a, V, n, L.scan_tmp, &L.ct);
+    codebook_emit(a, V, n, L.scan_tmp, &L.ct);
   }
 }
 
@@ -2247,7 +2242,7 @@ __device__ __forceinline__ void encode_tiles(const FusedEncodeArgs& a) {
       if (lane == 0) atomicOr(&sc->status, ST_RAW);
       continue;
     }
-    unsigned* const gw = words + pw;
+    unsigned* const cw = words + pw;  // the chunk's words
     if (steps) {
       const uint4* p = reinterpret_cast<const uint4*>(a.sym + cb) + lane;
       uint4 qn = eight(p, cb + 8 * lane);
@@ -2308,11 +2303,11 @@ __device__ __forceinline__ void encode_tiles(const FusedEncodeArgs& a) {
         b0 += tot & 0xFFFFu;
         const unsigned nfull = (b0 >> 5) - w0;
 #pragma unroll 1
-        for (unsigned i = lane; i < nfull; i += 32) gw[w0 + i] = buf[i];
+        for (unsigned i = lane; i < nfull; i += 32) cw[w0 + i] = buf[i];
         carry = (b0 & 31u) ? buf[nfull] : 0u;
         __syncwarp();
       }
-      if (lane == 0 && (b0 & 31u)) gw[b0 >> 5] = carry;
+      if (lane == 0 && (b0 & 31u)) cw[b0 >> 5] = carry;
     } else {  // zero the chunk's words; words shared by lanes are ORed
       unsigned long long epos = pe + (xe - nesc);
       if (a.esc && nesc) {
@@ -2323,11 +2318,11 @@ __device__ __forceinline__ void encode_tiles(const FusedEncodeArgs& a) {
           }
       }
       if ((lane & 3) == 0 && lane) a.splits[c * (kSplits - 1) + (lane >> 2) - 1] = (uint16_t)(xb - bits);
-      for (unsigned w = lane; w < W; w += 32) gw[w] = 0u;
+      for (unsigned w = lane; w < W; w += 32) cw[w] = 0u;
       __syncwarp();
       const unsigned bit0 = xb - bits;
       unsigned off = bit0 & 31u, cur = 0;
-      unsigned* wp = gw + (bit0 >> 5);
+      unsigned* wp = cw + (bit0 >> 5);
       bool head = off != 0u;  // the first word holds other lanes' bits
       for (int t = 0; t < cnt; ++t) {
         const unsigned s = CLAMP ? min((unsigned)a.sym[s0 + t], dmax) : (unsigned)a.sym[s0 + t];
