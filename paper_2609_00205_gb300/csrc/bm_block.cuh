@@ -53,7 +53,8 @@
 // row of B elements, rounded out to 16-byte boundaries, into shared memory
 // that is dead at a block's start (the transposed and coarse arrays and the
 // symbol staging area), then compacts the rows; blocks on the field's far
-// faces keep the element-wise zero-filling cp.async.  0 (default) =
+// faces keep the element-wise zero-filling cp.async, and so do the coded double
+// kernels (bm_block_class.cuh).  0 (default) =
 // element-wise cp.async for every block: a warp's 32 consecutive elements of
 // a row go out as coalesced requests, and on GB300 (513^3 FP32, B = 17, K = 2)
 // the kernel took 0.477 ms against 0.531 ms with 1 (289 bulk requests of 80

@@ -8,7 +8,7 @@
 // quantiser's range check, floor and conversions are integer arithmetic
 // (bm_common.cuh).  Per 9^3 block 293 instead of 480 warp instructions of that
 // unit.  385x385x257, B = 9, K = 2: forward 1.55 -> 1.04 ms, inverse 1.48 ->
-// 1.20.  (Single precision keeps the general expression for every line: the
+// 1.22.  (Single precision keeps the general expression for every line: the
 // classes' lines, every other one of every other plane, share shared-memory
 // banks, and the same split took 0.494 against 0.446 ms forward and 0.701
 // against 0.558 inverse at 513^3, B = 17.)

