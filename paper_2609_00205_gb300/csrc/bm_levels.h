@@ -18,8 +18,8 @@ cudaError_t level_lines(const GLevel<T>& L, const T* in, T* out, const T* U, con
 // the scans' segments and shared memory, or so many and so short that the
 // scans' work costs more than the sweeps.  The scans are bound by issue: a line
 // takes about 450 + 350 E cycles of an SM in double precision (whose unit runs
-// two lanes a clock) and 100 + 40 E in single, beside a launch's chain of about
-// 7,600; the sweeps by latency, about 1,350 cycles per coarse node along
+// two lanes a clock) and 100 + 40 E in single, beside a line's chain of about
+// 6,000 and 2,500; the sweeps by latency, about 1,350 cycles per coarse node along
 // dimensions 0 and 1 and 2,500 along dimension 2, where a thread's neighbours
 // are a line apart, and by 8 per line and coarse node.  Global levels of a
 // transposed decomposition with the scans (but for long lines) / the sweeps /
@@ -33,7 +33,8 @@ bool expand_serial(const GLevel<T>& L, int dim, int nsm) {
   if (E == 0) return true;
   const LineShape S = line_shape(L, dim);
   const int64_t lines = S.nb * S.ncol, c = L.d[dim].c, line = sizeof(T) == 8 ? 450 + 350 * E : 100 + 40 * E;
-  return 7600 + lines * line / nsm > c * (dim == 2 ? 2500 : 1350) + lines * c * 8 / nsm;
+  const int64_t chain = sizeof(T) == 8 ? 6000 : 2500;
+  return chain + lines * line / nsm > c * (dim == 2 ? 2500 : 1350) + lines * c * 8 / nsm;
 }
 
 // Expansion (M_f I M_c^-1) along dimension DIM, FIN as in expand_emit.  buf:

@@ -95,7 +95,7 @@ def test_loss_gradient_central_differences(bm):
 # ones, along each dimension, with a few lines (tiles of 8 or 4) and with many
 # (32 or 16).
 LINES = [(300, 20, 19), (19, 1000, 20), (20, 18, 3000), (4100, 18, 19), (18, 4100, 19), (18, 19, 4100),
-         (330, 340, 40), (3000, 40, 70)]
+         (330, 340, 40), (3000, 40, 70), (340, 18, 850)]
 
 
 @pytest.mark.parametrize("shape", LINES)
